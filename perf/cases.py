@@ -202,9 +202,8 @@ def exact(case, seed):
     """Plain torch in 64 bits, head by head over ranges of points; None where that takes long."""
     c = case
     train = c["kind"] == "train"
-    # Products and one exponential per triple, twice forward and twice backward, at the
-    # card's 64-bit rates.
-    if _pairs(c) * c["d"] * (3 if train else 1) > 1 << 38:
+    # At the card's 64-bit rates the largest listed cases take 12 to 18 seconds.
+    if _pairs(c) * c["d"] > 1 << 38:
         return None
     v = _inputs(c, seed)
     B, N, H, d, G = c["B"], c["N"], c["H"], c["d"], c["G"]
