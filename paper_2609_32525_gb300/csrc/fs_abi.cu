@@ -1,6 +1,6 @@
 // C ABI of the library: host-side validation, workspace layout, kernel dispatch.
 // Declarations and the contract of every entry point: include/flashslice.h.
-#include "fs_internal.h"
+#include "fs_simt_tiles.h"
 #include "fs_tc.h"
 
 #include <algorithm>
@@ -17,15 +17,26 @@ int num_sms() {
   return n;
 }
 
+// The tiled SIMT passes keep two blocks per SM resident (d = 64: one).  A block's time is
+// its point tiles plus about half a tile (its slot tile, its partial rows), so P minimises
+// waves * (tiles per split + 1/2); the smallest such P within 1%.  P stays below two
+// splits per SM and 128-slot block, which bounds the partials' workspace.
 int slot_splits(const Shape& s) {
-  const int64_t gblocks = (s.G + 127) / 128;
-  const int64_t units = s.BH() * gblocks;
-  int64_t P = (2LL * num_sms() + units - 1) / units;
-  const int64_t max_by_n = (s.N + 63) / 64;
-  if (P > max_by_n) P = max_by_n;
-  if (P < 1) P = 1;
-  if (P > 1024) P = 1024;
-  return (int)P;
+  const int64_t tg = simt_tile_slots(s);
+  const int64_t units = s.BH() * ((s.G + tg - 1) / tg), blocks = s.BH() * ((s.G + 127) / 128);
+  const int64_t cap = (int64_t)num_sms() * (s.d == 64 ? 1 : 2);
+  const int64_t tiles = (s.N + kSimtTP - 1) / kSimtTP;
+  const int64_t max_p = std::min<int64_t>({tiles, (2LL * num_sms() + blocks - 1) / blocks, 1024});
+  int64_t best = 1;
+  double best_t = 1e300;
+  for (int64_t p = 1; p <= max_p; p++) {
+    const double t = (double)((units * p + cap - 1) / cap) * ((double)((tiles + p - 1) / p) + 0.5);
+    if (t < 0.99 * best_t) {
+      best_t = t;
+      best = p;
+    }
+  }
+  return (int)best;
 }
 
 namespace {

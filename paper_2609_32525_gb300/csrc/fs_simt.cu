@@ -1,226 +1,14 @@
-// SIMT fp32 kernels: every step of the coupling with fp32 FMA products and fp32
-// accumulation (the paper's "ieee" dot level, Appendix G.2).  They serve every
-// shape the tensor-core kernels do not cover (d != 32, G above their limits, small
-// fp32 problems, the backward of fp32 inputs), and the small steps every path
-// shares: the fixed-order reductions, the mixes and their backward.
-//
-// Ownership follows the paper's G-blocked family (Appendix G.1): a statistics
-// pass per point; slot-owned split-N partial numerators and weight sums with a
-// fixed-order reduction afterwards; point-owned deslice; backward as
-// point-owned (input gradients, two sweeps over slots) plus slot-owned
-// (parameter and token gradients) kernels.  No float atomics anywhere.
-//
-// Logits are formed as a2 = x . (W * log2e/tau) + beta * log2e/tau, i.e. the
-// temperature-scaled logit in base-2 units, so that w = exp2(a2 - lse*log2e).
-#include "fs_internal.h"
+// SIMT path: dispatch of the tiled fp32 passes (fs_simt_tiles.cuh), which serve every shape
+// the tensor-core kernels do not cover (d != 32, G above their limits, small fp32
+// problems, the backward of fp32 inputs), and the small fp32 kernels that every path
+// shares: the fixed-order reductions, the mixes and their backward.  No float atomics
+// anywhere.
+#include "fs_simt_tiles.h"
 
 #include <cuda_bf16.h>
-#include <math_constants.h>
 
 namespace fs {
 namespace {
-
-constexpr int kThreads = 128;
-
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
-// Row of D contiguous elements -> floats (16-byte vector loads).
-template <int D>
-__device__ __forceinline__ void load_row(const float* p, float (&v)[D]) {
-  const float4* q = reinterpret_cast<const float4*>(p);
-#pragma unroll
-  for (int i = 0; i < D / 4; i++) {
-    float4 t = q[i];
-    v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
-  }
-}
-template <int D>
-__device__ __forceinline__ void load_row(const __nv_bfloat16* p, float (&v)[D]) {
-  const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-  for (int i = 0; i < D / 8; i++) {
-    uint4 t = q[i];
-    const uint32_t w[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      v[8 * i + 2 * j] = __uint_as_float(w[j] << 16);
-      v[8 * i + 2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
-    }
-  }
-}
-template <int D>
-__device__ __forceinline__ void store_row(float* p, const float (&v)[D]) {
-  float4* q = reinterpret_cast<float4*>(p);
-#pragma unroll
-  for (int i = 0; i < D / 4; i++) q[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-}
-template <int D>
-__device__ __forceinline__ void store_row(__nv_bfloat16* p, const float (&v)[D]) {
-  uint4* q = reinterpret_cast<uint4*>(p);
-#pragma unroll
-  for (int i = 0; i < D / 8; i++) {
-    uint32_t w[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      __nv_bfloat162 t = __floats2bfloat162_rn(v[8 * i + 2 * j], v[8 * i + 2 * j + 1]);
-      w[j] = *reinterpret_cast<uint32_t*>(&t);
-    }
-    q[i] = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-
-__device__ __forceinline__ void set_status(uint32_t* status, uint32_t code) {
-  if (status) atomicCAS(status, 0u, code);
-}
-
-// tau must be positive and finite; returns false (and flags the status word) otherwise.
-__device__ __forceinline__ bool tau_ok(float t, uint32_t* status) {
-  if (t > 0.f && t < CUDART_INF_F) return true;
-  if (threadIdx.x == 0) set_status(status, kDevBadTau);
-  return false;
-}
-
-__device__ __forceinline__ int64_t row_index(int64_t b, int64_t n, int h, int64_t N, int H) {
-  return (b * N + n) * H + h;
-}
-
-// Stage GC slots of W[h] (scaled by `scale`) as sW[g][k] plus the scaled bias.  The
-// rows are unpadded (16-byte aligned), so that the compute loops, in which every lane
-// reads the same row, take them four floats at a time; the staging stores are then
-// bank-conflicted, which costs little against the compute on each chunk.
-template <int D, int GC>
-__device__ __forceinline__ void stage_w(float (*sW)[D], float* sB, const float* W,
-                                        const float* bias, int h, int G, int g0, float scale) {
-  for (int i = threadIdx.x; i < GC * D; i += kThreads) {
-    const int g = i % GC, k = i / GC;
-    sW[g][k] = (g0 + g < G) ? W[((int64_t)h * D + k) * G + g0 + g] * scale : 0.f;
-  }
-  for (int i = threadIdx.x; i < GC; i += kThreads)
-    sB[i] = (g0 + i < G) ? bias[(int64_t)h * G + g0 + i] * scale : 0.f;
-}
-
-// ---- statistics: lse per (point, head) ------------------------------------------
-template <int D, typename T>
-__global__ void __launch_bounds__(kThreads) k_stats(const T* __restrict__ x, const float* __restrict__ W,
-                                                     const float* __restrict__ bias,
-                                                     const float* __restrict__ tau, float* __restrict__ lse,
-                                                     int64_t N, int H, int G, uint32_t* status) {
-  constexpr int GC = 32;
-  __shared__ __align__(16) float sW[GC][D];
-  __shared__ float sB[GC];
-  const int64_t bh = blockIdx.y;
-  const int64_t b = bh / H;
-  const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
-  const float scale = kLog2e / tau[h];
-  const int64_t n = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  const bool valid = n < N;
-  float xr[D];
-  if (valid) load_row<D>(x + row_index(b, n, h, N, H) * D, xr);
-  else {
-#pragma unroll
-    for (int k = 0; k < D; k++) xr[k] = 0.f;
-  }
-  float m = -CUDART_INF_F, l = 0.f;
-  for (int g0 = 0; g0 < G; g0 += GC) {
-    __syncthreads();
-    stage_w<D, GC>(sW, sB, W, bias, h, G, g0, scale);
-    __syncthreads();
-    const int gn = min(GC, G - g0);
-    float a[GC];
-    float cm = -CUDART_INF_F;
-#pragma unroll
-    for (int g = 0; g < GC; g++) {
-      float s = sB[g];
-#pragma unroll
-      for (int k = 0; k < D; k++) s = fmaf(xr[k], sW[g][k], s);
-      a[g] = (g < gn) ? s : -CUDART_INF_F;
-      cm = fmaxf(cm, a[g]);
-    }
-    const float mn = fmaxf(m, cm);
-    float acc = 0.f;
-#pragma unroll
-    for (int g = 0; g < GC; g++) acc += exp2f(a[g] - mn);
-    l = l * exp2f(m - mn) + acc;
-    m = mn;
-  }
-  if (valid) lse[bh * N + n] = (m + log2f(l)) * kLn2;
-}
-
-// ---- slice: slot-owned split-N partials ------------------------------------------
-// grid (ceil(G/128), B*H, P); thread = slot.  part[p][bh][g][0..D] = (U, S).
-template <int D, typename T>
-__global__ void __launch_bounds__(kThreads) k_slice_partial(
-    const T* __restrict__ x, const T* __restrict__ f, const float* __restrict__ W,
-    const float* __restrict__ bias, const float* __restrict__ tau, const float* __restrict__ lse,
-    float* __restrict__ part, int64_t B, int64_t N, int H, int G, int64_t per_split, uint32_t* status) {
-  constexpr int PT = 32;
-  __shared__ __align__(16) float sx[PT][D];
-  __shared__ float sf[PT][D];
-  __shared__ float sl[PT];
-  const int g = blockIdx.x * kThreads + threadIdx.x;
-  const int64_t bh = blockIdx.y;
-  const int64_t b = bh / H;
-  const int h = (int)(bh % H);
-  const int p = blockIdx.z;
-  if (!tau_ok(tau[h], status)) return;
-  const float scale = kLog2e / tau[h];
-  float wc[D], U[D];
-  float bb = 0.f, S = 0.f;
-#pragma unroll
-  for (int k = 0; k < D; k++) {
-    wc[k] = (g < G) ? W[((int64_t)h * D + k) * G + g] * scale : 0.f;
-    U[k] = 0.f;
-  }
-  if (g < G) bb = bias[(int64_t)h * G + g] * scale;
-  const int64_t n_begin = (int64_t)p * per_split;
-  const int64_t n_end = min(N, n_begin + per_split);
-  for (int64_t n0 = n_begin; n0 < n_end; n0 += PT) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < PT * D; i += kThreads) {
-      const int j = i / D, k = i % D;
-      const int64_t n = n0 + j;
-      float xv = 0.f, fv = 0.f;
-      if (n < n_end) {
-        const int64_t idx = row_index(b, n, h, N, H) * D + k;
-        xv = to_f(x[idx]);
-        fv = to_f(f[idx]);
-      }
-      sx[j][k] = xv;
-      sf[j][k] = fv;
-    }
-    for (int i = threadIdx.x; i < PT; i += kThreads) {
-      const int64_t n = n0 + i;
-      sl[i] = (n < n_end) ? lse[bh * N + n] * kLog2e : CUDART_INF_F;
-    }
-    __syncthreads();
-    // Four points at a time: their logits are independent chains; the sums take
-    // the points in order.
-#pragma unroll 1
-    for (int j = 0; j < PT; j += 4) {
-      float a[4] = {bb, bb, bb, bb};
-#pragma unroll
-      for (int k = 0; k < D; k++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) a[q] = fmaf(sx[j + q][k], wc[k], a[q]);
-      float w[4];
-#pragma unroll
-      for (int q = 0; q < 4; q++) w[q] = exp2f(a[q] - sl[j + q]);
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        S += w[q];
-#pragma unroll
-        for (int k = 0; k < D; k++) U[k] = fmaf(w[q], sf[j + q][k], U[k]);
-      }
-    }
-  }
-  if (g < G) {
-    float* o = part + (((int64_t)p * B * H + bh) * G + g) * (D + 1);
-#pragma unroll
-    for (int k = 0; k < D; k++) o[k] = U[k];
-    o[D] = S;
-  }
-}
 
 // Fixed-order sum of the P partials [P, BHG, D+1], then (optionally) the
 // normalisation.  The sum over splits runs in split order.  Partials hold Gs >= G
@@ -505,533 +293,6 @@ __global__ void __launch_bounds__(256) k_mix_bwd_dM(const float* __restrict__ z,
   }
 }
 
-// ---- deslice: point-owned ----------------------------------------------------------
-template <int D, typename T>
-__global__ void __launch_bounds__(kThreads) k_deslice(const T* __restrict__ x, const float* __restrict__ W,
-                                                       const float* __restrict__ bias,
-                                                       const float* __restrict__ tau,
-                                                       const float* __restrict__ zp,
-                                                       const float* __restrict__ lse, T* __restrict__ out,
-                                                       int64_t N, int H, int G, uint32_t* status) {
-  constexpr int GC = 32;
-  __shared__ __align__(16) float sW[GC][D];
-  __shared__ __align__(16) float sZ[GC][D];
-  __shared__ float sB[GC];
-  const int64_t bh = blockIdx.y;
-  const int64_t b = bh / H;
-  const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
-  const float scale = kLog2e / tau[h];
-  const int64_t n = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  const bool valid = n < N;
-  float xr[D], acc[D];
-#pragma unroll
-  for (int k = 0; k < D; k++) { xr[k] = 0.f; acc[k] = 0.f; }
-  float l2 = CUDART_INF_F;
-  if (valid) {
-    load_row<D>(x + row_index(b, n, h, N, H) * D, xr);
-    l2 = lse[bh * N + n] * kLog2e;
-  }
-  const float* zb = zp + bh * G * D;
-  for (int g0 = 0; g0 < G; g0 += GC) {
-    __syncthreads();
-    stage_w<D, GC>(sW, sB, W, bias, h, G, g0, scale);
-    for (int i = threadIdx.x; i < GC * D; i += kThreads) {
-      const int g = i / D, k = i % D;
-      sZ[g][k] = (g0 + g < G) ? zb[(int64_t)(g0 + g) * D + k] : 0.f;
-    }
-    __syncthreads();
-    const int gn = min(GC, G - g0);
-    // Four slots at a time (independent logit chains); the output sums the slots in
-    // order.  Slots past gn have zero z' rows and add exact zeros.
-#pragma unroll 1
-    for (int g = 0; g < gn; g += 4) {
-      float a[4];
-#pragma unroll
-      for (int q = 0; q < 4; q++) a[q] = sB[g + q];
-#pragma unroll
-      for (int k = 0; k < D; k++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) a[q] = fmaf(xr[k], sW[g + q][k], a[q]);
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        if (g + q >= gn) break;
-        const float w = exp2f(a[q] - l2);
-#pragma unroll
-        for (int k = 0; k < D; k++) acc[k] = fmaf(w, sZ[g + q][k], acc[k]);
-      }
-    }
-  }
-  if (valid) store_row<D>(out + row_index(b, n, h, N, H) * D, acc);
-}
-
-// ---- backward, point-owned -------------------------------------------------------------
-// Gradient w.r.t. the weights of point n at slot g:
-//   MODE 0 (deslice): dw_g = dO . z'_g
-//   MODE 1 (slice)  : dw_g = f . dU_g + dS_g      (dUS[bh][g] = (dU_g, dS_g))
-// Sweep 1 forms delta = sum_g w_g dw_g (and, for the slice, dfx = sum_g w_g dU_g);
-// sweep 2 forms dx = (1/tau) sum_g w_g (dw_g - delta) W[:,g].
-template <int D, typename T, int MODE>
-__global__ void __launch_bounds__(kThreads) k_bwd_point(
-    const T* __restrict__ x, const T* __restrict__ v /* dout (MODE 0) or fx (MODE 1) */,
-    const float* __restrict__ W, const float* __restrict__ bias, const float* __restrict__ tau,
-    const float* __restrict__ tok /* z' (MODE 0) or (dU,dS) (MODE 1) */, const float* __restrict__ lse,
-    T* __restrict__ dx, T* __restrict__ dfx, float* __restrict__ delta, float* __restrict__ dt_part,
-    int accumulate, int64_t N, int H, int G, uint32_t* status) {
-  constexpr int GC = 16;
-  __shared__ float s_dt[kThreads];
-  constexpr int TS = (MODE == 0) ? D : D + 1;  // token row stride in memory
-  __shared__ __align__(16) float sW[GC][D];
-  __shared__ __align__(16) float sT[GC][D];  // t_g (z' or dU)
-  __shared__ float sS[GC];                    // MODE 1: dS_g
-  __shared__ float sB[GC];
-  const int64_t bh = blockIdx.y;
-  const int64_t b = bh / H;
-  const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
-  const float scale = kLog2e / tau[h];
-  const int64_t n = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  const bool valid = n < N;
-  float xr[D], vr[D], acc[D];
-#pragma unroll
-  for (int k = 0; k < D; k++) { xr[k] = 0.f; vr[k] = 0.f; acc[k] = 0.f; }
-  float l2 = CUDART_INF_F;
-  const int64_t row = row_index(b, n, h, N, H);
-  if (valid) {
-    load_row<D>(x + row * D, xr);
-    load_row<D>(v + row * D, vr);
-    l2 = lse[bh * N + n] * kLog2e;
-  }
-  const float* tb = tok + bh * G * TS;
-  float dl = 0.f;
-  // The point's term of the temperature gradient, sum_g da_g (a_g - lse) in base-2
-  // units: with the logits centred on lse (exact, since sum_g da_g = 0) the row
-  // sum carries no large cancelling parts (App. G.2).
-  float dtn = 0.f;
-  for (int sweep = 0; sweep < 2; sweep++) {
-    for (int g0 = 0; g0 < G; g0 += GC) {
-      __syncthreads();
-      stage_w<D, GC>(sW, sB, W, bias, h, G, g0, scale);
-      for (int i = threadIdx.x; i < GC * TS; i += kThreads) {
-        const int g = i / TS, k = i % TS;
-        const float t = (g0 + g < G) ? tb[(int64_t)(g0 + g) * TS + k] : 0.f;
-        if (k < D)
-          sT[g][k] = t;
-        else
-          sS[g] = t;
-      }
-      __syncthreads();
-      const int gn = min(GC, G - g0);
-      // Four slots at a time: their logit and dw dot products are independent chains
-      // (one 32-long chain per slot would leave the FMA pipe waiting on each result).
-      // The per-slot updates below run in slot order, as one slot at a time would.
-#pragma unroll 1
-      for (int g = 0; g < gn; g += 4) {
-        float a[4], dwq[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          a[q] = sB[g + q];
-          dwq[q] = (MODE == 0) ? 0.f : sS[g + q];
-        }
-#pragma unroll
-        for (int k = 0; k < D; k++)
-#pragma unroll
-          for (int q = 0; q < 4; q++) {
-            a[q] = fmaf(xr[k], sW[g + q][k], a[q]);
-            dwq[q] = fmaf(vr[k], sT[g + q][k], dwq[q]);
-          }
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          if (g + q >= gn) break;
-          const float w = exp2f(a[q] - l2);
-          const float dw = dwq[q];
-          if (sweep == 0) {
-            dl = fmaf(w, dw, dl);
-            if (MODE == 1) {
-#pragma unroll
-              for (int k = 0; k < D; k++) acc[k] = fmaf(w, sT[g + q][k], acc[k]);
-            }
-          } else {
-            const float da = w * (dw - dl);
-#pragma unroll
-            for (int k = 0; k < D; k++) acc[k] = fmaf(da, sW[g + q][k], acc[k]);
-            if (valid) dtn = fmaf(da, a[q] - l2, dtn);
-          }
-        }
-      }
-    }
-    if (sweep == 0) {
-      if (MODE == 1 && valid) store_row<D>(dfx + row * D, acc);
-#pragma unroll
-      for (int k = 0; k < D; k++) acc[k] = 0.f;
-    }
-  }
-  // Block sum of the temperature terms (fixed tree order) -> dt_part[bh][block].
-  s_dt[threadIdx.x] = dtn;
-  __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) s_dt[threadIdx.x] += s_dt[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) dt_part[bh * gridDim.x + blockIdx.x] = s_dt[0] * kLn2;
-  if (!valid) return;
-  delta[bh * N + n] = dl;
-  // acc = sum_g da_g W[:,g] * log2e/tau ; dx = sum_g da_g W[:,g] / tau = acc * ln2.
-#pragma unroll
-  for (int k = 0; k < D; k++) acc[k] *= kLn2;
-  if (accumulate) {
-    float old[D];
-    load_row<D>(dx + row * D, old);
-#pragma unroll
-    for (int k = 0; k < D; k++) acc[k] += old[k];
-  }
-  store_row<D>(dx + row * D, acc);
-}
-
-// ---- backward, slot-owned ---------------------------------------------------------------
-// grid (ceil(G/128), B*H, P); thread = slot g.  For every point n of the split:
-//   da = w (dw - delta_n);  dWa += da x_n;  dba += da;  dta += da * a_n
-//   MODE 0 also accumulates dz'_g += w dO_n.
-// part[p][bh][g][...] = (MODE 0: dz'(D)) , dWa(D), dba, dta   (un-scaled by 1/tau)
-template <int D, typename T, int MODE>
-__global__ void __launch_bounds__(kThreads) k_bwd_slot(
-    const T* __restrict__ x, const T* __restrict__ v, const float* __restrict__ W,
-    const float* __restrict__ bias, const float* __restrict__ tau, const float* __restrict__ tok,
-    const float* __restrict__ lse, const float* __restrict__ delta, float* __restrict__ part, int64_t B,
-    int64_t N, int H, int G, int64_t per_split, uint32_t* status) {
-  constexpr int PT = 32;
-  constexpr int TS = (MODE == 0) ? D : D + 1;
-  constexpr int PS = (MODE == 0) ? 2 * D + 2 : D + 2;
-  __shared__ __align__(16) float sx[PT][D];
-  __shared__ __align__(16) float sv[PT][D];
-  __shared__ float sl[PT];
-  __shared__ float sd[PT];
-  const int g = blockIdx.x * kThreads + threadIdx.x;
-  const int64_t bh = blockIdx.y;
-  const int64_t b = bh / H;
-  const int h = (int)(bh % H);
-  const int p = blockIdx.z;
-  if (!tau_ok(tau[h], status)) return;
-  const float scale = kLog2e / tau[h];
-  float wc[D], tg[D], dzp[D], dWa[D];
-  float bb = 0.f, dSg = 0.f, dba = 0.f;
-#pragma unroll
-  for (int k = 0; k < D; k++) {
-    wc[k] = (g < G) ? W[((int64_t)h * D + k) * G + g] * scale : 0.f;
-    tg[k] = (g < G) ? tok[(bh * G + g) * TS + k] : 0.f;
-    dzp[k] = 0.f;
-    dWa[k] = 0.f;
-  }
-  if (g < G) {
-    bb = bias[(int64_t)h * G + g] * scale;
-    if (MODE == 1) dSg = tok[(bh * G + g) * TS + D];
-  }
-  const int64_t n_begin = (int64_t)p * per_split;
-  const int64_t n_end = min(N, n_begin + per_split);
-  for (int64_t n0 = n_begin; n0 < n_end; n0 += PT) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < PT * D; i += kThreads) {
-      const int j = i / D, k = i % D;
-      const int64_t n = n0 + j;
-      float xv = 0.f, vv = 0.f;
-      if (n < n_end) {
-        const int64_t idx = row_index(b, n, h, N, H) * D + k;
-        xv = to_f(x[idx]);
-        vv = to_f(v[idx]);
-      }
-      sx[j][k] = xv;
-      sv[j][k] = vv;
-    }
-    for (int i = threadIdx.x; i < PT; i += kThreads) {
-      const int64_t n = n0 + i;
-      const bool ok = n < n_end;
-      sl[i] = ok ? lse[bh * N + n] * kLog2e : CUDART_INF_F;
-      sd[i] = ok ? delta[bh * N + n] : 0.f;
-    }
-    __syncthreads();
-    // Four points at a time: independent logit and dw chains; the updates below run
-    // in point order, as one point at a time would.
-#pragma unroll 1
-    for (int j = 0; j < PT; j += 4) {
-      float a[4], dwq[4];
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        a[q] = bb;
-        dwq[q] = dSg;
-      }
-#pragma unroll
-      for (int k = 0; k < D; k++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          a[q] = fmaf(sx[j + q][k], wc[k], a[q]);
-          dwq[q] = fmaf(sv[j + q][k], tg[k], dwq[q]);
-        }
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const float w = exp2f(a[q] - sl[j + q]);
-        const float da = w * (dwq[q] - sd[j + q]);
-        if (MODE == 0) {
-#pragma unroll
-          for (int k = 0; k < D; k++) dzp[k] = fmaf(w, sv[j + q][k], dzp[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < D; k++) dWa[k] = fmaf(da, sx[j + q][k], dWa[k]);
-        dba += da;
-      }
-    }
-  }
-  if (g < G) {
-    float* o = part + (((int64_t)p * B * H + bh) * G + g) * PS;
-    int off = 0;
-    if (MODE == 0) {
-#pragma unroll
-      for (int k = 0; k < D; k++) o[k] = dzp[k];
-      off = D;
-    }
-#pragma unroll
-    for (int k = 0; k < D; k++) o[off + k] = dWa[k];
-    o[off + D] = dba;
-    o[off + D + 1] = 0.f;  // (the temperature gradient is formed per point, see k_bwd_point)
-  }
-}
-
-// ---- the coupling's whole backward, fused -------------------------------------------------
-// The deslice's and the slice's weight gradients share the weights, so their softmax
-// backward adds up: da = w (dw - delta) with dw_g = dO . z'_g + fx . dU_g + dS_g and
-// delta = sum_g w_g dw_g.  One point pass and one slot pass then serve both (the
-// separate calls make two of each).
-// Point pass: sweep 1 forms delta and dfx = sum_g w_g dU_g, sweep 2 dx = (1/tau) sum_g
-// da_g W[:,g] (added to dx when accumulate) and the points' temperature terms.
-template <int D, typename T>
-__global__ void __launch_bounds__(kThreads) k_bwd_point_comb(
-    const T* __restrict__ x, const T* __restrict__ dO, const T* __restrict__ fx, const float* __restrict__ W,
-    const float* __restrict__ bias, const float* __restrict__ tau, const float* __restrict__ zp,
-    const float* __restrict__ dUS, const float* __restrict__ lse, T* __restrict__ dx, T* __restrict__ dfx,
-    float* __restrict__ delta, float* __restrict__ dt_part, int accumulate, int64_t N, int H, int G,
-    uint32_t* status) {
-  constexpr int GC = 16;
-  __shared__ float s_dt[kThreads];
-  __shared__ __align__(16) float sW[GC][D];
-  __shared__ __align__(16) float sZ[GC][D];  // z'_g
-  __shared__ __align__(16) float sU[GC][D];  // dU_g
-  __shared__ float sS[GC];                    // dS_g
-  __shared__ float sB[GC];
-  const int64_t bh = blockIdx.y;
-  const int64_t b = bh / H;
-  const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
-  const float scale = kLog2e / tau[h];
-  const int64_t n = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  const bool valid = n < N;
-  float xr[D], dr[D], fr[D], acc[D];
-#pragma unroll
-  for (int k = 0; k < D; k++) { xr[k] = 0.f; dr[k] = 0.f; fr[k] = 0.f; acc[k] = 0.f; }
-  float l2 = CUDART_INF_F;
-  const int64_t row = row_index(b, n, h, N, H);
-  if (valid) {
-    load_row<D>(x + row * D, xr);
-    load_row<D>(dO + row * D, dr);
-    load_row<D>(fx + row * D, fr);
-    l2 = lse[bh * N + n] * kLog2e;
-  }
-  const float* zb = zp + bh * G * D;
-  const float* ub = dUS + bh * G * (D + 1);
-  auto stage = [&](int g0) {
-    __syncthreads();
-    stage_w<D, GC>(sW, sB, W, bias, h, G, g0, scale);
-    for (int i = threadIdx.x; i < GC * D; i += kThreads) {
-      const int g = i / D, k = i % D;
-      sZ[g][k] = (g0 + g < G) ? zb[(int64_t)(g0 + g) * D + k] : 0.f;
-    }
-    for (int i = threadIdx.x; i < GC * (D + 1); i += kThreads) {
-      const int g = i / (D + 1), k = i % (D + 1);
-      const float t = (g0 + g < G) ? ub[(int64_t)(g0 + g) * (D + 1) + k] : 0.f;
-      if (k < D)
-        sU[g][k] = t;
-      else
-        sS[g] = t;
-    }
-    __syncthreads();
-  };
-  // Logits and dw of kQ slots at a time (independent chains; the point's x, dO, fx and
-  // accumulator rows already hold 128 registers, so two rather than four).
-  constexpr int kQ = 2;
-  auto chains = [&](int g, float (&a)[kQ], float (&dwq)[kQ]) {
-#pragma unroll
-    for (int q = 0; q < kQ; q++) {
-      a[q] = sB[g + q];
-      dwq[q] = sS[g + q];
-    }
-#pragma unroll
-    for (int k = 0; k < D; k++)
-#pragma unroll
-      for (int q = 0; q < kQ; q++) {
-        a[q] = fmaf(xr[k], sW[g + q][k], a[q]);
-        dwq[q] = fmaf(dr[k], sZ[g + q][k], dwq[q]);
-        dwq[q] = fmaf(fr[k], sU[g + q][k], dwq[q]);
-      }
-  };
-  // Sweep 1: delta and dfx (updates in slot order).
-  float dl = 0.f;
-  for (int g0 = 0; g0 < G; g0 += GC) {
-    stage(g0);
-    const int gn = min(GC, G - g0);
-#pragma unroll 1
-    for (int g = 0; g < gn; g += kQ) {
-      float a[kQ], dwq[kQ];
-      chains(g, a, dwq);
-#pragma unroll
-      for (int q = 0; q < kQ; q++) {
-        if (g + q < gn) {
-          const float w = exp2f(a[q] - l2);
-          dl = fmaf(w, dwq[q], dl);
-#pragma unroll
-          for (int k = 0; k < D; k++) acc[k] = fmaf(w, sU[g + q][k], acc[k]);
-        }
-      }
-    }
-  }
-  if (valid) store_row<D>(dfx + row * D, acc);
-#pragma unroll
-  for (int k = 0; k < D; k++) acc[k] = 0.f;
-  // Sweep 2: dx and the temperature terms.
-  float dtn = 0.f;
-  for (int g0 = 0; g0 < G; g0 += GC) {
-    stage(g0);
-    const int gn = min(GC, G - g0);
-#pragma unroll 1
-    for (int g = 0; g < gn; g += kQ) {
-      float a[kQ], dwq[kQ];
-      chains(g, a, dwq);
-#pragma unroll
-      for (int q = 0; q < kQ; q++) {
-        if (g + q < gn) {
-          const float da = exp2f(a[q] - l2) * (dwq[q] - dl);
-#pragma unroll
-          for (int k = 0; k < D; k++) acc[k] = fmaf(da, sW[g + q][k], acc[k]);
-          if (valid) dtn = fmaf(da, a[q] - l2, dtn);
-        }
-      }
-    }
-  }
-  // Block sum of the temperature terms (fixed tree order) -> dt_part[bh][block].
-  s_dt[threadIdx.x] = dtn;
-  __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) s_dt[threadIdx.x] += s_dt[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) dt_part[bh * gridDim.x + blockIdx.x] = s_dt[0] * kLn2;
-  if (!valid) return;
-  delta[bh * N + n] = dl;
-#pragma unroll
-  for (int k = 0; k < D; k++) acc[k] *= kLn2;
-  if (accumulate) {
-    float old[D];
-    load_row<D>(dx + row * D, old);
-#pragma unroll
-    for (int k = 0; k < D; k++) acc[k] += old[k];
-  }
-  store_row<D>(dx + row * D, acc);
-}
-
-// Slot pass of the fused backward: thread = slot g; for every point n of the split,
-// da = w (dw - delta_n) with dw as above; dWa += da x_n; dba += da.
-// part[p][bh][g] = (dWa (D), dba, 0), un-scaled by 1/tau.
-template <int D, typename T>
-__global__ void __launch_bounds__(kThreads) k_bwd_slot_comb(
-    const T* __restrict__ x, const T* __restrict__ dO, const T* __restrict__ fx, const float* __restrict__ W,
-    const float* __restrict__ bias, const float* __restrict__ tau, const float* __restrict__ zp,
-    const float* __restrict__ dUS, const float* __restrict__ lse, const float* __restrict__ delta,
-    float* __restrict__ part, int64_t B, int64_t N, int H, int G, int64_t per_split, uint32_t* status) {
-  constexpr int PT = 32;
-  constexpr int PS = D + 2;
-  __shared__ __align__(16) float sx[PT][D];
-  __shared__ __align__(16) float sd[PT][D];  // dO
-  __shared__ __align__(16) float sf[PT][D];  // fx
-  __shared__ float sl[PT];
-  __shared__ float sdl[PT];
-  const int g = blockIdx.x * kThreads + threadIdx.x;
-  const int64_t bh = blockIdx.y;
-  const int64_t b = bh / H;
-  const int h = (int)(bh % H);
-  const int p = blockIdx.z;
-  if (!tau_ok(tau[h], status)) return;
-  const float scale = kLog2e / tau[h];
-  float wc[D], zg[D], ug[D], dWa[D];
-  float bb = 0.f, dSg = 0.f, dba = 0.f;
-#pragma unroll
-  for (int k = 0; k < D; k++) {
-    wc[k] = (g < G) ? W[((int64_t)h * D + k) * G + g] * scale : 0.f;
-    zg[k] = (g < G) ? zp[(bh * G + g) * D + k] : 0.f;
-    ug[k] = (g < G) ? dUS[(bh * G + g) * (D + 1) + k] : 0.f;
-    dWa[k] = 0.f;
-  }
-  if (g < G) {
-    bb = bias[(int64_t)h * G + g] * scale;
-    dSg = dUS[(bh * G + g) * (D + 1) + D];
-  }
-  const int64_t n_begin = (int64_t)p * per_split;
-  const int64_t n_end = min(N, n_begin + per_split);
-  for (int64_t n0 = n_begin; n0 < n_end; n0 += PT) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < PT * D; i += kThreads) {
-      const int j = i / D, k = i % D;
-      const int64_t n = n0 + j;
-      float xv = 0.f, dv = 0.f, fv = 0.f;
-      if (n < n_end) {
-        const int64_t idx = row_index(b, n, h, N, H) * D + k;
-        xv = to_f(x[idx]);
-        dv = to_f(dO[idx]);
-        fv = to_f(fx[idx]);
-      }
-      sx[j][k] = xv;
-      sd[j][k] = dv;
-      sf[j][k] = fv;
-    }
-    for (int i = threadIdx.x; i < PT; i += kThreads) {
-      const int64_t n = n0 + i;
-      const bool ok = n < n_end;
-      sl[i] = ok ? lse[bh * N + n] * kLog2e : CUDART_INF_F;
-      sdl[i] = ok ? delta[bh * N + n] : 0.f;
-    }
-    __syncthreads();
-    // Four points at a time (independent chains), updates in point order.
-#pragma unroll 1
-    for (int j = 0; j < PT; j += 4) {
-      float a[4], dwq[4];
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        a[q] = bb;
-        dwq[q] = dSg;
-      }
-#pragma unroll
-      for (int k = 0; k < D; k++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          a[q] = fmaf(sx[j + q][k], wc[k], a[q]);
-          dwq[q] = fmaf(sd[j + q][k], zg[k], dwq[q]);
-          dwq[q] = fmaf(sf[j + q][k], ug[k], dwq[q]);
-        }
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const float w = exp2f(a[q] - sl[j + q]);
-        const float da = w * (dwq[q] - sdl[j + q]);
-#pragma unroll
-        for (int k = 0; k < D; k++) dWa[k] = fmaf(da, sx[j + q][k], dWa[k]);
-        dba += da;
-      }
-    }
-  }
-  if (g < G) {
-    float* o = part + (((int64_t)p * B * H + bh) * G + g) * PS;
-#pragma unroll
-    for (int k = 0; k < D; k++) o[k] = dWa[k];
-    o[D] = dba;
-    o[D + 1] = 0.f;  // (the temperature gradient is formed per point, in the point pass)
-  }
-}
-
 // Token-gradient prep for the slice backward: dUS[bh][g] = (dz_g/(S_g+eps), -(dz_g.z_g)/(S_g+eps)).
 __global__ void k_slice_bwd_prep(const float* __restrict__ z, const float* __restrict__ wsum,
                                  const float* __restrict__ dz, float* __restrict__ dUS, int64_t BHG, int D,
@@ -1103,99 +364,6 @@ __global__ void k_reduce_dtau(const float* __restrict__ dt_part, int64_t B, int 
   if (threadIdx.x == 0) dtau[h] = (accumulate ? dtau[h] : 0.f) - s[0] / tau[h];
 }
 
-inline dim3 point_grid(const Shape& s) {
-  return dim3((unsigned)((s.N + kThreads - 1) / kThreads), (unsigned)s.BH());
-}
-inline dim3 slot_grid(const Shape& s, int P) {
-  return dim3((unsigned)((s.G + kThreads - 1) / kThreads), (unsigned)s.BH(), (unsigned)P);
-}
-inline int64_t per_split(const Shape& s, int P) { return (s.N + P - 1) / P; }
-
-template <int D, typename T>
-cudaError_t launch_stats(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
-                         float* lse, uint32_t* status, cudaStream_t st) {
-  k_stats<D, T><<<point_grid(s), kThreads, 0, st>>>((const T*)x, W, bias, tau, lse, s.N, s.H, s.G, status);
-  return cudaGetLastError();
-}
-
-template <int D, typename T>
-cudaError_t launch_slice_partials(const Shape& s, int P, const void* x, const void* f, const float* W,
-                                  const float* bias, const float* tau, const float* lse, float* part,
-                                  uint32_t* status, cudaStream_t st) {
-  k_slice_partial<D, T><<<slot_grid(s, P), kThreads, 0, st>>>((const T*)x, (const T*)f, W, bias, tau, lse,
-                                                               part, s.B, s.N, s.H, s.G, per_split(s, P),
-                                                               status);
-  return cudaGetLastError();
-}
-
-template <int D, typename T>
-cudaError_t launch_deslice(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
-                           const float* zp, const float* lse, void* out, uint32_t* status, cudaStream_t st) {
-  k_deslice<D, T><<<point_grid(s), kThreads, 0, st>>>((const T*)x, W, bias, tau, zp, lse, (T*)out, s.N, s.H,
-                                                       s.G, status);
-  return cudaGetLastError();
-}
-
-template <int D, typename T, int MODE>
-cudaError_t launch_bwd(const Shape& s, int P, const void* x, const void* v, const float* W, const float* bias,
-                       const float* tau, const float* tok, const float* lse, void* dx, void* dfx, float* delta,
-                       float* dt_part, float* part, int accumulate, uint32_t* status, cudaStream_t st) {
-  k_bwd_point<D, T, MODE><<<point_grid(s), kThreads, 0, st>>>((const T*)x, (const T*)v, W, bias, tau, tok, lse,
-                                                               (T*)dx, (T*)dfx, delta, dt_part, accumulate, s.N,
-                                                               s.H, s.G, status);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_bwd_slot<D, T, MODE><<<slot_grid(s, P), kThreads, 0, st>>>((const T*)x, (const T*)v, W, bias, tau, tok,
-                                                                lse, delta, part, s.B, s.N, s.H, s.G,
-                                                                per_split(s, P), status);
-  return cudaGetLastError();
-}
-
-template <int D, typename T>
-cudaError_t launch_bwd_comb(const Shape& s, int P, const void* x, const void* dO, const void* fx, const float* W,
-                            const float* bias, const float* tau, const float* zp, const float* dUS,
-                            const float* lse, void* dx, void* dfx, float* delta, float* dt_part, float* part,
-                            int accumulate, uint32_t* status, cudaStream_t st) {
-  k_bwd_point_comb<D, T><<<point_grid(s), kThreads, 0, st>>>((const T*)x, (const T*)dO, (const T*)fx, W, bias, tau,
-                                                              zp, dUS, lse, (T*)dx, (T*)dfx, delta, dt_part,
-                                                              accumulate, s.N, s.H, s.G, status);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_bwd_slot_comb<D, T><<<slot_grid(s, P), kThreads, 0, st>>>((const T*)x, (const T*)dO, (const T*)fx, W, bias, tau,
-                                                               zp, dUS, lse, delta, part, s.B, s.N, s.H, s.G,
-                                                               per_split(s, P), status);
-  return cudaGetLastError();
-}
-
-// Dispatch over (d, dtype).// Dispatch over (d, dtype).
-#define FS_DISPATCH(s, FN, ...)                                                        \
-  do {                                                                                 \
-    const bool bf = (s).dtype == FS_BF16;                                              \
-    switch ((s).d) {                                                                   \
-      case 16: return bf ? FN<16, __nv_bfloat16>(__VA_ARGS__) : FN<16, float>(__VA_ARGS__); \
-      case 32: return bf ? FN<32, __nv_bfloat16>(__VA_ARGS__) : FN<32, float>(__VA_ARGS__); \
-      case 64: return bf ? FN<64, __nv_bfloat16>(__VA_ARGS__) : FN<64, float>(__VA_ARGS__); \
-      default: return cudaErrorInvalidValue;                                           \
-    }                                                                                  \
-  } while (0)
-
-template <int D, typename T>
-cudaError_t launch_bwd_deslice(const Shape& s, int P, const void* x, const void* v, const float* W,
-                               const float* bias, const float* tau, const float* tok, const float* lse,
-                               void* dx, float* delta, float* dt_part, float* part, int accumulate,
-                               uint32_t* status, cudaStream_t st) {
-  return launch_bwd<D, T, 0>(s, P, x, v, W, bias, tau, tok, lse, dx, nullptr, delta, dt_part, part, accumulate,
-                             status, st);
-}
-template <int D, typename T>
-cudaError_t launch_bwd_slice(const Shape& s, int P, const void* x, const void* v, const float* W,
-                             const float* bias, const float* tau, const float* tok, const float* lse, void* dx,
-                             void* dfx, float* delta, float* dt_part, float* part, int accumulate,
-                             uint32_t* status, cudaStream_t st) {
-  return launch_bwd<D, T, 1>(s, P, x, v, W, bias, tau, tok, lse, dx, dfx, delta, dt_part, part, accumulate,
-                             status, st);
-}
-
 }  // namespace
 
 cudaError_t simt_reduce_bwd(const Shape& s, int P, const float* part, int Gs, int PS, int has_dzp, const float* tau,
@@ -1229,17 +397,54 @@ cudaError_t simt_slice_bwd_prep(const Shape& s, const float* z, const float* wsu
   return cudaGetLastError();
 }
 
-int64_t simt_point_blocks(const Shape& s) { return (s.N + kThreads - 1) / kThreads; }
+int64_t simt_point_blocks(const Shape& s) { return (s.N + kSimtTP - 1) / kSimtTP; }
+
+// Calls fn with a pointer of the shape's point type.
+#define FS_DISPATCH(s, FN, ...) \
+  ((s).dtype == FS_BF16 ? FN<__nv_bfloat16>(__VA_ARGS__) : FN<float>(__VA_ARGS__))
+
+namespace {
+
+template <typename T>
+const T* in(const void* p) { return static_cast<const T*>(p); }
+template <typename T>
+T* out(void* p) { return static_cast<T*>(p); }
+
+template <typename T>
+cudaError_t launch_stats(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
+                         float* lse, uint32_t* status, cudaStream_t st) {
+  return SimtTiles<T>::stats(s, in<T>(x), W, bias, tau, lse, status, st);
+}
+template <typename T>
+cudaError_t launch_slice(const Shape& s, int P, const void* x, const void* f, const float* W, const float* bias,
+                         const float* tau, const float* lse, float* part, uint32_t* status, cudaStream_t st) {
+  return SimtTiles<T>::slice(s, P, in<T>(x), in<T>(f), W, bias, tau, lse, part, status, st);
+}
+template <typename T>
+cudaError_t launch_deslice(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
+                           const float* zp, const float* lse, void* o, uint32_t* status, cudaStream_t st) {
+  return SimtTiles<T>::deslice(s, in<T>(x), W, bias, tau, zp, lse, out<T>(o), status, st);
+}
+template <typename T>
+cudaError_t launch_bwd(const Shape& s, int mode, int P, const void* x, const void* dO, const void* fx,
+                       const float* W, const float* bias, const float* tau, const float* zp, const float* dUS,
+                       const float* lse, void* dx, void* dfx, float* delta, float* dt_part, float* part,
+                       int accumulate, uint32_t* status, cudaStream_t st) {
+  return SimtTiles<T>::backward(s, mode, P, in<T>(x), in<T>(dO), in<T>(fx), W, bias, tau, zp, dUS, lse, out<T>(dx),
+                                out<T>(dfx), delta, dt_part, part, accumulate, status, st);
+}
+
+}  // namespace
 
 cudaError_t simt_stats(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
                        float* lse, uint32_t* status, cudaStream_t st) {
-  FS_DISPATCH(s, launch_stats, s, x, W, bias, tau, lse, status, st);
+  return FS_DISPATCH(s, launch_stats, s, x, W, bias, tau, lse, status, st);
 }
 
 cudaError_t simt_slice_partials(const Shape& s, int P, const void* x, const void* f, const float* W,
                                 const float* bias, const float* tau, const float* lse, float* part,
                                 uint32_t* status, cudaStream_t st) {
-  FS_DISPATCH(s, launch_slice_partials, s, P, x, f, W, bias, tau, lse, part, status, st);
+  return FS_DISPATCH(s, launch_slice, s, P, x, f, W, bias, tau, lse, part, status, st);
 }
 
 cudaError_t simt_reduce_tokens(const Shape& s, int P, const float* part, int Gs, float* tokens, float* wsum,
@@ -1297,18 +502,16 @@ cudaError_t simt_mix_channels_bwd(const Shape& s, const float* Wc, const float* 
 }
 
 cudaError_t simt_deslice(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
-                         const float* zp, const float* lse, void* out, uint32_t* status, cudaStream_t st) {
-  FS_DISPATCH(s, launch_deslice, s, x, W, bias, tau, zp, lse, out, status, st);
+                         const float* zp, const float* lse, void* o, uint32_t* status, cudaStream_t st) {
+  return FS_DISPATCH(s, launch_deslice, s, x, W, bias, tau, zp, lse, o, status, st);
 }
 
 cudaError_t simt_deslice_bwd(const Shape& s, int P, const void* x, const float* W, const float* bias,
                              const float* tau, const float* zp, const float* lse, const void* dout, float* dzp,
                              void* dx, float* dW, float* db, float* dtau, int accumulate, float* delta,
                              float* part, float* dt_part, uint32_t* status, cudaStream_t st) {
-  cudaError_t e = [&]() -> cudaError_t {
-    FS_DISPATCH(s, launch_bwd_deslice, s, P, x, dout, W, bias, tau, zp, lse, dx, delta, dt_part, part,
-                accumulate, status, st);
-  }();
+  cudaError_t e = FS_DISPATCH(s, launch_bwd, s, 0, P, x, dout, nullptr, W, bias, tau, zp, nullptr, lse, dx, nullptr,
+                              delta, dt_part, part, accumulate, status, st);
   if (e != cudaSuccess) return e;
   return simt_reduce_bwd(s, P, part, s.G, 2 * s.d + 2, 1, tau, dzp, dW, db, dtau, dt_part, simt_point_blocks(s),
                          accumulate, st);
@@ -1321,10 +524,8 @@ cudaError_t simt_slice_bwd(const Shape& s, int P, const void* x, const void* f, 
                            uint32_t* status, cudaStream_t st) {
   cudaError_t e = simt_slice_bwd_prep(s, z, wsum, dz, dUS, st);
   if (e != cudaSuccess) return e;
-  e = [&]() -> cudaError_t {
-    FS_DISPATCH(s, launch_bwd_slice, s, P, x, f, W, bias, tau, dUS, lse, dx, dfx, delta, dt_part, part,
-                accumulate, status, st);
-  }();
+  e = FS_DISPATCH(s, launch_bwd, s, 1, P, x, nullptr, f, W, bias, tau, nullptr, dUS, lse, dx, dfx, delta, dt_part,
+                  part, accumulate, status, st);
   if (e != cudaSuccess) return e;
   return simt_reduce_bwd(s, P, part, s.G, s.d + 2, 0, tau, nullptr, dW, db, dtau, dt_part, simt_point_blocks(s),
                          accumulate, st);
@@ -1332,7 +533,7 @@ cudaError_t simt_slice_bwd(const Shape& s, int P, const void* x, const void* f, 
 
 // The coupling's whole backward on the SIMT kernels: d z' as the forward slice's
 // unnormalised numerators with dO for fx, the mix backward, the slice's dU, dS, then
-// one point pass and one slot pass for da_D + da_S (k_bwd_point_comb, k_bwd_slot_comb)
+// one point pass and one slot pass for da_D + da_S (mode 2)
 // and the parameter reductions.  `part` holds the larger of the two partial sets;
 // the d z' reduction's weight sums go to dUS, which the prologue then overwrites.
 cudaError_t simt_coupling_bwd(const Shape& s, int P, const void* x, const void* fx, const void* dout,
@@ -1346,10 +547,8 @@ cudaError_t simt_coupling_bwd(const Shape& s, int P, const void* x, const void* 
   if ((e = simt_reduce_tokens(s, P, part, s.G, dzp, dUS, 0, st)) != cudaSuccess) return e;
   if ((e = simt_mix_bwd(s, M, z, dzp, dz, dM, st)) != cudaSuccess) return e;
   if ((e = simt_slice_bwd_prep(s, z, wsum, dz, dUS, st)) != cudaSuccess) return e;
-  e = [&]() -> cudaError_t {
-    FS_DISPATCH(s, launch_bwd_comb, s, P, x, dout, fx, W, bias, tau, zp, dUS, lse, dx, dfx, delta, dt_part, part,
-                accumulate, status, st);
-  }();
+  e = FS_DISPATCH(s, launch_bwd, s, 2, P, x, dout, fx, W, bias, tau, zp, dUS, lse, dx, dfx, delta, dt_part, part,
+                  accumulate, status, st);
   if (e != cudaSuccess) return e;
   return simt_reduce_bwd(s, P, part, s.G, s.d + 2, 0, tau, nullptr, dW, db, dtau, dt_part, simt_point_blocks(s),
                          accumulate, st);
