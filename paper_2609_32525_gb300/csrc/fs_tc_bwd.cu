@@ -103,44 +103,39 @@ __global__ void k_prep_dpx(const float* __restrict__ delta, const float* __restr
 
 // ---- device pieces -----------------------------------------------------------------------------
 
-// M = 128 x N = 64 product with K = 48 (80 with the residual half, lo_a or lo_b):
-// a0/b0 are the K-major 64B-swizzled 32-channel blocks, ae/be the extra blocks
-// (kExtra = false: K = 32 / 64, no extra block).
+// M = 128 x N = 64 product with K = 48 (80 with the residual half, lo of A or B): a, b the
+// low descriptor words of the K-major 64B-swizzled 32-channel blocks, ae, be those of the
+// extra blocks with high words kAeHi, kBeHi (kAeHi = 0: K = 32 / 64, no extra block).
 // acc0: add to what d holds (a second chain into the same accumulator).
-template <bool kLoA, bool kExtra = true>
-__device__ __forceinline__ void issue_dot64(uint32_t d, uint32_t a, uint32_t b, uint64_t ae, uint64_t be,
-                                            uint32_t lo, uint32_t acc0 = 0) {
+template <bool kLoA, uint32_t kAeHi, uint32_t kBeHi>
+__device__ __forceinline__ void issue_dot64(uint32_t d, uint32_t a, uint32_t b, uint32_t ae, uint32_t be, uint32_t lo,
+                                            uint32_t acc0 = 0) {
   constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
-  mma_ss_w(d, sdesc(a, 16, 512, kSw64), sdesc(b, 16, 512, kSw64), idesc, acc0);
-  mma_ss_w(d, sdesc(a + 32, 16, 512, kSw64), sdesc(b + 32, 16, 512, kSw64), idesc, 1);
+  mma_ss_w<kHi64, kHi64>(d, a, b, idesc, acc0);
+  mma_ss_w<kHi64, kHi64>(d, a + 2, b + 2, idesc, 1);
   if (lo) {
-    if (kLoA) {
-      mma_ss_w(d, sdesc(lo, 16, 512, kSw64), sdesc(b, 16, 512, kSw64), idesc, 1);
-      mma_ss_w(d, sdesc(lo + 32, 16, 512, kSw64), sdesc(b + 32, 16, 512, kSw64), idesc, 1);
-    } else {
-      mma_ss_w(d, sdesc(a, 16, 512, kSw64), sdesc(lo, 16, 512, kSw64), idesc, 1);
-      mma_ss_w(d, sdesc(a + 32, 16, 512, kSw64), sdesc(lo + 32, 16, 512, kSw64), idesc, 1);
-    }
+    mma_ss_w<kHi64, kHi64>(d, kLoA ? lo : a, kLoA ? b : lo, idesc, 1);
+    mma_ss_w<kHi64, kHi64>(d, kLoA ? lo + 2 : a + 2, kLoA ? b + 2 : lo + 2, idesc, 1);
   }
-  if (kExtra) mma_ss_w(d, ae, be, idesc, 1);
+  if (kAeHi != 0) mma_ss_w<kAeHi, kBeHi>(d, ae, be, idesc, 1);
 }
 
-// The same logits product with the slot side (A) in TMEM: tW holds a slot block's W'
-// image as packed bf16 pairs, K steps of 8 columns: W' (2 steps), its residual (2), the
-// extra block (1).  Only the point side (B) is read from shared memory.
-__device__ __forceinline__ void issue_logits64_ts(uint32_t d, uint32_t tW, uint32_t b, uint64_t be, bool lo) {
+// The main part of the same product with the slot side (A) in TMEM: tA holds a slot
+// block's rows as packed bf16 pairs, K steps of 8 columns: the bf16 half (2 steps), its
+// residual (2).  Only the point side (B) is read from shared memory.
+__device__ __forceinline__ void issue_dot64_ts(uint32_t d, uint32_t tA, uint32_t b, bool lo) {
   constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
-  mma_ts_w(d, tW, sdesc(b, 16, 512, kSw64), idesc, 0u);
-  mma_ts_w(d, tW + 8, sdesc(b + 32, 16, 512, kSw64), idesc, 1u);
+  mma_ts_w<kHi64>(d, tA, b, idesc, 0u);
+  mma_ts_w<kHi64>(d, tA + 8, b + 2, idesc, 1u);
   if (lo) {
-    mma_ts_w(d, tW + 16, sdesc(b, 16, 512, kSw64), idesc, 1u);
-    mma_ts_w(d, tW + 24, sdesc(b + 32, 16, 512, kSw64), idesc, 1u);
+    mma_ts_w<kHi64>(d, tA + 16, b, idesc, 1u);
+    mma_ts_w<kHi64>(d, tA + 24, b + 2, idesc, 1u);
   }
-  mma_ts_w(d, tW + 32, be, idesc, 1u);
 }
 
-// Point-extra descriptor (no swizzle, 16-byte rows) whose k = 8..15 half is the shared zero block.
-__device__ __forceinline__ uint64_t px_desc(uint32_t px_s, uint32_t zero_s) { return sdesc(px_s, zero_s - px_s, 128, 0); }
+// Low word of a point-extra descriptor (no swizzle, 16-byte rows) whose k = 8..15 half is
+// the shared zero block; n rows further on both its fields change.
+__device__ __forceinline__ uint32_t px_lo(uint32_t px_s, uint32_t zero_s) { return sdesc_lo(px_s, zero_s - px_s); }
 
 // One 64-column unit of a TMEM lane: L (log2 weights) at tL, dw - delta at tD.
 // da = 2^L (dw - delta) goes back in place into the L columns as bf16 pairs: columns
@@ -373,58 +368,52 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------ logits and dw issuer ------------------------------
-    const uint32_t sw = smem_u32(s_w), stt = smem_u32(s_t), stt2 = smem_u32(s_t2), sz = smem_u32(s_zero);
+    const uint32_t w = sdesc_lo(smem_u32(s_w), 16), t = sdesc_lo(smem_u32(s_t), 16), t2 = sdesc_lo(smem_u32(s_t2), 16);
+    const uint32_t sz = smem_u32(s_zero);
+    constexpr uint32_t kExt = kGC * 4, kLo = kGC * 6;  // the extra and residual rows of a slot block, in 16 bytes
+    constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
     bool ok = mbar_wait_w(w_full, 0, ab, status);
     if (kWT && ok) {
       ok = mbar_wait_w(wt_ready, 0, ab, status);
       tc_fence_after();
     }
-    for (int u = 0; ok && u < units; u++) {
-      const int i = u >> 1, half = u & 1;
-      const int s = i % kNSt;
-      const int bb = u % kSBuf;
-      if (half == 0 && !(ok = mbar_wait_w(&x_full[s], (uint32_t)((i / kNSt) & 1), ab, status))) break;
-      if (u >= kSBuf && !(ok = mbar_wait_w(&pv_done[bb], (uint32_t)(((u / kSBuf) - 1) & 1), ab, status))) break;
-      tc_fence_after();
-      const uint32_t st = smem_u32(s_st + s * kStgS);
-      const uint32_t rows = (uint32_t)half * 64 * 64;     // the unit's 64 points in the 64-byte-row tiles
-      const uint32_t prow = (uint32_t)half * 64 * 16;     // ... and in the 16-byte extra rows
-      const uint32_t tL = tmem + (uint32_t)bb * kGC;
-      if (kTT) {
-        constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
-        const uint32_t tW = tmem + kAccZ, tT = tW + 32;
-        const uint32_t xb = st + rows, vb = st + kVOff + rows;
-        mma_ts_w(tL, tW, sdesc(xb, 16, 512, kSw64), idesc, 0u);
-        mma_ts_w(tL, tW + 8, sdesc(xb + 32, 16, 512, kSw64), idesc, 1u);
-        if (split) {
-          mma_ts_w(tL, tW + 16, sdesc(xb, 16, 512, kSw64), idesc, 1u);
-          mma_ts_w(tL, tW + 24, sdesc(xb + 32, 16, 512, kSw64), idesc, 1u);
+    Ring<kNSt> stg;
+    Ring<kSBuf> sb;
+    for (int i = 0, u = 0; ok && i < wk.ntiles; i++, stg.next()) {
+      if (!(ok = mbar_wait_w(&x_full[stg.i], stg.pass, ab, status))) break;
+      const uint32_t st = smem_u32(s_st + stg.i * kStgS);
+      uint32_t x = sdesc_lo(st, 16);
+      uint32_t px = px_lo(st + kPOff, sz), dpx = px_lo(st + kDOff, sz);
+      // the second half's 64 points: 64-byte-row tiles, then 16-byte extra rows (whose
+      // leading offset to the zero block shrinks as the address grows)
+      constexpr uint32_t kHalf = 64 * 64 / 16, kHalfP = 64 * 16 / 16 - ((64u * 16 / 16) << 16);
+#pragma unroll 1
+      for (int half = 0; half < 2; half++, u++, sb.next(), x += kHalf, px += kHalfP, dpx += kHalfP) {
+        if (u >= kSBuf && !(ok = mbar_wait_w(&pv_done[sb.i], sb.pass ^ 1u, ab, status))) break;
+        tc_fence_after();
+        const uint32_t tL = tmem + (uint32_t)sb.i * kGC;
+        const uint32_t v = x + kVOff / 16, f = x + kBStage / 16;
+        if (kTT) {
+          issue_dot64_ts(tL, tmem + kAccZ, x, split);
+          mma_ss_w<kHi32, kHiPx>(tL, w + kExt, px, idesc, 1u);
+          // the deslice's chain: T (and its residual) from TMEM against dO, no extra block;
+          // the slice's extra block [dS_hi, dS_lo, 1, 1, 1] against delta's rows
+          // [1, 1, -delta parts] adds dS - delta in one K step.
+          issue_dot64_ts(tL + 64, tmem + kAccZ + 32, v, split);
+          issue_dot64<true, kHi32, kHiPx>(tL + 64, t2, f, t2 + kExt, dpx, split ? t2 + kLo : 0u, 1u);
+        } else {
+          if (kWT) {
+            issue_dot64_ts(tL, tmem + kAccZ, x, split);
+            mma_ts_w<kHiPx>(tL, tmem + kAccZ + 32, px, idesc, 1u);
+          } else {
+            issue_dot64<true, kHi32, kHiPx>(tL, w, x, w + kExt, px, split ? w + kLo : 0u);
+          }
+          if (MODE == 1 || MODE == 2)
+            issue_dot64<true, kHi32, kHiPx>(tL + 64, t, v, t + kExt, dpx, split ? t + kLo : 0u);
         }
-        mma_ss_w(tL, sdesc(sw + kGC * 64, 16, 256, kSw32), px_desc(st + kPOff + prow, sz), idesc, 1u);
-        // the deslice's chain: T (and its residual) from TMEM against dO, no extra block
-        mma_ts_w(tL + 64, tT, sdesc(vb, 16, 512, kSw64), idesc, 0u);
-        mma_ts_w(tL + 64, tT + 8, sdesc(vb + 32, 16, 512, kSw64), idesc, 1u);
-        if (split) {
-          mma_ts_w(tL + 64, tT + 16, sdesc(vb, 16, 512, kSw64), idesc, 1u);
-          mma_ts_w(tL + 64, tT + 24, sdesc(vb + 32, 16, 512, kSw64), idesc, 1u);
-        }
-      } else if (kWT)
-        issue_logits64_ts(tL, tmem + kAccZ, st + rows, px_desc(st + kPOff + prow, sz), split);
-      else
-        issue_dot64<true>(tL, sw, st + rows, sdesc(sw + kGC * 64, 16, 256, kSw32), px_desc(st + kPOff + prow, sz),
-                          split ? sw + kGC * 96 : 0u);
-      if (MODE == 1 || MODE == 2)
-        issue_dot64<true>(tL + 64, stt, st + kVOff + rows, sdesc(stt + kGC * 64, 16, 256, kSw32),
-                          px_desc(st + kDOff + prow, sz), split ? stt + kGC * 96 : 0u);
-      if (MODE == 3) {
-        // The deslice's T has c = 0, so its chain (issued above from TMEM) needs no extra
-        // block: the slice's extra block [dS_hi, dS_lo, 1, 1, 1] against delta's rows
-        // [1, 1, -delta parts] adds dS - delta in one K step.
-        issue_dot64<true>(tL + 64, stt2, st + kBStage + rows, sdesc(stt2 + kGC * 64, 16, 256, kSw32),
-                          px_desc(st + kDOff + prow, sz), split ? stt2 + kGC * 96 : 0u, 1u);
+        mma_commit_w(&s_full[sb.i]);
       }
-      mma_commit_w(&s_full[bb]);
-      if (half == 1) mma_commit_w(&st_empty[s]);
+      mma_commit_w(&st_empty[stg.i]);
     }
     mma_commit_w(&drain[0]);
     mbar_wait_w(&drain[0], 0, ab, nullptr, kWaitNs);
@@ -433,38 +422,37 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int j = warp - 2;  // units u with u % 2 == j (half j of every tile)
     constexpr uint32_t idesc = idesc_bf16(128, kD, false, true);
     bool ok = true;
-    for (int u = j; ok && u < units; u += 2) {
-      const int i = u >> 1;
-      const int s = i % kNSt;
-      const int bb = u % kSBuf;
-      // This issuer's units on set bb are 2 kSBuf apart.
-      if (!(ok = mbar_wait_w(&p_ready[j * kSBuf + bb], (uint32_t)((u / (2 * kSBuf)) & 1), ab, status))) break;
+    Ring<kNSt> stg;
+    Ring<kSBuf> sb;
+    uint32_t pass = 0;  // parity of this issuer's uses of a set (its units there are 2 kSBuf apart)
+    if (j == 1) sb.next();
+    for (int u = j; ok && u < units; u += 2, stg.next(), sb.next(), sb.next()) {
+      if (!(ok = mbar_wait_w(&p_ready[j * kSBuf + sb.i], pass, ab, status))) break;
       tc_fence_after();
-      const uint32_t st = smem_u32(s_st + s * kStgS) + (uint32_t)j * 64 * 64;
-      const uint32_t tL = tmem + (uint32_t)bb * kGC, tD = tL + 64;
+      // 16 points: two 8-row groups of the 64B-swizzled tile (MN-major: channels contiguous).
+      const uint32_t x = sdesc_lo(smem_u32(s_st + stg.i * kStgS) + (uint32_t)j * 64 * 64, 4096), v = x + kVOff / 16;
+      const uint32_t tL = tmem + (uint32_t)sb.i * kGC, tD = tL + 64;
+      const uint32_t tW = tmem + kAccW + (uint32_t)j * 32, tZ = tmem + kAccZ + (uint32_t)j * 32;
+      const bool fresh = u < 2 || (kFl && slot_flush_at(u));
 #pragma unroll
       for (int kk = 0; kk < 4; kk++) {
-        // 16 points: two 8-row groups of the 64B-swizzled tile (MN-major: channels contiguous).
-        const uint64_t xd = sdesc(st + (uint32_t)kk * 1024, 4096, 512, kSw64);
-        const bool fresh = u < 2 || (kFl && slot_flush_at(u));
         const uint32_t acc = (!fresh || kk > 0) ? 1u : 0u;
         if (MODE == 0) {  // the weights are in the L columns: dZ += w^T dO
-          const uint64_t vd = sdesc(st + kVOff + (uint32_t)kk * 1024, 4096, 512, kSw64);
-          mma_ts_w(tmem + kAccZ + (uint32_t)j * 32, tL + da_col(kk), vd, idesc, acc);
-          if (split) mma_ts_w(tmem + kAccZ + (uint32_t)j * 32, tL + da_col(kk) + 16, vd, idesc, 1u);
+          mma_ts_w<kHi64>(tZ, tL + da_col(kk), v + kk * 64, idesc, acc);
+          if (split) mma_ts_w<kHi64>(tZ, tL + da_col(kk) + 16, v + kk * 64, idesc, 1u);
           continue;
         }
-        mma_ts_w(tmem + kAccW + (uint32_t)j * 32, tL + da_col(kk), xd, idesc, acc);
-        if (split) mma_ts_w(tmem + kAccW + (uint32_t)j * 32, tL + da_col(kk) + 16, xd, idesc, 1u);
+        mma_ts_w<kHi64>(tW, tL + da_col(kk), x + kk * 64, idesc, acc);
+        if (split) mma_ts_w<kHi64>(tW, tL + da_col(kk) + 16, x + kk * 64, idesc, 1u);
         if (MODE == 1) {
-          const uint64_t vd = sdesc(st + kVOff + (uint32_t)kk * 1024, 4096, 512, kSw64);
-          mma_ts_w(tmem + kAccZ + (uint32_t)j * 32, tD + da_col(kk), vd, idesc, acc);
-          if (split) mma_ts_w(tmem + kAccZ + (uint32_t)j * 32, tD + da_col(kk) + 16, vd, idesc, 1u);
+          mma_ts_w<kHi64>(tZ, tD + da_col(kk), v + kk * 64, idesc, acc);
+          if (split) mma_ts_w<kHi64>(tZ, tD + da_col(kk) + 16, v + kk * 64, idesc, 1u);
         }
       }
-      mma_commit_w(&pv_done[bb]);
-      mma_commit_w(&st_empty[s]);
+      mma_commit_w(&pv_done[sb.i]);
+      mma_commit_w(&st_empty[stg.i]);
       if (kFl) mma_commit_w(&acc_done[j]);
+      if ((u >> 1) % kSBuf == kSBuf - 1) pass ^= 1u;
     }
     if (ok) mma_commit_w(acc_full);
     mma_commit_w(&drain[1 + j]);
@@ -748,34 +736,34 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     if (wk.ntiles > 0) {
-      const uint32_t sw = smem_u32(s_w), stt = smem_u32(s_t), stt2 = smem_u32(s_t2), sz = smem_u32(s_zero);
+      const uint32_t w0 = sdesc_lo(smem_u32(s_w), 16), t0 = sdesc_lo(smem_u32(s_t), 16), t20 = sdesc_lo(smem_u32(s_t2), 16);
+      const uint32_t sz = smem_u32(s_zero), ext = (uint32_t)G * 4;
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
-      BlockPos pos(0, nch);
-      for (int q = 0; ok && q < total; q++, pos.step(1, nch)) {
-        const int i = pos.i, c = pos.c;
-        const int s = i % kDxStages;
-        const int bb = q % kSBuf;
-        if (c == 0 && !(ok = mbar_wait_w(&x_full[s], (uint32_t)((i / kDxStages) & 1), ab, status))) break;
-        if (q >= kSBuf && !(ok = mbar_wait_w(&pv_done[bb], (uint32_t)(((q / kSBuf) - 1) & 1), ab, status))) break;
-        tc_fence_after();
-        const uint32_t st = smem_u32(s_st + s * kStg);
-        const uint32_t tL = tmem + (uint32_t)bb * kGC;
-        const uint32_t rows = (uint32_t)c * 64 * 64, erows = (uint32_t)c * 64 * 32;
-        issue_dot64<false>(tL, st, sw + rows, px_desc(st + kPOff, sz),
-                           sdesc(sw + (uint32_t)G * 64 + erows, 16, 256, kSw32),
-                           hilo ? sw + (uint32_t)G * 96 + rows : 0u);
-        if (kComb) {
-          // As in the slot pass: the deslice's chain without an extra block, the slice's
-          // extra block against delta's rows (dS - delta in one K step).
-          issue_dot64<false, false>(tL + 64, st + kVOff, stt + rows, 0ull, 0ull, 0u);
-          issue_dot64<false>(tL + 64, st + kBStage, stt2 + rows, px_desc(st + kDOff, sz),
-                             sdesc(stt2 + (uint32_t)G * 64 + erows, 16, 256, kSw32), 0u, 1u);
-        } else {
-          issue_dot64<false>(tL + 64, st + kVOff, stt + rows, px_desc(st + kDOff, sz),
-                             sdesc(stt + (uint32_t)G * 64 + erows, 16, 256, kSw32), 0u);
+      Ring<kDxStages> stg;
+      Ring<kSBuf> sb;
+      for (int i = 0, q = 0; ok && i < wk.ntiles; i++, stg.next()) {
+        if (!(ok = mbar_wait_w(&x_full[stg.i], stg.pass, ab, status))) break;
+        const uint32_t st = smem_u32(s_st + stg.i * kStg);
+        const uint32_t x = sdesc_lo(st, 16), v = x + kVOff / 16, f = x + kBStage / 16;
+        const uint32_t px = px_lo(st + kPOff, sz), dpx = px_lo(st + kDOff, sz);
+        uint32_t r = 0, e = ext;  // the chunk's rows in the 64-byte and 32-byte images, in 16 bytes
+#pragma unroll 1
+        for (int c = 0; c < nch; c++, q++, sb.next(), r += 64 * 4, e += 64 * 2) {
+          if (q >= kSBuf && !(ok = mbar_wait_w(&pv_done[sb.i], sb.pass ^ 1u, ab, status))) break;
+          tc_fence_after();
+          const uint32_t tL = tmem + (uint32_t)sb.i * kGC;
+          issue_dot64<false, kHiPx, kHi32>(tL, x, w0 + r, px, w0 + e, hilo ? w0 + (uint32_t)G * 6 + r : 0u);
+          if (kComb) {
+            // As in the slot pass: the deslice's chain without an extra block, the slice's
+            // extra block against delta's rows (dS - delta in one K step).
+            issue_dot64<false, 0, 0>(tL + 64, v, t0 + r, 0u, 0u, 0u);
+            issue_dot64<false, kHiPx, kHi32>(tL + 64, f, t20 + r, dpx, t20 + e, 0u, 1u);
+          } else {
+            issue_dot64<false, kHiPx, kHi32>(tL + 64, v, t0 + r, dpx, t0 + e, 0u);
+          }
+          mma_commit_w(&s_full[sb.i]);
         }
-        mma_commit_w(&s_full[bb]);
-        if (c == nch - 1) mma_commit_w(&x_empty[s]);
+        mma_commit_w(&x_empty[stg.i]);
       }
       mma_commit_w(&drain[0]);
       mbar_wait_w(&drain[0], 0, ab, nullptr, kWaitNs);
@@ -784,27 +772,28 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int j = warp - 2;
     if (wk.ntiles > 0) {
       constexpr uint32_t idesc = idesc_bf16(128, kD, false, false);
-      const uint32_t swt = smem_u32(s_wt);
+      // K-steps [2 j, 2 j + 2) of a 64-slot chunk
+      const uint32_t wt0 = sdesc_lo(smem_u32(s_wt), 16) + (uint32_t)j * 4;
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
-      BlockPos pos(0, nch);
-      for (int q = 0; ok && q < total; q++, pos.step(1, nch)) {
-        const int i = pos.i, c = pos.c;
+      Ring<kSBuf> sb;
+      for (int i = 0; ok && i < wk.ntiles; i++) {
         const int ob = i & 1;
-        const int bb = q % kSBuf;
-        if (c == 0 && i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
-        if (!(ok = mbar_wait_w(&p_ready[bb], (uint32_t)((q / kSBuf) & 1), ab, status))) break;
-        tc_fence_after();
-        const uint32_t tL = tmem + (uint32_t)bb * kGC;
         const uint32_t tO = tmem + kO + (uint32_t)(j * 2 + ob) * kD;
+        if (i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
+        uint32_t wt = wt0;
+#pragma unroll 1
+        for (int c = 0; c < nch; c++, wt += 256, sb.next()) {
+          if (!(ok = mbar_wait_w(&p_ready[sb.i], sb.pass, ab, status))) break;
+          tc_fence_after();
+          const uint32_t tL = tmem + (uint32_t)sb.i * kGC + (uint32_t)j * 32;  // da_col(2 j)
 #pragma unroll
-        for (int e = 0; e < 2; e++) {
-          const int kk = 2 * j + e;
-          const uint64_t bd = sdesc(swt + (uint32_t)c * 4096 + (uint32_t)kk * 32, 16, 1024, kSw128);
-          mma_ts_w(tO, tL + da_col(kk), bd, idesc, (c > 0 || e > 0) ? 1u : 0u);
-          if (split) mma_ts_w(tO, tL + da_col(kk) + 16, bd, idesc, 1u);
+          for (int e = 0; e < 2; e++) {
+            mma_ts_w<kHi128>(tO, tL + da_col(e), wt + e * 2, idesc, (c > 0 || e > 0) ? 1u : 0u);
+            if (split) mma_ts_w<kHi128>(tO, tL + da_col(e) + 16, wt + e * 2, idesc, 1u);
+          }
+          mma_commit_w(&pv_done[sb.i]);
         }
-        mma_commit_w(&pv_done[bb]);
-        if (c == nch - 1) mma_commit_w(&o_full[ob]);
+        mma_commit_w(&o_full[ob]);
       }
       mma_commit_w(&drain[1 + j]);
       mbar_wait_w(&drain[1 + j], 0, ab, nullptr, kWaitNs);

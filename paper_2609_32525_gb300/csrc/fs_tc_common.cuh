@@ -171,61 +171,42 @@ __device__ __forceinline__ void write_const_extra(uint8_t* ex) {
   }
 }
 
-// Descriptors of the two kinds of point-side extra block: the constant one
-// (32B swizzle) and the per-tile one loaded by TMA (no swizzle; the k = 0..7
+// Low descriptor words of the two kinds of point-side extra block: the constant one
+// (32B swizzle, kHi32) and the per-tile one loaded by TMA (no swizzle, kHiPx; the k = 0..7
 // core matrices at px, the zero k = 8..15 half kPxBytes further on).
-__device__ __forceinline__ uint64_t const_extra_desc(uint32_t ex_s) { return sdesc(ex_s, 16, 256, kSw32); }
-__device__ __forceinline__ uint64_t point_extra_desc(uint32_t px_s) { return sdesc(px_s, kPxBytes, 128, 0); }
+__device__ __forceinline__ uint32_t const_extra_lo(uint32_t ex_s) { return sdesc_lo(ex_s, 16); }
+__device__ __forceinline__ uint32_t point_extra_lo(uint32_t px_s) { return sdesc_lo(px_s, kPxBytes); }
 __device__ __forceinline__ void zero_smem(uint8_t* p, uint32_t bytes) {
   for (uint32_t o = threadIdx.x * 16; o < bytes; o += blockDim.x * 16) st_shared_v4(smem_u32(p) + o, 0u, 0u, 0u, 0u);
 }
 
-// Base-2 logits of 128 points x 128 slots (chunk c of the W image) into TMEM.
-//   point_major: A = points (x tile), B = slots (W);  else A = slots, B = points.
-//   xe: descriptor of the point-side extra block.
-//   wl_img: the residual half of W' (0: bf16 W' only, K = 48; else K = 80).
-//   xr_s: the residual half of x, fp32 inputs (0: none; else two more K-steps, x_r W'_hi).
-__device__ __forceinline__ void issue_logits(uint32_t tmem_d, uint32_t x_s, uint64_t xe, uint32_t w_img,
-                                             uint32_t we_img, uint32_t wl_img, int c, bool point_major,
-                                             uint32_t xr_s = 0) {
+// Base-2 logits of 128 points x 128 slots into TMEM.  Operands by their low descriptor
+// words:
+//   kPointMajor: A = points (x tile), B = slots (W);  else A = slots, B = points.
+//   x, xe: the point tile and its extra block (kXeHi: its high word); w, we: the slot block's
+//   W' rows and extra rows; wl: the residual half of W' (0: bf16 W' only, K = 48; else K = 80);
+//   xr: the residual half of x, fp32 inputs (0: none; else two more K-steps, x_r W'_hi).
+template <bool kPointMajor, uint32_t kXeHi>
+__device__ __forceinline__ void issue_logits(uint32_t tmem_d, uint32_t x, uint32_t xe, uint32_t w, uint32_t we,
+                                             uint32_t wl, uint32_t xr) {
   constexpr uint32_t idesc = idesc_bf16(128, kGC, false, false);
-  const uint32_t wc = w_img + (uint32_t)c * kGC * 64;
-  const uint32_t wec = we_img + (uint32_t)c * kGC * 32;
-  const uint64_t x0 = sdesc(x_s, 16, 512, kSw64), x1 = sdesc(x_s + 32, 16, 512, kSw64);
-  const uint64_t w0 = sdesc(wc, 16, 512, kSw64), w1 = sdesc(wc + 32, 16, 512, kSw64);
-  const uint64_t we = sdesc(wec, 16, 256, kSw32);
-  if (point_major) {
-    mma_ss_w(tmem_d, x0, w0, idesc, 0);
-    mma_ss_w(tmem_d, x1, w1, idesc, 1);
-  } else {
-    mma_ss_w(tmem_d, w0, x0, idesc, 0);
-    mma_ss_w(tmem_d, w1, x1, idesc, 1);
+  auto mma = [&](uint32_t pt, uint32_t sl, uint32_t acc) {
+    mma_ss_w<kHi64, kHi64>(tmem_d, kPointMajor ? pt : sl, kPointMajor ? sl : pt, idesc, acc);
+  };
+  mma(x, w, 0);
+  mma(x + 2, w + 2, 1);
+  if (wl) {
+    mma(x, wl, 1);
+    mma(x + 2, wl + 2, 1);
   }
-  if (wl_img) {
-    const uint32_t wlc = wl_img + (uint32_t)c * kGC * 64;
-    const uint64_t l0 = sdesc(wlc, 16, 512, kSw64), l1 = sdesc(wlc + 32, 16, 512, kSw64);
-    if (point_major) {
-      mma_ss_w(tmem_d, x0, l0, idesc, 1);
-      mma_ss_w(tmem_d, x1, l1, idesc, 1);
-    } else {
-      mma_ss_w(tmem_d, l0, x0, idesc, 1);
-      mma_ss_w(tmem_d, l1, x1, idesc, 1);
-    }
+  if (xr) {
+    mma(xr, w, 1);
+    mma(xr + 2, w + 2, 1);
   }
-  if (xr_s) {
-    const uint64_t r0 = sdesc(xr_s, 16, 512, kSw64), r1 = sdesc(xr_s + 32, 16, 512, kSw64);
-    if (point_major) {
-      mma_ss_w(tmem_d, r0, w0, idesc, 1);
-      mma_ss_w(tmem_d, r1, w1, idesc, 1);
-    } else {
-      mma_ss_w(tmem_d, w0, r0, idesc, 1);
-      mma_ss_w(tmem_d, w1, r1, idesc, 1);
-    }
-  }
-  if (point_major)
-    mma_ss_w(tmem_d, xe, we, idesc, 1);
+  if (kPointMajor)
+    mma_ss_w<kXeHi, kHi32>(tmem_d, xe, we, idesc, 1);
   else
-    mma_ss_w(tmem_d, we, xe, idesc, 1);
+    mma_ss_w<kHi32, kXeHi>(tmem_d, we, xe, idesc, 1);
 }
 
 // fp32 point tensors -> bf16 hi and residual lo tensors of the same layout (v = hi + lo
@@ -272,28 +253,9 @@ __device__ __forceinline__ void weights32_hilo(const uint32_t (&v)[32], uint32_t
   }
 }
 
-// The 128 log2-weights of one TMEM lane of an S buffer -> bf16 weights written back
-// in place, packed in pairs, into the first 64 columns, in two halves: columns
-// [64 h, 64 h + 64) -> packed weights in columns [32 h, 32 h + 32), which this
-// thread has already read.
-__device__ __forceinline__ void weights_in_halves(uint32_t tS) {
-#pragma unroll 1
-  for (int half = 0; half < 2; half++) {
-    uint32_t v0[32], v1[32];
-    tmem_ld32(tS + half * 64, v0);
-    tmem_ld32(tS + half * 64 + 32, v1);
-    tmem_wait_ld2(v0, v1);
-    uint32_t pk0[16], pk1[16];
-    weights32(v0, pk0);
-    weights32(v1, pk1);
-    tmem_st16(tS + half * 32, pk0);
-    tmem_st16(tS + half * 32 + 16, pk1);
-  }
-}
-
-// One 64-slot half of the row: the log2-weights in columns [0, 64) from tS -> bf16
-// weights packed in pairs into columns [0, 32) from tS, which this thread has read.
-__device__ __forceinline__ void weights_half(uint32_t tS) {
+// 64 log2-weights of one TMEM lane in columns [0, 64) from tS -> bf16 weights packed in
+// pairs into columns [0, 32) from tP (which may be columns this thread has read).
+__device__ __forceinline__ void weights_half(uint32_t tS, uint32_t tP) {
   uint32_t v0[32], v1[32];
   tmem_ld32(tS, v0);
   tmem_ld32(tS + 32, v1);
@@ -301,8 +263,17 @@ __device__ __forceinline__ void weights_half(uint32_t tS) {
   uint32_t pk0[16], pk1[16];
   weights32(v0, pk0);
   weights32(v1, pk1);
-  tmem_st16(tS, pk0);
-  tmem_st16(tS + 16, pk1);
+  tmem_st16(tP, pk0);
+  tmem_st16(tP + 16, pk1);
+}
+
+// The 128 log2-weights of one TMEM lane of an S buffer -> bf16 weights written back
+// in place, packed in pairs, into the first 64 columns, in two halves: columns
+// [64 h, 64 h + 64) -> packed weights in columns [32 h, 32 h + 32), which this
+// thread has already read.
+__device__ __forceinline__ void weights_in_halves(uint32_t tS) {
+#pragma unroll 1
+  for (int half = 0; half < 2; half++) weights_half(tS + half * 64, tS + half * 32);
 }
 
 // One 64-column half with split products: the log2-weights in columns [0, 64) from tS

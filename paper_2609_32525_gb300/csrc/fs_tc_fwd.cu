@@ -38,8 +38,8 @@
 // products into accumulators of their own, which are summed in a fixed order,
 // so the result is deterministic.
 //
-// CTA (384 threads): warp 0 TMA producer, warps 1..3 MMA issuers, warps 4..11
-// two softmax warpgroups that take alternate blocks (so they run out of phase);
+// CTA: warp 0 TMA producer, warps 1..3 MMA issuers, warps 4 and up softmax warpgroups
+// (two to four) that take blocks in turn (so they run out of phase);
 // a thread owns one TMEM lane (tcgen05.ld/st 32x32b).  Every wait is bounded
 // (2 s): a wait that gives up writes FS_ERR_TIMEOUT to the status word, the CTA
 // drains its copies and MMAs, frees TMEM and exits.
@@ -62,12 +62,22 @@ using namespace tc;
 // =========================================================================================
 // Deslice: out_n = sum_g w_ng z'_g.
 // smem: [W img G*96][Z' img G*64][stages: x | point extra (TMA half, zero half)][barriers]
-// TMEM: S buffers [0, 384); P x Z' accumulators O_0 [384, 448), O_1 [448, 512),
-// each double-buffered by tile parity.  Block q (tile q / nb, slot block q % nb)
-// uses S buffer q % 3 and softmax warpgroup q % 2, which writes the bf16 weights
-// of its 128 slots, packed in pairs, into columns [0, 64) of the same buffer;
-// warp 2 + j turns slots [64 j, 64 j + 64) of every block into products
-// (K-steps [4 j, 4 j + 4)) accumulated in O_j.
+// TMEM: S buffers [0, 384); P x Z' accumulators O_0 [384, 448), O_1 [448, 512), each
+// double-buffered by tile parity.  Block q (tile q / nb, slot block q % nb) uses S buffer
+// q % 3; a softmax warpgroup writes the bf16 weights of its 128 slots, packed in pairs,
+// into columns [0, 64) of the same buffer; warp 2 + j turns slots [64 j, 64 j + 64) of every
+// block into products (K-steps [4 j, 4 j + 4)) accumulated in O_j.
+//
+// What bounds it is each buffer's cycle logits -> exponentials -> products -> logits: a
+// block takes ~760 clocks where its exponentials need 512 of MUFU and a loop of loads,
+// exponentials and stores alone runs at 620 (synchronisation included, measured).  The
+// forward with single-level products (MODE 0, !PS) therefore runs three softmax warpgroups
+// (512 threads), one per S buffer, and hands each 64-slot half of the weights over as soon as
+// it is written, so that its products run under the other half's exponentials (N = 262,144,
+// H = 8, call: G = 1024 373 -> 355 us, G = 512 232 -> 211, G = 256 133 -> 118, against four
+// warpgroups on half rows).  Weights in a buffer of their own with two S buffers, which frees
+// S before the exponentials, was slower (375 with three warpgroups, 411 with four).  The other
+// modes need more registers: two warpgroups, warpgroup q % 2 taking block q.
 //
 // The same pass serves the backward (Sec. 3.3): with R_n = sum_g w_ng t_g,
 //   MODE 1 (deslice backward, t = z', v = dO): delta_n = dO_n . R_n (fp32);
@@ -87,16 +97,16 @@ constexpr uint32_t kDStage = kXBytes + 2 * kPxBytes;  // x tile, point extra (bo
 
 // X3 (fp32 inputs, MODE 0 with PS): each stage also holds x's residual tile
 // (xrmap), the logits add x_r W'_hi, and out is fp32.
-// The forward with single-level products (MODE 0, !PS) runs four softmax
-// warpgroups (640 threads): warpgroups 2p and 2p + 1 take the blocks q with
-// q % 2 == p, each one 64-slot half of every row, and half j's packed weights go to
-// columns [64 j, 64 j + 32) of the S buffer, where product issuer j reads them as
-// soon as half j is ready.  The other modes keep two warpgroups on whole rows.
 template <int MODE, bool PS>
-constexpr bool desl_wg4() { return MODE == 0 && !PS; }
-constexpr int kDesl4Threads = 640;
+constexpr bool desl_wg3() { return MODE == 0 && !PS; }
+constexpr int kDesl3Threads = 512;
+// Barriers of completed tiles.  With three warpgroups the one that drains tile t has not
+// waited for tile t - 2 (the accumulator's previous tile), and a parity wait on a barrier
+// two phases behind would pass at once; what it has seen (the logits of a block at most three
+// blocks back, so the products three blocks before that: tile t - 5) covers tile t - 8.
+constexpr int kOFull = 8;
 template <int MODE, bool PS, bool X3 = false>
-__global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThreads, 1)
+__global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThreads, 1)
     k_deslice(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap pmap,
               const __grid_constant__ CUtensorMap xrmap,
               const uint8_t* __restrict__ wimg, const uint8_t* __restrict__ zimg, __nv_bfloat16* __restrict__ out,
@@ -119,11 +129,11 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
   uint64_t* x_full = bars + 1;
   uint64_t* x_empty = x_full + kStages;
   uint64_t* s_full = x_empty + kStages;
-  constexpr bool kWG4 = desl_wg4<MODE, PS>();
-  uint64_t* p_ready = s_full + kSBuf;  // [kSBuf][2 halves] with four warpgroups, else [kSBuf]
+  constexpr bool kWG3 = desl_wg3<MODE, PS>();
+  uint64_t* p_ready = s_full + kSBuf;  // [S buffer][half] (two warpgroups: half 0 stands for both)
   uint64_t* pv_done = p_ready + 2 * kSBuf;
   uint64_t* o_full = pv_done + kSBuf;
-  uint64_t* o_free = o_full + 2;
+  uint64_t* o_free = o_full + kOFull;
   uint64_t* drain = o_free + 2;  // one per issuing warp
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 3);
   Abort* ab = reinterpret_cast<Abort*>(tmem_slot + 1);
@@ -134,6 +144,7 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
   const int h = (int)(wk.bh % H);
   const int nch = G / kGC;
   constexpr uint32_t kO = kSBuf * kGC;  // TMEM column base of the O accumulators
+  constexpr int kWGs = kWG3 ? 3 : 2;    // softmax warpgroups
   const int total = wk.ntiles * nch;
 
   if (threadIdx.x == 0) {
@@ -144,14 +155,12 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
     }
     for (int i = 0; i < kSBuf; i++) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&p_ready[2 * i], 4);  // the four warps of the warpgroup that owns the block (half)
+      mbar_init(&p_ready[2 * i], 4);  // the four warps of the warpgroup that owns the block
       mbar_init(&p_ready[2 * i + 1], 4);
       mbar_init(&pv_done[i], 2);
     }
-    for (int i = 0; i < 2; i++) {
-      mbar_init(&o_full[i], 2);
-      mbar_init(&o_free[i], 4);
-    }
+    for (int i = 0; i < kOFull; i++) mbar_init(&o_full[i], 2);
+    for (int i = 0; i < 2; i++) mbar_init(&o_free[i], 4);
     for (int i = 0; i < 3; i++) mbar_init(&drain[i], 1);
     ab->flag = 0;
     fence_mbar_init();
@@ -195,21 +204,28 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
     // Block q uses S buffer q % 3; it is rewritten only after the products of
     // block q - 3 (issued by the other warps) have completed.
     if (wk.ntiles > 0) {
-      const uint32_t sw = smem_u32(s_w), swe = sw + (uint32_t)G * 64;
+      const uint32_t w0 = sdesc_lo(smem_u32(s_w), 16), we0 = w0 + (uint32_t)G * 4;
+      const uint32_t wl0 = hilo ? w0 + (uint32_t)G * 6 : 0u, wl_step = hilo ? kGC * 4u : 0u;
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
-      BlockPos pos(0, nch);
-      for (int q = 0; ok && q < total; q++, pos.step(1, nch)) {
-        const int i = pos.i, c = pos.c;
-        const int s = i % kStages;
-        const int bb = q % kSBuf;
-        if (c == 0 && !(ok = mbar_wait_w(&x_full[s], (uint32_t)((i / kStages) & 1), ab, status))) break;
-        if (q >= kSBuf && !(ok = mbar_wait_w(&pv_done[bb], (uint32_t)(((q / kSBuf) - 1) & 1), ab, status))) break;
-        tc_fence_after();
-        const uint32_t xs = smem_u32(s_x + s * kDSt);
-        issue_logits(tmem + (uint32_t)bb * kGC, xs, point_extra_desc(xs + kXBytes), sw, swe,
-                     hilo ? sw + (uint32_t)G * 96 : 0u, c, true, X3 ? xs + kDStage : 0u);
-        mma_commit_w(&s_full[bb]);
-        if (c == nch - 1) mma_commit_w(&x_empty[s]);
+      Ring<kSBuf> sb;
+      Ring<kStages> st;
+      int q = 0;
+      for (int i = 0; ok && i < wk.ntiles; i++, st.next()) {
+        if (!(ok = mbar_wait_w(&x_full[st.i], st.pass, ab, status))) break;
+        const uint32_t xs = smem_u32(s_x + st.i * kDSt);
+        const uint32_t x = sdesc_lo(xs, 16), xe = point_extra_lo(xs + kXBytes);
+        const uint32_t xr = X3 ? sdesc_lo(xs + kDStage, 16) : 0u;
+        uint32_t w = w0, we = we0, wl = wl0;
+        for (int c = 0; c < nch; c++, q++, sb.next()) {
+          if (q >= kSBuf && !(ok = mbar_wait_w(&pv_done[sb.i], sb.pass ^ 1u, ab, status))) break;
+          tc_fence_after();
+          issue_logits<true, kHiPx>(tmem + (uint32_t)sb.i * kGC, x, xe, w, we, wl, xr);
+          mma_commit_w(&s_full[sb.i]);
+          w += kGC * 4;
+          we += kGC * 2;
+          wl += wl_step;
+        }
+        mma_commit_w(&x_empty[st.i]);
       }
       mma_commit_w(&drain[0]);
       mbar_wait_w(&drain[0], 0, ab, nullptr, kWaitNs);
@@ -219,40 +235,38 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
     const int j = warp - 2;  // K-steps [4j, 4j + 4) of every block, accumulator O_j
     if (wk.ntiles > 0) {
       constexpr uint32_t idesc_pv = idesc_bf16(128, kD, false, false);
-      const uint32_t sz = smem_u32(s_z);
+      // slots [64 j, 64 j + 64) of a block: 64-slot block 2 c + j of the Z' image
+      const uint32_t z0 = sdesc_lo(smem_u32(s_z) + (uint32_t)j * 4096, 16);
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
-      BlockPos pos(0, nch);
-      for (int q = 0; ok && q < total; q++, pos.step(1, nch)) {
-        const int i = pos.i, c = pos.c;
+      Ring<kSBuf> sb;
+      for (int i = 0; ok && i < wk.ntiles; i++) {
         const int ob = i & 1;
-        const int bb = q % kSBuf;
-        if (c == 0 && i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
-        if (!(ok = mbar_wait_w(&p_ready[kWG4 ? 2 * bb + j : 2 * bb], (uint32_t)((q / kSBuf) & 1), ab, status))) break;
-        tc_fence_after();
-        // weights of slots 64j.. (packed pairs; PS: hi pairs, then lo pairs 32 on)
-        const uint32_t tP = tmem + (uint32_t)bb * kGC + (uint32_t)j * ((kWG4 || PS) ? 64 : 32);
         const uint32_t tO = tmem + kO + (uint32_t)(j * 2 + ob) * kD;
+        if (i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
+        uint32_t z = z0;
+        for (int c = 0; c < nch; c++, z += 512, sb.next()) {
+          if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + (kWG3 ? j : 0)], sb.pass, ab, status))) break;
+          tc_fence_after();
+          // weights of slots 64j.. (packed pairs; PS: hi pairs, then lo pairs 32 on)
+          const uint32_t tP = tmem + (uint32_t)sb.i * kGC + (uint32_t)j * (PS ? 64 : 32);
 #pragma unroll
-        for (int kk = 0; kk < 4; kk++) {
-          const int g0 = c * kGC + (4 * j + kk) * 16;
-          const uint32_t zaddr = sz + (uint32_t)((g0 >> 6) * 4096 + (g0 & 63) * 2);
-          mma_ts_w(tO, tP + (uint32_t)kk * 8, sdesc(zaddr, 16, 1024, kSw128), idesc_pv, (c > 0 || kk > 0) ? 1u : 0u);
-          if (PS) {
-            mma_ts_w(tO, tP + 32 + (uint32_t)kk * 8, sdesc(zaddr, 16, 1024, kSw128), idesc_pv, 1u);
-            mma_ts_w(tO, tP + (uint32_t)kk * 8, sdesc(zaddr + (uint32_t)G * 64, 16, 1024, kSw128), idesc_pv, 1u);
+          for (int kk = 0; kk < 4; kk++) {
+            mma_ts_w<kHi128>(tO, tP + (uint32_t)kk * 8, z + kk * 2, idesc_pv, (c > 0 || kk > 0) ? 1u : 0u);
+            if (PS) {
+              mma_ts_w<kHi128>(tO, tP + 32 + (uint32_t)kk * 8, z + kk * 2, idesc_pv, 1u);
+              mma_ts_w<kHi128>(tO, tP + (uint32_t)kk * 8, z + (uint32_t)G * 4 + kk * 2, idesc_pv, 1u);
+            }
           }
+          mma_commit_w(&pv_done[sb.i]);
         }
-        mma_commit_w(&pv_done[bb]);
-        if (c == nch - 1) mma_commit_w(&o_full[ob]);
+        mma_commit_w(&o_full[i % kOFull]);
       }
       mma_commit_w(&drain[1 + j]);
       mbar_wait_w(&drain[1 + j], 0, ab, nullptr, kWaitNs);
     }
   } else if (warp >= kSoftmaxWarp0) {
     // ------------------------------ softmax warpgroups ------------------------------
-    const int wg4 = (warp - kSoftmaxWarp0) >> 2;
-    const int wg = kWG4 ? wg4 >> 1 : wg4;  // the block parity this warpgroup takes
-    const int hf = kWG4 ? wg4 & 1 : 0;     // four warpgroups: the half of each row
+    const int wg = (warp - kSoftmaxWarp0) >> 2;
     const int wq = warp & 3;  // TMEM sub-partition of this warp
     const int r = wq * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
@@ -260,7 +274,7 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
     // Output of tile t: O_0 + O_1 (fixed order) -> bf16 -> global, 64 B per point.
     auto epilogue = [&](int t) -> bool {
       const int ob = (int)(t & 1);
-      if (!mbar_wait(&o_full[ob], (uint32_t)((t >> 1) & 1), ab, status)) return false;
+      if (!mbar_wait(&o_full[t % kOFull], (uint32_t)((t / kOFull) & 1), ab, status)) return false;
       tc_fence_after();
       float R[kD];  // O_0 + O_1, in that order
       {
@@ -331,15 +345,23 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
       }
       wds_acc = 0.f;
     };
-    // Warpgroup wg takes the whole blocks q with q % 2 == wg, so the two warpgroups
-    // run half a block out of phase: one exponentiates while the other waits.
+    // Warpgroup wg takes the whole blocks q with q % kWGs == wg, so the warpgroups run
+    // out of phase: one exponentiates while another waits.
     BlockPos pos(wg, nch);
-    for (int q = wg; ok && q < total; q += 2, pos.step(2, nch)) {
+    for (int q = wg; ok && q < total; q += kWGs, pos.step(kWGs, nch)) {
       const int i = pos.i, c = pos.c;
-      const int bb = q % kSBuf;
+      const int bb = kWG3 ? wg : q % kSBuf;
       if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((q / kSBuf) & 1), ab, status))) break;
       tc_fence_after();
-      if (MODE == 2) {
+      if constexpr (kWG3) {
+        const uint32_t tS = tmem + lane_addr + (uint32_t)bb * kGC;
+        weights_half(tS, tS);
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_ready[2 * bb]);
+        weights_half(tS + 64, tS + 32);
+      } else if constexpr (MODE == 2) {
         if (i != wds_tile) {
           flush_wds();
           wds_tile = i;
@@ -349,24 +371,21 @@ __global__ void __launch_bounds__(desl_wg4<MODE, PS>() ? kDesl4Threads : kThread
           weights_hilo_half_ds(tmem + lane_addr + (uint32_t)bb * kGC + 64, s_ds + c * kGC + 64, wds_acc);
         } else
           weights_in_halves_ds(tmem + lane_addr + (uint32_t)bb * kGC, s_ds + c * kGC, wds_acc);
-      } else if (PS) {
+      } else if constexpr (PS) {
         weights_hilo_half(tmem + lane_addr + (uint32_t)bb * kGC);
         weights_hilo_half(tmem + lane_addr + (uint32_t)bb * kGC + 64);
-      } else if (kWG4) {
-        weights_half(tmem + lane_addr + (uint32_t)bb * kGC + (uint32_t)hf * 64);
       } else {
         weights_in_halves(tmem + lane_addr + (uint32_t)bb * kGC);
       }
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&p_ready[2 * bb + hf]);
-      // The output of the previous tile is drained by the warpgroup (half 0 of the
-      // pair) that took the first block of this tile, when the last products of that
-      // tile have long finished.
-      if (c == 0 && i > 0 && hf == 0 && !(ok = epilogue(i - 1))) break;
+      if (lane == 0) mbar_arrive(&p_ready[2 * bb + (kWG3 ? 1 : 0)]);
+      // The output of the previous tile is drained by the warpgroup that took the first
+      // block of this tile, when the last products of that tile have long finished.
+      if (c == 0 && i > 0 && !(ok = epilogue(i - 1))) break;
     }
-    if (ok && total > 0 && total % 2 == wg && hf == 0) epilogue(wk.ntiles - 1);
+    if (ok && total > 0 && total % kWGs == wg) epilogue(wk.ntiles - 1);
     if (ok) flush_wds();
   }
   tc_fence_before();
@@ -479,7 +498,8 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     const int j = warp - 1;
     const int nis = nch >= 2 ? 2 : 1;
     if (wk.ntiles > 0 && j < nis) {
-      const uint32_t sw = smem_u32(s_w), swe = sw + (uint32_t)G * 64;
+      const uint32_t w0 = sdesc_lo(smem_u32(s_w), 16), we0 = w0 + (uint32_t)G * 4;
+      const uint32_t wl0 = split ? w0 + (uint32_t)G * 6 : 0u, xe = const_extra_lo(smem_u32(s_ex));
       bool ok = mbar_wait_w(w_full, 0, ab, status);
       const int total = wk.ntiles * nch;
       BlockPos pos(j, nch);
@@ -491,8 +511,9 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
         if (q >= 2 && !(ok = mbar_wait_w(&s_free[bb], (uint32_t)(((q >> 1) - 1) & 1), ab, status))) break;
         tc_fence_after();
         const uint32_t xs = smem_u32(s_x + s * kXSt);
-        issue_logits(tmem + (uint32_t)bb * kGC, xs, const_extra_desc(smem_u32(s_ex)), sw, swe,
-                     split ? sw + (uint32_t)G * 96 : 0u, c, true, X3 ? xs + kXBytes : 0u);
+        issue_logits<true, kHi32>(tmem + (uint32_t)bb * kGC, sdesc_lo(xs, 16), xe, w0 + (uint32_t)c * (kGC * 4),
+                                  we0 + (uint32_t)c * (kGC * 2), split ? wl0 + (uint32_t)c * (kGC * 4) : 0u,
+                                  X3 ? sdesc_lo(xs + kXBytes, 16) : 0u);
         mma_commit_w(&s_full[bb]);
         if (c >= nch - nis) mma_commit_w(&x_empty[s]);
       }
@@ -662,7 +683,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap xrmap,
             const __grid_constant__ CUtensorMap frmap, const uint8_t* __restrict__ wimg, float* __restrict__ part,
             int64_t N, int64_t Np, int H, int G, int splits, uint32_t* status) {
-  constexpr int kNSt = X3 ? kSliceStages / 2 : kSliceStages;
+  constexpr int kSBuft = X3 ? kSliceStages / 2 : kSliceStages;
   constexpr uint32_t kStB = kStageBytes + (X3 ? kXBytes + 2 * kFBlock : 0u);
   constexpr uint32_t kXROff = kStageBytes, kFROff = kStageBytes + kXBytes;
   // split (FS_DOT_BF16X2): logits with both halves of W' (K = 80), and the
@@ -675,11 +696,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* s_w = smem;
   uint8_t* s_st = s_w + kWBlock;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_st + kNSt * kStB);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_st + kSBuft * kStB);
   uint64_t* w_full = bars;
   uint64_t* x_full = bars + 1;
-  uint64_t* st_empty = x_full + kNSt;
-  uint64_t* s_full = st_empty + kNSt;
+  uint64_t* st_empty = x_full + kSBuft;
+  uint64_t* s_full = st_empty + kSBuft;
   uint64_t* p_ready = s_full + kSBuf;   // [issuer][S buffer]
   uint64_t* pv_done = p_ready + 2 * kSBuf;
   uint64_t* acc_full = pv_done + kSBuf;
@@ -703,7 +724,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (threadIdx.x == 0) {
     mbar_init(w_full, 1);
-    for (int s = 0; s < kNSt; s++) {
+    for (int s = 0; s < kSBuft; s++) {
       mbar_init(&x_full[s], 1);
       mbar_init(&st_empty[s], 2);  // the logits issuer and the tile's product issuer
     }
@@ -721,9 +742,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     ab->flag = 0;
     fence_mbar_init();
   }
-  for (int s = 0; s < kNSt; s++) zero_smem(s_st + s * kStB + kPOff + kPxBytes, kPxBytes);
+  for (int s = 0; s < kSBuft; s++) zero_smem(s_st + s * kStB + kPOff + kPxBytes, kPxBytes);
   // Constant "ones" block of every stage: row n = [1, 0 x 15] (32B swizzle).
-  for (int idx = threadIdx.x; idx < kNSt * kTile; idx += kThreads) {
+  for (int idx = threadIdx.x; idx < kSBuft * kTile; idx += kThreads) {
     const int s = idx / kTile, r = idx % kTile;
     const uint32_t base = smem_u32(s_st + s * kStB + kFOff + 2 * kFBlock) +
                           (uint32_t)((r >> 3) * 256 + (r & 7) * 32);
@@ -756,9 +777,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (split) load_images(s_w + kGC * 96, src + (size_t)G * 96 + (size_t)g_base * 64, kGC * 64, w_full);
       int i = 0;
       for (; i < wk.ntiles; i++) {
-        const int s = i % kNSt;
-        if (i >= kNSt &&
-            !mbar_wait(&st_empty[s], (uint32_t)(((i / kNSt) - 1) & 1), ab, status))
+        const int s = i % kSBuft;
+        if (i >= kSBuft &&
+            !mbar_wait(&st_empty[s], (uint32_t)(((i / kSBuft) - 1) & 1), ab, status))
           break;
         uint8_t* st = s_st + s * kStB;
         const int n0 = (int)((wk.tile0 + i) * kTile);
@@ -773,38 +794,38 @@ __global__ void __launch_bounds__(kThreads, 1)
           tma_load_3d(st + kFROff + kFBlock, &frmap, h * kD + 16, n0, (int)b, &x_full[s]);
         }
       }
-      for (int j = (i > kNSt ? i - kNSt : 0); j < i; j++)
-        mbar_wait(&x_full[j % kNSt], (uint32_t)((j / kNSt) & 1), ab, nullptr, kWaitNs);
+      for (int j = (i > kSBuft ? i - kSBuft : 0); j < i; j++)
+        mbar_wait(&x_full[j % kSBuft], (uint32_t)((j / kSBuft) & 1), ab, nullptr, kWaitNs);
       mbar_wait(w_full, 0, ab, nullptr, kWaitNs);
     }
   } else if (warp == 1) {
     // ------------------------------ logits issuer (transposed) ------------------------------
     {
-      const uint32_t sw = smem_u32(s_w), swe = sw + kGC * 64;
+      const uint32_t w = sdesc_lo(smem_u32(s_w), 16), we = w + kGC * 4;
       bool ok = mbar_wait_w(w_full, 0, ab, status);
       if (kWT && ok) {
         ok = mbar_wait_w(wt_ready, 0, ab, status);
         tc_fence_after();
       }
-      for (int i = 0; ok && i < wk.ntiles; i++) {
-        const int s = i % kNSt;
-        const int bb = i % kSBuf;
-        if (!(ok = mbar_wait_w(&x_full[s], (uint32_t)((i / kNSt) & 1), ab, status))) break;
-        if (i >= kSBuf && !(ok = mbar_wait_w(&pv_done[bb], (uint32_t)(((i / kSBuf) - 1) & 1), ab, status))) break;
+      Ring<kSBuft> st;
+      Ring<kSBuf> sb;
+      for (int i = 0; ok && i < wk.ntiles; i++, st.next(), sb.next()) {
+        if (!(ok = mbar_wait_w(&x_full[st.i], st.pass, ab, status))) break;
+        if (i >= kSBuf && !(ok = mbar_wait_w(&pv_done[sb.i], sb.pass ^ 1u, ab, status))) break;
         tc_fence_after();
-        const uint32_t xs = smem_u32(s_st + s * kStB);
+        const uint32_t xs = smem_u32(s_st + st.i * kStB);
+        const uint32_t x = sdesc_lo(xs, 16), xe = point_extra_lo(xs + kPOff);
+        const uint32_t tD = tmem + (uint32_t)sb.i * kGC;
         if (kWT) {
           constexpr uint32_t idesc = idesc_bf16(128, kGC, false, false);
-          const uint32_t tD = tmem + (uint32_t)bb * kGC;
-          mma_ts_w(tD, tmem + kTW, sdesc(xs, 16, 512, kSw64), idesc, 0u);
-          mma_ts_w(tD, tmem + kTW + 8, sdesc(xs + 32, 16, 512, kSw64), idesc, 1u);
-          mma_ts_w(tD, tmem + kTW + 16, point_extra_desc(xs + kPOff), idesc, 1u);
+          mma_ts_w<kHi64>(tD, tmem + kTW, x, idesc, 0u);
+          mma_ts_w<kHi64>(tD, tmem + kTW + 8, x + 2, idesc, 1u);
+          mma_ts_w<kHiPx>(tD, tmem + kTW + 16, xe, idesc, 1u);
         } else {
-          issue_logits(tmem + (uint32_t)bb * kGC, xs, point_extra_desc(xs + kPOff), sw, swe,
-                       split ? sw + kGC * 96 : 0u, 0, false, X3 ? xs + kXROff : 0u);
+          issue_logits<false, kHiPx>(tD, x, xe, w, we, split ? w + kGC * 6 : 0u, X3 ? sdesc_lo(xs + kXROff, 16) : 0u);
         }
-        mma_commit_w(&s_full[bb]);
-        mma_commit_w(&st_empty[s]);
+        mma_commit_w(&s_full[sb.i]);
+        mma_commit_w(&st_empty[st.i]);
       }
       mma_commit_w(&drain[0]);
       mbar_wait_w(&drain[0], 0, ab, nullptr, kWaitNs);
@@ -815,34 +836,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     {
       constexpr uint32_t idesc_sl = idesc_bf16(128, 48, false, true);
       bool ok = true;
+      Ring<kSBuft> st;
+      Ring<kSBuf> sb;
+      uint32_t half = 0;  // parity of this issuer's uses of a buffer (its tiles there are 2 kSBuf apart)
+      if (j == 1) st.next(), sb.next();
       for (int i = j; ok && i < wk.ntiles; i += 2) {
-        const int s = i % kNSt;
-        const int bb = i % kSBuf;
-        // This issuer's tiles on buffer bb are 2 kSBuf apart.
-        if (!(ok = mbar_wait_w(&p_ready[j * kSBuf + bb], (uint32_t)((i / (2 * kSBuf)) & 1), ab, status))) break;
+        if (!(ok = mbar_wait_w(&p_ready[j * kSBuf + sb.i], half, ab, status))) break;
         tc_fence_after();
-        const uint32_t tE = tmem + (uint32_t)bb * kGC;  // packed weights of the 128 points
-        const uint32_t fs = smem_u32(s_st + s * kStB) + kFOff;
+        const uint32_t tE = tmem + (uint32_t)sb.i * kGC;  // packed weights of the 128 points
+        const uint32_t f = sdesc_lo(smem_u32(s_st + st.i * kStB) + kFOff, kFBlock);
+        const uint32_t fr = f - kFOff / 16 + kFROff / 16;
         const uint32_t tacc = tmem + kA + (uint32_t)j * 48;
         // A chain restarts at this issuer's first tile and at every flush tile (its
         // warpgroup has moved the earlier tiles' sums to registers by then).
         const bool fresh = i < 2 || slice_flush_at<split || X3>(i);
 #pragma unroll
         for (int kk = 0; kk < 8; kk++) {
-          const uint64_t fdesc = sdesc(fs + (uint32_t)kk * 512, kFBlock, 256, kSw32);
           // 16 points' packed weights: columns kk * 8, or with split products the hi
           // pairs of half kk / 4 at (kk / 4) * 64 + (kk % 4) * 8, their residuals 32 on
           const uint32_t tw = tE + (split ? (uint32_t)(kk >> 2) * 64 + (uint32_t)(kk & 3) * 8 : (uint32_t)kk * 8);
-          mma_ts_w(tacc, tw, fdesc, idesc_sl, (!fresh || kk > 0) ? 1u : 0u);
+          mma_ts_w<kHi32>(tacc, tw, f + kk * 32, idesc_sl, (!fresh || kk > 0) ? 1u : 0u);
           // The residual halves of the weights: U and S to ~2^-16.
-          if (split) mma_ts_w(tacc, tw + 32, fdesc, idesc_sl, 1u);
+          if (split) mma_ts_w<kHi32>(tacc, tw + 32, f + kk * 32, idesc_sl, 1u);
           if (X3)  // the weights against fx's residual half (U only)
-            mma_ts_w(tacc, tw, sdesc(fs - kFOff + kFROff + (uint32_t)kk * 512, kFBlock, 256, kSw32),
-                     idesc_bf16(128, 32, false, true), 1u);
+            mma_ts_w<kHi32>(tacc, tw, fr + kk * 32, idesc_bf16(128, 32, false, true), 1u);
         }
-        mma_commit_w(&pv_done[bb]);
-        mma_commit_w(&st_empty[s]);
+        mma_commit_w(&pv_done[sb.i]);
+        mma_commit_w(&st_empty[st.i]);
         if (split || X3) mma_commit_w(&acc_done[j]);
+        st.next(), st.next();
+        // kSBuf is odd: after each full pass over the ring the issuer has visited every buffer
+        // once, in an order that repeats every kSBuf of its tiles
+        sb.next(), sb.next();
+        if ((i >> 1) % kSBuf == kSBuf - 1) half ^= 1u;
       }
       if (ok) mma_commit_w(acc_full);
       mma_commit_w(&drain[1 + j]);
@@ -891,11 +917,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int bb = i % kSBuf;
       if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((i / kSBuf) & 1), ab, status))) break;
       tc_fence_after();
-      if (split) {
-        weights_hilo_half(tmem + lane_addr + (uint32_t)bb * kGC);
-        weights_hilo_half(tmem + lane_addr + (uint32_t)bb * kGC + 64);
+      const uint32_t tS = tmem + lane_addr + (uint32_t)bb * kGC;
+      if constexpr (split) {
+        weights_hilo_half(tS);
+        weights_hilo_half(tS + 64);
       } else {
-        weights_in_halves(tmem + lane_addr + (uint32_t)bb * kGC);
+        weights_in_halves(tS);
       }
       tmem_wait_st();
       if (i >= 2 && slice_flush_at<split || X3>(i)) {
@@ -1220,7 +1247,7 @@ cudaError_t tc_deslice_fwd(const Shape& s0, const void* x, const float* W, const
     else
       k_prep_z<<<(unsigned)((nz + 255) / 256), 256, 0, st>>>(zk, zimg, s.BH(), G, s.G);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    kernel<<<dim3((unsigned)P, (unsigned)s.BH()), x3 ? kThreads : kDesl4Threads, sm, st>>>(
+    kernel<<<dim3((unsigned)P, (unsigned)s.BH()), x3 ? kThreads : kDesl3Threads, sm, st>>>(
         xmap, pmap, xrmap, wimg, zimg, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr, s.N, Np,
         s.H, s.G, P, hilo ? 1 : 0, (uint32_t)s.G * (ps ? 128 : 64), k > 0 ? 1 : 0, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -223,20 +223,30 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
 // issues a small tcgen05.mma in ~25 cycles, a lone lane inside a divergent branch
 // in ~50-130.  With the full mask elect.sync picks the same lane every time, so
 // that lane's commits cover every MMA the warp issued.
-__device__ __forceinline__ void mma_ss_w(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+//
+// Operands in shared memory are given by the low word of their descriptor (address and
+// leading offset), which the issue loops keep in a register and advance by additions; the
+// high word (stride, version, swizzle) is a constant of the instruction.  Building both
+// words anew per MMA put ~40 clocks between two MMAs next to busy softmax warps: four
+// N = 32 products took 207 clocks to issue, with advanced low words 108.
+template <uint32_t kAHi, uint32_t kBHi>
+__device__ __forceinline__ void mma_ss_w(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, e;\n .reg .b64 a, b;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+      " setp.ne.b32 p, %6, 0;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_lo), "n"(kAHi), "r"(b_lo), "n"(kBHi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void mma_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+template <uint32_t kBHi>
+__device__ __forceinline__ void mma_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, e;\n .reg .b64 b;\n mov.b64 b, {%2, %3};\n"
+      " setp.ne.b32 p, %5, 0;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b_lo), "n"(kBHi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit_w(uint64_t* bar) {
@@ -252,18 +262,34 @@ __device__ __forceinline__ bool mbar_wait_w(uint64_t* bar, uint32_t parity, Abor
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, ab, status, limit_ns));
 }
 
-// Shared-memory matrix descriptor (tcgen05 format).
+// Shared-memory matrix descriptor (tcgen05 format) as its two words.
 //   swizzle: 0 none, 2 128B, 4 64B, 6 32B.  lbo/sbo in bytes.
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo, uint32_t swizzle) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version for tcgen05
-  d |= (uint64_t)(swizzle & 7u) << 61;
-  return d;
+// A low word plus n moves the operand by 16 n bytes (shared memory ends below 2^18).
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr, uint32_t lbo) {
+  return ((saddr & 0x3FFFFu) >> 4) | (((lbo >> 4) & 0x3FFFu) << 16);
+}
+constexpr uint32_t sdesc_hi(uint32_t sbo, uint32_t swizzle) {
+  return ((sbo >> 4) & 0x3FFFu) | (1u << 14) /* descriptor version for tcgen05 */ | (swizzle << 29);
 }
 constexpr uint32_t kSw128 = 2, kSw64 = 4, kSw32 = 6;
+// The operand layouts in use: 64B- and 32B-swizzled K-major rows (x, W', T; extra blocks),
+// the unswizzled point-extra rows, 128B-swizzled channel rows (Z', W'^T), and MN-major
+// tiles ([F | 1] blocks: 32B swizzle; x, dO tiles: 64B swizzle).
+constexpr uint32_t kHi64 = sdesc_hi(512, kSw64), kHi32 = sdesc_hi(256, kSw32), kHiPx = sdesc_hi(128, 0),
+                   kHi128 = sdesc_hi(1024, kSw128);
+
+// Position in a ring of N buffers and the parity of the pass over it, without divisions.
+template <int N>
+struct Ring {
+  int i = 0;
+  uint32_t pass = 0;
+  __device__ __forceinline__ void next() {
+    if (++i == N) {
+      i = 0;
+      pass ^= 1u;
+    }
+  }
+};
 
 // Instruction descriptor for kind::f16 with bf16 A/B and fp32 D.
 //   a_mn / b_mn: operand is MN-major (else K-major).
