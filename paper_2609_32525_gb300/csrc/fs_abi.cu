@@ -131,12 +131,12 @@ Regions regions(const Shape& s, int op) {
       r.tc = take(tc_deslice_prep_bytes(s));
       break;
     case FS_OP_SLICE_BWD:
-      r.dus = take(BHG * (s.d + 1) * sizeof(float));
       if (tc_backward_supported(s)) {
         r.stats = take(pts * sizeof(float));
         r.tc = take(std::max(tc_backward_bytes(s, 2), tc_deslice_prep_bytes(s)));
         break;
       }
+      r.dus = take(BHG * (s.d + 1) * sizeof(float));
       r.delta = take(pts * sizeof(float));
       r.partials = take((size_t)P * BHG * (s.d + 2) * sizeof(float));
       r.dtau_p = take((size_t)s.BH() * simt_point_blocks(s) * sizeof(float));
@@ -145,7 +145,6 @@ Regions regions(const Shape& s, int op) {
       break;
     case FS_OP_COUPLING_BWD:
       if (tc_backward_supported(s)) {
-        r.dus = take(BHG * (s.d + 1) * sizeof(float));
         r.stats = take(pts * sizeof(float));
         r.tc = take(std::max(tc_coupling_bwd_bytes(s), tc_deslice_prep_bytes(s)));
         break;
@@ -179,7 +178,8 @@ fs_status check_ws(const Shape& s, int op, void* ws, size_t ws_bytes) {
 
 fs_status cuda_status(cudaError_t e) { return e == cudaSuccess ? FS_OK : FS_ERR_CUDA; }
 
-// Every ws-using call starts by clearing its status word.
+// Every ws-using call starts by clearing its status word: the tensor-core calls in their
+// first kernel (the preparation), the others with a memset.
 cudaError_t reset_status(void* ws, cudaStream_t st) { return cudaMemsetAsync(ws, 0, sizeof(uint32_t), st); }
 
 // The backward forms its weights from fp32 logits, so it needs lse to ~1e-5.  On
@@ -191,7 +191,12 @@ cudaError_t reset_status(void* ws, cudaStream_t st) { return cudaMemsetAsync(ws,
 // backward computes them.
 cudaError_t backward_stats(const Shape& sh, const void* x_mid, const float* W_slice, const float* bias,
                            const float* tau, const float* lse, void* ws, const Regions& r, uint32_t* status,
-                           cudaStream_t st, const float** lse_use) {
+                           cudaStream_t st, const float** lse_use, bool* reset) {
+  // *reset: the status word is still to be cleared by the call's next launch (a SIMT backward
+  // has no preparation that could).
+  *reset = tc_backward_supported(sh);
+  if (!*reset)
+    if (cudaError_t e = reset_status(ws, st)) return e;
   *lse_use = lse;
   // fp32 shapes take the fp32 SIMT backward: it gets exact fp32 statistics (the
   // forward's come from split bf16 products on the tensor cores).
@@ -200,10 +205,16 @@ cudaError_t backward_stats(const Shape& sh, const void* x_mid, const float* W_sl
   if (lse && !fp32_tc && (!tc || sh.dot == FS_DOT_BF16X2)) return cudaSuccess;
   float* buf = at<float>(ws, r.stats);
   *lse_use = buf;
-  if (!tc) return simt_stats(sh, x_mid, W_slice, bias, tau, buf, status, st);
+  const bool clear = *reset;
+  *reset = false;
+  if (!tc) {
+    if (clear)
+      if (cudaError_t e = reset_status(ws, st)) return e;
+    return simt_stats(sh, x_mid, W_slice, bias, tau, buf, status, st);
+  }
   Shape split = sh;
   split.dot = FS_DOT_BF16X2;
-  return tc_stats(split, x_mid, W_slice, bias, tau, buf, at<void>(ws, r.tc), status, st);
+  return tc_stats(split, x_mid, W_slice, bias, tau, buf, at<void>(ws, r.tc), clear, status, st);
 }
 
 #define FS_CHECK_SHAPE(s)                               \
@@ -309,11 +320,11 @@ fs_status fs_slice_fwd(const fs_shape* s, const void* x_mid, const void* fx, con
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint32_t* status = at<uint32_t>(ws, r.status);
   float* lse_buf = lse ? lse : at<float>(ws, r.stats);
-  FS_CUDA(reset_status(ws, st));
   if (tc_forward_supported(sh)) {
     return cuda_status(tc_slice_fwd(sh, x_mid, fx, W_slice, bias, tau, tokens, wsum, lse_buf, finalize,
-                                    at<float>(ws, r.partials), at<void>(ws, r.tc), status, st));
+                                    at<float>(ws, r.partials), at<void>(ws, r.tc), true, status, st));
   }
+  FS_CUDA(reset_status(ws, st));
   const int P = slot_splits(sh);
   float* part = at<float>(ws, r.partials);
   FS_CUDA(simt_stats(sh, x_mid, W_slice, bias, tau, lse_buf, status, st));
@@ -331,9 +342,9 @@ fs_status fs_stats(const fs_shape* s, const void* x_mid, const float* W_slice, c
   const Regions r = regions(sh, FS_OP_STATS);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint32_t* status = at<uint32_t>(ws, r.status);
-  FS_CUDA(reset_status(ws, st));
   if (tc_forward_supported(sh))
-    return cuda_status(tc_stats(sh, x_mid, W_slice, bias, tau, lse, at<void>(ws, r.tc), status, st));
+    return cuda_status(tc_stats(sh, x_mid, W_slice, bias, tau, lse, at<void>(ws, r.tc), true, status, st));
+  FS_CUDA(reset_status(ws, st));
   return cuda_status(simt_stats(sh, x_mid, W_slice, bias, tau, lse, status, st));
 }
 
@@ -348,10 +359,10 @@ fs_status fs_slice_fwd_lse(const fs_shape* s, const void* x_mid, const void* fx,
   const Regions r = regions(sh, FS_OP_SLICE_FWD);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint32_t* status = at<uint32_t>(ws, r.status);
-  FS_CUDA(reset_status(ws, st));
   if (tc_forward_supported(sh))
     return cuda_status(tc_slice_fwd_lse(sh, x_mid, fx, W_slice, bias, tau, lse, tokens, wsum, finalize,
-                                        at<float>(ws, r.partials), at<void>(ws, r.tc), status, st));
+                                        at<float>(ws, r.partials), at<void>(ws, r.tc), true, status, st));
+  FS_CUDA(reset_status(ws, st));
   const int P = slot_splits(sh);
   float* part = at<float>(ws, r.partials);
   FS_CUDA(simt_slice_partials(sh, P, x_mid, fx, W_slice, bias, tau, lse, part, status, st));
@@ -405,17 +416,18 @@ fs_status fs_deslice_fwd(const fs_shape* s, const void* x_mid, const float* W_sl
   const Regions r = regions(sh, FS_OP_DESLICE_FWD);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint32_t* status = at<uint32_t>(ws, r.status);
+  float* buf = at<float>(ws, r.stats);
+  if (tc_forward_supported(sh)) {
+    if (!lse) FS_CUDA(tc_stats(sh, x_mid, W_slice, bias, tau, buf, at<void>(ws, r.tc), true, status, st));
+    return cuda_status(tc_deslice_fwd(sh, x_mid, W_slice, bias, tau, tokens_mixed, lse ? lse : buf, out,
+                                      at<void>(ws, r.tc), lse != nullptr, status, st));
+  }
   FS_CUDA(reset_status(ws, st));
   const float* lse_use = lse;
   if (!lse_use) {
-    float* buf = at<float>(ws, r.stats);
-    if (tc_forward_supported(sh)) FS_CUDA(tc_stats(sh, x_mid, W_slice, bias, tau, buf, at<void>(ws, r.tc), status, st));
-    else FS_CUDA(simt_stats(sh, x_mid, W_slice, bias, tau, buf, status, st));
+    FS_CUDA(simt_stats(sh, x_mid, W_slice, bias, tau, buf, status, st));
     lse_use = buf;
   }
-  if (tc_forward_supported(sh))
-    return cuda_status(tc_deslice_fwd(sh, x_mid, W_slice, bias, tau, tokens_mixed, lse_use, out,
-                                      at<void>(ws, r.tc), status, st));
   return cuda_status(simt_deslice(sh, x_mid, W_slice, bias, tau, tokens_mixed, lse_use, out, status, st));
 }
 
@@ -432,12 +444,12 @@ fs_status fs_deslice_bwd(const fs_shape* s, const void* x_mid, const float* W_sl
   if (fs_status e = check_ws(sh, FS_OP_DESLICE_BWD, ws, ws_bytes)) return e;
   const Regions r = regions(sh, FS_OP_DESLICE_BWD);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  FS_CUDA(reset_status(ws, st));
   const float* lse_use = nullptr;
-  FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, at<uint32_t>(ws, r.status), st, &lse_use));
+  bool reset = true;
+  FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, at<uint32_t>(ws, r.status), st, &lse_use, &reset));
   if (tc_backward_supported(sh))
     return cuda_status(tc_deslice_bwd(sh, x_mid, W_slice, bias, tau, tokens_mixed, lse_use, dout, d_tokens_mixed,
-                                      dx_mid, dW, dbias, dtau, accumulate, at<void>(ws, r.tc),
+                                      dx_mid, dW, dbias, dtau, accumulate, at<void>(ws, r.tc), reset,
                                       at<uint32_t>(ws, r.status), st));
   return cuda_status(simt_deslice_bwd(sh, slot_splits(sh), x_mid, W_slice, bias, tau, tokens_mixed, lse_use, dout,
                                       d_tokens_mixed, dx_mid, dW, dbias, dtau, accumulate, at<float>(ws, r.delta),
@@ -468,12 +480,12 @@ fs_status fs_slice_bwd(const fs_shape* s, const void* x_mid, const void* fx, con
   if (fs_status e = check_ws(sh, FS_OP_SLICE_BWD, ws, ws_bytes)) return e;
   const Regions r = regions(sh, FS_OP_SLICE_BWD);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  FS_CUDA(reset_status(ws, st));
   const float* lse_use = nullptr;
-  FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, at<uint32_t>(ws, r.status), st, &lse_use));
+  bool reset = true;
+  FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, at<uint32_t>(ws, r.status), st, &lse_use, &reset));
   if (tc_backward_supported(sh))
     return cuda_status(tc_slice_bwd(sh, x_mid, fx, W_slice, bias, tau, tokens, wsum, lse_use, d_tokens, dx_mid, dfx,
-                                    dW, dbias, dtau, accumulate, at<float>(ws, r.dus), at<void>(ws, r.tc),
+                                    dW, dbias, dtau, accumulate, at<void>(ws, r.tc), reset,
                                     at<uint32_t>(ws, r.status), st));
   return cuda_status(simt_slice_bwd(sh, slot_splits(sh), x_mid, fx, W_slice, bias, tau, tokens, wsum, lse_use,
                                     d_tokens, dx_mid, dfx, dW, dbias, dtau, accumulate, at<float>(ws, r.delta),
@@ -502,9 +514,9 @@ fs_status fs_coupling_bwd(const fs_shape* s, const void* x_mid, const void* fx, 
     const Regions r = regions(sh, FS_OP_COUPLING_BWD);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     uint32_t* status = at<uint32_t>(ws, r.status);
-    FS_CUDA(reset_status(ws, st));
     const float* lse_use = nullptr;
-    FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, status, st, &lse_use));
+    bool reset = true;
+    FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, status, st, &lse_use, &reset));
     return cuda_status(simt_coupling_bwd(sh, slot_splits(sh), x_mid, fx, dout, W_slice, bias, tau, M, tokens, wsum,
                                          tokens_mixed, lse_use, d_tokens_mixed, d_tokens, dM, dx_mid, dfx, dW, dbias,
                                          dtau, accumulate, at<float>(ws, r.delta), at<float>(ws, r.dus),
@@ -512,12 +524,12 @@ fs_status fs_coupling_bwd(const fs_shape* s, const void* x_mid, const void* fx, 
   }
   const Regions r = regions(sh, FS_OP_COUPLING_BWD);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  FS_CUDA(reset_status(ws, st));
   const float* lse_use = nullptr;
-  FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, at<uint32_t>(ws, r.status), st, &lse_use));
+  bool reset = true;
+  FS_CUDA(backward_stats(sh, x_mid, W_slice, bias, tau, lse, ws, r, at<uint32_t>(ws, r.status), st, &lse_use, &reset));
   return cuda_status(tc_coupling_bwd(sh, x_mid, fx, dout, W_slice, bias, tau, M, tokens, wsum, tokens_mixed, lse_use,
                                      d_tokens_mixed, d_tokens, dM, dx_mid, dfx, dW, dbias, dtau, accumulate,
-                                     at<float>(ws, r.dus), at<void>(ws, r.tc), at<uint32_t>(ws, r.status), st));
+                                     at<void>(ws, r.tc), reset, at<uint32_t>(ws, r.status), st));
 }
 
 fs_status fs_device_status(const void* ws, fs_stream_t stream) {

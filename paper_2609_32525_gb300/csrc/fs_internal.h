@@ -51,6 +51,9 @@ cudaError_t simt_mix(const Shape& s, const float* M, const float* z, float* zp, 
 cudaError_t simt_mix_channels(const Shape& s, const float* Wc, const float* z, float* zp, cudaStream_t st);
 cudaError_t simt_mix_channels_bwd(const Shape& s, const float* Wc, const float* z, const float* dzp, float* dz,
                                   float* dWc, cudaStream_t st);
+// simt_mix_bwd in one launch.
+cudaError_t mix_bwd(const Shape& s, const float* M, const float* z, const float* dzp, float* dz, float* dM,
+                    cudaStream_t st);
 cudaError_t simt_mix_bwd(const Shape& s, const float* M, const float* z, const float* dzp,
                          float* dz, float* dM, cudaStream_t st);
 cudaError_t simt_deslice(const Shape& s, const void* x, const float* W, const float* bias,
@@ -71,7 +74,10 @@ cudaError_t simt_slice_bwd_prep(const Shape& s, const float* z, const float* wsu
 cudaError_t simt_reduce_bwd(const Shape& s, int P, const float* part, int Gs, int PS, int has_dzp, const float* tau,
                             float* dzp, float* dW, float* db, float* dtau, const float* dt_part, int64_t nblk,
                             int accumulate, cudaStream_t st);
-// The token gradient alone from partials whose first d words per slot are dz'.
+// simt_reduce_bwd in one launch (dzp null: partials without the token gradient).
+cudaError_t reduce_bwd(const Shape& s, int P, const float* part, int Gs, int PS, const float* tau, float* dzp,
+                       float* dW, float* db, float* dtau, const float* dt_part, int64_t nblk, int accumulate,
+                       cudaStream_t st);
 // The coupling's whole backward on the SIMT kernels (fs_coupling_bwd on shapes the
 // tensor-core backward does not take); delta, dUS, part, dt_part as in the calls above
 // (part holds P * B*H * G * (d + 2) floats).
@@ -82,6 +88,7 @@ cudaError_t simt_coupling_bwd(const Shape& s, int P, const void* x, const void* 
                               float* delta, float* dUS, float* part, float* dt_part, uint32_t* status,
                               cudaStream_t st);
 int simt_coupling_bwd_launch_count();
+// The token gradient alone from partials whose first d words per slot are dz'.
 cudaError_t simt_reduce_dzp(const Shape& s, int P, const float* part, int Gs, int PS, float* dzp, cudaStream_t st);
 cudaError_t simt_slice_bwd(const Shape& s, int P, const void* x, const void* f, const float* W,
                            const float* bias, const float* tau, const float* z,

@@ -87,15 +87,17 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+template <bool kTrans>
+constexpr int mix_words() { return kMixStages * (mix_a_words<kTrans>() + kMixKC * kMixTC); }
+
+// Tile (gx, bh, cx) of the product, with mix_words() floats of shared memory.
 template <bool kTrans, bool kVec>
-__global__ void __launch_bounds__(256) k_mix_tiled(const float* __restrict__ M, const float* __restrict__ in,
-                                                   float* __restrict__ out, int H, int G, int D) {
+__device__ __forceinline__ void mix_tile(float* sm, const float* __restrict__ M, const float* __restrict__ in,
+                                         float* __restrict__ out, int H, int G, int D, int gx, int64_t bh, int cx) {
   constexpr int TG = kMixTG, TC = kMixTC, KC = kMixKC, S = kMixStages;
   constexpr int AW = mix_a_words<kTrans>(), BW = KC * TC, SW = AW + BW;
-  __shared__ __align__(16) float sm[S * SW];
-  const int64_t bh = blockIdx.y;
   const int h = (int)(bh % H);
-  const int g0 = blockIdx.x * TG, c0 = blockIdx.z * TC;
+  const int g0 = gx * TG, c0 = cx * TC;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const float* Mh = M + (int64_t)h * G * G;
   const float* X = in + bh * (int64_t)G * D;
@@ -207,6 +209,12 @@ __global__ void __launch_bounds__(256) k_mix_tiled(const float* __restrict__ M, 
     if (g0 + g < G && c0 + c < D) out[(bh * G + g0 + g) * (int64_t)D + c0 + c] = v;
   }
 }
+template <bool kTrans, bool kVec>
+__global__ void __launch_bounds__(256) k_mix_tiled(const float* __restrict__ M, const float* __restrict__ in,
+                                                   float* __restrict__ out, int H, int G, int D) {
+  __shared__ __align__(16) float sm[mix_words<kTrans>()];
+  mix_tile<kTrans, kVec>(sm, M, in, out, H, G, D, blockIdx.x, blockIdx.y, blockIdx.z);
+}
 static_assert(8 * kMixTG * kMixTC <= kMixStages * (kMixKC * kMixTC + kMixTG * (kMixKC + 4)),
               "the partial tiles fit in the staging buffers");
 
@@ -246,13 +254,15 @@ __global__ void k_mix_channels_dW(const float* __restrict__ z, const float* __re
 // K = B*D, tiled 64 x 64 per block (16 x 16 threads, 4 x 4 outputs each), the two
 // operand tiles staged in shared memory 16 channels at a time; the sum runs over
 // b, then c, in a fixed order.
-__global__ void __launch_bounds__(256) k_mix_bwd_dM(const float* __restrict__ z, const float* __restrict__ dzp,
-                                                    float* __restrict__ dM, int64_t B, int H, int G, int D) {
-  constexpr int T = 64, KC = 16;
-  __shared__ float sa[KC][T + 1];
-  __shared__ float sb[KC][T + 1];
-  const int h = blockIdx.z;
-  const int g0 = blockIdx.y * T, k0 = blockIdx.x * T;
+constexpr int kDmT = 64, kDmKC = 16;
+constexpr int kDmWords = 2 * kDmKC * (kDmT + 1);
+__device__ __forceinline__ void dM_tile(float* sm, const float* __restrict__ z, const float* __restrict__ dzp,
+                                        float* __restrict__ dM, int64_t B, int H, int G, int D, int kx, int gx,
+                                        int h) {
+  constexpr int T = kDmT, KC = kDmKC;
+  float(*sa)[T + 1] = reinterpret_cast<float(*)[T + 1]>(sm);
+  float(*sb)[T + 1] = sa + KC;
+  const int g0 = gx * T, k0 = kx * T;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   float acc[4][4] = {};
   for (int64_t b = 0; b < B; b++) {
@@ -293,20 +303,53 @@ __global__ void __launch_bounds__(256) k_mix_bwd_dM(const float* __restrict__ z,
   }
 }
 
-// Token-gradient prep for the slice backward: dUS[bh][g] = (dz_g/(S_g+eps), -(dz_g.z_g)/(S_g+eps)).
-__global__ void k_slice_bwd_prep(const float* __restrict__ z, const float* __restrict__ wsum,
-                                 const float* __restrict__ dz, float* __restrict__ dUS, int64_t BHG, int D,
-                                 float eps) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= BHG) return;
+__global__ void __launch_bounds__(256) k_mix_bwd_dM(const float* __restrict__ z, const float* __restrict__ dzp,
+                                                    float* __restrict__ dM, int64_t B, int H, int G, int D) {
+  __shared__ float sm[kDmWords];
+  dM_tile(sm, z, dzp, dM, B, H, G, D, blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// Both halves of the mix backward in one launch: blocks [0, nx * BH * nc) the tiles of
+// dz = M^T dz' (gx fastest, then bh), the rest dM's.
+template <bool kVec>
+__global__ void __launch_bounds__(256) k_mix_bwd(const float* __restrict__ M, const float* __restrict__ z,
+                                                 const float* __restrict__ dzp, float* __restrict__ dz,
+                                                 float* __restrict__ dM, int64_t B, int H, int G, int D, int nx,
+                                                 int nc) {
+  constexpr int kWords = mix_words<true>() > kDmWords ? mix_words<true>() : kDmWords;
+  __shared__ __align__(16) float sm[kWords];
+  const int64_t n = (int64_t)nx * B * H * nc;
+  int64_t i = blockIdx.x;
+  if (i < n) {
+    const int gx = (int)(i % nx);
+    i /= nx;
+    mix_tile<true, kVec>(sm, M, dzp, dz, H, G, D, gx, i % (B * H), (int)(i / (B * H)));
+    return;
+  }
+  i -= n;
+  const int nt = (G + kDmT - 1) / kDmT;
+  dM_tile(sm, z, dzp, dM, B, H, G, D, (int)(i % nt), (int)((i / nt) % nt), (int)(i / ((int64_t)nt * nt)));
+}
+
+// Token-gradient prep for the slice backward: dUS[bh][g] = (dz_g/(S_g+eps),
+// -(dz_g.z_g)/(S_g+eps)).  A warp per slot row (a thread per row read 32-word rows word by
+// word: 20 us at 2,048 rows, 5 us this way).
+__global__ void __launch_bounds__(256) k_slice_bwd_prep(const float* __restrict__ z, const float* __restrict__ wsum,
+                                                        const float* __restrict__ dz, float* __restrict__ dUS,
+                                                        int64_t BHG, int D, float eps) {
+  const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= BHG) return;  // whole warps
   const float den = wsum[i] + eps;
   float s = 0.f;
-  for (int c = 0; c < D; c++) {
+  for (int c = lane; c < D; c += 32) {
     const float g = dz[i * D + c];
     dUS[i * (D + 1) + c] = g / den;
     s = fmaf(g, z[i * D + c], s);
   }
-  dUS[i * (D + 1) + D] = -s / den;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) dUS[i * (D + 1) + D] = -s / den;
 }
 
 // Fixed-order reduction of slot-owned backward partials over (b, p), one thread
@@ -314,18 +357,20 @@ __global__ void k_slice_bwd_prep(const float* __restrict__ z, const float* __res
 //   k_reduce_bwd_params: dW[h][k][g], db[h][g] (written, or added), sums over b then p;
 //   k_reduce_bwd_tokens: d_tokens_mixed[b][h][g][c], sums over p.
 // The temperature gradient is reduced separately, from its own partials.
-__global__ void k_reduce_bwd_params(const float* __restrict__ part, int P, int64_t B, int H, int G, int Gs, int D,
-                                    int PS, int off, const float* __restrict__ tau, float* __restrict__ dW,
-                                    float* __restrict__ db, int accumulate) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void reduce_params(int64_t idx, const float* __restrict__ part, int P, int64_t B, int H,
+                                              int G, int Gs, int D, int PS, int off, const float* __restrict__ tau,
+                                              float* __restrict__ dW, float* __restrict__ db, int accumulate) {
   if (idx >= (int64_t)H * G * (D + 1)) return;
   const int k = (int)(idx % (D + 1));
   const int64_t hg = idx / (D + 1);
   const int h = (int)(hg / G), g = (int)(hg % G);
   const int64_t BH = B * H;
   float s = 0.f;
-  for (int64_t b = 0; b < B; b++)
-    for (int p = 0; p < P; p++) s += part[(((int64_t)p * BH + b * H + h) * Gs + g) * PS + off + k];
+  for (int64_t b = 0; b < B; b++) {
+    const float* src = part + ((b * H + h) * Gs + g) * PS + off + k;
+#pragma unroll 4
+    for (int p = 0; p < P; p++) s += src[(int64_t)p * BH * Gs * PS];
+  }
   s *= 1.f / tau[h];
   if (k < D) {
     const int64_t o = ((int64_t)h * D + k) * G + g;
@@ -334,24 +379,22 @@ __global__ void k_reduce_bwd_params(const float* __restrict__ part, int P, int64
     db[hg] = (accumulate ? db[hg] : 0.f) + s;
   }
 }
-__global__ void k_reduce_bwd_tokens(const float* __restrict__ part, int P, int64_t BH, int G, int Gs, int D, int PS,
-                                    float* __restrict__ dzp) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void reduce_dzp(int64_t idx, const float* __restrict__ part, int P, int64_t BH, int G,
+                                           int Gs, int D, int PS, float* __restrict__ dzp) {
   if (idx >= BH * G * D) return;
   const int c = (int)(idx % D);
   const int64_t i = idx / D;                  // output row bh * G + g
   const int64_t row = (i / G) * Gs + i % G;  // its partial row
   float s = 0.f;
+#pragma unroll 4
   for (int p = 0; p < P; p++) s += part[((int64_t)p * BH * Gs + row) * PS + c];
   dzp[idx] = s;
 }
-
 // dtau[h] (+)= -(1/tau_h) * sum over batches and point blocks of the block sums of
-// sum_g da (a - lse) (fixed order: strided per thread, then a tree).
-__global__ void k_reduce_dtau(const float* __restrict__ dt_part, int64_t B, int H, int64_t nblk,
-                              const float* __restrict__ tau, float* __restrict__ dtau, int accumulate) {
+// sum_g da (a - lse) (fixed order: strided per thread, then a tree).  256 threads.
+__device__ __forceinline__ void reduce_dtau(int h, const float* __restrict__ dt_part, int64_t B, int H, int64_t nblk,
+                                            const float* __restrict__ tau, float* __restrict__ dtau, int accumulate) {
   __shared__ float s[256];
-  const int h = blockIdx.x;
   float v = 0.f;
   for (int64_t b = 0; b < B; b++)
     for (int64_t i = threadIdx.x; i < nblk; i += 256) v += dt_part[(b * H + h) * nblk + i];
@@ -362,6 +405,33 @@ __global__ void k_reduce_dtau(const float* __restrict__ dt_part, int64_t B, int 
     __syncthreads();
   }
   if (threadIdx.x == 0) dtau[h] = (accumulate ? dtau[h] : 0.f) - s[0] / tau[h];
+}
+
+__global__ void __launch_bounds__(256) k_reduce_bwd_params(const float* part, int P, int64_t B, int H, int G, int Gs,
+                                                           int D, int PS, int off, const float* tau, float* dW,
+                                                           float* db, int accumulate) {
+  reduce_params((int64_t)blockIdx.x * 256 + threadIdx.x, part, P, B, H, G, Gs, D, PS, off, tau, dW, db, accumulate);
+}
+__global__ void __launch_bounds__(256) k_reduce_bwd_tokens(const float* part, int P, int64_t BH, int G, int Gs, int D,
+                                                           int PS, float* dzp) {
+  reduce_dzp((int64_t)blockIdx.x * 256 + threadIdx.x, part, P, BH, G, Gs, D, PS, dzp);
+}
+__global__ void __launch_bounds__(256) k_reduce_dtau(const float* dt_part, int64_t B, int H, int64_t nblk,
+                                                     const float* tau, float* dtau, int accumulate) {
+  reduce_dtau(blockIdx.x, dt_part, B, H, nblk, tau, dtau, accumulate);
+}
+// All of a backward call's reductions in one launch: blocks [0, n_par) dW and dbias,
+// [n_par, n_par + H) dtau, the rest d z' (dzp may be null).
+__global__ void __launch_bounds__(256) k_reduce_bwd(const float* part, int P, int64_t B, int H, int G, int Gs, int D,
+                                                    int PS, const float* tau, float* dzp, float* dW, float* db,
+                                                    float* dtau, const float* dt_part, int64_t nblk, int accumulate,
+                                                    int64_t n_par) {
+  int64_t blk = blockIdx.x;
+  if (blk < n_par)
+    return reduce_params(blk * 256 + threadIdx.x, part, P, B, H, G, Gs, D, PS, dzp ? D : 0, tau, dW, db, accumulate);
+  blk -= n_par;
+  if (blk < H) return reduce_dtau((int)blk, dt_part, B, H, nblk, tau, dtau, accumulate);
+  reduce_dzp((blk - H) * 256 + threadIdx.x, part, P, B * H, G, Gs, D, PS, dzp);
 }
 
 }  // namespace
@@ -384,6 +454,27 @@ cudaError_t simt_reduce_bwd(const Shape& s, int P, const float* part, int Gs, in
   return cudaGetLastError();
 }
 
+cudaError_t reduce_bwd(const Shape& s, int P, const float* part, int Gs, int PS, const float* tau, float* dzp,
+                       float* dW, float* db, float* dtau, const float* dt_part, int64_t nblk, int accumulate,
+                       cudaStream_t st) {
+  const int64_t n_par = ((int64_t)s.H * s.G * (s.d + 1) + 255) / 256;
+  const int64_t n = n_par + s.H + (dzp ? (s.BH() * s.G * s.d + 255) / 256 : 0);
+  k_reduce_bwd<<<(unsigned)n, 256, 0, st>>>(part, P, s.B, s.H, s.G, Gs, s.d, PS, tau, dzp, dW, db, dtau, dt_part, nblk,
+                                            accumulate, n_par);
+  return cudaGetLastError();
+}
+
+cudaError_t mix_bwd(const Shape& s, const float* M, const float* z, const float* dzp, float* dz, float* dM,
+                    cudaStream_t st) {
+  const int nx = (s.G + kMixTG - 1) / kMixTG, nc = (s.d + kMixTC - 1) / kMixTC, nt = (s.G + kDmT - 1) / kDmT;
+  const int64_t n = (int64_t)nx * s.BH() * nc + (int64_t)nt * nt * s.H;
+  if (s.G % 4 == 0)
+    k_mix_bwd<true><<<(unsigned)n, 256, 0, st>>>(M, z, dzp, dz, dM, s.B, s.H, s.G, s.d, nx, nc);
+  else
+    k_mix_bwd<false><<<(unsigned)n, 256, 0, st>>>(M, z, dzp, dz, dM, s.B, s.H, s.G, s.d, nx, nc);
+  return cudaGetLastError();
+}
+
 cudaError_t simt_reduce_dzp(const Shape& s, int P, const float* part, int Gs, int PS, float* dzp, cudaStream_t st) {
   const int64_t BHG = s.BH() * s.G;
   k_reduce_bwd_tokens<<<(unsigned)((BHG * s.d + 255) / 256), 256, 0, st>>>(part, P, s.BH(), s.G, Gs, s.d, PS, dzp);
@@ -393,7 +484,7 @@ cudaError_t simt_reduce_dzp(const Shape& s, int P, const float* part, int Gs, in
 cudaError_t simt_slice_bwd_prep(const Shape& s, const float* z, const float* wsum, const float* dz, float* dUS,
                                 cudaStream_t st) {
   const int64_t BHG = s.BH() * s.G;
-  k_slice_bwd_prep<<<(unsigned)((BHG + 255) / 256), 256, 0, st>>>(z, wsum, dz, dUS, BHG, s.d, s.eps);
+  k_slice_bwd_prep<<<(unsigned)((BHG + 7) / 8), 256, 0, st>>>(z, wsum, dz, dUS, BHG, s.d, s.eps);
   return cudaGetLastError();
 }
 

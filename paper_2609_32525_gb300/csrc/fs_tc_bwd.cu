@@ -30,58 +30,59 @@ constexpr uint32_t kWBlockB = kGC * kWRow;             // one 128-slot block of 
 
 // ---- prep kernels ------------------------------------------------------------------------------
 
-// T image of (b,h), in the W image's layout (kWRow bytes per slot): t_g rounded to
-// bf16, the extra rows [c_hi, c_lo, 1, 1, 1, 0...] (k = 2..4 meet -delta's three
-// parts), the residual t_g - bf16(t_g).
-// t: [BH][G][tstride] fp32, c_g = t[..][32] when has_c.  Also writes c_g to c_out
-// [BH][Gp].  Padding slots [G, Gp) get t = 0 and c = 0 (their weights are 0).
-__global__ void k_prep_t(const float* __restrict__ t, int tstride, int has_c, uint8_t* __restrict__ img,
-                         float* __restrict__ c_out, int64_t BH, int G, int Gp) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= BH * Gp) return;
-  const int64_t bh = i / Gp;
-  const int g = (int)(i % Gp);
-  const bool real = g < G;
-  const float* src = t + (bh * G + (real ? g : 0)) * tstride;
-  uint8_t* base = img + (size_t)bh * Gp * kWRow;
-  __nv_bfloat16* hp = reinterpret_cast<__nv_bfloat16*>(base);
-  __nv_bfloat16* lp = reinterpret_cast<__nv_bfloat16*>(base + (size_t)Gp * 96);
-  for (int k = 0; k < kD; k++) {
-    const float v = real ? src[k] : 0.f;
-    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-    hp[off_sw64(g, k) / 2] = hi;
-    lp[off_sw64(g, k) / 2] = __float2bfloat16_rn(v - __bfloat162float(hi));
+// The slice's token gradients as images: per (b,h) and slot, u_g = dz_g / (S_g + eps) and
+// c_g = -(dz_g . z_g) / (S_g + eps).  T image in the W image's layout (kWRow bytes per slot):
+// u rounded to bf16, the extra rows [c_hi, c_lo, 1, 1, 1, 0...] (k = 2..4 meet -delta's three
+// parts), the residuals; the Z-layout image of u (hi, then residual); c itself.  Padding
+// slots [G, Gp) get u = 0 and c = 0 (their weights are 0).
+// A block takes 64 slots of one (b,h): a warp per slot row, then 16-byte pieces of the images
+// from shared memory.
+__global__ void __launch_bounds__(256) k_prep_us(const float* __restrict__ z, const float* __restrict__ wsum,
+                                                 const float* __restrict__ dz, uint8_t* __restrict__ timg,
+                                                 uint8_t* __restrict__ zimg, float* __restrict__ c_out, int G, int Gp,
+                                                 float eps) {
+  __shared__ float su[64][kD + 1];
+  const int64_t bh = blockIdx.y;
+  const int g0 = blockIdx.x * 64, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint8_t* base = timg + (size_t)bh * Gp * kWRow;
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    const int w = warp * 8 + i, g = g0 + w;
+    const bool real = g < G;
+    const int64_t row = (bh * G + (real ? g : 0)) * kD + lane;
+    const float d = real ? dz[row] : 0.f;
+    const float den = real ? wsum[bh * G + g] + eps : 1.f;
+    float s = real ? d * z[row] : 0.f;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    su[w][lane] = d / den;
+    if (lane == 0) {
+      const float c = -s / den;
+      c_out[bh * Gp + g] = c;
+      const uint32_t hi = pack_bf16(c, 0.f) & 0xFFFFu;
+      const uint32_t lo = pack_bf16(c - __uint_as_float(hi << 16), 0.f) & 0xFFFFu;
+      uint8_t* ep = base + (size_t)Gp * 64;
+      *reinterpret_cast<uint4*>(ep + off_sw32(g, 0)) = make_uint4(hi | (lo << 16), 0x3F803F80u, 0x3F80u, 0u);
+      *reinterpret_cast<uint4*>(ep + off_sw32(g, 8)) = make_uint4(0u, 0u, 0u, 0u);
+    }
   }
-  const float c = (has_c && real) ? src[kD] : 0.f;
-  if (c_out) c_out[i] = c;
-  const __nv_bfloat16 chi = __float2bfloat16_rn(c);
-  const __nv_bfloat16 clo = __float2bfloat16_rn(c - __bfloat162float(chi));
-  __nv_bfloat16* ep = reinterpret_cast<__nv_bfloat16*>(base + (size_t)Gp * 64);
-  for (int k = 0; k < 16; k++)
-    ep[off_sw32(g, k) / 2] = k == 0 ? chi : (k == 1 ? clo : __float2bfloat16_rn((k >= 2 && k <= 4) ? 1.f : 0.f));
-}
-
-// W'^T image of head h in the Z layout (channel rows, slots along K), W' =
-// W log2(e)/tau: the bf16 half, then the residual half (Gp*128 bytes per head;
-// padding slots zero).  It is the B operand of dx += da W'^T.
-__global__ void k_prep_wt(const float* __restrict__ W, const float* __restrict__ tau, uint8_t* __restrict__ img,
-                          int H, int G, int Gp, uint32_t* status) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)H * kD * Gp) return;
-  const int g = (int)(i % Gp);
-  const int c = (int)((i / Gp) % kD);
-  const int h = (int)(i / ((int64_t)kD * Gp));
-  const float tv = tau[h];
-  if (!(tv > 0.f && tv < INFINITY)) {
-    atomicCAS(status, 0u, (uint32_t)FS_ERR_BAD_TAU);
-    return;
+  __syncthreads();
+  {
+    const int w = threadIdx.x >> 2, q = threadIdx.x & 3;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) v[e] = su[w][8 * q + e];
+    const uint32_t off = off_sw64(g0 + w, 8 * q);
+    split8(v, *reinterpret_cast<uint4*>(base + off), *reinterpret_cast<uint4*>(base + (size_t)Gp * 96 + off));
   }
-  const float v = g < G ? W[((int64_t)h * kD + c) * G + g] * (kLog2e / tv) : 0.f;
-  __nv_bfloat16* hp = reinterpret_cast<__nv_bfloat16*>(img + (size_t)h * Gp * 128);
-  __nv_bfloat16* lp = reinterpret_cast<__nv_bfloat16*>(img + (size_t)h * Gp * 128 + (size_t)Gp * 64);
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  hp[off_z(c, g) / 2] = hi;
-  lp[off_z(c, g) / 2] = __float2bfloat16_rn(v - __bfloat162float(hi));
+  {
+    const int c = threadIdx.x & 31, w8 = threadIdx.x >> 5;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) v[e] = su[w8 * 8 + e][c];
+    uint8_t* zi = zimg + (size_t)bh * Gp * 128 + off_z(c, g0 + w8 * 8);
+    split8(v, *reinterpret_cast<uint4*>(zi), *reinterpret_cast<uint4*>(zi + (size_t)Gp * 64));
+  }
 }
 
 // delta's point-extra rows [1, 1, -delta in three bf16 parts, 0, 0, 0] into dpx [BH, Np, 8];
@@ -622,7 +623,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // =========================================================================================
-// Point pass: dx_n = ln2 * sum_g da_ng W'_g (W' = W log2(e)/tau).  CTA (split, bh)
+// Point pass: dx_n = ln2 * sum_g da_ng W'_g (W' = W log2(e)/tau) over slots [g0, g0 + G) of
+// images of Gi slots; accumulate: added to what dx holds.  CTA (split, bh)
 // walks its point tiles; block q is (tile q / nb, 64-slot chunk q % nb).  Warp 1
 // forms L (x tile vs W rows) and dw - delta (v tile vs T rows), M = 128 points,
 // N = 64 slots, into set q % 3; softmax warpgroup q % 2 writes da in place (hi, lo
@@ -645,7 +647,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const __grid_constant__ CUtensorMap fmap, const uint8_t* __restrict__ wimg,
                 const uint8_t* __restrict__ timg, const uint8_t* __restrict__ timg2,
                 const uint8_t* __restrict__ wtimg, __nv_bfloat16* __restrict__ dx, int64_t N, int64_t Np, int H,
-                int G, int splits, int hilo, int accumulate, uint32_t* status) {
+                int Gi, int g0, int G, int splits, int hilo, int accumulate, uint32_t* status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr uint32_t kStg = kBStage + (kComb ? kXBytes : 0u);  // x | v | px | dpx [| fx]
@@ -713,10 +715,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       prefetch_tmap(&dmap);
       if (kComb) prefetch_tmap(&fmap);
       mbar_expect_tx(wz_full, wbytes + (uint32_t)G * 96 * (kComb ? 2u : 1u) + (uint32_t)G * 64);
-      load_images(s_w, wimg + (size_t)h * G * kWRow, wbytes, wz_full);
-      load_images(s_t, timg + (size_t)wk.bh * G * kWRow, (uint32_t)G * 96, wz_full);
-      if (kComb) load_images(s_t2, timg2 + (size_t)wk.bh * G * kWRow, (uint32_t)G * 96, wz_full);
-      load_images(s_wt, wtimg + (size_t)h * G * 128, (uint32_t)G * 64, wz_full);
+      load_slots(s_w, wimg + (size_t)h * Gi * kWRow, Gi, g0, G, hilo, wz_full);
+      load_slots(s_t, timg + (size_t)wk.bh * Gi * kWRow, Gi, g0, G, false, wz_full);
+      if (kComb) load_slots(s_t2, timg2 + (size_t)wk.bh * Gi * kWRow, Gi, g0, G, false, wz_full);
+      load_images(s_wt, wtimg + (size_t)h * Gi * 128 + (size_t)g0 * 64, (uint32_t)G * 64, wz_full);
       int i = 0;
       for (; i < wk.ntiles; i++) {
         const int s = i % kDxStages;
@@ -885,26 +887,27 @@ size_t smem_bwd_dx(int G, bool hilo, bool comb = false) {
 int bwd_slot_blocks(const Shape& s) { return s.G / kGC; }
 int bwd_slot_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * bwd_slot_blocks(s))); }
 
-// Slot ranges.  The point pass holds three images of its slots in shared memory,
-// which fits up to kBwdSlotsMax slots.  A larger G runs every pass over ranges of
-// `size` slots (a multiple of 128; the last range may hold fewer real slots), all
-// with the full problem's lse, so that the weights of a range are those of the
-// softmax over all G.  The sums over slots (delta, dfx, dx) add up over the
-// ranges; the slot-owned gradients of a range are its own.  `size` minimises the
-// padded slots plus half a block per range (a range re-reads x and v); ties go to
-// the larger size.
-constexpr int kBwdSlotsMax = 640;
+// Slot ranges.  The images of a call cover all of its slots; the rows and point passes, which
+// hold images in shared memory (a rows pass W' and t with their residuals, the point pass
+// W', W'^T and one T image, in fs_coupling_bwd two), run over ranges of at most so many
+// slots, all with the full problem's lse, so that the weights of a range are those of the
+// softmax over all G.  The sums over slots (delta, dfx, dx) add up over the ranges.  The slot
+// pass holds one 128-slot block and needs no ranges.  As few ranges as fit (a range re-reads
+// x and v), of equal size but for the last.
+// (The separate calls' point pass holds the residual half of W' up to 512 slots: past 640,
+// where it runs over ranges anyway, no range is longer, which keeps dx of a sum over many
+// ranges accurate.)
+constexpr int kBwdSlotsMax = 640, kCombSlotsMax = 256, kPointSlotsMax = 512;
 struct SlotRanges {
   int n, size;
 };
-SlotRanges slot_ranges(int G) {
-  if (G <= kBwdSlotsMax) return {1, (G + kGC - 1) / kGC * kGC};
-  SlotRanges best{0, 0};
-  for (int size = kGC; size <= kBwdSlotsMax; size += kGC) {
-    const int n = (G + size - 1) / size;
-    if (best.n == 0 || (int64_t)n * (size + kGC / 2) <= (int64_t)best.n * (best.size + kGC / 2)) best = {n, size};
-  }
-  return best;
+SlotRanges slot_ranges(int Gp, int most) {
+  const int n = (Gp + most - 1) / most;
+  return {n, (Gp / kGC + n - 1) / n * kGC};
+}
+
+SlotRanges point_ranges(int Gp, bool comb) {
+  return slot_ranges(Gp, comb ? kCombSlotsMax : (Gp <= kBwdSlotsMax ? kBwdSlotsMax : kPointSlotsMax));
 }
 
 // The backward forms every weight with split products whatever the forward's
@@ -916,21 +919,16 @@ Shape split_shape(const Shape& s) {
   r.dot = FS_DOT_BF16X2;
   return r;
 }
+// The shape the passes see: split products, whole 128-slot blocks.
+Shape pass_shape(const Shape& s0) { return tc_padded(split_shape(s0)); }
 
-// The shape the passes see: split products, G = the slot range.
-Shape pass_shape(const Shape& s0) {
-  Shape s = split_shape(s0);
-  s.G = slot_ranges(s0.G).size;
-  return s;
-}
+enum BwdKind { kDesliceBwd = 1, kSliceBwd = 2, kCouplingBwd = 3 };
 
 // Workspace layout of one tensor-core backward call (offsets from the tc region).
-// With several slot ranges it also holds a range's slice of W, bias and t (wc, bc,
-// tc) and its slot-owned gradients (dwc, dbc, dzc) before they go to their places.
 struct BwdLayout {
-  size_t wimg, wtimg, timg, zimg, px, dpx, delta, wds, ds, dtp, part, wc, bc, tc, dwc, dbc, dzc, total;
+  size_t wimg, wtimg, timg, timg2, zimg, px, dpx, delta, delta_d, wds, ds, dtp, part, sl_part, sl_wsum, total;
 };
-BwdLayout bwd_layout(const Shape& s0, int mode) {
+BwdLayout bwd_layout(const Shape& s0, BwdKind kind) {
   BwdLayout L{};
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -942,435 +940,121 @@ BwdLayout bwd_layout(const Shape& s0, int mode) {
   const size_t BHG = (size_t)s.BH() * s.G;
   const size_t pts = (size_t)s.BH() * s.N;
   const int P = bwd_slot_splits(s), R = bwd_slot_blocks(s);
+  const bool comb = kind == kCouplingBwd;
   L.wimg = take(w_image_bytes(s));
   L.wtimg = take((size_t)s.H * s.G * 128);
   L.timg = take(BHG * kWRow);
+  L.timg2 = take(comb ? BHG * kWRow : 0);
   L.zimg = take(BHG * 128);
   L.px = take(px_bytes(s));
   L.dpx = take(px_bytes(s));
   L.delta = take(pts * sizeof(float));
-  L.wds = take(mode == 2 ? 2 * pts * sizeof(float) : 0);
+  L.delta_d = take(comb ? pts * sizeof(float) : 0);
+  L.wds = take(kind != kDesliceBwd ? 2 * pts * sizeof(float) : 0);
   L.ds = take(BHG * sizeof(float));
   L.dtp = take((size_t)s.BH() * P * R * sizeof(float));
-  L.part = take((size_t)P * BHG * (mode == 1 ? 2 * kD + 2 : kD + 2) * sizeof(float));
-  const size_t rs = slot_ranges(s0.G).n > 1 ? (size_t)s.G : 0;
-  L.wc = take((size_t)s.H * kD * rs * sizeof(float));
-  L.bc = take((size_t)s.H * rs * sizeof(float));
-  L.tc = take((size_t)s.BH() * rs * (kD + 1) * sizeof(float));
-  L.dwc = take((size_t)s.H * kD * rs * sizeof(float));
-  L.dbc = take((size_t)s.H * rs * sizeof(float));
-  L.dzc = take(mode == 1 ? (size_t)s.BH() * rs * kD * sizeof(float) : 0);
+  L.part = take((size_t)P * BHG * (kind == kDesliceBwd ? 2 * kD + 2 : kD + 2) * sizeof(float));
+  // d z' of the coupling through the forward's slice
+  const bool via_slice = comb && tc_forward_supported(split_shape(s0));
+  L.sl_part = take(via_slice ? tc_slice_partials_bytes(split_shape(s0)) : 0);
+  L.sl_wsum = take(via_slice ? (size_t)s.BH() * s0.G * sizeof(float) : 0);
   L.total = off;
   return L;
 }
 
-bool make_maps(const Shape& s, const void* x, const void* v, const void* px, const void* dpx, CUtensorMap* xmap,
-               CUtensorMap* vmap, CUtensorMap* pmap, CUtensorMap* dmap) {
-  const int64_t Np = padded_n(s);
-  return make_point_map(xmap, x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B) &&
-         make_point_map(vmap, v, s, kD, CU_TENSOR_MAP_SWIZZLE_64B) && make_px_map(pmap, px, s.BH(), Np) &&
-         make_px_map(dmap, dpx, s.BH(), Np);
-}
+// The passes of a call on its layout.
+struct BwdCall {
+  const Shape &s0, s;  // the caller's shape; the padded one
+  const BwdLayout L;
+  uint8_t* ws;
+  uint32_t* status;
+  cudaStream_t st;
+  BwdCall(const Shape& s0_, BwdKind kind, void* w, uint32_t* status_, cudaStream_t st_)
+      : s0(s0_), s(pass_shape(s0_)), L(bwd_layout(s0_, kind)), ws(static_cast<uint8_t*>(w)), status(status_), st(st_) {}
+  float* f(size_t off) const { return reinterpret_cast<float*>(ws + off); }
 
-// Slot-side images of t (T image, its c column, Z-layout image) for G slots.
-cudaError_t prep_t_images(const Shape& s, int G, const float* t, int tstride, int has_c, uint8_t* ws,
-                          const BwdLayout& L, cudaStream_t st) {
-  const int64_t BHG = s.BH() * s.G;
-  k_prep_t<<<(unsigned)((BHG + 127) / 128), 128, 0, st>>>(t, tstride, has_c, ws + L.timg,
-                                                            reinterpret_cast<float*>(ws + L.ds), s.BH(), G, s.G);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_prep_z2<<<(unsigned)((BHG * kD + 255) / 256), 256, 0, st>>>(t, tstride, ws + L.zimg, s.BH(), G, s.G);
-  return cudaGetLastError();
-}
-
-// One backward call: mode 1 (deslice; t = z', v = dO, writes dzp) or 2 (slice; t =
-// dU | dS with tstride 33, v = fx, writes dfx).  t: [BH][G][tstride] fp32.
-//   1. lse rows; for each slot range: its images, then the rows pass (delta, dfx
-//      and the wds partials add up over the ranges);
-//   2. delta's rows; for each slot range: the slot pass, its reduction into the
-//      range's dW, dbias, dtau (and dz') partials, and the point pass (dx; skipped
-//      when dx is null).
-// delta_out: where delta goes (null: the layout's own buffer).
-cudaError_t run_backward(const Shape& s0, int mode, const void* x, const void* v, const float* W,
-                         const float* bias, const float* tau, const float* t, int tstride, const float* lse,
-                         void* dfx, void* dx, float* dzp, float* dW, float* db, float* dtau, int accumulate,
-                         uint8_t* ws, uint32_t* status, cudaStream_t st, float* delta_out = nullptr) {
-  const SlotRanges sr = slot_ranges(s0.G);
-  const Shape s = pass_shape(s0);
-  const BwdLayout L = bwd_layout(s0, mode);
-  const bool ranged = sr.n > 1;
-  const int64_t Np = padded_n(s);
-  const int64_t npx = s.BH() * Np;
-  const int has_c = mode == 2 ? 1 : 0;
-  cudaError_t e;
-  auto range_g = [&](int k) { return k < sr.n - 1 ? sr.size : s0.G - (sr.n - 1) * sr.size; };
-
-  // Images of range k: t's, W's (and W'^T's when wt).
-  auto prep_range = [&](int k, bool wt) -> cudaError_t {
-    const int g0 = k * sr.size, G = range_g(k);
-    const float *Wk = W, *bk = bias, *tk = t;
-    cudaError_t r;
-    if (ranged) {
-      float* wc = reinterpret_cast<float*>(ws + L.wc);
-      float* bc = reinterpret_cast<float*>(ws + L.bc);
-      float* tc = reinterpret_cast<float*>(ws + L.tc);
-      if ((r = copy_rows(wc, G, W + g0, s0.G, G, (int64_t)s.H * kD, st)) != cudaSuccess) return r;
-      if ((r = copy_rows(bc, G, bias + g0, s0.G, G, s.H, st)) != cudaSuccess) return r;
-      if ((r = copy_rows(tc, (int64_t)G * tstride, t + (int64_t)g0 * tstride, (int64_t)s0.G * tstride,
-                         (int64_t)G * tstride, s.BH(), st)) != cudaSuccess)
-        return r;
-      Wk = wc, bk = bc, tk = tc;
-    }
-    if ((r = prep_t_images(s, G, tk, tstride, has_c, ws, L, st)) != cudaSuccess) return r;
-    if ((r = prep_w(s, G, Wk, bk, tau, ws + L.wimg, status, st)) != cudaSuccess) return r;
-    if (wt) {
-      const int64_t nwt = (int64_t)s.H * kD * s.G;
-      k_prep_wt<<<(unsigned)((nwt + 255) / 256), 256, 0, st>>>(Wk, tau, ws + L.wtimg, s.H, G, s.G, status);
-      r = cudaGetLastError();
-    }
-    return r;
-  };
-
-  k_prep_px<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(lse, reinterpret_cast<uint4*>(ws + L.px), s.BH(), s.N,
-                                                             Np);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  float* delta = delta_out ? delta_out : reinterpret_cast<float*>(ws + L.delta);
-  float* wds = mode == 2 ? reinterpret_cast<float*>(ws + L.wds) : nullptr;
-  if (wds && (e = cudaMemsetAsync(wds, 0, 2 * (size_t)s.BH() * s.N * sizeof(float), st)) != cudaSuccess) return e;
-  for (int k = 0; k < sr.n; k++) {
-    if ((e = prep_range(k, false)) != cudaSuccess) return e;
-    if ((e = tc_rows_bwd(s, mode, x, ws + L.wimg, ws + L.zimg, ws + L.px, v, dfx, delta, wds,
-                         reinterpret_cast<const float*>(ws + L.ds), k > 0 ? 1 : 0, status, st)) != cudaSuccess)
-      return e;
-  }
-  k_prep_dpx<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(delta, nullptr, wds,
-                                                              reinterpret_cast<uint4*>(ws + L.dpx), s.BH(), s.N, Np);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-
-  CUtensorMap xmap, vmap, pmap, dmap;
-  if (!make_maps(s, x, v, ws + L.px, ws + L.dpx, &xmap, &vmap, &pmap, &dmap)) return cudaErrorInvalidValue;
-  const int R = bwd_slot_blocks(s), P = bwd_slot_splits(s);
-  for (int k = 0; k < sr.n; k++) {
-    const int g0 = k * sr.size, G = range_g(k);
-    // The images of the last range are still in place after the rows passes; W'^T
-    // (for the point pass, when dx is wanted) is not.
-    if (ranged) {
-      if ((e = prep_range(k, dx != nullptr)) != cudaSuccess) return e;
-    } else if (dx) {
-      const int64_t nwt = (int64_t)s.H * kD * s.G;
-      k_prep_wt<<<(unsigned)((nwt + 255) / 256), 256, 0, st>>>(W, tau, ws + L.wtimg, s.H, G, s.G, status);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    {
-      const size_t sm = smem_bwd_slot(mode);
-      const auto kernel = mode == 1 ? k_bwd_slot_tc<1, true> : k_bwd_slot_tc<2, true>;
-      if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
-      kernel<<<dim3((unsigned)R, (unsigned)P, (unsigned)s.BH()), kThreads, sm, st>>>(
-          xmap, vmap, pmap, dmap, xmap, ws + L.wimg, ws + L.timg, nullptr, reinterpret_cast<float*>(ws + L.part),
-          reinterpret_cast<float*>(ws + L.dtp), s.N, Np, s.H, s.G, P, status);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    // The slot-owned gradients of range k: straight into dW, dbias (and dz') with
-    // one range; else into the range's buffers (holding dW, dbias's values when
-    // they are added to), then to their places.  dtau sums over the ranges.
-    const int acc = accumulate || k > 0;
-    Shape sk = s0;
-    sk.G = G;
-    float *dWk = dW, *dbk = db, *dzk = dzp;
-    if (ranged) {
-      dWk = reinterpret_cast<float*>(ws + L.dwc);
-      dbk = reinterpret_cast<float*>(ws + L.dbc);
-      dzk = mode == 1 ? reinterpret_cast<float*>(ws + L.dzc) : nullptr;
-      if (accumulate) {
-        if ((e = copy_rows(dWk, G, dW + g0, s0.G, G, (int64_t)s.H * kD, st)) != cudaSuccess) return e;
-        if ((e = copy_rows(dbk, G, db + g0, s0.G, G, s.H, st)) != cudaSuccess) return e;
-      } else if (acc) {
-        if ((e = cudaMemsetAsync(dWk, 0, (size_t)s.H * kD * G * sizeof(float), st)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(dbk, 0, (size_t)s.H * G * sizeof(float), st)) != cudaSuccess) return e;
-      }
-    }
-    if ((e = simt_reduce_bwd(sk, P, reinterpret_cast<const float*>(ws + L.part), s.G,
-                             mode == 1 ? 2 * kD + 2 : kD + 2, mode == 1 ? 1 : 0, tau, dzk, dWk, dbk, dtau,
-                             reinterpret_cast<const float*>(ws + L.dtp), (int64_t)P * R, acc, st)) != cudaSuccess)
-      return e;
-    if (ranged) {
-      if ((e = copy_rows(dW + g0, s0.G, dWk, G, G, (int64_t)s.H * kD, st)) != cudaSuccess) return e;
-      if ((e = copy_rows(db + g0, s0.G, dbk, G, G, s.H, st)) != cudaSuccess) return e;
-      if (mode == 1 && (e = copy_rows(dzp + (int64_t)g0 * kD, (int64_t)s0.G * kD, dzk, (int64_t)G * kD,
-                                      (int64_t)G * kD, s.BH(), st)) != cudaSuccess)
+  // delta and, mode 2, dfx and the sums of w dS, over the slot ranges; zimg holds t.
+  cudaError_t rows(int mode, const void* x, const void* v, void* dfx, float* delta) const {
+    const SlotRanges r = slot_ranges(s.G, kBwdSlotsMax);
+    for (int k = 0; k < r.n; k++) {
+      const int g0 = k * r.size;
+      Shape sr = s;
+      sr.G = std::min(r.size, s.G - g0);
+      if (cudaError_t e = tc_rows_bwd(sr, s.G, g0, mode, x, ws + L.wimg, ws + L.zimg, ws + L.px, v, dfx, delta,
+                                      mode == 2 ? f(L.wds) : nullptr, f(L.ds), k > 0 ? 1 : 0, status, st))
         return e;
-    }
-    if (dx) {
-      const bool hilo = smem_bwd_dx(s.G, true) <= kMaxSmem;
-      const size_t sm = smem_bwd_dx(s.G, hilo);
-      const int Pd = point_splits(s, (int)s.BH());
-      const auto kernel = k_bwd_dx_tc<true>;
-      if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
-      kernel<<<dim3((unsigned)Pd, (unsigned)s.BH()), kThreads, sm, st>>>(
-          xmap, vmap, pmap, dmap, xmap, ws + L.wimg, ws + L.timg, nullptr, ws + L.wtimg,
-          static_cast<__nv_bfloat16*>(dx), s.N, Np, s.H, s.G, Pd, hilo ? 1 : 0, acc, status);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-  }
-  return cudaSuccess;
-}
-
-// The coupling's backward in one call (fs_coupling_bwd).  The deslice's and the
-// slice's da share the weights, so their slot-owned and point-owned products can be
-// formed once from da_D + da_S; what has to come first is d z' (it feeds the mix
-// backward, and so dU, dS and the slice's part).  Per slot range (as in the separate
-// calls):
-//   1. the deslice part's rows pass: delta_D;
-//   2. d z' = sum_n w_ng dO_n: the forward's slice with dO for fx (its unnormalised
-//      numerators) where the forward's kernels take the shape, else the slot pass in
-//      mode 0 (the weights alone);
-//   3. the mix backward and the dU | dS prologue;
-//   4. the slice part's rows pass: delta_S, dfx, the sum_g w dS partials;
-//   5. delta = delta_S + delta_D + sum_g w dS into the point rows;
-//   6. the slot pass in mode 3: dW, dbias, dtau of da_D + da_S;
-//   7. one point pass (k_bwd_dx_tc<., true>) for dx, over ranges of at most 256
-//      slots (it holds two T images besides W' and W'^T).
-constexpr int kCombSlotsMax = 256;
-SlotRanges comb_ranges(const Shape& s0) {
-  const int cap = std::min(kCombSlotsMax, pass_shape(s0).G);
-  const int Gp = (s0.G + kGC - 1) / kGC * kGC;
-  if (Gp <= cap) return {1, Gp};
-  SlotRanges best{0, 0};
-  for (int size = kGC; size <= cap; size += kGC) {
-    const int n = (s0.G + size - 1) / size;
-    if (best.n == 0 || (int64_t)n * (size + kGC / 2) <= (int64_t)best.n * (best.size + kGC / 2)) best = {n, size};
-  }
-  return best;
-}
-
-// Workspace of the coupling backward: the slice backward's layout, then delta_D, a
-// second T image (the slice's, beside the deslice's), the ranges' d z' slices, and a
-// range's slices of W, bias, z' and dU | dS (for the passes' ranges and the point
-// pass's, whichever are larger).
-struct CoupLayout {
-  size_t deltaD, timg2, dzc, wc, bc, zc, uc, sl_part, sl_prep, sl_wsum, total;
-};
-CoupLayout coup_layout(const Shape& s0) {
-  CoupLayout C{};
-  size_t off = bwd_layout(s0, 2).total;
-  auto take = [&](size_t bytes) {
-    const size_t o = off;
-    off = align_up(off + bytes, 256);
-    return o;
-  };
-  const Shape s = pass_shape(s0);
-  const SlotRanges sr = slot_ranges(s0.G), cr = comb_ranges(s0);
-  const size_t rp = sr.n > 1 ? (size_t)sr.size : 0;
-  const size_t rs = std::max(rp, cr.n > 1 ? (size_t)cr.size : 0);
-  C.deltaD = take((size_t)s.BH() * s.N * sizeof(float));
-  C.timg2 = take((size_t)s.BH() * std::max(s.G, cr.size) * kWRow);
-  C.dzc = take((size_t)s.BH() * rp * kD * sizeof(float));
-  C.wc = take((size_t)s.H * kD * rs * sizeof(float));
-  C.bc = take((size_t)s.H * rs * sizeof(float));
-  C.zc = take((size_t)s.BH() * rs * kD * sizeof(float));
-  C.uc = take((size_t)s.BH() * rs * (kD + 1) * sizeof(float));
-  // d z' through the forward's slice (split products, as the backward's weights)
-  const Shape ss = split_shape(s0);
-  const bool via_slice = tc_forward_supported(ss);
-  C.sl_part = take(via_slice ? tc_slice_partials_bytes(ss) : 0);
-  C.sl_prep = take(via_slice ? tc_slice_prep_bytes(ss) : 0);
-  C.sl_wsum = take(via_slice ? (size_t)s.BH() * s0.G * sizeof(float) : 0);
-  C.total = off;
-  return C;
-}
-
-cudaError_t run_coupling_bwd(const Shape& s0, const void* x, const void* f, const void* dout, const float* W,
-                             const float* bias, const float* tau, const float* M, const float* z, const float* wsum,
-                             const float* zp, const float* lse, float* dzp, float* dz, float* dM, void* dx, void* dfx,
-                             float* dW, float* db, float* dtau, int accumulate, float* dUS, uint8_t* ws,
-                             uint32_t* status, cudaStream_t st) {
-  const SlotRanges sr = slot_ranges(s0.G);
-  const Shape s = pass_shape(s0);
-  const BwdLayout L = bwd_layout(s0, 2);
-  const CoupLayout C = coup_layout(s0);
-  const bool ranged = sr.n > 1;
-  const int64_t Np = padded_n(s), npx = s.BH() * Np;
-  float* deltaD = reinterpret_cast<float*>(ws + C.deltaD);
-  float* deltaS = reinterpret_cast<float*>(ws + L.delta);
-  float* wds = reinterpret_cast<float*>(ws + L.wds);
-  float* wc = reinterpret_cast<float*>(ws + C.wc);
-  float* bc = reinterpret_cast<float*>(ws + C.bc);
-  float* zc = reinterpret_cast<float*>(ws + C.zc);
-  float* uc = reinterpret_cast<float*>(ws + C.uc);
-  cudaError_t e;
-  // Slices [g0, g0 + G) of W, bias, z' and dU | dS (the gathered ones when `slice`).
-  struct Src {
-    const float *W, *b, *z, *u;
-  };
-  auto gather = [&](int g0, int G, bool slice, bool wz, bool zt, bool ut, Src* o) -> cudaError_t {
-    *o = {W, bias, zp, dUS};
-    if (!slice) return cudaSuccess;
-    cudaError_t r;
-    if (wz) {
-      if ((r = copy_rows(wc, G, W + g0, s0.G, G, (int64_t)s.H * kD, st)) != cudaSuccess) return r;
-      if ((r = copy_rows(bc, G, bias + g0, s0.G, G, s.H, st)) != cudaSuccess) return r;
-      o->W = wc, o->b = bc;
-    }
-    if (zt) {
-      if ((r = copy_rows(zc, (int64_t)G * kD, zp + (int64_t)g0 * kD, (int64_t)s0.G * kD, (int64_t)G * kD, s.BH(),
-                         st)) != cudaSuccess)
-        return r;
-      o->z = zc;
-    }
-    if (ut) {
-      if ((r = copy_rows(uc, (int64_t)G * (kD + 1), dUS + (int64_t)g0 * (kD + 1), (int64_t)s0.G * (kD + 1),
-                         (int64_t)G * (kD + 1), s.BH(), st)) != cudaSuccess)
-        return r;
-      o->u = uc;
     }
     return cudaSuccess;
-  };
-  auto range_g = [&](int k) { return k < sr.n - 1 ? sr.size : s0.G - (sr.n - 1) * sr.size; };
+  }
+  // u = dz / (S + eps) and c as images (T at `timg`, zimg) and ds.
+  cudaError_t images_us(const float* z, const float* wsum, const float* dz, size_t timg) const {
+    k_prep_us<<<dim3((unsigned)(s.G / 64), (unsigned)s.BH()), 256, 0, st>>>(z, wsum, dz, ws + timg, ws + L.zimg,
+                                                                              f(L.ds), s0.G, s.G, s.eps);
+    return cudaGetLastError();
+  }
+  // delta's point rows from delta (+ delta2) (+ the sums of w dS).
+  cudaError_t delta_rows(const float* delta, const float* delta2, const float* wds) const {
+    const int64_t n = s.BH() * padded_n(s);
+    k_prep_dpx<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(delta, delta2, wds, reinterpret_cast<uint4*>(ws + L.dpx),
+                                                              s.BH(), s.N, padded_n(s));
+    return cudaGetLastError();
+  }
+  // The slot pass over all slots (v, f: the deslice's and the slice's points of MODE 3).
+  template <int MODE>
+  cudaError_t slot(const void* x, const void* v, const void* f3) const {
+    CUtensorMap xmap, vmap, pmap, dmap, fmap;
+    if (!make_maps(x, v, f3, &xmap, &vmap, &pmap, &dmap, &fmap)) return cudaErrorInvalidValue;
+    const size_t sm = smem_bwd_slot(MODE);
+    const auto kernel = k_bwd_slot_tc<MODE, true>;
+    if (cudaError_t e = set_smem(kernel, sm)) return e;
+    const int P = bwd_slot_splits(s);
+    kernel<<<dim3((unsigned)bwd_slot_blocks(s), (unsigned)P, (unsigned)s.BH()), kThreads, sm, st>>>(
+        xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, f(L.part), f(L.dtp), s.N, padded_n(s),
+        s.H, s.G, P, status);
+    return cudaGetLastError();
+  }
+  // dW, dbias, dtau (and d z' into dzp) from the slot pass's partials.
+  cudaError_t reduce(const float* tau, float* dzp, float* dW, float* db, float* dtau, int accumulate) const {
+    const int P = bwd_slot_splits(s);
+    return reduce_bwd(s0, P, f(L.part), s.G, dzp ? 2 * kD + 2 : kD + 2, tau, dzp, dW, db, dtau, f(L.dtp),
+                      (int64_t)P * bwd_slot_blocks(s), accumulate, st);
+  }
+  // dx over the slot ranges.
+  template <bool kComb>
+  cudaError_t point(const void* x, const void* v, const void* f3, void* dx, int accumulate) const {
+    CUtensorMap xmap, vmap, pmap, dmap, fmap;
+    if (!make_maps(x, v, f3, &xmap, &vmap, &pmap, &dmap, &fmap)) return cudaErrorInvalidValue;
+    const SlotRanges r = point_ranges(s.G, kComb);
+    const bool hilo = smem_bwd_dx(r.size, true, kComb) <= kMaxSmem;
+    const size_t sm = smem_bwd_dx(r.size, hilo, kComb);
+    if (sm > kMaxSmem) return cudaErrorInvalidValue;
+    const auto kernel = k_bwd_dx_tc<true, kComb>;
+    if (cudaError_t e = set_smem(kernel, sm)) return e;
+    const int P = point_splits(s, (int)s.BH());
+    for (int k = 0; k < r.n; k++) {
+      const int g0 = k * r.size;
+      kernel<<<dim3((unsigned)P, (unsigned)s.BH()), kThreads, sm, st>>>(
+          xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, ws + L.wtimg,
+          static_cast<__nv_bfloat16*>(dx), s.N, padded_n(s), s.H, s.G, g0, std::min(r.size, s.G - g0), P,
+          hilo ? 1 : 0, (accumulate || k > 0) ? 1 : 0, status);
+      if (cudaError_t e = cudaGetLastError()) return e;
+    }
+    return cudaSuccess;
+  }
+  bool make_maps(const void* x, const void* v, const void* f3, CUtensorMap* xmap, CUtensorMap* vmap, CUtensorMap* pmap,
+                 CUtensorMap* dmap, CUtensorMap* fmap) const {
+    const int64_t Np = padded_n(s);
+    return make_point_map(xmap, x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B) &&
+           make_point_map(vmap, v, s, kD, CU_TENSOR_MAP_SWIZZLE_64B) && make_px_map(pmap, ws + L.px, s.BH(), Np) &&
+           make_px_map(dmap, ws + L.dpx, s.BH(), Np) &&
+           make_point_map(fmap, f3 ? f3 : x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B);
+  }
+};
 
-  k_prep_px<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(lse, reinterpret_cast<uint4*>(ws + L.px), s.BH(), s.N,
-                                                             Np);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // 1. delta_D
-  for (int k = 0; k < sr.n; k++) {
-    const int g0 = k * sr.size, G = range_g(k);
-    Src a;
-    if ((e = gather(g0, G, ranged, true, true, false, &a)) != cudaSuccess) return e;
-    if ((e = prep_w(s, G, a.W, a.b, tau, ws + L.wimg, status, st)) != cudaSuccess) return e;
-    if ((e = prep_t_images(s, G, a.z, kD, 0, ws, L, st)) != cudaSuccess) return e;
-    if ((e = tc_rows_bwd(s, 1, x, ws + L.wimg, ws + L.zimg, ws + L.px, dout, nullptr, deltaD, nullptr,
-                         reinterpret_cast<const float*>(ws + L.ds), k > 0 ? 1 : 0, status, st)) != cudaSuccess)
-      return e;
-  }
-  const int R = bwd_slot_blocks(s), P = bwd_slot_splits(s);
-  CUtensorMap xmap, vmap, pmap, dmap, fmap;
-  if (!make_maps(s, x, dout, ws + L.px, ws + L.dpx, &xmap, &vmap, &pmap, &dmap) ||
-      !make_point_map(&fmap, f, s, kD, CU_TENSOR_MAP_SWIZZLE_64B))
-    return cudaErrorInvalidValue;
-  // 2. d z'
-  const Shape ssl = split_shape(s0);
-  if (tc_forward_supported(ssl)) {
-    if ((e = tc_slice_fwd_lse(ssl, x, dout, W, bias, tau, lse, dzp, reinterpret_cast<float*>(ws + C.sl_wsum), 0,
-                              reinterpret_cast<float*>(ws + C.sl_part), ws + C.sl_prep, status, st)) != cudaSuccess)
-      return e;
-  } else {  // the slot pass in mode 0 (the W image of the last range is in place)
-    const size_t sm = smem_bwd_slot(0);
-    const auto kernel = k_bwd_slot_tc<0, true>;
-    if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
-    for (int k = 0; k < sr.n; k++) {
-      const int g0 = k * sr.size, G = range_g(k);
-      if (ranged) {
-        Src a;
-        if ((e = gather(g0, G, true, true, false, false, &a)) != cudaSuccess) return e;
-        if ((e = prep_w(s, G, a.W, a.b, tau, ws + L.wimg, status, st)) != cudaSuccess) return e;
-      }
-      kernel<<<dim3((unsigned)R, (unsigned)P, (unsigned)s.BH()), kThreads, sm, st>>>(
-          xmap, vmap, pmap, pmap, xmap, ws + L.wimg, ws + L.timg, nullptr, reinterpret_cast<float*>(ws + L.part),
-          reinterpret_cast<float*>(ws + L.dtp), s.N, Np, s.H, s.G, P, status);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      Shape sk = s0;
-      sk.G = G;
-      float* dzk = ranged ? reinterpret_cast<float*>(ws + C.dzc) : dzp;
-      if ((e = simt_reduce_dzp(sk, P, reinterpret_cast<const float*>(ws + L.part), s.G, kD, dzk, st)) != cudaSuccess)
-        return e;
-      if (ranged && (e = copy_rows(dzp + (int64_t)g0 * kD, (int64_t)s0.G * kD, dzk, (int64_t)G * kD, (int64_t)G * kD,
-                                   s.BH(), st)) != cudaSuccess)
-        return e;
-    }
-  }
-  // 3. the mix backward and dU | dS
-  if ((e = simt_mix_bwd(s0, M, z, dzp, dz, dM, st)) != cudaSuccess) return e;
-  if ((e = simt_slice_bwd_prep(s0, z, wsum, dz, dUS, st)) != cudaSuccess) return e;
-  // 4. delta_S, dfx, sum_g w dS
-  if ((e = cudaMemsetAsync(wds, 0, 2 * (size_t)s.BH() * s.N * sizeof(float), st)) != cudaSuccess) return e;
-  for (int k = 0; k < sr.n; k++) {
-    const int g0 = k * sr.size, G = range_g(k);
-    Src a;
-    if ((e = gather(g0, G, ranged, true, false, true, &a)) != cudaSuccess) return e;
-    if ((e = prep_w(s, G, a.W, a.b, tau, ws + L.wimg, status, st)) != cudaSuccess) return e;
-    if ((e = prep_t_images(s, G, a.u, kD + 1, 1, ws, L, st)) != cudaSuccess) return e;
-    if ((e = tc_rows_bwd(s, 2, x, ws + L.wimg, ws + L.zimg, ws + L.px, f, dfx, deltaS, wds,
-                         reinterpret_cast<const float*>(ws + L.ds), k > 0 ? 1 : 0, status, st)) != cudaSuccess)
-      return e;
-  }
-  // 5. delta's point rows
-  k_prep_dpx<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(deltaS, deltaD, wds, reinterpret_cast<uint4*>(ws + L.dpx),
-                                                              s.BH(), s.N, Np);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // 6. dW, dbias, dtau of da_D + da_S
-  {
-    const size_t sm = smem_bwd_slot(3);
-    const auto kernel = k_bwd_slot_tc<3, true>;
-    if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
-    for (int k = 0; k < sr.n; k++) {
-      const int g0 = k * sr.size, G = range_g(k);
-      Src a;
-      if ((e = gather(g0, G, ranged, true, true, true, &a)) != cudaSuccess) return e;
-      if ((e = prep_w(s, G, a.W, a.b, tau, ws + L.wimg, status, st)) != cudaSuccess) return e;
-      const int64_t BHG = s.BH() * s.G;
-      k_prep_t<<<(unsigned)((BHG + 127) / 128), 128, 0, st>>>(a.z, kD, 0, ws + L.timg, nullptr, s.BH(), G, s.G);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      k_prep_t<<<(unsigned)((BHG + 127) / 128), 128, 0, st>>>(a.u, kD + 1, 1, ws + C.timg2, nullptr, s.BH(), G, s.G);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      kernel<<<dim3((unsigned)R, (unsigned)P, (unsigned)s.BH()), kThreads, sm, st>>>(
-          xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + C.timg2, reinterpret_cast<float*>(ws + L.part),
-          reinterpret_cast<float*>(ws + L.dtp), s.N, Np, s.H, s.G, P, status);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      const int acc = accumulate || k > 0;
-      Shape sk = s0;
-      sk.G = G;
-      float *dWk = dW, *dbk = db;
-      if (ranged) {
-        dWk = reinterpret_cast<float*>(ws + L.dwc);
-        dbk = reinterpret_cast<float*>(ws + L.dbc);
-        if (accumulate) {
-          if ((e = copy_rows(dWk, G, dW + g0, s0.G, G, (int64_t)s.H * kD, st)) != cudaSuccess) return e;
-          if ((e = copy_rows(dbk, G, db + g0, s0.G, G, s.H, st)) != cudaSuccess) return e;
-        } else if (acc) {
-          if ((e = cudaMemsetAsync(dWk, 0, (size_t)s.H * kD * G * sizeof(float), st)) != cudaSuccess) return e;
-          if ((e = cudaMemsetAsync(dbk, 0, (size_t)s.H * G * sizeof(float), st)) != cudaSuccess) return e;
-        }
-      }
-      if ((e = simt_reduce_bwd(sk, P, reinterpret_cast<const float*>(ws + L.part), s.G, kD + 2, 0, tau, nullptr, dWk,
-                               dbk, dtau, reinterpret_cast<const float*>(ws + L.dtp), (int64_t)P * R, acc, st)) !=
-          cudaSuccess)
-        return e;
-      if (ranged) {
-        if ((e = copy_rows(dW + g0, s0.G, dWk, G, G, (int64_t)s.H * kD, st)) != cudaSuccess) return e;
-        if ((e = copy_rows(db + g0, s0.G, dbk, G, G, s.H, st)) != cudaSuccess) return e;
-      }
-    }
-  }
-  // 7. dx from da_D + da_S
-  const SlotRanges cr = comb_ranges(s0);
-  Shape sc = s;
-  sc.G = cr.size;
-  const bool hilo = smem_bwd_dx(sc.G, true, true) <= kMaxSmem;
-  const size_t sm = smem_bwd_dx(sc.G, hilo, true);
-  if (sm > kMaxSmem) return cudaErrorInvalidValue;
-  const auto kernel = k_bwd_dx_tc<true, true>;
-  if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
-  const int Pd = point_splits(sc, (int)sc.BH());
-  for (int k = 0; k < cr.n; k++) {
-    const int g0 = k * cr.size, G = k < cr.n - 1 ? cr.size : s0.G - (cr.n - 1) * cr.size;
-    Src a;
-    if ((e = gather(g0, G, cr.n > 1, true, true, true, &a)) != cudaSuccess) return e;
-    if ((e = prep_w(sc, G, a.W, a.b, tau, ws + L.wimg, status, st)) != cudaSuccess) return e;
-    const int64_t nwt = (int64_t)sc.H * kD * sc.G, BHG = sc.BH() * sc.G;
-    k_prep_wt<<<(unsigned)((nwt + 255) / 256), 256, 0, st>>>(a.W, tau, ws + L.wtimg, sc.H, G, sc.G, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_prep_t<<<(unsigned)((BHG + 127) / 128), 128, 0, st>>>(a.z, kD, 0, ws + L.timg, nullptr, sc.BH(), G, sc.G);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_prep_t<<<(unsigned)((BHG + 127) / 128), 128, 0, st>>>(a.u, kD + 1, 1, ws + C.timg2, nullptr, sc.BH(), G, sc.G);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    kernel<<<dim3((unsigned)Pd, (unsigned)sc.BH()), kThreads, sm, st>>>(
-        xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + C.timg2, ws + L.wtimg,
-        static_cast<__nv_bfloat16*>(dx), sc.N, Np, sc.H, sc.G, Pd, hilo ? 1 : 0, (accumulate || k > 0) ? 1 : 0,
-        status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
+#define FS_TRY(call)                                  \
+  do {                                                \
+    if (cudaError_t e_ = (call)) return e_;           \
+  } while (0)
 
 }  // namespace
 
@@ -1380,63 +1064,114 @@ cudaError_t run_coupling_bwd(const Shape& s0, const void* x, const void* f, cons
 // to ~2^-17 of that size.
 bool tc_backward_supported(const Shape& s0) {
   if (s0.dtype != FS_BF16 || s0.d != kD || s0.N < 2 || s0.G > 4096) return false;
-  const Shape s = pass_shape(s0);
+  Shape s = pass_shape(s0);
+  s.G = slot_ranges(s.G, kBwdSlotsMax).size;
   return tc_forward_supported(s) && smem_bwd_dx(s.G, false) <= kMaxSmem &&
          tc_rows_smem(s, 2, false, false) <= kMaxSmem;
 }
 
 size_t tc_backward_bytes(const Shape& s, int mode) {
-  return tc_backward_supported(s) ? bwd_layout(s, mode).total : 0;
+  return tc_backward_supported(s) ? bwd_layout(s, mode == 1 ? kDesliceBwd : kSliceBwd).total : 0;
 }
 
 int tc_backward_launch_count(const Shape& s, int mode) {
-  const SlotRanges sr = slot_ranges(s.G);
-  // per range: prep_t, prep_z2, prep_w, rows; then prep_px, prep_dpx; per range: the
-  // images again (or prep_wt alone with one range), slot, dx and the reductions of
-  // the parameters and dtau (and of dz' in mode 1); mode 2 also the dU/dS prologue.
-  const int images = sr.n > 1 ? 4 : 1;
-  const int reduce = mode == 1 ? 3 : 2;
-  return 4 * sr.n + 2 + sr.n * (images + 2 + reduce) + (mode == 2 ? 1 : 0);
+  const int G = pass_shape(s).G;
+  // prep, delta's rows, slot, reductions; rows and point per range; mode 2 also u's images
+  return 4 + slot_ranges(G, kBwdSlotsMax).n + point_ranges(G, false).n + (mode == 2 ? 1 : 0);
 }
 
+// dz' (the slot pass, MODE 1), dW, dbias, dtau, dx of the deslice: the rows pass forms delta,
+// the slot pass the slot-owned gradients, the point pass dx.
 cudaError_t tc_deslice_bwd(const Shape& s0, const void* x, const float* W, const float* bias, const float* tau,
                            const float* zp, const float* lse, const void* dout, float* dzp, void* dx, float* dW,
-                           float* db, float* dtau, int accumulate, void* ws_tc, uint32_t* status, cudaStream_t st) {
-  return run_backward(s0, 1, x, dout, W, bias, tau, zp, kD, lse, nullptr, dx, dzp, dW, db, dtau, accumulate,
-                      static_cast<uint8_t*>(ws_tc), status, st);
-}
-
-size_t tc_coupling_bwd_bytes(const Shape& s) { return tc_backward_supported(s) ? coup_layout(s).total : 0; }
-
-int tc_coupling_bwd_launch_count(const Shape& s) {
-  const SlotRanges sr = slot_ranges(s.G), cr = comb_ranges(s);
-  const int n = sr.n, r = n > 1 ? 1 : 0;
-  // lse rows; per range: the deslice rows pass with its images (4), the d z' slot
-  // pass with its reduction (2, and the W image again with several ranges); the mix
-  // backward (2) and the dU | dS prologue; per range the slice rows pass with its
-  // images (4); delta's rows; per range the combined slot pass with its images and
-  // reductions (6); per point-pass range its images and the pass (5)
-  const int dz = tc_forward_supported(split_shape(s)) ? 4 /*prep_w, prep_px, slice, reduce*/ : n * (2 + r);
-  return 1 + 4 * n + dz + 3 + 4 * n + 1 + 6 * n + 5 * cr.n;
-}
-
-cudaError_t tc_coupling_bwd(const Shape& s0, const void* x, const void* f, const void* dout, const float* W,
-                            const float* bias, const float* tau, const float* M, const float* z, const float* wsum,
-                            const float* zp, const float* lse, float* dzp, float* dz, float* dM, void* dx, void* dfx,
-                            float* dW, float* db, float* dtau, int accumulate, float* dUS, void* ws_tc,
-                            uint32_t* status, cudaStream_t st) {
-  return run_coupling_bwd(s0, x, f, dout, W, bias, tau, M, z, wsum, zp, lse, dzp, dz, dM, dx, dfx, dW, db, dtau,
-                          accumulate, dUS, static_cast<uint8_t*>(ws_tc), status, st);
+                           float* db, float* dtau, int accumulate, void* ws_tc, bool reset, uint32_t* status,
+                           cudaStream_t st) {
+  const BwdCall c(s0, kDesliceBwd, ws_tc, status, st);
+  Prepare p(c.s, s0.G, tau, status, reset);
+  p.weights(W, bias, c.ws + c.L.wimg);
+  p.weights_t(W, c.ws + c.L.wtimg);
+  p.tokens(zp, c.ws + c.L.timg, c.ws + c.L.zimg, true);
+  p.rows(lse, c.ws + c.L.px);
+  FS_TRY(p.run(st));
+  FS_TRY(c.rows(1, x, dout, nullptr, c.f(c.L.delta)));
+  FS_TRY(c.delta_rows(c.f(c.L.delta), nullptr, nullptr));
+  FS_TRY(c.slot<1>(x, dout, nullptr));
+  FS_TRY(c.reduce(tau, dzp, dW, db, dtau, accumulate));
+  return c.point<false>(x, dout, nullptr, dx, accumulate);
 }
 
 cudaError_t tc_slice_bwd(const Shape& s0, const void* x, const void* f, const float* W, const float* bias,
                          const float* tau, const float* z, const float* wsum, const float* lse, const float* dz,
-                         void* dx, void* dfx, float* dW, float* db, float* dtau, int accumulate, float* dUS,
-                         void* ws_tc, uint32_t* status, cudaStream_t st) {
-  cudaError_t e = simt_slice_bwd_prep(s0, z, wsum, dz, dUS, st);
-  if (e != cudaSuccess) return e;
-  return run_backward(s0, 2, x, f, W, bias, tau, dUS, kD + 1, lse, dfx, dx, nullptr, dW, db, dtau, accumulate,
-                      static_cast<uint8_t*>(ws_tc), status, st);
+                         void* dx, void* dfx, float* dW, float* db, float* dtau, int accumulate, void* ws_tc,
+                         bool reset, uint32_t* status, cudaStream_t st) {
+  const BwdCall c(s0, kSliceBwd, ws_tc, status, st);
+  Prepare p(c.s, s0.G, tau, status, reset);
+  p.weights(W, bias, c.ws + c.L.wimg);
+  p.weights_t(W, c.ws + c.L.wtimg);
+  p.rows(lse, c.ws + c.L.px);
+  p.clear(c.f(c.L.wds), 2 * c.s.BH() * c.s.N);
+  FS_TRY(p.run(st));
+  FS_TRY(c.images_us(z, wsum, dz, c.L.timg));
+  FS_TRY(c.rows(2, x, f, dfx, c.f(c.L.delta)));
+  FS_TRY(c.delta_rows(c.f(c.L.delta), nullptr, c.f(c.L.wds)));
+  FS_TRY(c.slot<2>(x, f, nullptr));
+  FS_TRY(c.reduce(tau, nullptr, dW, db, dtau, accumulate));
+  return c.point<false>(x, f, nullptr, dx, accumulate);
+}
+
+size_t tc_coupling_bwd_bytes(const Shape& s) {
+  return tc_backward_supported(s) ? bwd_layout(s, kCouplingBwd).total : 0;
+}
+
+int tc_coupling_bwd_launch_count(const Shape& s) {
+  const int G = pass_shape(s).G, n = slot_ranges(G, kBwdSlotsMax).n;
+  // prep; d z' (slice or slot pass, reduction), the mix backward, u's images; delta's rows,
+  // slot, reductions; both rows passes and the point pass per range
+  return 1 + 2 + 1 + 1 + 3 + 2 * n + point_ranges(G, true).n;
+}
+
+// The coupling's backward in one call (fs_coupling_bwd).  The deslice's and the
+// slice's da share the weights, so their slot-owned and point-owned products can be
+// formed once from da_D + da_S; what has to come first is d z' (it feeds the mix
+// backward, and so dU, dS and the slice's part):
+//   1. the deslice part's rows pass: delta_D;
+//   2. d z' = sum_n w_ng dO_n: the forward's slice with dO for fx (its unnormalised
+//      numerators) where the forward's kernels take the shape, else the slot pass in
+//      mode 0 (the weights alone);
+//   3. the mix backward and the images of dU | dS;
+//   4. the slice part's rows pass: delta_S, dfx, the sum_g w dS partials;
+//   5. delta = delta_S + delta_D + sum_g w dS into the point rows;
+//   6. the slot pass in mode 3: dW, dbias, dtau of da_D + da_S;
+//   7. the point pass for dx.
+cudaError_t tc_coupling_bwd(const Shape& s0, const void* x, const void* f, const void* dout, const float* W,
+                            const float* bias, const float* tau, const float* M, const float* z, const float* wsum,
+                            const float* zp, const float* lse, float* dzp, float* dz, float* dM, void* dx, void* dfx,
+                            float* dW, float* db, float* dtau, int accumulate, void* ws_tc, bool reset,
+                            uint32_t* status, cudaStream_t st) {
+  const BwdCall c(s0, kCouplingBwd, ws_tc, status, st);
+  const BwdLayout& L = c.L;
+  Prepare p(c.s, s0.G, tau, status, reset);
+  p.weights(W, bias, c.ws + L.wimg);
+  p.weights_t(W, c.ws + L.wtimg);
+  p.tokens(zp, c.ws + L.timg, c.ws + L.zimg, true);
+  p.rows(lse, c.ws + L.px);
+  p.clear(c.f(L.wds), 2 * c.s.BH() * c.s.N);
+  FS_TRY(p.run(st));
+  FS_TRY(c.rows(1, x, dout, nullptr, c.f(L.delta_d)));
+  if (tc_forward_supported(split_shape(s0))) {
+    FS_TRY(run_slice(c.s, s0.G, x, dout, nullptr, nullptr, c.ws + L.wimg, c.ws + L.px, dzp, c.f(L.sl_wsum), 0,
+                     c.f(L.sl_part), status, st));
+  } else {
+    FS_TRY(c.slot<0>(x, dout, nullptr));
+    FS_TRY(simt_reduce_dzp(s0, bwd_slot_splits(c.s), c.f(L.part), c.s.G, kD, dzp, st));
+  }
+  FS_TRY(mix_bwd(s0, M, z, dzp, dz, dM, st));
+  FS_TRY(c.images_us(z, wsum, dz, L.timg2));
+  FS_TRY(c.rows(2, x, f, dfx, c.f(L.delta)));
+  FS_TRY(c.delta_rows(c.f(L.delta), c.f(L.delta_d), c.f(L.wds)));
+  FS_TRY(c.slot<3>(x, dout, f));
+  FS_TRY(c.reduce(tau, nullptr, dW, db, dtau, accumulate));
+  return c.point<true>(x, dout, f, dx, accumulate);
 }
 
 }  // namespace fs

@@ -53,81 +53,166 @@ __device__ __forceinline__ uint32_t off_z(int c, int g) {
   return (uint32_t)(kb * 4096 + (c >> 3) * 1024 + (c & 7) * 128 + (((w >> 3) ^ (c & 7)) << 4) + (w & 7) * 2);
 }
 
-// Slots [G, Gp) pad the image to whole 128-slot blocks: W' = 0 and b' = -1e30, so
-// their logits are -1e30 and their weights exactly 0 in every pass.
-// Thread (h, q, g): for q < 4 the 16-byte pieces of channels [8q, 8q + 8) of slot g
-// in both halves of W'; for q = 4 the slot's extra row.  Consecutive threads take
-// consecutive slots, so the reads of W [H, d, G] coalesce.
-__global__ void k_prep_w(const float* __restrict__ W, const float* __restrict__ bias, const float* __restrict__ tau,
-                         uint8_t* __restrict__ img, int H, int G, int Gp, uint32_t* status) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)H * 5 * Gp) return;
-  const int g = (int)(i % Gp);
-  const int q = (int)((i / Gp) % 5);
-  const int h = (int)(i / ((int64_t)5 * Gp));
-  const float t = tau[h];
-  if (!(t > 0.f && t < INFINITY)) {
-    atomicCAS(status, 0u, (uint32_t)FS_ERR_BAD_TAU);
-    return;
-  }
-  const float scale = kLog2e / t;
-  const bool real = g < G;
-  uint8_t* base = img + (size_t)h * Gp * kWRow;
-  if (q < 4) {
-    uint32_t hi[4], lo[4];
+// One launch prepares everything a call's passes read: its blocks are divided among jobs
+// (images of W and of the tokens, point rows, splits of fp32 points, a buffer to clear), in
+// the order below.  Each job alone is a few microseconds of launch and latency, and a small
+// call used to spend more time in them than in its passes (a training step at N = 32,768,
+// G = 64: 29 small kernels of 165 us beside 180 us of passes).
+//
+// Images cover slots [0, Gp), Gp = G rounded up to whole 128-slot blocks.  Padding slots
+// [G, Gp) have W' = 0 and b' = -1e30 (their logits are -1e30 and their weights exactly 0 in
+// every pass) and zero token rows.
+struct Prep {
+  // blocks of 256 threads up to and including each job
+  int64_t e_w, e_wt, e_t, e_z, e_px, e_split0, e_split1, e_zero;
+  const float *W, *bias, *tau, *t /* tokens [BH][G][32] */, *lse, *split_src[2];
+  uint8_t *wimg, *wtimg, *timg, *zimg;
+  uint4* px;
+  __nv_bfloat16 *split_hi[2], *split_lo[2];
+  float4* zero;
+  int64_t BH, N, Np, n_split8, n_zero4;
+  int H, G, Gp, z_lo /* zimg with the residual half */, reset;
+  uint32_t* status;
+};
+
+__device__ __forceinline__ bool good_tau(float t) { return t > 0.f && t < INFINITY; }
+// 8 floats -> 8 bf16 (hi) and the bf16 of the residuals (lo).
+__device__ __forceinline__ void split8(const float (&v)[8], uint4& hi, uint4& lo) {
+  uint32_t h[4], l[4];
 #pragma unroll
-    for (int e = 0; e < 4; e++) {
-      const int k = 8 * q + 2 * e;
-      const float w0 = real ? W[((int64_t)h * kD + k) * G + g] * scale : 0.f;
-      const float w1 = real ? W[((int64_t)h * kD + k + 1) * G + g] * scale : 0.f;
-      const uint32_t p = pack_bf16(w0, w1);
-      hi[e] = p;
-      lo[e] = pack_bf16(w0 - __uint_as_float(p << 16), w1 - __uint_as_float(p & 0xFFFF0000u));
-    }
+  for (int e = 0; e < 4; e++) {
+    h[e] = pack_bf16(v[2 * e], v[2 * e + 1]);
+    l[e] = pack_bf16(v[2 * e] - __uint_as_float(h[e] << 16), v[2 * e + 1] - __uint_as_float(h[e] & 0xFFFF0000u));
+  }
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+}
+
+// W image, thread (h, q, g): for q < 4 the 16-byte pieces of channels [8q, 8q + 8) of slot g
+// in both halves of W'; for q = 4 the slot's extra row [b'_hi, b'_lo, 1, 1, 1, 0 ...]
+// (k = 2, 3, 4 multiply the three bf16 parts of the point side's -lse2, zero in the
+// statistics pass).  Consecutive threads take consecutive slots, so the reads of W
+// [H, d, G] coalesce.
+__device__ __forceinline__ void prep_w_piece(const Prep& a, int64_t i) {
+  if (i >= (int64_t)a.H * 5 * a.Gp) return;
+  const int g = (int)(i % a.Gp), q = (int)((i / a.Gp) % 5), h = (int)(i / ((int64_t)5 * a.Gp));
+  if (!good_tau(a.tau[h])) return;
+  const float scale = kLog2e / a.tau[h];
+  const bool real = g < a.G;
+  uint8_t* base = a.wimg + (size_t)h * a.Gp * kWRow;
+  if (q < 4) {
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) v[e] = real ? a.W[((int64_t)h * kD + 8 * q + e) * a.G + g] * scale : 0.f;
     const uint32_t off = off_sw64(g, 8 * q);
-    *reinterpret_cast<uint4*>(base + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    *reinterpret_cast<uint4*>(base + (size_t)Gp * 96 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    split8(v, *reinterpret_cast<uint4*>(base + off), *reinterpret_cast<uint4*>(base + (size_t)a.Gp * 96 + off));
     return;
   }
-  // The extra row [b'_hi, b'_lo, 1, 1, 1, 0 ...]; k = 2, 3, 4 multiply the three bf16
-  // parts of the point side's -lse2 (zero in the statistics pass).
-  const float b2 = real ? bias[(int64_t)h * G + g] * scale : -1e30f;
+  const float b2 = real ? a.bias[(int64_t)h * a.G + g] * scale : -1e30f;
   const uint32_t bp = pack_bf16(b2, 0.f) & 0xFFFFu;
   const float bhi = __uint_as_float(bp << 16);
   const uint32_t blo = pack_bf16(b2 - bhi, 0.f) & 0xFFFFu;
-  uint8_t* ep = base + (size_t)Gp * 64;
+  uint8_t* ep = base + (size_t)a.Gp * 64;
   *reinterpret_cast<uint4*>(ep + off_sw32(g, 0)) = make_uint4(bp | (blo << 16), 0x3F803F80u, 0x3F80u, 0u);
   *reinterpret_cast<uint4*>(ep + off_sw32(g, 8)) = make_uint4(0u, 0u, 0u, 0u);
 }
-
-// Padding slots [G, Gp) get zero rows (their weights are 0, and 0 * 0 stays 0).
-__global__ void k_prep_z(const float* __restrict__ zp, uint8_t* __restrict__ img, int64_t BH, int G, int Gp) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t total = BH * Gp * kD;
-  if (i >= total) return;
-  const int c = (int)(i % kD);
-  const int g = (int)((i / kD) % Gp);
-  const int64_t bh = i / ((int64_t)kD * Gp);
-  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(img + (size_t)bh * Gp * 64);
-  out[off_z(c, g) / 2] = __float2bfloat16_rn(g < G ? zp[(bh * G + g) * kD + c] : 0.f);
+// W'^T image of head h in the Z layout (channel rows, slots along K): the bf16 half, then
+// the residual half (Gp*128 bytes per head).  Thread (h, c, 8 slots).
+__device__ __forceinline__ void prep_wt_piece(const Prep& a, int64_t i) {
+  const int n8 = a.Gp / 8;
+  if (i >= (int64_t)a.H * kD * n8) return;
+  const int g = (int)(i % n8) * 8, c = (int)((i / n8) % kD), h = (int)(i / ((int64_t)kD * n8));
+  if (!good_tau(a.tau[h])) return;
+  const float scale = kLog2e / a.tau[h];
+  float v[8];
+#pragma unroll
+  for (int e = 0; e < 8; e++) v[e] = g + e < a.G ? a.W[((int64_t)h * kD + c) * a.G + g + e] * scale : 0.f;
+  uint8_t* base = a.wtimg + (size_t)h * a.Gp * 128 + off_z(c, g);
+  split8(v, *reinterpret_cast<uint4*>(base), *reinterpret_cast<uint4*>(base + (size_t)a.Gp * 64));
+}
+// T image of tokens without an added column (c = 0), in the W image's layout.
+__device__ __forceinline__ void prep_t_piece(const Prep& a, int64_t i) {
+  if (i >= a.BH * 5 * a.Gp) return;
+  const int g = (int)(i % a.Gp), q = (int)((i / a.Gp) % 5);
+  const int64_t bh = i / ((int64_t)5 * a.Gp);
+  uint8_t* base = a.timg + (size_t)bh * a.Gp * kWRow;
+  if (q < 4) {
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (g < a.G) load8(a.t + (bh * a.G + g) * kD + 8 * q, v);
+    const uint32_t off = off_sw64(g, 8 * q);
+    split8(v, *reinterpret_cast<uint4*>(base + off), *reinterpret_cast<uint4*>(base + (size_t)a.Gp * 96 + off));
+    return;
+  }
+  uint8_t* ep = base + (size_t)a.Gp * 64;
+  *reinterpret_cast<uint4*>(ep + off_sw32(g, 0)) = make_uint4(0u, 0x3F803F80u, 0x3F80u, 0u);
+  *reinterpret_cast<uint4*>(ep + off_sw32(g, 8)) = make_uint4(0u, 0u, 0u, 0u);
+}
+// Z-layout image of tokens (blocks of 64 slots, 32 channel rows x 128 B, 128B swizzle): the
+// bf16 half, with z_lo then the residual half.  Thread (bh, 8 slots, channel).
+__device__ __forceinline__ void prep_z_piece(const Prep& a, int64_t i) {
+  const int n8 = a.Gp / 8;
+  if (i >= a.BH * n8 * kD) return;
+  const int c = (int)(i % kD), g = (int)((i / kD) % n8) * 8;
+  const int64_t bh = i / ((int64_t)kD * n8);
+  float v[8];
+#pragma unroll
+  for (int e = 0; e < 8; e++) v[e] = g + e < a.G ? a.t[(bh * a.G + g + e) * kD + c] : 0.f;
+  uint4 hi, lo;
+  split8(v, hi, lo);
+  uint8_t* base = a.zimg + (size_t)bh * a.Gp * (a.z_lo ? 128 : 64) + off_z(c, g);
+  *reinterpret_cast<uint4*>(base) = hi;
+  if (a.z_lo) *reinterpret_cast<uint4*>(base + (size_t)a.Gp * 64) = lo;
 }
 
-// Z-layout image (blocks of 64 slots, 32 channel rows x 128 B, 128B swizzle) of
-// t [BH][G][tstride] per (b,h): the bf16 half, then the residual half (Gp*128 bytes
-// per (b,h)); padding slots [G, Gp) are zero.
-__global__ void k_prep_z2(const float* __restrict__ t, int tstride, uint8_t* __restrict__ img, int64_t BH, int G,
-                          int Gp) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= BH * Gp * kD) return;
-  const int c = (int)(i % kD);
-  const int g = (int)((i / kD) % Gp);
-  const int64_t bh = i / ((int64_t)kD * Gp);
-  const float v = g < G ? t[(bh * G + g) * tstride + c] : 0.f;
-  __nv_bfloat16* hp = reinterpret_cast<__nv_bfloat16*>(img + (size_t)bh * Gp * 128);
-  __nv_bfloat16* lp = reinterpret_cast<__nv_bfloat16*>(img + (size_t)bh * Gp * 128 + (size_t)Gp * 64);
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  hp[off_z(c, g) / 2] = hi;
-  lp[off_z(c, g) / 2] = __float2bfloat16_rn(v - __bfloat162float(hi));
+__device__ __forceinline__ uint4 extra_row3(float nv);  // below
+
+__global__ void __launch_bounds__(256) k_prep(const __grid_constant__ Prep a) {
+  const int64_t blk = blockIdx.x;
+  if (blk == 0) {
+    // The status word: cleared by the first launch of a call; bad temperatures flagged.
+    int bad = 0;
+    for (int h = threadIdx.x; h < a.H; h += 256) bad |= !good_tau(a.tau[h]);
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) {
+      if (a.reset)
+        *a.status = bad ? (uint32_t)FS_ERR_BAD_TAU : 0u;
+      else if (bad)
+        atomicCAS(a.status, 0u, (uint32_t)FS_ERR_BAD_TAU);
+    }
+  }
+  if (blk < a.e_w) return prep_w_piece(a, blk * 256 + threadIdx.x);
+  if (blk < a.e_wt) return prep_wt_piece(a, (blk - a.e_w) * 256 + threadIdx.x);
+  if (blk < a.e_t) return prep_t_piece(a, (blk - a.e_wt) * 256 + threadIdx.x);
+  if (blk < a.e_z) return prep_z_piece(a, (blk - a.e_t) * 256 + threadIdx.x);
+  if (blk < a.e_px) {
+    // Point-extra rows [1, 1, -lse2 in three parts, 0, 0, 0]; padded points get -1e30 so that
+    // their weights vanish.
+    const int64_t i = (blk - a.e_z) * 256 + threadIdx.x;
+    if (i >= a.BH * a.Np) return;
+    const int64_t bh = i / a.Np, n = i % a.Np;
+    a.px[i] = extra_row3(n < a.N ? -a.lse[bh * a.N + n] * kLog2e : -1e30f);
+    return;
+  }
+  if (blk < a.e_split1) {
+    // fp32 points -> bf16 hi and residual tensors of the same layout (v = hi + lo to ~2^-16
+    // relative), 8 values per thread in 16-byte loads and stores.
+    const int k = blk < a.e_split0 ? 0 : 1;
+    const int64_t i = (blk - (k ? a.e_split0 : a.e_px)) * 256 + threadIdx.x;
+    if (i >= a.n_split8) return;
+    float v[8];
+    load8(a.split_src[k] + 8 * i, v);
+    uint4 hi, lo;
+    split8(v, hi, lo);
+    reinterpret_cast<uint4*>(a.split_hi[k])[i] = hi;
+    reinterpret_cast<uint4*>(a.split_lo[k])[i] = lo;
+    return;
+  }
+  const int64_t i = (blk - a.e_split1) * 256 + threadIdx.x;
+  if (i < a.n_zero4) a.zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // ---- shared pieces -------------------------------------------------------------------------
@@ -209,22 +294,6 @@ __device__ __forceinline__ void issue_logits(uint32_t tmem_d, uint32_t x, uint32
     mma_ss_w<kHi32, kXeHi>(tmem_d, we, xe, idesc, 1);
 }
 
-// fp32 point tensors -> bf16 hi and residual lo tensors of the same layout (v = hi + lo
-// to ~2^-16 relative): the tensor-core path's operands for fp32 inputs.
-__global__ void k_split_bf16(const float* __restrict__ v, __nv_bfloat16* __restrict__ hi,
-                             __nv_bfloat16* __restrict__ lo, int64_t n) {
-  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (i >= n) return;
-  const float4 a = *reinterpret_cast<const float4*>(v + i);
-  const float e[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-  for (int k = 0; k < 4; k++) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(e[k]);
-    hi[i + k] = h;
-    lo[i + k] = __float2bfloat16_rn(e[k] - __bfloat162float(h));
-  }
-}
-
 // Producer-side bulk loads of an image into smem (pieces of at most 32 KB).
 __device__ __forceinline__ void load_images(uint8_t* dst, const uint8_t* src, uint32_t bytes, uint64_t* bar) {
   constexpr uint32_t kPiece = 32768;
@@ -232,6 +301,15 @@ __device__ __forceinline__ void load_images(uint8_t* dst, const uint8_t* src, ui
     const uint32_t n = (bytes - off) < kPiece ? (bytes - off) : kPiece;
     bulk_load(dst + off, src + off, n, bar);
   }
+}
+
+// Slots [g0, g0 + n) of a slot image (W or T layout, Gi slots in all): the bf16 rows, the
+// extra rows and, with `lo`, the residual rows, one after the other.
+__device__ __forceinline__ void load_slots(uint8_t* dst, const uint8_t* img, int Gi, int g0, int n, bool lo,
+                                           uint64_t* bar) {
+  load_images(dst, img + (size_t)g0 * 64, (uint32_t)n * 64, bar);
+  load_images(dst + (size_t)n * 64, img + (size_t)Gi * 64 + (size_t)g0 * 32, (uint32_t)n * 32, bar);
+  if (lo) load_images(dst + (size_t)n * 96, img + (size_t)Gi * 96 + (size_t)g0 * 64, (uint32_t)n * 64, bar);
 }
 
 // 2^t for 32 log2-weights -> 16 bf16x2 words.
@@ -378,16 +456,6 @@ __device__ __forceinline__ uint4 extra_row3(float nv) {
                     (uint32_t)__bfloat16_as_ushort(p3), 0u);
 }
 
-// Point-extra rows [1, 1, -lse2 in three parts, 0, 0, 0] from lse [B,H,N] (natural
-// log) into px [B*H, Np, 8]; padded points (n >= N) get -1e30 so that their weights
-// vanish.
-__global__ void k_prep_px(const float* __restrict__ lse, uint4* __restrict__ px, int64_t BH, int64_t N, int64_t Np) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= BH * Np) return;
-  const int64_t bh = i / Np, n = i % Np;
-  px[i] = extra_row3(n < N ? -lse[bh * N + n] * kLog2e : -1e30f);
-}
-
 // ---- host side -------------------------------------------------------------------------------
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -463,27 +531,59 @@ int point_splits(const Shape& s, int units) {
   return (int)best;
 }
 
-// rows x cols floats from src (row pitch spitch floats) to dst (row pitch dpitch
-// floats): a slot range's slice of W [H, d, G], bias [H, G] or a per-slot tensor.
-cudaError_t copy_rows(float* dst, int64_t dpitch, const float* src, int64_t spitch, int64_t cols, int64_t rows,
-                      cudaStream_t st) {
-  return cudaMemcpy2DAsync(dst, (size_t)dpitch * sizeof(float), src, (size_t)spitch * sizeof(float),
-                           (size_t)cols * sizeof(float), (size_t)rows, cudaMemcpyDeviceToDevice, st);
-}
-
 constexpr size_t kMaxSmem = 232448;  // opt-in shared memory per block on sm_103
 template <typename K>
 cudaError_t set_smem(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// W image of the padded shape sp (sp.G = G rounded up) from W [H, d, G].
-cudaError_t prep_w(const Shape& sp, int G, const float* W, const float* bias, const float* tau, uint8_t* img,
-                   uint32_t* status, cudaStream_t st) {
-  const int64_t n = (int64_t)sp.H * 5 * sp.G;
-  k_prep_w<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(W, bias, tau, img, sp.H, G, sp.G, status);
-  return cudaGetLastError();
-}
+// A call's preparation: jobs are added in any order, run() launches them as one kernel.
+struct Prepare {
+  Prep a{};
+  int64_t w = 0, wt = 0, t = 0, z = 0, px = 0, sp[2] = {0, 0}, zero = 0;  // threads of each job
+  // sp.G: slots of the images, G: the caller's.
+  Prepare(const Shape& sp_, int G, const float* tau, uint32_t* status, bool reset) {
+    a.H = sp_.H, a.G = G, a.Gp = sp_.G, a.BH = sp_.BH(), a.N = sp_.N, a.Np = padded_n(sp_);
+    a.tau = tau, a.status = status, a.reset = reset ? 1 : 0;
+  }
+  void weights(const float* W, const float* bias, uint8_t* img) {
+    a.W = W, a.bias = bias, a.wimg = img;
+    w = (int64_t)a.H * 5 * a.Gp;
+  }
+  void weights_t(const float* W, uint8_t* img) {
+    a.W = W, a.wtimg = img;
+    wt = (int64_t)a.H * kD * (a.Gp / 8);
+  }
+  void tokens(const float* tok, uint8_t* timg, uint8_t* zimg, bool z_lo) {
+    a.t = tok, a.timg = timg, a.zimg = zimg, a.z_lo = z_lo ? 1 : 0;
+    t = timg ? a.BH * 5 * a.Gp : 0;
+    z = a.BH * (a.Gp / 8) * kD;
+  }
+  void rows(const float* lse, void* dst) {
+    a.lse = lse, a.px = static_cast<uint4*>(dst);
+    px = a.BH * a.Np;
+  }
+  // fp32 points v -> bf16 hi at dst, residuals at dst + half.
+  void split(const Shape& s, const void* v, uint8_t* dst, size_t half) {
+    const int k = sp[0] ? 1 : 0;
+    a.split_src[k] = static_cast<const float*>(v);
+    a.split_hi[k] = reinterpret_cast<__nv_bfloat16*>(dst);
+    a.split_lo[k] = reinterpret_cast<__nv_bfloat16*>(dst + half);
+    a.n_split8 = sp[k] = s.B * s.N * s.H * s.d / 8;
+  }
+  void clear(float* p, int64_t n) {  // n rounded up to 4 floats
+    a.zero = reinterpret_cast<float4*>(p);
+    a.n_zero4 = zero = (n + 3) / 4;
+  }
+  cudaError_t run(cudaStream_t st) {
+    int64_t e = 0;
+    auto end = [&](int64_t threads) { return e += (threads + 255) / 256; };
+    a.e_w = end(w), a.e_wt = end(wt), a.e_t = end(t), a.e_z = end(z), a.e_px = end(px);
+    a.e_split0 = end(sp[0]), a.e_split1 = end(sp[1]), a.e_zero = end(zero);
+    k_prep<<<(unsigned)(e > 0 ? e : 1), 256, 0, st>>>(a);
+    return cudaGetLastError();
+  }
+};
 
 }  // namespace
 }  // namespace fs

@@ -2,7 +2,7 @@
 // of the backward (the deslice kernel in modes 1 and 2, see k_deslice).
 //
 // Inputs: bf16 point tensors as they are; fp32 point tensors split beforehand
-// into bf16 hi and residual tensors (k_split_bf16), with the residual products
+// into bf16 hi and residual tensors (k_prep), with the residual products
 // added in the X3 instantiations.  G is padded to whole 128-slot blocks whose
 // padding slots carry weight 0.
 //
@@ -85,8 +85,8 @@ using namespace tc;
 //     delta_n = fx_n . R_n + sum_g w_ng dS_g.  The second sum is formed by the
 //     softmax warpgroups from the fp32 weights; each warpgroup adds its own
 //     partial per point to wds[wg][bh][n] (cleared beforehand) and the consumer adds them.
-// accumulate (MODES 1, 2, and MODE 0 with X3): the pass covers a later range of the
-// slots, whose contributions to delta and dfx (to the fp32 out) are added to those of
+// The pass covers slots [g0, g0 + G) of images of Gi slots.  accumulate (MODES 1, 2, and
+// MODE 0 with X3): a later range of the slots, whose contributions to delta and dfx (to the fp32 out) are added to those of
 // the earlier ranges.
 // PS (split products): the weights and t as bf16 hi + lo halves, P t = Phi thi +
 // Plo thi + Phi tlo; the image then holds t's residual half after its bf16 half.
@@ -111,8 +111,8 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
               const __grid_constant__ CUtensorMap xrmap,
               const uint8_t* __restrict__ wimg, const uint8_t* __restrict__ zimg, __nv_bfloat16* __restrict__ out,
               const __nv_bfloat16* __restrict__ v, float* __restrict__ delta, float* __restrict__ wds,
-              const float* __restrict__ dS, int64_t N, int64_t Np, int H, int G, int splits, int hilo,
-              uint32_t zstride, int accumulate, uint32_t* status) {
+              const float* __restrict__ dS, int64_t N, int64_t Np, int H, int Gi, int g0, int G, int splits,
+              int hilo, uint32_t zstride, int accumulate, uint32_t* status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // hilo: the residual half of W' fits in shared memory too (K = 80 logits, as in
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
   }
   for (int s = 0; s < kStages; s++) zero_smem(s_x + s * kDSt + kXBytes + kPxBytes, kPxBytes);
   if (MODE == 2)
-    for (int g = threadIdx.x; g < G; g += kThreads) s_ds[g] = dS[wk.bh * G + g];
+    for (int g = threadIdx.x; g < G; g += kThreads) s_ds[g] = dS[wk.bh * Gi + g0 + g];
   fence_proxy_async_smem();
   if (warp == 1) tmem_alloc(tmem_slot, 512);
   tc_fence_before();
@@ -182,8 +182,10 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       prefetch_tmap(&pmap);
       if (X3) prefetch_tmap(&xrmap);
       mbar_expect_tx(wz_full, wbytes + zbytes);
-      load_images(s_w, wimg + (size_t)h * G * kWRow, wbytes, wz_full);
-      load_images(s_z, zimg + (size_t)wk.bh * zstride, zbytes, wz_full);
+      load_slots(s_w, wimg + (size_t)h * Gi * kWRow, Gi, g0, G, hilo, wz_full);
+      const uint8_t* zi = zimg + (size_t)wk.bh * zstride + (size_t)g0 * 64;
+      load_images(s_z, zi, (uint32_t)G * 64, wz_full);
+      if (PS) load_images(s_z + (uint32_t)G * 64, zi + (size_t)Gi * 64, (uint32_t)G * 64, wz_full);
       int i = 0;
       for (; i < wk.ntiles; i++) {
         const int s = i % kStages;
@@ -991,14 +993,13 @@ int slice_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * slice_b
 
 // fp32 point tensors take the tensor-core path with every operand as two bf16 halves
 // (x, fx and W', the weights, z'): the X3 kernels.  Their inputs are first split
-// into bf16 hi and residual tensors in the workspace (k_split_bf16).
+// into bf16 hi and residual tensors in the workspace (k_prep).
 bool x3_shape(const Shape& s) { return s.dtype == FS_F32; }
 
 // The X3 deslice holds both halves of W' and of z' in shared memory, which fits up to
 // 512 slots; past that it runs over ranges of `size` slots (a multiple of 128), each
-// with the full lse, adding its output to the earlier ranges'.  `size` minimises the
-// padded slots plus half a block per range (a range re-reads x); ties go to the
-// larger size.
+// with the full lse, adding its output to the earlier ranges': as few as fit (a range
+// re-reads x), of equal size but for the last.
 constexpr int kX3SlotsMax = 512;
 struct X3Ranges {
   int n, size;
@@ -1006,12 +1007,8 @@ struct X3Ranges {
 X3Ranges x3_ranges(const Shape& s0) {
   const int Gp = (s0.G + kGC - 1) / kGC * kGC;
   if (s0.dtype != FS_F32 || s0.G <= kX3SlotsMax) return {1, Gp};
-  X3Ranges best{0, 0};
-  for (int size = kGC; size <= kX3SlotsMax; size += kGC) {
-    const int n = (s0.G + size - 1) / size;
-    if (best.n == 0 || (int64_t)n * (size + kGC / 2) <= (int64_t)best.n * (best.size + kGC / 2)) best = {n, size};
-  }
-  return best;
+  const int n = (Gp + kX3SlotsMax - 1) / kX3SlotsMax;
+  return {n, (Gp / kGC + n - 1) / n * kGC};
 }
 size_t half_bytes(const Shape& s) { return align_up((size_t)s.B * s.N * s.H * s.d * 2, 256); }
 
@@ -1026,15 +1023,6 @@ size_t smem_slice(bool x3 = false) {
   return 1024 + (size_t)kWBlock +
          (x3 ? (size_t)(kSliceStages / 2) * (kStageBytes + kXBytes + 2 * kFBlock) : (size_t)kSliceStages * kStageBytes) +
          512;
-}
-
-// v (fp32 [B,N,H,d]) -> bf16 hi at dst, bf16 residual at dst + half_bytes(s).
-cudaError_t split_points(const Shape& s, const void* v, uint8_t* dst, cudaStream_t st) {
-  const int64_t n = s.B * s.N * s.H * s.d;
-  k_split_bf16<<<(unsigned)((n / 4 + 255) / 256), 256, 0, st>>>(
-      static_cast<const float*>(v), reinterpret_cast<__nv_bfloat16*>(dst),
-      reinterpret_cast<__nv_bfloat16*>(dst + half_bytes(s)), n);
-  return cudaGetLastError();
 }
 
 // Statistics into lse [B,H,N] and the point-extra rows at px.  xr: x's residual
@@ -1074,11 +1062,10 @@ bool tc_forward_supported(const Shape& s) {
          s.BH() * np < (int64_t(1) << 31) && encode_fn() != nullptr;
 }
 
-int tc_stats_launch_count(const Shape& s) { return 2 /*prep_w, stats*/ + (x3_shape(s) ? 1 : 0); }
+int tc_stats_launch_count(const Shape& s) { return 2 /*prep, stats*/; }
 
 int tc_forward_launch_count(const Shape& s) {
-  return 4 /*prep_w, stats, slice, reduce*/ + 1 /*prep_px*/ + 3 * x3_ranges(s).n /*prep_w, prep_z, deslice*/ +
-         (x3_shape(s) ? 3 /*splits of x, fx; of x*/ : 0);
+  return 4 /*prep, stats, slice, reduce*/ + 1 /*prep*/ + x3_ranges(s).n /*deslice*/;
 }
 
 size_t tc_slice_partials_bytes(const Shape& s0) {
@@ -1096,50 +1083,61 @@ size_t tc_slice_prep_bytes(const Shape& s0) {
 }
 size_t tc_deslice_prep_bytes(const Shape& s0) {
   const Shape s = tc_padded(s0);
-  const X3Ranges xr = x3_ranges(s0);
-  // with several X3 ranges, a range's slices of W, bias and z' too
-  const size_t gather = xr.n > 1 ? align_up((size_t)s.H * (kD + 1) * xr.size * sizeof(float), 256) +
-                                       align_up((size_t)s.BH() * xr.size * kD * sizeof(float), 256)
-                                 : 0;
   return tc_forward_supported(s0) ? align_up(w_image_bytes(s), 256) + align_up(z_image_bytes(s), 256) +
-                                        align_up(px_bytes(s), 256) + (x3_shape(s) ? 2 * half_bytes(s) : 0) + gather
+                                        align_up(px_bytes(s), 256) + (x3_shape(s) ? 2 * half_bytes(s) : 0)
                                   : 0;
 }
 
 cudaError_t tc_stats(const Shape& s0, const void* x, const float* W, const float* bias, const float* tau, float* lse,
-                     void* prep, uint32_t* status, cudaStream_t st) {
+                     void* prep, bool reset, uint32_t* status, cudaStream_t st) {
   const Shape s = tc_padded(s0);
   uint8_t* wimg = static_cast<uint8_t*>(prep);
   uint8_t* px = wimg + align_up(w_image_bytes(s), 256) + align_up(z_image_bytes(s), 256);
   uint8_t* xh = px + align_up(px_bytes(s), 256);
-  cudaError_t e = prep_w(s, s0.G, W, bias, tau, wimg, status, st);
-  if (e != cudaSuccess) return e;
-  if (!x3_shape(s)) return run_stats(s, x, nullptr, wimg, lse, px, status, st);
-  if ((e = split_points(s, x, xh, st)) != cudaSuccess) return e;
-  return run_stats(s, xh, xh + half_bytes(s), wimg, lse, px, status, st);
+  const bool x3 = x3_shape(s);
+  Prepare p(s, s0.G, tau, status, reset);
+  p.weights(W, bias, wimg);
+  if (x3) p.split(s, x, xh, half_bytes(s));
+  if (cudaError_t e = p.run(st)) return e;
+  return run_stats(s, x3 ? xh : x, x3 ? xh + half_bytes(s) : nullptr, wimg, lse, px, status, st);
 }
 
-cudaError_t tc_slice_fwd(const Shape& s0, const void* x, const void* f, const float* W, const float* bias,
-                         const float* tau, float* tokens, float* wsum, float* lse, int finalize, float* part,
-                         void* prep, uint32_t* status, cudaStream_t st) {
+// The slice with its statistics pass (lse an output) or, with given, without it.
+static cudaError_t slice_with_prep(const Shape& s0, const void* x, const void* f, const float* W, const float* bias,
+                                   const float* tau, float* tokens, float* wsum, float* lse, const float* given,
+                                   int finalize, float* part, void* prep, bool reset, uint32_t* status,
+                                   cudaStream_t st) {
   const Shape s = tc_padded(s0);
   uint8_t* wimg = static_cast<uint8_t*>(prep);
   uint8_t* px = wimg + align_up(w_image_bytes(s), 256);
   uint8_t* xh = px + align_up(px_bytes(s), 256);
   uint8_t* fh = xh + 2 * half_bytes(s);
-  cudaError_t e = prep_w(s, s0.G, W, bias, tau, wimg, status, st);
-  if (e != cudaSuccess) return e;
+  Prepare p(s, s0.G, tau, status, reset);
+  p.weights(W, bias, wimg);
+  if (given) p.rows(given, px);
   const void *xr = nullptr, *fr = nullptr;
   if (x3_shape(s)) {
-    if ((e = split_points(s, x, xh, st)) != cudaSuccess) return e;
-    if ((e = split_points(s, f, fh, st)) != cudaSuccess) return e;
-    x = xh;
-    xr = xh + half_bytes(s);
-    f = fh;
-    fr = fh + half_bytes(s);
+    p.split(s, x, xh, half_bytes(s));
+    p.split(s, f, fh, half_bytes(s));
+    x = xh, xr = xh + half_bytes(s);
+    f = fh, fr = fh + half_bytes(s);
   }
-  if ((e = run_stats(s, x, xr, wimg, lse, px, status, st)) != cudaSuccess) return e;
+  cudaError_t e = p.run(st);
+  if (e != cudaSuccess) return e;
+  if (!given && (e = run_stats(s, x, xr, wimg, lse, px, status, st)) != cudaSuccess) return e;
   return run_slice(s, s0.G, x, f, xr, fr, wimg, px, tokens, wsum, finalize, part, status, st);
+}
+
+cudaError_t tc_slice_fwd(const Shape& s0, const void* x, const void* f, const float* W, const float* bias,
+                         const float* tau, float* tokens, float* wsum, float* lse, int finalize, float* part,
+                         void* prep, bool reset, uint32_t* status, cudaStream_t st) {
+  return slice_with_prep(s0, x, f, W, bias, tau, tokens, wsum, lse, nullptr, finalize, part, prep, reset, status, st);
+}
+
+cudaError_t tc_slice_fwd_lse(const Shape& s0, const void* x, const void* f, const float* W, const float* bias,
+                             const float* tau, const float* lse, float* tokens, float* wsum, int finalize,
+                             float* part, void* prep, bool reset, uint32_t* status, cudaStream_t st) {
+  return slice_with_prep(s0, x, f, W, bias, tau, tokens, wsum, nullptr, lse, finalize, part, prep, reset, status, st);
 }
 
 // The slice on prepared operands: the W image and the point-extra rows at px; xr and
@@ -1168,88 +1166,43 @@ cudaError_t run_slice(const Shape& s, int G, const void* x, const void* f, const
   return simt_reduce_tokens(so, P, part, s.G, tokens, wsum, finalize, st);
 }
 
-cudaError_t tc_slice_fwd_lse(const Shape& s0, const void* x, const void* f, const float* W, const float* bias,
-                             const float* tau, const float* lse, float* tokens, float* wsum, int finalize,
-                             float* part, void* prep, uint32_t* status, cudaStream_t st) {
-  const Shape s = tc_padded(s0);
-  uint8_t* wimg = static_cast<uint8_t*>(prep);
-  uint8_t* px = wimg + align_up(w_image_bytes(s), 256);
-  uint8_t* xh = px + align_up(px_bytes(s), 256);
-  uint8_t* fh = xh + 2 * half_bytes(s);
-  cudaError_t e = prep_w(s, s0.G, W, bias, tau, wimg, status, st);
-  if (e != cudaSuccess) return e;
-  const int64_t Np = padded_n(s), npx = s.BH() * Np;
-  k_prep_px<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(lse, reinterpret_cast<uint4*>(px), s.BH(), s.N, Np);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const void *xr = nullptr, *fr = nullptr;
-  if (x3_shape(s)) {
-    if ((e = split_points(s, x, xh, st)) != cudaSuccess) return e;
-    if ((e = split_points(s, f, fh, st)) != cudaSuccess) return e;
-    x = xh;
-    xr = xh + half_bytes(s);
-    f = fh;
-    fr = fh + half_bytes(s);
-  }
-  return run_slice(s, s0.G, x, f, xr, fr, wimg, px, tokens, wsum, finalize, part, status, st);
-}
-
 cudaError_t tc_deslice_fwd(const Shape& s0, const void* x, const float* W, const float* bias, const float* tau,
-                           const float* zp, const float* lse, void* out, void* prep, uint32_t* status,
+                           const float* zp, const float* lse, void* out, void* prep, bool reset, uint32_t* status,
                            cudaStream_t st) {
-  const Shape sf = tc_padded(s0);  // the whole problem (layout of the workspace)
-  const bool x3 = x3_shape(sf);
+  const Shape s = tc_padded(s0);
+  const bool x3 = x3_shape(s);
   const X3Ranges xr = x3_ranges(s0);
-  const bool ranged = xr.n > 1;
-  Shape s = sf;  // the shape the kernel sees: G = the range's slots
-  s.G = xr.size;
   uint8_t* wimg = static_cast<uint8_t*>(prep);
-  uint8_t* zimg = wimg + align_up(w_image_bytes(sf), 256);
-  uint8_t* px = zimg + align_up(z_image_bytes(sf), 256);
-  uint8_t* xh = px + align_up(px_bytes(sf), 256);
-  float* wc = reinterpret_cast<float*>(xh + (x3 ? 2 * half_bytes(sf) : 0));  // range slices (ranged only)
-  float* bc = wc + (size_t)s.H * kD * xr.size;
-  float* zc = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(wc) +
-                                       align_up((size_t)s.H * (kD + 1) * xr.size * sizeof(float), 256));
-  cudaError_t e;
-  const int64_t Np = padded_n(s), npx = s.BH() * Np;
-  k_prep_px<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(lse, reinterpret_cast<uint4*>(px), s.BH(), s.N, Np);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (x3 && (e = split_points(s, x, xh, st)) != cudaSuccess) return e;
+  uint8_t* zimg = wimg + align_up(w_image_bytes(s), 256);
+  uint8_t* px = zimg + align_up(z_image_bytes(s), 256);
+  uint8_t* xh = px + align_up(px_bytes(s), 256);
+  // With split products the z' image holds z' hi then its residual (G*128 bytes per (b,h)).
+  Prepare p(s, s0.G, tau, status, reset);
+  p.weights(W, bias, wimg);
+  p.tokens(zp, nullptr, zimg, x3);
+  p.rows(lse, px);
+  if (x3) p.split(s, x, xh, half_bytes(s));
+  cudaError_t e = p.run(st);
+  if (e != cudaSuccess) return e;
   CUtensorMap xmap, pmap, xrmap;
   if (!make_point_map(&xmap, x3 ? xh : x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B)) return cudaErrorInvalidValue;
   if (!make_point_map(&xrmap, x3 ? xh + half_bytes(s) : x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B))
     return cudaErrorInvalidValue;
-  if (!make_px_map(&pmap, px, s.BH(), Np)) return cudaErrorInvalidValue;
+  if (!make_px_map(&pmap, px, s.BH(), padded_n(s))) return cudaErrorInvalidValue;
   const int P = point_splits(s, (int)s.BH());
   const bool split = s.dot == FS_DOT_BF16X2 || x3;
-  // With split products the image holds z' hi then its residual (G*128 bytes per (b,h)).
   const bool ps = x3;
-  const bool hilo = split && smem_deslice(s.G, true, 0, ps, x3) <= kMaxSmem;  // up to G = 768 (bf16)
-  const size_t sm = smem_deslice(s.G, hilo, 0, ps, x3);
+  const bool hilo = split && smem_deslice(xr.size, true, 0, ps, x3) <= kMaxSmem;  // up to G = 768 (bf16)
+  const size_t sm = smem_deslice(xr.size, hilo, 0, ps, x3);
   if (sm > kMaxSmem) return cudaErrorInvalidValue;
   const auto kernel = x3 ? k_deslice<0, true, true> : k_deslice<0, false>;
   if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
   for (int k = 0; k < xr.n; k++) {
-    const int g0 = k * xr.size, G = ranged ? std::min(xr.size, s0.G - g0) : s0.G;
-    const float *Wk = W, *bk = bias, *zk = zp;
-    if (ranged) {
-      if ((e = copy_rows(wc, G, W + g0, s0.G, G, (int64_t)s.H * kD, st)) != cudaSuccess) return e;
-      if ((e = copy_rows(bc, G, bias + g0, s0.G, G, s.H, st)) != cudaSuccess) return e;
-      if ((e = copy_rows(zc, (int64_t)G * kD, zp + (int64_t)g0 * kD, (int64_t)s0.G * kD, (int64_t)G * kD, s.BH(),
-                         st)) != cudaSuccess)
-        return e;
-      Wk = wc, bk = bc, zk = zc;
-    }
-    if ((e = prep_w(s, G, Wk, bk, tau, wimg, status, st)) != cudaSuccess) return e;
-    const int64_t nz = s.BH() * s.G * kD;
-    if (ps)
-      k_prep_z2<<<(unsigned)((nz + 255) / 256), 256, 0, st>>>(zk, kD, zimg, s.BH(), G, s.G);
-    else
-      k_prep_z<<<(unsigned)((nz + 255) / 256), 256, 0, st>>>(zk, zimg, s.BH(), G, s.G);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int g0 = k * xr.size;
     kernel<<<dim3((unsigned)P, (unsigned)s.BH()), x3 ? kThreads : kDesl3Threads, sm, st>>>(
-        xmap, pmap, xrmap, wimg, zimg, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr, s.N, Np,
-        s.H, s.G, P, hilo ? 1 : 0, (uint32_t)s.G * (ps ? 128 : 64), k > 0 ? 1 : 0, status);
+        xmap, pmap, xrmap, wimg, zimg, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr, s.N,
+        padded_n(s), s.H, s.G, g0, std::min(xr.size, s.G - g0), P, hilo ? 1 : 0, (uint32_t)s.G * (ps ? 128 : 64),
+        k > 0 ? 1 : 0, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1257,9 +1210,9 @@ cudaError_t tc_deslice_fwd(const Shape& s0, const void* x, const float* W, const
 
 size_t tc_rows_smem(const Shape& s, int mode, bool ps, bool hilo) { return smem_deslice(s.G, hilo, mode, ps); }
 
-cudaError_t tc_rows_bwd(const Shape& s, int mode, const void* x, const uint8_t* wimg, const uint8_t* zimg,
-                        const void* px, const void* v, void* dfx, float* delta, float* wds, const float* dS,
-                        int accumulate, uint32_t* status, cudaStream_t st) {
+cudaError_t tc_rows_bwd(const Shape& s, int Gi, int g0, int mode, const void* x, const uint8_t* wimg,
+                        const uint8_t* zimg, const void* px, const void* v, void* dfx, float* delta, float* wds,
+                        const float* dS, int accumulate, uint32_t* status, cudaStream_t st) {
   const bool split = s.dot == FS_DOT_BF16X2;
   const bool ps = split && smem_deslice(s.G, false, mode, true) <= kMaxSmem;
   const bool hilo = split && smem_deslice(s.G, true, mode, ps) <= kMaxSmem;
@@ -1276,8 +1229,8 @@ cudaError_t tc_rows_bwd(const Shape& s, int mode, const void* x, const uint8_t* 
   cudaError_t e = set_smem(kernel, sm);
   if (e != cudaSuccess) return e;
   kernel<<<grid, kThreads, sm, st>>>(xmap, pmap, xmap, wimg, zimg, static_cast<__nv_bfloat16*>(dfx),
-                                     static_cast<const __nv_bfloat16*>(v), delta, wds, dS, s.N, Np, s.H, s.G, P,
-                                     hilo ? 1 : 0, (uint32_t)s.G * 128, accumulate, status);
+                                     static_cast<const __nv_bfloat16*>(v), delta, wds, dS, s.N, Np, s.H, Gi, g0, s.G,
+                                     P, hilo ? 1 : 0, (uint32_t)Gi * 128, accumulate, status);
   return cudaGetLastError();
 }
 
