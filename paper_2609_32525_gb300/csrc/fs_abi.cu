@@ -178,9 +178,8 @@ fs_status check_ws(const Shape& s, int op, void* ws, size_t ws_bytes) {
 
 fs_status cuda_status(cudaError_t e) { return e == cudaSuccess ? FS_OK : FS_ERR_CUDA; }
 
-// Every ws-using call starts by clearing its status word: the tensor-core calls in their
-// first kernel (the preparation), the others with a memset.
-cudaError_t reset_status(void* ws, cudaStream_t st) { return cudaMemsetAsync(ws, 0, sizeof(uint32_t), st); }
+// Every ws-using call writes its status word anew: the first of its kernels that knows the
+// temperatures does (`reset`), so that no memset breaks the chain of kernels.
 
 // The backward forms its weights from fp32 logits, so it needs lse to ~1e-5.  On
 // tensor-core shapes with bf16 products the forward's lse comes from logits with
@@ -192,11 +191,7 @@ cudaError_t reset_status(void* ws, cudaStream_t st) { return cudaMemsetAsync(ws,
 cudaError_t backward_stats(const Shape& sh, const void* x_mid, const float* W_slice, const float* bias,
                            const float* tau, const float* lse, void* ws, const Regions& r, uint32_t* status,
                            cudaStream_t st, const float** lse_use, bool* reset) {
-  // *reset: the status word is still to be cleared by the call's next launch (a SIMT backward
-  // has no preparation that could).
-  *reset = tc_backward_supported(sh);
-  if (!*reset)
-    if (cudaError_t e = reset_status(ws, st)) return e;
+  *reset = true;  // no kernel has written the status word yet
   *lse_use = lse;
   // fp32 shapes take the fp32 SIMT backward: it gets exact fp32 statistics (the
   // forward's come from split bf16 products on the tensor cores).
@@ -205,16 +200,11 @@ cudaError_t backward_stats(const Shape& sh, const void* x_mid, const float* W_sl
   if (lse && !fp32_tc && (!tc || sh.dot == FS_DOT_BF16X2)) return cudaSuccess;
   float* buf = at<float>(ws, r.stats);
   *lse_use = buf;
-  const bool clear = *reset;
   *reset = false;
-  if (!tc) {
-    if (clear)
-      if (cudaError_t e = reset_status(ws, st)) return e;
-    return simt_stats(sh, x_mid, W_slice, bias, tau, buf, status, st);
-  }
+  if (!tc) return simt_stats(sh, x_mid, W_slice, bias, tau, buf, true, status, st);
   Shape split = sh;
   split.dot = FS_DOT_BF16X2;
-  return tc_stats(split, x_mid, W_slice, bias, tau, buf, at<void>(ws, r.tc), clear, status, st);
+  return tc_stats(split, x_mid, W_slice, bias, tau, buf, at<void>(ws, r.tc), true, status, st);
 }
 
 #define FS_CHECK_SHAPE(s)                               \
@@ -324,11 +314,10 @@ fs_status fs_slice_fwd(const fs_shape* s, const void* x_mid, const void* fx, con
     return cuda_status(tc_slice_fwd(sh, x_mid, fx, W_slice, bias, tau, tokens, wsum, lse_buf, finalize,
                                     at<float>(ws, r.partials), at<void>(ws, r.tc), true, status, st));
   }
-  FS_CUDA(reset_status(ws, st));
   const int P = slot_splits(sh);
   float* part = at<float>(ws, r.partials);
-  FS_CUDA(simt_stats(sh, x_mid, W_slice, bias, tau, lse_buf, status, st));
-  FS_CUDA(simt_slice_partials(sh, P, x_mid, fx, W_slice, bias, tau, lse_buf, part, status, st));
+  FS_CUDA(simt_stats(sh, x_mid, W_slice, bias, tau, lse_buf, true, status, st));
+  FS_CUDA(simt_slice_partials(sh, P, x_mid, fx, W_slice, bias, tau, lse_buf, part, false, status, st));
   FS_CUDA(simt_reduce_tokens(sh, P, part, sh.G, tokens, wsum, finalize, st));
   return FS_OK;
 }
@@ -344,8 +333,7 @@ fs_status fs_stats(const fs_shape* s, const void* x_mid, const float* W_slice, c
   uint32_t* status = at<uint32_t>(ws, r.status);
   if (tc_forward_supported(sh))
     return cuda_status(tc_stats(sh, x_mid, W_slice, bias, tau, lse, at<void>(ws, r.tc), true, status, st));
-  FS_CUDA(reset_status(ws, st));
-  return cuda_status(simt_stats(sh, x_mid, W_slice, bias, tau, lse, status, st));
+  return cuda_status(simt_stats(sh, x_mid, W_slice, bias, tau, lse, true, status, st));
 }
 
 fs_status fs_slice_fwd_lse(const fs_shape* s, const void* x_mid, const void* fx, const float* W_slice,
@@ -362,10 +350,9 @@ fs_status fs_slice_fwd_lse(const fs_shape* s, const void* x_mid, const void* fx,
   if (tc_forward_supported(sh))
     return cuda_status(tc_slice_fwd_lse(sh, x_mid, fx, W_slice, bias, tau, lse, tokens, wsum, finalize,
                                         at<float>(ws, r.partials), at<void>(ws, r.tc), true, status, st));
-  FS_CUDA(reset_status(ws, st));
   const int P = slot_splits(sh);
   float* part = at<float>(ws, r.partials);
-  FS_CUDA(simt_slice_partials(sh, P, x_mid, fx, W_slice, bias, tau, lse, part, status, st));
+  FS_CUDA(simt_slice_partials(sh, P, x_mid, fx, W_slice, bias, tau, lse, part, true, status, st));
   FS_CUDA(simt_reduce_tokens(sh, P, part, sh.G, tokens, wsum, finalize, st));
   return FS_OK;
 }
@@ -422,13 +409,9 @@ fs_status fs_deslice_fwd(const fs_shape* s, const void* x_mid, const float* W_sl
     return cuda_status(tc_deslice_fwd(sh, x_mid, W_slice, bias, tau, tokens_mixed, lse ? lse : buf, out,
                                       at<void>(ws, r.tc), lse != nullptr, status, st));
   }
-  FS_CUDA(reset_status(ws, st));
-  const float* lse_use = lse;
-  if (!lse_use) {
-    FS_CUDA(simt_stats(sh, x_mid, W_slice, bias, tau, buf, status, st));
-    lse_use = buf;
-  }
-  return cuda_status(simt_deslice(sh, x_mid, W_slice, bias, tau, tokens_mixed, lse_use, out, status, st));
+  if (!lse) FS_CUDA(simt_stats(sh, x_mid, W_slice, bias, tau, buf, true, status, st));
+  return cuda_status(simt_deslice(sh, x_mid, W_slice, bias, tau, tokens_mixed, lse ? lse : buf, out, lse != nullptr,
+                                  status, st));
 }
 
 fs_status fs_deslice_bwd(const fs_shape* s, const void* x_mid, const float* W_slice, const float* bias,
@@ -454,7 +437,7 @@ fs_status fs_deslice_bwd(const fs_shape* s, const void* x_mid, const float* W_sl
   return cuda_status(simt_deslice_bwd(sh, slot_splits(sh), x_mid, W_slice, bias, tau, tokens_mixed, lse_use, dout,
                                       d_tokens_mixed, dx_mid, dW, dbias, dtau, accumulate, at<float>(ws, r.delta),
                                       at<float>(ws, r.partials), at<float>(ws, r.dtau_p),
-                                      at<uint32_t>(ws, r.status), st));
+                                      reset, at<uint32_t>(ws, r.status), st));
 }
 
 fs_status fs_mix_bwd(const fs_shape* s, const float* M, const float* tokens, const float* d_tokens_mixed,
@@ -490,7 +473,7 @@ fs_status fs_slice_bwd(const fs_shape* s, const void* x_mid, const void* fx, con
   return cuda_status(simt_slice_bwd(sh, slot_splits(sh), x_mid, fx, W_slice, bias, tau, tokens, wsum, lse_use,
                                     d_tokens, dx_mid, dfx, dW, dbias, dtau, accumulate, at<float>(ws, r.delta),
                                     at<float>(ws, r.dus), at<float>(ws, r.partials), at<float>(ws, r.dtau_p),
-                                    at<uint32_t>(ws, r.status), st));
+                                    reset, at<uint32_t>(ws, r.status), st));
 }
 
 fs_status fs_coupling_bwd(const fs_shape* s, const void* x_mid, const void* fx, const float* W_slice,
@@ -520,7 +503,7 @@ fs_status fs_coupling_bwd(const fs_shape* s, const void* x_mid, const void* fx, 
     return cuda_status(simt_coupling_bwd(sh, slot_splits(sh), x_mid, fx, dout, W_slice, bias, tau, M, tokens, wsum,
                                          tokens_mixed, lse_use, d_tokens_mixed, d_tokens, dM, dx_mid, dfx, dW, dbias,
                                          dtau, accumulate, at<float>(ws, r.delta), at<float>(ws, r.dus),
-                                         at<float>(ws, r.partials), at<float>(ws, r.dtau_p), status, st));
+                                         at<float>(ws, r.partials), at<float>(ws, r.dtau_p), reset, status, st));
   }
   const Regions r = regions(sh, FS_OP_COUPLING_BWD);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

@@ -36,10 +36,10 @@ int slot_splits(const Shape& s);
 // buffer holds one float per (b, h, point block).
 int64_t simt_point_blocks(const Shape& s);
 cudaError_t simt_stats(const Shape& s, const void* x, const float* W, const float* bias,
-                       const float* tau, float* lse, uint32_t* status, cudaStream_t st);
+                       const float* tau, float* lse, bool reset, uint32_t* status, cudaStream_t st);
 cudaError_t simt_slice_partials(const Shape& s, int P, const void* x, const void* f,
                                 const float* W, const float* bias, const float* tau,
-                                const float* lse, float* part, uint32_t* status, cudaStream_t st);
+                                const float* lse, float* part, bool reset, uint32_t* status, cudaStream_t st);
 // Fixed-order sum of split partials [P, B*H, Gs, d+1] (Gs >= G slot rows per (b, h);
 // the first G are reduced) into tokens (normalised when finalize) and wsum.
 cudaError_t simt_reduce_tokens(const Shape& s, int P, const float* part, int Gs, float* tokens,
@@ -58,12 +58,12 @@ cudaError_t simt_mix_bwd(const Shape& s, const float* M, const float* z, const f
                          float* dz, float* dM, cudaStream_t st);
 cudaError_t simt_deslice(const Shape& s, const void* x, const float* W, const float* bias,
                          const float* tau, const float* zp, const float* lse, void* out,
-                         uint32_t* status, cudaStream_t st);
+                         bool reset, uint32_t* status, cudaStream_t st);
 cudaError_t simt_deslice_bwd(const Shape& s, int P, const void* x, const float* W,
                              const float* bias, const float* tau, const float* zp,
                              const float* lse, const void* dout, float* dzp, void* dx,
                              float* dW, float* db, float* dtau, int accumulate, float* delta,
-                             float* part, float* dt_part, uint32_t* status, cudaStream_t st);
+                             float* part, float* dt_part, bool reset, uint32_t* status, cudaStream_t st);
 // dUS[bh][g] = (dz_g / (S_g + eps), -(dz_g . z_g) / (S_g + eps)) (d + 1 floats per slot).
 cudaError_t simt_slice_bwd_prep(const Shape& s, const float* z, const float* wsum, const float* dz, float* dUS,
                                 cudaStream_t st);
@@ -85,7 +85,7 @@ cudaError_t simt_coupling_bwd(const Shape& s, int P, const void* x, const void* 
                               const float* W, const float* bias, const float* tau, const float* M, const float* z,
                               const float* wsum, const float* zp, const float* lse, float* dzp, float* dz,
                               float* dM, void* dx, void* dfx, float* dW, float* db, float* dtau, int accumulate,
-                              float* delta, float* dUS, float* part, float* dt_part, uint32_t* status,
+                              float* delta, float* dUS, float* part, float* dt_part, bool reset, uint32_t* status,
                               cudaStream_t st);
 int simt_coupling_bwd_launch_count();
 // The token gradient alone from partials whose first d words per slot are dz'.
@@ -95,6 +95,6 @@ cudaError_t simt_slice_bwd(const Shape& s, int P, const void* x, const void* f, 
                            const float* wsum, const float* lse, const float* dz, void* dx,
                            void* dfx, float* dW, float* db, float* dtau, int accumulate,
                            float* delta, float* dUS, float* part, float* dt_part,
-                           uint32_t* status, cudaStream_t st);
+                           bool reset, uint32_t* status, cudaStream_t st);
 
 }  // namespace fs

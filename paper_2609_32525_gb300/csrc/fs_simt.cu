@@ -3,6 +3,7 @@
 // problems, the backward of fp32 inputs), and the small fp32 kernels that every path
 // shares: the fixed-order reductions, the mixes and their backward.  No float atomics
 // anywhere.
+#include "fs_launch.h"
 #include "fs_simt_tiles.h"
 
 #include <cuda_bf16.h>
@@ -17,6 +18,7 @@ namespace {
 __global__ void k_reduce_tokens(const float* __restrict__ part, int P, int64_t BH, int G, int Gs, int D,
                                 float* __restrict__ tokens, float* __restrict__ wsum, int finalize,
                                 float eps) {
+  grid_begin(part);
   // One warp per output row bh * G + g; lane l sums columns l, l + 32, l + 64 (<= D)
   // of its partial row over the splits, loads four splits ahead.
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -52,6 +54,7 @@ __global__ void k_reduce_tokens(const float* __restrict__ part, int P, int64_t B
 
 __global__ void k_finalize(float* __restrict__ tokens, const float* __restrict__ wsum, int64_t BHG,
                            int D, float eps) {
+  grid_begin(tokens, wsum);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= BHG * D) return;
   tokens[i] = tokens[i] / (wsum[i / D] + eps);
@@ -212,6 +215,7 @@ __device__ __forceinline__ void mix_tile(float* sm, const float* __restrict__ M,
 template <bool kTrans, bool kVec>
 __global__ void __launch_bounds__(256) k_mix_tiled(const float* __restrict__ M, const float* __restrict__ in,
                                                    float* __restrict__ out, int H, int G, int D) {
+  grid_begin(M, in);
   __shared__ __align__(16) float sm[mix_words<kTrans>()];
   mix_tile<kTrans, kVec>(sm, M, in, out, H, G, D, blockIdx.x, blockIdx.y, blockIdx.z);
 }
@@ -224,6 +228,7 @@ static_assert(8 * kMixTG * kMixTC <= kMixStages * (kMixKC * kMixTC + kMixTG * (k
 template <bool kTrans>
 __global__ void k_mix_channels(const float* __restrict__ Wc, const float* __restrict__ in, float* __restrict__ out,
                                int64_t BHG, int H, int G, int D) {
+  grid_begin(Wc, in);
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= BHG * D) return;
   const int c = (int)(idx % D);
@@ -239,6 +244,7 @@ __global__ void k_mix_channels(const float* __restrict__ Wc, const float* __rest
 // dWc[h][c][k] = sum over b and g of dzp[b,h,g,c] z[b,h,g,k] (fixed order: b, then g).
 __global__ void k_mix_channels_dW(const float* __restrict__ z, const float* __restrict__ dzp, float* __restrict__ dWc,
                                   int64_t B, int H, int G, int D) {
+  grid_begin(z, dzp);
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)H * D * D) return;
   const int k = (int)(idx % D), c = (int)((idx / D) % D), h = (int)(idx / ((int64_t)D * D));
@@ -305,6 +311,7 @@ __device__ __forceinline__ void dM_tile(float* sm, const float* __restrict__ z, 
 
 __global__ void __launch_bounds__(256) k_mix_bwd_dM(const float* __restrict__ z, const float* __restrict__ dzp,
                                                     float* __restrict__ dM, int64_t B, int H, int G, int D) {
+  grid_begin(z, dzp);
   __shared__ float sm[kDmWords];
   dM_tile(sm, z, dzp, dM, B, H, G, D, blockIdx.x, blockIdx.y, blockIdx.z);
 }
@@ -316,6 +323,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd(const float* __restrict__ M, co
                                                  const float* __restrict__ dzp, float* __restrict__ dz,
                                                  float* __restrict__ dM, int64_t B, int H, int G, int D, int nx,
                                                  int nc) {
+  grid_begin(M, z, dzp);
   constexpr int kWords = mix_words<true>() > kDmWords ? mix_words<true>() : kDmWords;
   __shared__ __align__(16) float sm[kWords];
   const int64_t n = (int64_t)nx * B * H * nc;
@@ -337,6 +345,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd(const float* __restrict__ M, co
 __global__ void __launch_bounds__(256) k_slice_bwd_prep(const float* __restrict__ z, const float* __restrict__ wsum,
                                                         const float* __restrict__ dz, float* __restrict__ dUS,
                                                         int64_t BHG, int D, float eps) {
+  grid_begin(z, wsum, dz);
   const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= BHG) return;  // whole warps
@@ -410,14 +419,17 @@ __device__ __forceinline__ void reduce_dtau(int h, const float* __restrict__ dt_
 __global__ void __launch_bounds__(256) k_reduce_bwd_params(const float* part, int P, int64_t B, int H, int G, int Gs,
                                                            int D, int PS, int off, const float* tau, float* dW,
                                                            float* db, int accumulate) {
+  grid_begin(part, tau);
   reduce_params((int64_t)blockIdx.x * 256 + threadIdx.x, part, P, B, H, G, Gs, D, PS, off, tau, dW, db, accumulate);
 }
 __global__ void __launch_bounds__(256) k_reduce_bwd_tokens(const float* part, int P, int64_t BH, int G, int Gs, int D,
                                                            int PS, float* dzp) {
+  grid_begin(part);
   reduce_dzp((int64_t)blockIdx.x * 256 + threadIdx.x, part, P, BH, G, Gs, D, PS, dzp);
 }
 __global__ void __launch_bounds__(256) k_reduce_dtau(const float* dt_part, int64_t B, int H, int64_t nblk,
                                                      const float* tau, float* dtau, int accumulate) {
+  grid_begin(dt_part, tau);
   reduce_dtau(blockIdx.x, dt_part, B, H, nblk, tau, dtau, accumulate);
 }
 // All of a backward call's reductions in one launch: blocks [0, n_par) dW and dbias,
@@ -426,6 +438,7 @@ __global__ void __launch_bounds__(256) k_reduce_bwd(const float* part, int P, in
                                                     int PS, const float* tau, float* dzp, float* dW, float* db,
                                                     float* dtau, const float* dt_part, int64_t nblk, int accumulate,
                                                     int64_t n_par) {
+  grid_begin(part, tau, dt_part);
   int64_t blk = blockIdx.x;
   if (blk < n_par)
     return reduce_params(blk * 256 + threadIdx.x, part, P, B, H, G, Gs, D, PS, dzp ? D : 0, tau, dW, db, accumulate);
@@ -440,18 +453,15 @@ cudaError_t simt_reduce_bwd(const Shape& s, int P, const float* part, int Gs, in
                             float* dzp, float* dW, float* db, float* dtau, const float* dt_part, int64_t nblk,
                             int accumulate, cudaStream_t st) {
   const int64_t nw = (int64_t)s.H * s.G * (s.d + 1);
-  k_reduce_bwd_params<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(part, P, s.B, s.H, s.G, Gs, s.d, PS,
-                                                                     has_dzp ? s.d : 0, tau, dW, db, accumulate);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch(k_reduce_bwd_params, dim3((unsigned)((nw + 255) / 256)), dim3(256), 0, st, part, P, s.B, s.H,
+                         s.G, Gs, s.d, PS, has_dzp ? s.d : 0, tau, dW, db, accumulate);
   if (e != cudaSuccess) return e;
   if (has_dzp) {
     const int64_t BHG = s.BH() * s.G;
-    k_reduce_bwd_tokens<<<(unsigned)((BHG * s.d + 255) / 256), 256, 0, st>>>(part, P, s.BH(), s.G, Gs, s.d, PS,
-                                                                              dzp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch(k_reduce_bwd_tokens, dim3((unsigned)((BHG * s.d + 255) / 256)), dim3(256), 0, st, part, P, s.BH(),
+                    s.G, Gs, s.d, PS, dzp)) != cudaSuccess) return e;
   }
-  k_reduce_dtau<<<s.H, 256, 0, st>>>(dt_part, s.B, s.H, nblk, tau, dtau, accumulate);
-  return cudaGetLastError();
+  return launch(k_reduce_dtau, dim3(s.H), dim3(256), 0, st, dt_part, s.B, s.H, nblk, tau, dtau, accumulate);
 }
 
 cudaError_t reduce_bwd(const Shape& s, int P, const float* part, int Gs, int PS, const float* tau, float* dzp,
@@ -459,33 +469,28 @@ cudaError_t reduce_bwd(const Shape& s, int P, const float* part, int Gs, int PS,
                        cudaStream_t st) {
   const int64_t n_par = ((int64_t)s.H * s.G * (s.d + 1) + 255) / 256;
   const int64_t n = n_par + s.H + (dzp ? (s.BH() * s.G * s.d + 255) / 256 : 0);
-  k_reduce_bwd<<<(unsigned)n, 256, 0, st>>>(part, P, s.B, s.H, s.G, Gs, s.d, PS, tau, dzp, dW, db, dtau, dt_part, nblk,
-                                            accumulate, n_par);
-  return cudaGetLastError();
+  return launch(k_reduce_bwd, dim3((unsigned)n), dim3(256), 0, st, part, P, s.B, s.H, s.G, Gs, s.d, PS, tau, dzp, dW,
+                db, dtau, dt_part, nblk, accumulate, n_par);
 }
 
 cudaError_t mix_bwd(const Shape& s, const float* M, const float* z, const float* dzp, float* dz, float* dM,
                     cudaStream_t st) {
   const int nx = (s.G + kMixTG - 1) / kMixTG, nc = (s.d + kMixTC - 1) / kMixTC, nt = (s.G + kDmT - 1) / kDmT;
   const int64_t n = (int64_t)nx * s.BH() * nc + (int64_t)nt * nt * s.H;
-  if (s.G % 4 == 0)
-    k_mix_bwd<true><<<(unsigned)n, 256, 0, st>>>(M, z, dzp, dz, dM, s.B, s.H, s.G, s.d, nx, nc);
-  else
-    k_mix_bwd<false><<<(unsigned)n, 256, 0, st>>>(M, z, dzp, dz, dM, s.B, s.H, s.G, s.d, nx, nc);
-  return cudaGetLastError();
+  return launch(s.G % 4 == 0 ? k_mix_bwd<true> : k_mix_bwd<false>, dim3((unsigned)n), dim3(256), 0, st, M, z, dzp, dz,
+                dM, s.B, s.H, s.G, s.d, nx, nc);
 }
 
 cudaError_t simt_reduce_dzp(const Shape& s, int P, const float* part, int Gs, int PS, float* dzp, cudaStream_t st) {
   const int64_t BHG = s.BH() * s.G;
-  k_reduce_bwd_tokens<<<(unsigned)((BHG * s.d + 255) / 256), 256, 0, st>>>(part, P, s.BH(), s.G, Gs, s.d, PS, dzp);
-  return cudaGetLastError();
+  return launch(k_reduce_bwd_tokens, dim3((unsigned)((BHG * s.d + 255) / 256)), dim3(256), 0, st, part, P, s.BH(), s.G,
+                Gs, s.d, PS, dzp);
 }
 
 cudaError_t simt_slice_bwd_prep(const Shape& s, const float* z, const float* wsum, const float* dz, float* dUS,
                                 cudaStream_t st) {
   const int64_t BHG = s.BH() * s.G;
-  k_slice_bwd_prep<<<(unsigned)((BHG + 7) / 8), 256, 0, st>>>(z, wsum, dz, dUS, BHG, s.d, s.eps);
-  return cudaGetLastError();
+  return launch(k_slice_bwd_prep, dim3((unsigned)((BHG + 7) / 8)), dim3(256), 0, st, z, wsum, dz, dUS, BHG, s.d, s.eps);
 }
 
 int64_t simt_point_blocks(const Shape& s) { return (s.N + kSimtTP - 1) / kSimtTP; }
@@ -503,106 +508,97 @@ T* out(void* p) { return static_cast<T*>(p); }
 
 template <typename T>
 cudaError_t launch_stats(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
-                         float* lse, uint32_t* status, cudaStream_t st) {
-  return SimtTiles<T>::stats(s, in<T>(x), W, bias, tau, lse, status, st);
+                         float* lse, bool reset, uint32_t* status, cudaStream_t st) {
+  return SimtTiles<T>::stats(s, in<T>(x), W, bias, tau, lse, reset, status, st);
 }
 template <typename T>
 cudaError_t launch_slice(const Shape& s, int P, const void* x, const void* f, const float* W, const float* bias,
-                         const float* tau, const float* lse, float* part, uint32_t* status, cudaStream_t st) {
-  return SimtTiles<T>::slice(s, P, in<T>(x), in<T>(f), W, bias, tau, lse, part, status, st);
+                         const float* tau, const float* lse, float* part, bool reset, uint32_t* status, cudaStream_t st) {
+  return SimtTiles<T>::slice(s, P, in<T>(x), in<T>(f), W, bias, tau, lse, part, reset, status, st);
 }
 template <typename T>
 cudaError_t launch_deslice(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
-                           const float* zp, const float* lse, void* o, uint32_t* status, cudaStream_t st) {
-  return SimtTiles<T>::deslice(s, in<T>(x), W, bias, tau, zp, lse, out<T>(o), status, st);
+                           const float* zp, const float* lse, void* o, bool reset, uint32_t* status, cudaStream_t st) {
+  return SimtTiles<T>::deslice(s, in<T>(x), W, bias, tau, zp, lse, out<T>(o), reset, status, st);
 }
 template <typename T>
 cudaError_t launch_bwd(const Shape& s, int mode, int P, const void* x, const void* dO, const void* fx,
                        const float* W, const float* bias, const float* tau, const float* zp, const float* dUS,
                        const float* lse, void* dx, void* dfx, float* delta, float* dt_part, float* part,
-                       int accumulate, uint32_t* status, cudaStream_t st) {
+                       int accumulate, bool reset, uint32_t* status, cudaStream_t st) {
   return SimtTiles<T>::backward(s, mode, P, in<T>(x), in<T>(dO), in<T>(fx), W, bias, tau, zp, dUS, lse, out<T>(dx),
-                                out<T>(dfx), delta, dt_part, part, accumulate, status, st);
+                                out<T>(dfx), delta, dt_part, part, accumulate, reset, status, st);
 }
 
 }  // namespace
 
 cudaError_t simt_stats(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
-                       float* lse, uint32_t* status, cudaStream_t st) {
-  return FS_DISPATCH(s, launch_stats, s, x, W, bias, tau, lse, status, st);
+                       float* lse, bool reset, uint32_t* status, cudaStream_t st) {
+  return FS_DISPATCH(s, launch_stats, s, x, W, bias, tau, lse, reset, status, st);
 }
 
 cudaError_t simt_slice_partials(const Shape& s, int P, const void* x, const void* f, const float* W,
                                 const float* bias, const float* tau, const float* lse, float* part,
-                                uint32_t* status, cudaStream_t st) {
-  return FS_DISPATCH(s, launch_slice, s, P, x, f, W, bias, tau, lse, part, status, st);
+                                bool reset, uint32_t* status, cudaStream_t st) {
+  return FS_DISPATCH(s, launch_slice, s, P, x, f, W, bias, tau, lse, part, reset, status, st);
 }
 
 cudaError_t simt_reduce_tokens(const Shape& s, int P, const float* part, int Gs, float* tokens, float* wsum,
                                int finalize, cudaStream_t st) {
   const int64_t n = s.BH() * s.G * 32;  // a warp per output row
-  k_reduce_tokens<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part, P, s.BH(), s.G, Gs, s.d, tokens, wsum, finalize,
-                                                               s.eps);
-  return cudaGetLastError();
+  return launch(k_reduce_tokens, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, part, P, s.BH(), s.G, Gs, s.d,
+                tokens, wsum, finalize, s.eps);
 }
 
 cudaError_t simt_finalize(const Shape& s, float* tokens, const float* wsum, cudaStream_t st) {
   const int64_t BHG = s.BH() * s.G;
-  k_finalize<<<(unsigned)((BHG * s.d + 255) / 256), 256, 0, st>>>(tokens, wsum, BHG, s.d, s.eps);
-  return cudaGetLastError();
+  return launch(k_finalize, dim3((unsigned)((BHG * s.d + 255) / 256)), dim3(256), 0, st, tokens, wsum, BHG, s.d, s.eps);
 }
 
 cudaError_t simt_mix(const Shape& s, const float* M, const float* z, float* zp, cudaStream_t st) {
   const dim3 grid((unsigned)((s.G + kMixTG - 1) / kMixTG), (unsigned)s.BH(), (unsigned)((s.d + kMixTC - 1) / kMixTC));
-  if (s.G % 4 == 0)
-    k_mix_tiled<false, true><<<grid, 256, 0, st>>>(M, z, zp, s.H, s.G, s.d);
-  else
-    k_mix_tiled<false, false><<<grid, 256, 0, st>>>(M, z, zp, s.H, s.G, s.d);
-  return cudaGetLastError();
+  return launch(s.G % 4 == 0 ? k_mix_tiled<false, true> : k_mix_tiled<false, false>, grid, dim3(256), 0, st, M, z, zp,
+                s.H, s.G, s.d);
 }
 
 cudaError_t simt_mix_bwd(const Shape& s, const float* M, const float* z, const float* dzp, float* dz, float* dM,
                          cudaStream_t st) {
   const dim3 grid((unsigned)((s.G + kMixTG - 1) / kMixTG), (unsigned)s.BH(), (unsigned)((s.d + kMixTC - 1) / kMixTC));
-  if (s.G % 4 == 0)
-    k_mix_tiled<true, true><<<grid, 256, 0, st>>>(M, dzp, dz, s.H, s.G, s.d);
-  else
-    k_mix_tiled<true, false><<<grid, 256, 0, st>>>(M, dzp, dz, s.H, s.G, s.d);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch(s.G % 4 == 0 ? k_mix_tiled<true, true> : k_mix_tiled<true, false>, grid, dim3(256), 0, st, M,
+                         dzp, dz, s.H, s.G, s.d);
   if (e != cudaSuccess) return e;
   const dim3 tiles((unsigned)((s.G + 63) / 64), (unsigned)((s.G + 63) / 64), (unsigned)s.H);
-  k_mix_bwd_dM<<<tiles, 256, 0, st>>>(z, dzp, dM, s.B, s.H, s.G, s.d);
-  return cudaGetLastError();
+  return launch(k_mix_bwd_dM, tiles, dim3(256), 0, st, z, dzp, dM, s.B, s.H, s.G, s.d);
 }
 
 cudaError_t simt_mix_channels(const Shape& s, const float* Wc, const float* z, float* zp, cudaStream_t st) {
   const int64_t BHG = s.BH() * s.G;
-  k_mix_channels<false><<<(unsigned)((BHG * s.d + 255) / 256), 256, 0, st>>>(Wc, z, zp, BHG, s.H, s.G, s.d);
-  return cudaGetLastError();
+  return launch(k_mix_channels<false>, dim3((unsigned)((BHG * s.d + 255) / 256)), dim3(256), 0, st, Wc, z, zp, BHG, s.H,
+                s.G, s.d);
 }
 
 cudaError_t simt_mix_channels_bwd(const Shape& s, const float* Wc, const float* z, const float* dzp, float* dz,
                                   float* dWc, cudaStream_t st) {
   const int64_t BHG = s.BH() * s.G;
-  k_mix_channels<true><<<(unsigned)((BHG * s.d + 255) / 256), 256, 0, st>>>(Wc, dzp, dz, BHG, s.H, s.G, s.d);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch(k_mix_channels<true>, dim3((unsigned)((BHG * s.d + 255) / 256)), dim3(256), 0, st, Wc, dzp, dz,
+                         BHG, s.H, s.G, s.d);
   if (e != cudaSuccess) return e;
   const int64_t n = (int64_t)s.H * s.d * s.d;
-  k_mix_channels_dW<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(z, dzp, dWc, s.B, s.H, s.G, s.d);
-  return cudaGetLastError();
+  return launch(k_mix_channels_dW, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, st, z, dzp, dWc, s.B, s.H, s.G,
+                s.d);
 }
 
 cudaError_t simt_deslice(const Shape& s, const void* x, const float* W, const float* bias, const float* tau,
-                         const float* zp, const float* lse, void* o, uint32_t* status, cudaStream_t st) {
-  return FS_DISPATCH(s, launch_deslice, s, x, W, bias, tau, zp, lse, o, status, st);
+                         const float* zp, const float* lse, void* o, bool reset, uint32_t* status, cudaStream_t st) {
+  return FS_DISPATCH(s, launch_deslice, s, x, W, bias, tau, zp, lse, o, reset, status, st);
 }
 
 cudaError_t simt_deslice_bwd(const Shape& s, int P, const void* x, const float* W, const float* bias,
                              const float* tau, const float* zp, const float* lse, const void* dout, float* dzp,
                              void* dx, float* dW, float* db, float* dtau, int accumulate, float* delta,
-                             float* part, float* dt_part, uint32_t* status, cudaStream_t st) {
+                             float* part, float* dt_part, bool reset, uint32_t* status, cudaStream_t st) {
   cudaError_t e = FS_DISPATCH(s, launch_bwd, s, 0, P, x, dout, nullptr, W, bias, tau, zp, nullptr, lse, dx, nullptr,
-                              delta, dt_part, part, accumulate, status, st);
+                              delta, dt_part, part, accumulate, reset, status, st);
   if (e != cudaSuccess) return e;
   return simt_reduce_bwd(s, P, part, s.G, 2 * s.d + 2, 1, tau, dzp, dW, db, dtau, dt_part, simt_point_blocks(s),
                          accumulate, st);
@@ -612,11 +608,11 @@ cudaError_t simt_slice_bwd(const Shape& s, int P, const void* x, const void* f, 
                            const float* bias, const float* tau, const float* z, const float* wsum,
                            const float* lse, const float* dz, void* dx, void* dfx, float* dW, float* db,
                            float* dtau, int accumulate, float* delta, float* dUS, float* part, float* dt_part,
-                           uint32_t* status, cudaStream_t st) {
+                           bool reset, uint32_t* status, cudaStream_t st) {
   cudaError_t e = simt_slice_bwd_prep(s, z, wsum, dz, dUS, st);
   if (e != cudaSuccess) return e;
   e = FS_DISPATCH(s, launch_bwd, s, 1, P, x, nullptr, f, W, bias, tau, nullptr, dUS, lse, dx, dfx, delta, dt_part,
-                  part, accumulate, status, st);
+                  part, accumulate, reset, status, st);
   if (e != cudaSuccess) return e;
   return simt_reduce_bwd(s, P, part, s.G, s.d + 2, 0, tau, nullptr, dW, db, dtau, dt_part, simt_point_blocks(s),
                          accumulate, st);
@@ -631,15 +627,15 @@ cudaError_t simt_coupling_bwd(const Shape& s, int P, const void* x, const void* 
                               const float* W, const float* bias, const float* tau, const float* M, const float* z,
                               const float* wsum, const float* zp, const float* lse, float* dzp, float* dz,
                               float* dM, void* dx, void* dfx, float* dW, float* db, float* dtau, int accumulate,
-                              float* delta, float* dUS, float* part, float* dt_part, uint32_t* status,
+                              float* delta, float* dUS, float* part, float* dt_part, bool reset, uint32_t* status,
                               cudaStream_t st) {
-  cudaError_t e = simt_slice_partials(s, P, x, dout, W, bias, tau, lse, part, status, st);
+  cudaError_t e = simt_slice_partials(s, P, x, dout, W, bias, tau, lse, part, reset, status, st);
   if (e != cudaSuccess) return e;
   if ((e = simt_reduce_tokens(s, P, part, s.G, dzp, dUS, 0, st)) != cudaSuccess) return e;
   if ((e = simt_mix_bwd(s, M, z, dzp, dz, dM, st)) != cudaSuccess) return e;
   if ((e = simt_slice_bwd_prep(s, z, wsum, dz, dUS, st)) != cudaSuccess) return e;
   e = FS_DISPATCH(s, launch_bwd, s, 2, P, x, dout, fx, W, bias, tau, zp, dUS, lse, dx, dfx, delta, dt_part, part,
-                  accumulate, status, st);
+                  accumulate, false, status, st);
   if (e != cudaSuccess) return e;
   return simt_reduce_bwd(s, P, part, s.G, s.d + 2, 0, tau, nullptr, dW, db, dtau, dt_part, simt_point_blocks(s),
                          accumulate, st);

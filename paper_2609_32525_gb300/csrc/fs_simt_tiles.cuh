@@ -37,6 +37,7 @@
 // stays finite.
 #pragma once
 
+#include "fs_launch.h"
 #include "fs_simt_tiles.h"
 
 #include <cuda_bf16.h>
@@ -77,10 +78,14 @@ struct Tile {
   static constexpr size_t kVectors = 2 * TP + 2 * TG + kWarps * TP;  // lse2, delta | beta, dS | sums of a pass
 };
 
-__device__ __forceinline__ bool tau_ok(float t, uint32_t* status) {
-  if (t > 0.f && t < INFINITY) return true;
-  if (threadIdx.x == 0 && status) atomicCAS(status, 0u, kDevBadTau);
-  return false;
+__device__ __forceinline__ bool tau_ok(float t) { return t > 0.f && t < INFINITY; }
+// The call's first launch writes the status word: one block looks at every temperature.
+__device__ __forceinline__ void write_status(bool reset, const float* tau, int H, uint32_t* status) {
+  if (!reset || blockIdx.x + blockIdx.y + blockIdx.z != 0) return;
+  int bad = 0;
+  for (int h = threadIdx.x; h < H; h += blockDim.x) bad |= !tau_ok(tau[h]);
+  bad = __syncthreads_or(bad);
+  if (threadIdx.x == 0) *status = bad ? kDevBadTau : kDevOk;
 }
 
 // ---- staging ---------------------------------------------------------------------------------
@@ -321,7 +326,10 @@ constexpr int resident(int blocks) { return D == 64 ? 1 : blocks; }
 template <int D, int TG, typename T>
 __global__ void __launch_bounds__(Tile<D, TG>::kThreads)
     k_tile_stats(const T* __restrict__ x, const float* __restrict__ W, const float* __restrict__ bias,
-                 const float* __restrict__ tau, float* __restrict__ lse, int64_t N, int H, int G, uint32_t* status) {
+                 const float* __restrict__ tau, float* __restrict__ lse, int64_t N, int H, int G, int reset,
+                 uint32_t* status) {
+  grid_begin(x, W, bias, tau);
+  write_status(reset, tau, H, status);
   using C = Tile<D, TG>;
   constexpr int NT = C::kThreads, NJ = C::kPairN;
   extern __shared__ __align__(16) float sm[];
@@ -331,7 +339,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads)
   float2* red = reinterpret_cast<float2*>(sB + TG);  // [warp columns][TP]
   const int64_t bh = blockIdx.y, b = bh / H;
   const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
+  if (!tau_ok(tau[h])) return;
   const float scale = kLog2e / tau[h];
   const int64_t n0 = (int64_t)blockIdx.x * TP;
   const Place<D, TG> pl;
@@ -414,7 +422,9 @@ template <int D, int TG, typename T>
 __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     k_tile_slice(const T* __restrict__ x, const T* __restrict__ f, const float* __restrict__ W,
                  const float* __restrict__ bias, const float* __restrict__ tau, const float* __restrict__ lse,
-                 float* __restrict__ part, int64_t N, int H, int G, int P, uint32_t* status) {
+                 float* __restrict__ part, int64_t N, int H, int G, int P, int reset, uint32_t* status) {
+  grid_begin(x, f, W, bias, tau, lse);
+  write_status(reset, tau, H, status);
   using C = Tile<D, TG>;
   constexpr int NT = C::kThreads, NJ = C::kPairN;
   extern __shared__ __align__(16) float sm[];
@@ -428,7 +438,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   const int g0 = blockIdx.x * TG;
   const int64_t bh = blockIdx.y, b = bh / H;
   const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
+  if (!tau_ok(tau[h])) return;
   const Place<D, TG> pl;
   stage_w<D, TG, NT>(sw, sB, W, bias, h, G, g0, kLog2e / tau[h]);
   float U[C::kSlM][C::kSlN], S[NJ];
@@ -486,7 +496,9 @@ template <int D, int TG, typename T>
 __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     k_tile_deslice(const T* __restrict__ x, const float* __restrict__ W, const float* __restrict__ bias,
                    const float* __restrict__ tau, const float* __restrict__ zp, const float* __restrict__ lse,
-                   T* __restrict__ out, int64_t N, int H, int G, uint32_t* status) {
+                   T* __restrict__ out, int64_t N, int H, int G, int reset, uint32_t* status) {
+  grid_begin(x, W, bias, tau, zp, lse);
+  write_status(reset, tau, H, status);
   using C = Tile<D, TG>;
   constexpr int NT = C::kThreads, NJ = C::kPairN;
   extern __shared__ __align__(16) float sm[];
@@ -498,7 +510,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   float* sB = sl + TP;
   const int64_t bh = blockIdx.y, b = bh / H;
   const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
+  if (!tau_ok(tau[h])) return;
   const float scale = kLog2e / tau[h];
   const int64_t n0 = (int64_t)blockIdx.x * TP;
   const Place<D, TG> pl;
@@ -545,7 +557,9 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
                      const float* __restrict__ W, const float* __restrict__ bias, const float* __restrict__ tau,
                      const float* __restrict__ zp, const float* __restrict__ dUS, const float* __restrict__ lse,
                      T* __restrict__ dx, T* __restrict__ dfx, float* __restrict__ delta, float* __restrict__ dt_part,
-                     int accumulate, int64_t N, int H, int G, uint32_t* status) {
+                     int accumulate, int64_t N, int H, int G, int reset, uint32_t* status) {
+  grid_begin(x, dO, fx, W, bias, tau, zp, dUS, lse);
+  write_status(reset, tau, H, status);
   using C = Tile<D, TG>;
   constexpr int NT = C::kThreads, NJ = C::kPairN, M2 = C::kPtM;
   constexpr bool kD = MODE != 1, kS = MODE != 0;
@@ -564,7 +578,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   float* red = sS + TG;  // [4][TP]
   const int64_t bh = blockIdx.y, b = bh / H;
   const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
+  if (!tau_ok(tau[h])) return;
   const float scale = kLog2e / tau[h];
   const int64_t n0 = (int64_t)blockIdx.x * TP;
   const Place<D, TG> pl;
@@ -702,8 +716,8 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     k_tile_bwd_slot(const T* __restrict__ x, const T* __restrict__ dO, const T* __restrict__ fx,
                     const float* __restrict__ W, const float* __restrict__ bias, const float* __restrict__ tau,
                     const float* __restrict__ zp, const float* __restrict__ dUS, const float* __restrict__ lse,
-                    const float* __restrict__ delta, float* __restrict__ part, int64_t N, int H, int G, int P,
-                    uint32_t* status) {
+                    const float* __restrict__ delta, float* __restrict__ part, int64_t N, int H, int G, int P) {
+  grid_begin(x, dO, fx, W, bias, tau, zp, dUS, lse, delta);
   using C = Tile<D, TG>;
   constexpr int NT = C::kThreads, NJ = C::kPairN;
   constexpr bool kD = MODE != 1, kS = MODE != 0;
@@ -724,7 +738,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   const int g0 = blockIdx.x * TG;
   const int64_t bh = blockIdx.y, b = bh / H;
   const int h = (int)(bh % H);
-  if (!tau_ok(tau[h], status)) return;
+  if (!tau_ok(tau[h])) return;
   const Place<D, TG> pl;
   stage_w<D, TG, NT>(sw, sB, W, bias, h, G, g0, kLog2e / tau[h]);
   if (kD) stage_tokens<D, TG, NT>(sz, zp + bh * G * D, G, g0);
@@ -837,40 +851,42 @@ cudaError_t with_tile(const Shape& s, Fn fn) {
 
 template <typename T>
 cudaError_t SimtTiles<T>::stats(const Shape& s, const T* x, const float* W, const float* bias, const float* tau,
-                                float* lse, uint32_t* status, cudaStream_t st) {
+                                float* lse, bool reset, uint32_t* status, cudaStream_t st) {
   return with_tile(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value;
     constexpr size_t sm = tile_bytes<D, TG>(1, 1, 0);
     const auto k = k_tile_stats<D, TG, T>;
     if (cudaError_t e = allow_smem(k, sm)) return e;
-    k<<<point_grid(s), Tile<D, TG>::kThreads, sm, st>>>(x, W, bias, tau, lse, s.N, s.H, s.G, status);
-    return cudaGetLastError();
+    return launch(k, point_grid(s), dim3(Tile<D, TG>::kThreads), sm, st, x, W, bias, tau, lse, s.N, s.H, s.G, reset,
+                  status);
   });
 }
 
 template <typename T>
 cudaError_t SimtTiles<T>::slice(const Shape& s, int P, const T* x, const T* f, const float* W, const float* bias,
-                                const float* tau, const float* lse, float* part, uint32_t* status, cudaStream_t st) {
+                                const float* tau, const float* lse, float* part, bool reset, uint32_t* status,
+                                cudaStream_t st) {
   return with_tile(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value;
     constexpr size_t sm = tile_bytes<D, TG>(2, 1, 1);
     const auto k = k_tile_slice<D, TG, T>;
     if (cudaError_t e = allow_smem(k, sm)) return e;
-    k<<<slot_grid<TG>(s, P), Tile<D, TG>::kThreads, sm, st>>>(x, f, W, bias, tau, lse, part, s.N, s.H, s.G, P, status);
-    return cudaGetLastError();
+    return launch(k, slot_grid<TG>(s, P), dim3(Tile<D, TG>::kThreads), sm, st, x, f, W, bias, tau, lse, part, s.N, s.H,
+                  s.G, P, reset, status);
   });
 }
 
 template <typename T>
 cudaError_t SimtTiles<T>::deslice(const Shape& s, const T* x, const float* W, const float* bias, const float* tau,
-                                  const float* zp, const float* lse, T* out, uint32_t* status, cudaStream_t st) {
+                                  const float* zp, const float* lse, T* out, bool reset, uint32_t* status,
+                                  cudaStream_t st) {
   return with_tile(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value;
     constexpr size_t sm = tile_bytes<D, TG>(1, 2, 1);
     const auto k = k_tile_deslice<D, TG, T>;
     if (cudaError_t e = allow_smem(k, sm)) return e;
-    k<<<point_grid(s), Tile<D, TG>::kThreads, sm, st>>>(x, W, bias, tau, zp, lse, out, s.N, s.H, s.G, status);
-    return cudaGetLastError();
+    return launch(k, point_grid(s), dim3(Tile<D, TG>::kThreads), sm, st, x, W, bias, tau, zp, lse, out, s.N, s.H, s.G,
+                  reset, status);
   });
 }
 
@@ -878,7 +894,7 @@ template <typename T>
 cudaError_t SimtTiles<T>::backward(const Shape& s, int mode, int P, const T* x, const T* dO, const T* fx,
                                    const float* W, const float* bias, const float* tau, const float* zp,
                                    const float* dUS, const float* lse, T* dx, T* dfx, float* delta, float* dt_part,
-                                   float* part, int accumulate, uint32_t* status, cudaStream_t st) {
+                                   float* part, int accumulate, bool reset, uint32_t* status, cudaStream_t st) {
   return with_tile(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value, NT = Tile<D, TG>::kThreads;
     auto run = [&](auto m) -> cudaError_t {
@@ -886,14 +902,13 @@ cudaError_t SimtTiles<T>::backward(const Shape& s, int mode, int P, const T* x, 
       constexpr size_t sm = tile_bytes<D, TG>(V, V, 1);
       const auto kp = k_tile_bwd_point<D, TG, T, MODE>;
       if (cudaError_t e = allow_smem(kp, sm)) return e;
-      kp<<<point_grid(s), NT, sm, st>>>(x, dO, fx, W, bias, tau, zp, dUS, lse, dx, dfx, delta, dt_part, accumulate,
-                                        s.N, s.H, s.G, status);
-      if (cudaError_t e = cudaGetLastError()) return e;
+      if (cudaError_t e = launch(kp, point_grid(s), dim3(NT), sm, st, x, dO, fx, W, bias, tau, zp, dUS, lse, dx, dfx,
+                                 delta, dt_part, accumulate, s.N, s.H, s.G, reset, status))
+        return e;
       const auto ks = k_tile_bwd_slot<D, TG, T, MODE>;
       if (cudaError_t e = allow_smem(ks, sm)) return e;
-      ks<<<slot_grid<TG>(s, P), NT, sm, st>>>(x, dO, fx, W, bias, tau, zp, dUS, lse, delta, part, s.N, s.H, s.G, P,
-                                              status);
-      return cudaGetLastError();
+      return launch(ks, slot_grid<TG>(s, P), dim3(NT), sm, st, x, dO, fx, W, bias, tau, zp, dUS, lse, delta, part, s.N,
+                    s.H, s.G, P);
     };
     if (mode == 0) return run(std::integral_constant<int, 0>{});
     if (mode == 1) return run(std::integral_constant<int, 1>{});

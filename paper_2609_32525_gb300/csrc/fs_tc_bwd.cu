@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(256) k_prep_us(const float* __restrict__ z, co
                                                  const float* __restrict__ dz, uint8_t* __restrict__ timg,
                                                  uint8_t* __restrict__ zimg, float* __restrict__ c_out, int G, int Gp,
                                                  float eps) {
+  grid_begin(z, wsum, dz);
   __shared__ float su[64][kD + 1];
   const int64_t bh = blockIdx.y;
   const int g0 = blockIdx.x * 64, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(256) k_prep_us(const float* __restrict__ z, co
 // when wds is given).
 __global__ void k_prep_dpx(const float* __restrict__ delta, const float* __restrict__ delta2,
                            const float* __restrict__ wds, uint4* __restrict__ dpx, int64_t BH, int64_t N, int64_t Np) {
+  grid_begin(delta, delta2, wds);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= BH * Np) return;
   const int64_t bh = i / Np, n = i % Np;
@@ -329,6 +331,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_trigger();
+  grid_wait(wimg, timg, timg2);
 
   if (warp == 0) {
     // ------------------------------ producer ------------------------------
@@ -706,6 +710,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_trigger();
+  grid_wait(wimg, timg, timg2, wtimg, dx);
 
   if (warp == 0) {
     if (lane == 0 && wk.ntiles > 0) {
@@ -988,16 +994,14 @@ struct BwdCall {
   }
   // u = dz / (S + eps) and c as images (T at `timg`, zimg) and ds.
   cudaError_t images_us(const float* z, const float* wsum, const float* dz, size_t timg) const {
-    k_prep_us<<<dim3((unsigned)(s.G / 64), (unsigned)s.BH()), 256, 0, st>>>(z, wsum, dz, ws + timg, ws + L.zimg,
-                                                                              f(L.ds), s0.G, s.G, s.eps);
-    return cudaGetLastError();
+    return launch(k_prep_us, dim3((unsigned)(s.G / 64), (unsigned)s.BH()), dim3(256), 0, st, z, wsum, dz, ws + timg,
+                  ws + L.zimg, f(L.ds), s0.G, s.G, s.eps);
   }
   // delta's point rows from delta (+ delta2) (+ the sums of w dS).
   cudaError_t delta_rows(const float* delta, const float* delta2, const float* wds) const {
     const int64_t n = s.BH() * padded_n(s);
-    k_prep_dpx<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(delta, delta2, wds, reinterpret_cast<uint4*>(ws + L.dpx),
-                                                              s.BH(), s.N, padded_n(s));
-    return cudaGetLastError();
+    return launch(k_prep_dpx, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, delta, delta2, wds,
+                  reinterpret_cast<uint4*>(ws + L.dpx), s.BH(), s.N, padded_n(s));
   }
   // The slot pass over all slots (v, f: the deslice's and the slice's points of MODE 3).
   template <int MODE>
@@ -1008,10 +1012,9 @@ struct BwdCall {
     const auto kernel = k_bwd_slot_tc<MODE, true>;
     if (cudaError_t e = set_smem(kernel, sm)) return e;
     const int P = bwd_slot_splits(s);
-    kernel<<<dim3((unsigned)bwd_slot_blocks(s), (unsigned)P, (unsigned)s.BH()), kThreads, sm, st>>>(
-        xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, f(L.part), f(L.dtp), s.N, padded_n(s),
-        s.H, s.G, P, status);
-    return cudaGetLastError();
+    return launch(kernel, dim3((unsigned)bwd_slot_blocks(s), (unsigned)P, (unsigned)s.BH()), dim3(kThreads), sm, st,
+                  xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, f(L.part), f(L.dtp), s.N,
+                  padded_n(s), s.H, s.G, P, status);
   }
   // dW, dbias, dtau (and d z' into dzp) from the slot pass's partials.
   cudaError_t reduce(const float* tau, float* dzp, float* dW, float* db, float* dtau, int accumulate) const {
@@ -1033,11 +1036,11 @@ struct BwdCall {
     const int P = point_splits(s, (int)s.BH());
     for (int k = 0; k < r.n; k++) {
       const int g0 = k * r.size;
-      kernel<<<dim3((unsigned)P, (unsigned)s.BH()), kThreads, sm, st>>>(
-          xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, ws + L.wtimg,
-          static_cast<__nv_bfloat16*>(dx), s.N, padded_n(s), s.H, s.G, g0, std::min(r.size, s.G - g0), P,
-          hilo ? 1 : 0, (accumulate || k > 0) ? 1 : 0, status);
-      if (cudaError_t e = cudaGetLastError()) return e;
+      if (cudaError_t e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kThreads), sm, st, xmap, vmap, pmap,
+                                 dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, ws + L.wtimg,
+                                 static_cast<__nv_bfloat16*>(dx), s.N, padded_n(s), s.H, s.G, g0,
+                                 std::min(r.size, s.G - g0), P, hilo ? 1 : 0, (accumulate || k > 0) ? 1 : 0,
+                                 status)) return e;
     }
     return cudaSuccess;
   }

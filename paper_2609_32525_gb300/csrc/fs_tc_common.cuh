@@ -5,6 +5,7 @@
 // translation unit that includes it gets its own copy.
 #pragma once
 
+#include "fs_launch.h"
 #include "fs_tc.h"
 #include "fs_tc_ptx.cuh"
 
@@ -62,6 +63,7 @@ __device__ __forceinline__ uint32_t off_z(int c, int g) {
 // Images cover slots [0, Gp), Gp = G rounded up to whole 128-slot blocks.  Padding slots
 // [G, Gp) have W' = 0 and b' = -1e30 (their logits are -1e30 and their weights exactly 0 in
 // every pass) and zero token rows.
+constexpr int kSplitPieces = 4, kRowsPerBlock = 1024;
 struct Prep {
   // blocks of 256 threads up to and including each job
   int64_t e_w, e_wt, e_t, e_z, e_px, e_split0, e_split1, e_zero;
@@ -171,11 +173,12 @@ __device__ __forceinline__ void prep_z_piece(const Prep& a, int64_t i) {
 __device__ __forceinline__ uint4 extra_row3(float nv);  // below
 
 __global__ void __launch_bounds__(256) k_prep(const __grid_constant__ Prep a) {
-  const int64_t blk = blockIdx.x;
+  const int64_t zero = grid_begin();
+  const int64_t blk = blockIdx.x + zero;
   if (blk == 0) {
     // The status word: cleared by the first launch of a call; bad temperatures flagged.
     int bad = 0;
-    for (int h = threadIdx.x; h < a.H; h += 256) bad |= !good_tau(a.tau[h]);
+    for (int h = threadIdx.x + (int)zero; h < a.H; h += 256) bad |= !good_tau(a.tau[h]);
     bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
       if (a.reset)
@@ -191,24 +194,35 @@ __global__ void __launch_bounds__(256) k_prep(const __grid_constant__ Prep a) {
   if (blk < a.e_px) {
     // Point-extra rows [1, 1, -lse2 in three parts, 0, 0, 0]; padded points get -1e30 so that
     // their weights vanish.
-    const int64_t i = (blk - a.e_z) * 256 + threadIdx.x;
-    if (i >= a.BH * a.Np) return;
-    const int64_t bh = i / a.Np, n = i % a.Np;
-    a.px[i] = extra_row3(n < a.N ? -a.lse[bh * a.N + n] * kLog2e : -1e30f);
+    const int64_t per = (a.Np + kRowsPerBlock - 1) / kRowsPerBlock, i = blk - a.e_z, bh = i / per;
+    const int64_t n0 = (i - bh * per) * kRowsPerBlock + threadIdx.x;
+    float v[kRowsPerBlock / 256];
+#pragma unroll
+    for (int e = 0; e < kRowsPerBlock / 256; e++)
+      v[e] = n0 + e * 256 < a.N ? -a.lse[bh * a.N + n0 + e * 256] * kLog2e : -1e30f;
+#pragma unroll
+    for (int e = 0; e < kRowsPerBlock / 256; e++)
+      if (n0 + e * 256 < a.Np) a.px[bh * a.Np + n0 + e * 256] = extra_row3(v[e]);
     return;
   }
   if (blk < a.e_split1) {
     // fp32 points -> bf16 hi and residual tensors of the same layout (v = hi + lo to ~2^-16
-    // relative), 8 values per thread in 16-byte loads and stores.
+    // relative), kSplitPieces pieces of 8 values per thread in 16-byte loads and stores.
     const int k = blk < a.e_split0 ? 0 : 1;
-    const int64_t i = (blk - (k ? a.e_split0 : a.e_px)) * 256 + threadIdx.x;
-    if (i >= a.n_split8) return;
-    float v[8];
-    load8(a.split_src[k] + 8 * i, v);
-    uint4 hi, lo;
-    split8(v, hi, lo);
-    reinterpret_cast<uint4*>(a.split_hi[k])[i] = hi;
-    reinterpret_cast<uint4*>(a.split_lo[k])[i] = lo;
+    const int64_t i0 = (blk - (k ? a.e_split0 : a.e_px)) * (256 * kSplitPieces) + threadIdx.x;
+    float v[kSplitPieces][8];
+#pragma unroll
+    for (int e = 0; e < kSplitPieces; e++)
+      if (i0 + e * 256 < a.n_split8) load8(a.split_src[k] + 8 * (i0 + e * 256), v[e]);
+#pragma unroll
+    for (int e = 0; e < kSplitPieces; e++) {
+      const int64_t i = i0 + e * 256;
+      if (i >= a.n_split8) break;
+      uint4 hi, lo;
+      split8(v[e], hi, lo);
+      reinterpret_cast<uint4*>(a.split_hi[k])[i] = hi;
+      reinterpret_cast<uint4*>(a.split_lo[k])[i] = lo;
+    }
     return;
   }
   const int64_t i = (blk - a.e_split1) * 256 + threadIdx.x;
@@ -561,7 +575,7 @@ struct Prepare {
   }
   void rows(const float* lse, void* dst) {
     a.lse = lse, a.px = static_cast<uint4*>(dst);
-    px = a.BH * a.Np;
+    px = a.BH * ((a.Np + kRowsPerBlock - 1) / kRowsPerBlock) * 256;
   }
   // fp32 points v -> bf16 hi at dst, residuals at dst + half.
   void split(const Shape& s, const void* v, uint8_t* dst, size_t half) {
@@ -569,7 +583,8 @@ struct Prepare {
     a.split_src[k] = static_cast<const float*>(v);
     a.split_hi[k] = reinterpret_cast<__nv_bfloat16*>(dst);
     a.split_lo[k] = reinterpret_cast<__nv_bfloat16*>(dst + half);
-    a.n_split8 = sp[k] = s.B * s.N * s.H * s.d / 8;
+    a.n_split8 = s.B * s.N * s.H * s.d / 8;
+    sp[k] = (a.n_split8 + kSplitPieces - 1) / kSplitPieces;
   }
   void clear(float* p, int64_t n) {  // n rounded up to 4 floats
     a.zero = reinterpret_cast<float4*>(p);
@@ -580,8 +595,7 @@ struct Prepare {
     auto end = [&](int64_t threads) { return e += (threads + 255) / 256; };
     a.e_w = end(w), a.e_wt = end(wt), a.e_t = end(t), a.e_z = end(z), a.e_px = end(px);
     a.e_split0 = end(sp[0]), a.e_split1 = end(sp[1]), a.e_zero = end(zero);
-    k_prep<<<(unsigned)(e > 0 ? e : 1), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch(k_prep, dim3((unsigned)(e > 0 ? e : 1)), dim3(256), 0, st, a);
   }
 };
 

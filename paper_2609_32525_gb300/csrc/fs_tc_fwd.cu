@@ -166,17 +166,23 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
     fence_mbar_init();
   }
   for (int s = 0; s < kStages; s++) zero_smem(s_x + s * kDSt + kXBytes + kPxBytes, kPxBytes);
-  if (MODE == 2)
-    for (int g = threadIdx.x; g < G; g += kThreads) s_ds[g] = dS[wk.bh * Gi + g0 + g];
   fence_proxy_async_smem();
   if (warp == 1) tmem_alloc(tmem_slot, 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_trigger();
+  grid_wait(wimg, zimg, out, v, delta, wds, dS);
+  if (MODE == 2) {
+    for (int g = threadIdx.x; g < G; g += kThreads) s_ds[g] = dS[wk.bh * Gi + g0 + g];
+    __syncthreads();
+  }
 
   if (warp == 0) {
     // ------------------------------ producer ------------------------------
+    // (Point rows formed here from lse instead of loaded from px were slower below eight slot
+    // blocks per tile: at G = 256 the call took 465 us against 425, at G = 1024 0.8% less.)
     if (lane == 0 && wk.ntiles > 0) {
       prefetch_tmap(&xmap);
       prefetch_tmap(&pmap);
@@ -186,15 +192,16 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       const uint8_t* zi = zimg + (size_t)wk.bh * zstride + (size_t)g0 * 64;
       load_images(s_z, zi, (uint32_t)G * 64, wz_full);
       if (PS) load_images(s_z + (uint32_t)G * 64, zi + (size_t)Gi * 64, (uint32_t)G * 64, wz_full);
+      Ring<kStages> st;
       int i = 0;
-      for (; i < wk.ntiles; i++) {
-        const int s = i % kStages;
-        if (i >= kStages && !mbar_wait(&x_empty[s], (uint32_t)(((i / kStages) - 1) & 1), ab, status)) break;
+      for (; i < wk.ntiles; i++, st.next()) {
+        if (i >= kStages && !mbar_wait(&x_empty[st.i], st.pass ^ 1u, ab, status)) break;
+        uint8_t* stage = s_x + st.i * kDSt;
         const int n0 = (int)((wk.tile0 + i) * kTile);
-        mbar_expect_tx(&x_full[s], kXBytes + kPxBytes + (X3 ? kXBytes : 0u));
-        tma_load_3d(s_x + s * kDSt, &xmap, h * kD, n0, (int)b, &x_full[s]);
-        tma_load_2d(s_x + s * kDSt + kXBytes, &pmap, 0, (int)(wk.bh * Np + n0), &x_full[s]);
-        if (X3) tma_load_3d(s_x + s * kDSt + kDStage, &xrmap, h * kD, n0, (int)b, &x_full[s]);
+        mbar_expect_tx(&x_full[st.i], kXBytes + kPxBytes + (X3 ? kXBytes : 0u));
+        tma_load_3d(stage, &xmap, h * kD, n0, (int)b, &x_full[st.i]);
+        tma_load_2d(stage + kXBytes, &pmap, 0, (int)(wk.bh * Np + n0), &x_full[st.i]);
+        if (X3) tma_load_3d(stage + kDStage, &xrmap, h * kD, n0, (int)b, &x_full[st.i]);
       }
       // Drain: the newest load of each stage has landed before the CTA exits.
       for (int j = (i > kStages ? i - kStages : 0); j < i; j++)
@@ -474,6 +481,8 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_trigger();
+  grid_wait(wimg);
 
   if (warp == 0) {
     if (lane == 0 && wk.ntiles > 0) {
@@ -760,6 +769,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_trigger();
+  grid_wait(wimg);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1039,9 +1050,8 @@ cudaError_t run_stats(const Shape& s, const void* x, const void* xr, const uint8
   const auto kernel = x3 ? k_stats<true, true> : (split ? k_stats<true, false> : k_stats<false, false>);
   cudaError_t e = set_smem(kernel, sm);
   if (e != cudaSuccess) return e;
-  kernel<<<dim3((unsigned)P, (unsigned)s.BH()), kStatsThreads, sm, st>>>(xmap, xrmap, wimg, lse, static_cast<uint4*>(px),
-                                                                    s.N, padded_n(s), s.H, s.G, P, status);
-  return cudaGetLastError();
+  return launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kStatsThreads), sm, st, xmap, xrmap, wimg, lse,
+                static_cast<uint4*>(px), s.N, padded_n(s), s.H, s.G, P, status);
 }
 
 }  // namespace
@@ -1158,9 +1168,8 @@ cudaError_t run_slice(const Shape& s, int G, const void* x, const void* f, const
   const size_t sm = smem_slice(x3);
   const auto kernel = x3 ? k_slice<true, true> : (s.dot == FS_DOT_BF16X2 ? k_slice<true, false> : k_slice<false, false>);
   if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
-  kernel<<<grid, kThreads, sm, st>>>(xmap, fmap, pmap, xrmap, frmap, wimg, part, s.N, padded_n(s), s.H, s.G, P,
-                                     status);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch(kernel, grid, dim3(kThreads), sm, st, xmap, fmap, pmap, xrmap, frmap, wimg, part, s.N, padded_n(s),
+                  s.H, s.G, P, status)) != cudaSuccess) return e;
   Shape so = s;
   so.G = G;
   return simt_reduce_tokens(so, P, part, s.G, tokens, wsum, finalize, st);
@@ -1199,11 +1208,10 @@ cudaError_t tc_deslice_fwd(const Shape& s0, const void* x, const float* W, const
   if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
   for (int k = 0; k < xr.n; k++) {
     const int g0 = k * xr.size;
-    kernel<<<dim3((unsigned)P, (unsigned)s.BH()), x3 ? kThreads : kDesl3Threads, sm, st>>>(
-        xmap, pmap, xrmap, wimg, zimg, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr, s.N,
-        padded_n(s), s.H, s.G, g0, std::min(xr.size, s.G - g0), P, hilo ? 1 : 0, (uint32_t)s.G * (ps ? 128 : 64),
-        k > 0 ? 1 : 0, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(x3 ? kThreads : kDesl3Threads), sm, st, xmap,
+                    pmap, xrmap, wimg, zimg, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr,
+                    s.N, padded_n(s), s.H, s.G, g0, std::min(xr.size, s.G - g0), P, hilo ? 1 : 0,
+                    (uint32_t)s.G * (ps ? 128 : 64), k > 0 ? 1 : 0, status)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -1228,10 +1236,9 @@ cudaError_t tc_rows_bwd(const Shape& s, int Gi, int g0, int mode, const void* x,
                                 : (ps ? k_deslice<2, true> : k_deslice<2, false>);
   cudaError_t e = set_smem(kernel, sm);
   if (e != cudaSuccess) return e;
-  kernel<<<grid, kThreads, sm, st>>>(xmap, pmap, xmap, wimg, zimg, static_cast<__nv_bfloat16*>(dfx),
-                                     static_cast<const __nv_bfloat16*>(v), delta, wds, dS, s.N, Np, s.H, Gi, g0, s.G,
-                                     P, hilo ? 1 : 0, (uint32_t)Gi * 128, accumulate, status);
-  return cudaGetLastError();
+  return launch(kernel, grid, dim3(kThreads), sm, st, xmap, pmap, xmap, wimg, zimg, static_cast<__nv_bfloat16*>(dfx),
+                static_cast<const __nv_bfloat16*>(v), delta, wds, dS, s.N, Np, s.H, Gi, g0, s.G, P, hilo ? 1 : 0,
+                (uint32_t)Gi * 128, accumulate, status);
 }
 
 }  // namespace fs
