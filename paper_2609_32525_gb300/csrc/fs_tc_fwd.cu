@@ -34,7 +34,7 @@
 //
 // Issue.  Each MMA-issuing role is a whole converged warp in which one elected
 // lane issues (a lone lane in a divergent branch issues several times slower).
-// Warp 1 issues the logits (stats: warps 1 and 2); warps 2 and 3 issue the
+// Warp 1 issues the logits; warps 2 and 3 issue the
 // products into accumulators of their own, which are summed in a fixed order,
 // so the result is deterministic.
 //
@@ -408,28 +408,30 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
 // the point-extra row [1, 1, -lse2 in three bf16 parts, 0 x 3] (lse2 = lse*log2(e)) to
 // px[bh*Np + n] (Np = N rounded up to a whole tile; padded points get -1e30 so
 // that their weights vanish).
-// Two logits issuers and four softmax warpgroups (640 threads): block q (tile
-// q / nb, slot block q % nb) goes through S buffer p = q % 2, issuer 1 + p and
-// warpgroups 2p and 2p + 1, each of which takes one half (64 slots) of every row,
-// so that each SM sub-partition holds four softmax warps whose exponentials and
-// reductions interleave.  Each warpgroup keeps a running (max, sum) over the slots
-// it took and hands it over through shared memory after its last block of the tile.
-// With two or more blocks per tile all four warpgroups take blocks of every tile and
-// warp 3 combines their shares and writes lse and the px rows, so no softmax warp
-// waits for the others.  With one block per tile (G <= 128) the pair that takes it
-// combines in place: half 1 hands its share to half 0, which writes (at two tiles or
-// so per CTA an extra hop to warp 3 would lengthen each CTA's tail).
-// smem: [W img G*96][x stages][constant extra][ml exchange][barriers]
-// TMEM: two S buffers [0, 256).
+// nw softmax warpgroups (kStatsWGs, fewer where shared memory holds fewer x stages) take
+// whole tiles (warpgroup w the tiles i with i % nw == w) and own S buffer w: a thread keeps its point's running (max, sum) over
+// all slot blocks in registers and writes the point's results, so nothing is exchanged
+// between warpgroups.  Warp 1 issues the logits of nw tiles in turn, block by block; an S
+// buffer is rewritten once its second half is in registers, under the exponentials.
+// MUFU and the softmax warps' issue slots bound it (a block's exponentials take 512 clocks
+// and a loop of loads, maxima, exponentials and sums alone 640).  Warpgroups that shared
+// tiles, each one half of every row, had to exchange their (max, sum) and waited on twice as
+// many barriers per row (call at N = 262,144, H = 8: G = 1024 359 us, 256 118, 64 70; three
+// warpgroups on whole tiles 349, 98, 56; four 330, 93, 54; four with a second issuing warp
+// 356, 100, 56).
+// smem: [W img G*96][x stages][constant extra][barriers]
+// TMEM: S buffers [0, 128 kStatsWGs).
 // =========================================================================================
 // X3 (fp32 inputs): x arrives as bf16 hi and residual tiles (xmap, xrmap), one stage
 // holding both, and the logits add x_r W'_hi.
-constexpr int kStatsThreads = 640;
+constexpr int kStatsWGs = 4;
+constexpr int kStatsThreads = 128 + 128 * kStatsWGs;
+constexpr int kStatsMaxStages = 8;
 template <bool split, bool X3>
 __global__ void __launch_bounds__(kStatsThreads, 1)
     k_stats(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap xrmap,
             const uint8_t* __restrict__ wimg, float* __restrict__ lse, uint4* __restrict__ px, int64_t N,
-            int64_t Np, int H, int G, int splits, uint32_t* status) {
+            int64_t Np, int H, int G, int splits, int nst, int nw, uint32_t* status) {
   constexpr uint32_t kXSt = X3 ? 2 * kXBytes : kXBytes;  // x stage
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -437,18 +439,15 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   const uint32_t wbytes = (uint32_t)G * (split ? kWRow : 96);
   uint8_t* s_w = smem;
   uint8_t* s_x = s_w + wbytes;
-  uint8_t* s_ex = s_x + kStages * kXSt;
-  float2* s_ml = reinterpret_cast<float2*>(s_ex + kExBytes);  // [2 tile parities][4 warpgroups][128 rows]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_ml + 8 * kTile);
+  uint8_t* s_ex = s_x + (uint32_t)nst * kXSt;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_ex + kExBytes);
   uint64_t* w_full = bars;
   uint64_t* x_full = bars + 1;
-  uint64_t* x_empty = x_full + kStages;
-  uint64_t* s_full = x_empty + kStages;
-  uint64_t* s_free = s_full + 2;
-  uint64_t* ml_full = s_free + 2;   // the warpgroups' shares of a tile written (per tile parity)
-  uint64_t* ml_empty = ml_full + 2; // warp 3 has read them
-  uint64_t* drain = ml_empty + 2;   // one per issuing warp
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 2);
+  uint64_t* x_empty = x_full + kStatsMaxStages;
+  uint64_t* s_full = x_empty + kStatsMaxStages;
+  uint64_t* s_free = s_full + kStatsWGs;
+  uint64_t* drain = s_free + kStatsWGs;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   Abort* ab = reinterpret_cast<Abort*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -459,24 +458,21 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 
   if (threadIdx.x == 0) {
     mbar_init(w_full, 1);
-    for (int s = 0; s < kStages; s++) {
+    for (int s = 0; s < nst; s++) {
       mbar_init(&x_full[s], 1);
-      mbar_init(&x_empty[s], (uint32_t)(nch < 2 ? nch : 2));
+      mbar_init(&x_empty[s], 1);
     }
-    for (int i = 0; i < 2; i++) {
+    for (int i = 0; i < kStatsWGs; i++) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&s_free[i], 8);
-      mbar_init(&ml_full[i], nch >= 2 ? 16 : 4);
-      mbar_init(&ml_empty[i], nch >= 2 ? 1 : 4);
+      mbar_init(&s_free[i], 4);
     }
-    mbar_init(&drain[0], 1);
-    mbar_init(&drain[1], 1);
+    mbar_init(drain, 1);
     ab->flag = 0;
     fence_mbar_init();
   }
   write_const_extra(s_ex);
   fence_proxy_async_smem();
-  if (warp == 1) tmem_alloc(tmem_slot, 256);
+  if (warp == 1) tmem_alloc(tmem_slot, 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -490,165 +486,121 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       if (X3) prefetch_tmap(&xrmap);
       mbar_expect_tx(w_full, wbytes);
       load_images(s_w, wimg + (size_t)h * G * kWRow, wbytes, w_full);
-      int i = 0;
+      int i = 0, s = 0;
+      uint32_t pass = 0;
       for (; i < wk.ntiles; i++) {
-        const int s = i % kStages;
-        if (i >= kStages && !mbar_wait(&x_empty[s], (uint32_t)(((i / kStages) - 1) & 1), ab, status)) break;
+        if (i >= nst && !mbar_wait(&x_empty[s], pass ^ 1u, ab, status)) break;
+        const int n0 = (int)((wk.tile0 + i) * kTile);
         mbar_expect_tx(&x_full[s], kXSt);
-        tma_load_3d(s_x + s * kXSt, &xmap, h * kD, (int)((wk.tile0 + i) * kTile), (int)b, &x_full[s]);
-        if (X3) tma_load_3d(s_x + s * kXSt + kXBytes, &xrmap, h * kD, (int)((wk.tile0 + i) * kTile), (int)b, &x_full[s]);
+        tma_load_3d(s_x + s * kXSt, &xmap, h * kD, n0, (int)b, &x_full[s]);
+        if (X3) tma_load_3d(s_x + s * kXSt + kXBytes, &xrmap, h * kD, n0, (int)b, &x_full[s]);
+        if (++s == nst) s = 0, pass ^= 1u;
       }
-      for (int j = (i > kStages ? i - kStages : 0); j < i; j++)
-        mbar_wait(&x_full[j % kStages], (uint32_t)((j / kStages) & 1), ab, nullptr, kWaitNs);
+      for (int j = (i > nst ? i - nst : 0); j < i; j++)
+        mbar_wait(&x_full[j % nst], (uint32_t)((j / nst) & 1), ab, nullptr, kWaitNs);
       mbar_wait(w_full, 0, ab, nullptr, kWaitNs);
     }
-  } else if (warp == 1 || warp == 2) {
-    // With two or more blocks per tile, issuer j takes the blocks q with q % 2 == j
-    // (always S buffer j, so each buffer has one producer and one consumer and
-    // both issuers touch every tile); with one block per tile issuer 0 takes all.
-    const int j = warp - 1;
-    const int nis = nch >= 2 ? 2 : 1;
-    if (wk.ntiles > 0 && j < nis) {
+  } else if (warp == 1) {
+    if (wk.ntiles > 0) {
       const uint32_t w0 = sdesc_lo(smem_u32(s_w), 16), we0 = w0 + (uint32_t)G * 4;
       const uint32_t wl0 = split ? w0 + (uint32_t)G * 6 : 0u, xe = const_extra_lo(smem_u32(s_ex));
       bool ok = mbar_wait_w(w_full, 0, ab, status);
-      const int total = wk.ntiles * nch;
-      BlockPos pos(j, nch);
-      for (int q = j; ok && q < total; q += nis, pos.step(nis, nch)) {
-        const int i = pos.i, c = pos.c;
-        const int s = i % kStages;
-        const int bb = q & 1;
-        if (c < nis && !(ok = mbar_wait_w(&x_full[s], (uint32_t)((i / kStages) & 1), ab, status))) break;
-        if (q >= 2 && !(ok = mbar_wait_w(&s_free[bb], (uint32_t)(((q >> 1) - 1) & 1), ab, status))) break;
-        tc_fence_after();
-        const uint32_t xs = smem_u32(s_x + s * kXSt);
-        issue_logits<true, kHi32>(tmem + (uint32_t)bb * kGC, sdesc_lo(xs, 16), xe, w0 + (uint32_t)c * (kGC * 4),
-                                  we0 + (uint32_t)c * (kGC * 2), split ? wl0 + (uint32_t)c * (kGC * 4) : 0u,
-                                  X3 ? sdesc_lo(xs + kXBytes, 16) : 0u);
-        mma_commit_w(&s_full[bb]);
-        if (c >= nch - nis) mma_commit_w(&x_empty[s]);
-      }
-      mma_commit_w(&drain[j]);
-      mbar_wait_w(&drain[j], 0, ab, nullptr, kWaitNs);
-    }
-  } else if (warp == 3) {
-    // ------------------------------ combiner ------------------------------
-    // Tile i: the four warpgroups' shares -> lse and px rows (two or more blocks per
-    // tile).  Lane l takes the points l, l + 32, l + 64, l + 96 of the tile.
-    bool ok = nch >= 2;
-    for (int i = 0; ok && i < wk.ntiles; i++) {
-      const int pb = i & 1;
-      if (!(ok = mbar_wait(&ml_full[pb], (uint32_t)((i >> 1) & 1), ab, status))) break;
-      float2 sh[4][4];
-#pragma unroll
-      for (int k = 0; k < 4; k++)
-#pragma unroll
-        for (int w = 0; w < 4; w++) sh[k][w] = s_ml[(pb * 4 + w) * kTile + lane + 32 * k];
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&ml_empty[pb]);
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const float M = fmaxf(fmaxf(sh[k][0].x, sh[k][1].x), fmaxf(sh[k][2].x, sh[k][3].x));
-        float L = 0.f;
-#pragma unroll
-        for (int w = 0; w < 4; w++) L += sh[k][w].y * ex2(sh[k][w].x - M);
-        const int64_t n = (wk.tile0 + i) * kTile + lane + 32 * k;
-        const float lse2 = M + log2f(L);
-        if (n < Np) {
-          px[wk.bh * Np + n] = extra_row3(n < N ? -lse2 : -1e30f);
-          if (n < N) lse[wk.bh * N + n] = lse2 * kLn2;
+      uint32_t par = 1;  // parity of the S buffers' previous release
+      int s0 = 0;        // stage of the first of the tiles taken together
+      uint32_t pass0 = 0;
+      for (int i0 = 0; ok && i0 < wk.ntiles; i0 += nw) {
+        const int nt = min(nw, wk.ntiles - i0);
+        for (int c = 0; ok && c < nch; c++, par ^= 1u) {
+          const uint32_t w = w0 + (uint32_t)c * (kGC * 4), we = we0 + (uint32_t)c * (kGC * 2);
+          const uint32_t wl = split ? wl0 + (uint32_t)c * (kGC * 4) : 0u;
+          int s = s0;
+          uint32_t pass = pass0;
+          for (int k = 0; k < nt; k++) {
+            if (c == 0 && !(ok = mbar_wait_w(&x_full[s], pass, ab, status))) break;
+            if (i0 + c > 0 && !(ok = mbar_wait_w(&s_free[k], par, ab, status))) break;
+            tc_fence_after();
+            const uint32_t xs = smem_u32(s_x + s * kXSt);
+            issue_logits<true, kHi32>(tmem + (uint32_t)k * kGC, sdesc_lo(xs, 16), xe, w, we, wl,
+                                      X3 ? sdesc_lo(xs + kXBytes, 16) : 0u);
+            mma_commit_w(&s_full[k]);
+            if (c == nch - 1) mma_commit_w(&x_empty[s]);
+            if (++s == nst) s = 0, pass ^= 1u;
+          }
         }
+        s0 += nt;
+        if (s0 >= nst) s0 -= nst, pass0 ^= 1u;
       }
+      mma_commit_w(drain);
+      mbar_wait_w(drain, 0, ab, nullptr, kWaitNs);
     }
   } else if (warp >= kSoftmaxWarp0) {
     const int wg = (warp - kSoftmaxWarp0) >> 2;
-    const int pr = wg >> 1, hf = wg & 1;  // S buffer (block parity) and the half of each row
     const int wq = warp & 3;
     const int r = wq * 32 + lane;
-    const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
-    const int total = wk.ntiles * nch;
+    const uint32_t tS = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)wg * kGC;
     bool ok = true;
-    float m = -INFINITY, l = 0.f;
-    // The pair of warpgroups of S buffer pr takes the whole blocks q with q % 2 == pr,
-    // warpgroup hf the slots [64 hf, 64 hf + 64) of each.  A pair's last block of a
-    // tile is one of its last two (c >= nch - 2); after it the warpgroup hands its
-    // (max, sum) over the slots it took to warp 3.
-    BlockPos pos(pr, nch);
-    for (int q = pr; ok && q < total; q += 2, pos.step(2, nch)) {
-      const int i = pos.i, c = pos.c;
-      if (!(ok = mbar_wait(&s_full[pr], (uint32_t)((q >> 1) & 1), ab, status))) break;
-      tc_fence_after();
-      const uint32_t tS = tmem + lane_addr + (uint32_t)pr * kGC + (uint32_t)hf * 64;
-      uint32_t v[2][32];
-      tmem_ld32(tS, v[0]);
-      tmem_ld32(tS + 32, v[1]);
-      tmem_wait_ld2(v[0], v[1]);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&s_free[pr]);
-      float t[22];
+    uint32_t par = 0;
+    for (int i = wg; ok && wg < nw && i < wk.ntiles; i += nw) {
+      float m = -INFINITY, l = 0.f;
+      for (int c = 0; c < nch; c++, par ^= 1u) {
+        if (!(ok = mbar_wait(&s_full[wg], par, ab, status))) break;
+        tc_fence_after();
+#pragma unroll 1
+        for (int hf = 0; hf < 2; hf++) {
+          uint32_t v[2][32];
+          tmem_ld32(tS + 64 * hf, v[0]);
+          tmem_ld32(tS + 64 * hf + 32, v[1]);
+          tmem_wait_ld2(v[0], v[1]);
+          if (hf == 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_free[wg]);
+          }
+          float t[22];
 #pragma unroll
-      for (int k = 0; k < 21; k++)
-        t[k] = max3(__uint_as_float(v[(3 * k) >> 5][(3 * k) & 31]), __uint_as_float(v[(3 * k + 1) >> 5][(3 * k + 1) & 31]),
-                    __uint_as_float(v[(3 * k + 2) >> 5][(3 * k + 2) & 31]));
-      t[21] = fmaxf(__uint_as_float(v[1][31]), m);
+          for (int k = 0; k < 21; k++)
+            t[k] = max3(__uint_as_float(v[(3 * k) >> 5][(3 * k) & 31]),
+                        __uint_as_float(v[(3 * k + 1) >> 5][(3 * k + 1) & 31]),
+                        __uint_as_float(v[(3 * k + 2) >> 5][(3 * k + 2) & 31]));
+          t[21] = fmaxf(__uint_as_float(v[1][31]), m);
 #pragma unroll
-      for (int k = 0; k < 7; k++) t[k] = max3(t[3 * k], t[3 * k + 1], t[3 * k + 2]);
-      const float mn = max3(max3(t[0], t[1], t[2]), max3(t[3], t[4], t[5]), fmaxf(t[6], t[21]));
-      const uint32_t nmb = __float_as_uint(-mn);
-      const uint64_t nm2 = pack2(nmb, nmb);
+          for (int k = 0; k < 7; k++) t[k] = max3(t[3 * k], t[3 * k + 1], t[3 * k + 2]);
+          const float mn = max3(max3(t[0], t[1], t[2]), max3(t[3], t[4], t[5]), fmaxf(t[6], t[21]));
+          const uint32_t nmb = __float_as_uint(-mn);
+          const uint64_t nm2 = pack2(nmb, nmb);
 #pragma unroll
-      for (int j = 0; j < 2; j++)
+          for (int j = 0; j < 2; j++)
 #pragma unroll
-        for (int k = 0; k < 16; k++) {
-          const uint64_t a = add2(pack2(v[j][2 * k], v[j][2 * k + 1]), nm2);
-          v[j][2 * k] = __float_as_uint(ex2(lo_f(a)));
-          v[j][2 * k + 1] = __float_as_uint(ex2(hi_f(a)));
+            for (int k = 0; k < 16; k++) {
+              const uint64_t a = add2(pack2(v[j][2 * k], v[j][2 * k + 1]), nm2);
+              v[j][2 * k] = __float_as_uint(ex2(lo_f(a)));
+              v[j][2 * k + 1] = __float_as_uint(ex2(hi_f(a)));
+            }
+          uint64_t acc[16];
+#pragma unroll
+          for (int k = 0; k < 16; k++)
+            acc[k] = add2(pack2(v[0][2 * k], v[0][2 * k + 1]), pack2(v[1][2 * k], v[1][2 * k + 1]));
+#pragma unroll
+          for (int w = 8; w >= 1; w >>= 1)
+#pragma unroll
+            for (int k = 0; k < w; k++) acc[k] = add2(acc[k], acc[k + w]);
+          l = l * ex2(m - mn) + (lo_f(acc[0]) + hi_f(acc[0]));
+          m = mn;
         }
-      uint64_t acc[16];
-#pragma unroll
-      for (int k = 0; k < 16; k++)
-        acc[k] = add2(pack2(v[0][2 * k], v[0][2 * k + 1]), pack2(v[1][2 * k], v[1][2 * k + 1]));
-#pragma unroll
-      for (int w = 8; w >= 1; w >>= 1)
-#pragma unroll
-        for (int k = 0; k < w; k++) acc[k] = add2(acc[k], acc[k + w]);
-      const float sum = lo_f(acc[0]) + hi_f(acc[0]);
-      l = l * ex2(m - mn) + sum;
-      m = mn;
-      const int pb = i & 1;
-      if (nch == 1 && hf == 0) {
-        // One block per tile: combine with half 1's share and write.
-        if (!(ok = mbar_wait(&ml_full[pb], (uint32_t)((i >> 1) & 1), ab, status))) break;
-        const float2 o = s_ml[(pb * 4 + wg + 1) * kTile + r];
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ml_empty[pb]);
-        const float M = fmaxf(m, o.x);
-        const float L = l * ex2(m - M) + o.y * ex2(o.x - M);
-        const int64_t n = (wk.tile0 + i) * kTile + r;
-        const float lse2 = M + log2f(L);
-        if (n < Np) {
-          px[wk.bh * Np + n] = extra_row3(n < N ? -lse2 : -1e30f);
-          if (n < N) lse[wk.bh * N + n] = lse2 * kLn2;
-        }
-        m = -INFINITY;
-        l = 0.f;
-      } else if (c >= nch - 2) {
-        // This warpgroup's last block of the tile: hand the share over (to warp 3, or
-        // with one block per tile to half 0 of the pair).
-        if (i >= 2 && !(ok = mbar_wait(&ml_empty[pb], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
-        s_ml[(pb * 4 + wg) * kTile + r] = make_float2(m, l);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ml_full[pb]);
-        m = -INFINITY;
-        l = 0.f;
+      }
+      if (!ok) break;
+      const int64_t n = (wk.tile0 + i) * kTile + r;
+      const float lse2 = m + log2f(l);
+      if (n < Np) {
+        px[wk.bh * Np + n] = extra_row3(n < N ? -lse2 : -1e30f);
+        if (n < N) lse[wk.bh * N + n] = lse2 * kLn2;
       }
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, 256);
+  if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
 // =========================================================================================
@@ -1027,8 +979,9 @@ size_t smem_deslice(int G, bool hilo, int mode = 0, bool ps = false, bool x3 = f
   return 1024 + (size_t)G * ((hilo ? kWRow : 96) + (ps ? 128 : 64)) + (mode == 2 ? align_up((size_t)G * 4, 1024) : 0) +
          kStages * (kDStage + (x3 ? kXBytes : 0)) + 512;
 }
-size_t smem_stats(int G, bool split, bool x3 = false) {
-  return 1024 + (size_t)G * (split ? kWRow : 96) + kStages * kXBytes * (x3 ? 2 : 1) + kExBytes + 8 * kTile * 8 + 512;
+// Shared memory of the statistics pass and, from what W' leaves, its x stages.
+size_t smem_stats(int G, bool split, bool x3, int nst) {
+  return 1024 + (size_t)G * (split ? kWRow : 96) + (size_t)nst * kXBytes * (x3 ? 2 : 1) + kExBytes + 512;
 }
 size_t smem_slice(bool x3 = false) {
   return 1024 + (size_t)kWBlock +
@@ -1046,12 +999,14 @@ cudaError_t run_stats(const Shape& s, const void* x, const void* xr, const uint8
   const int P = point_splits(s, (int)s.BH());
   const bool x3 = xr != nullptr;
   const bool split = s.dot == FS_DOT_BF16X2 || x3;
-  const size_t sm = smem_stats(s.G, split, x3);
+  int nst = kStatsMaxStages;
+  while (nst > 1 && smem_stats(s.G, split, x3, nst) > kMaxSmem) nst--;
+  const size_t sm = smem_stats(s.G, split, x3, nst);
   const auto kernel = x3 ? k_stats<true, true> : (split ? k_stats<true, false> : k_stats<false, false>);
   cudaError_t e = set_smem(kernel, sm);
   if (e != cudaSuccess) return e;
   return launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kStatsThreads), sm, st, xmap, xrmap, wimg, lse,
-                static_cast<uint4*>(px), s.N, padded_n(s), s.H, s.G, P, status);
+                static_cast<uint4*>(px), s.N, padded_n(s), s.H, s.G, P, nst, std::min(nst, kStatsWGs), status);
 }
 
 }  // namespace
