@@ -140,78 +140,40 @@ __device__ __forceinline__ void issue_dot64_ts(uint32_t d, uint32_t tA, uint32_t
 // the shared zero block; n rows further on both its fields change.
 __device__ __forceinline__ uint32_t px_lo(uint32_t px_s, uint32_t zero_s) { return sdesc_lo(px_s, zero_s - px_s); }
 
-// One 64-column unit of a TMEM lane: L (log2 weights) at tL, dw - delta at tD.
+// One half (32 columns) of a unit of a TMEM lane: L (log2 weights) at tL, dw - delta at tD.
 // da = 2^L (dw - delta) goes back in place into the L columns as bf16 pairs: columns
-// [32 h, 32 h + 16) the hi halves of entries [32 h, 32 h + 32), [32 h + 16, 32 h + 32)
-// their lo halves (kSplit).  kW: the weights too, into the dw columns, same layout.
+// [0, 16) the hi halves of the 32 entries, [16, 32) their lo halves (kSplit).  kW: the
+// weights too, into the dw columns, same layout.
 // kSums: dt += sum da L, db += sum da.
-template <bool kSplit, bool kW, bool kSums>
-__device__ __forceinline__ void da_unit(uint32_t tL, uint32_t tD, float& dt, float& db) {
+// loaded(): called once the half's columns are in registers.
+template <bool kSplit, bool kW, bool kSums, typename F>
+__device__ __forceinline__ void da_half(uint32_t tL, uint32_t tD, float& dt, float& db, F loaded) {
   // Pairs of entries go through the packed f32x2 forms (one instruction for both).
   const uint64_t neg1 = pack2(__float_as_uint(-1.f), __float_as_uint(-1.f));
-#pragma unroll 1
-  for (int h2 = 0; h2 < 2; h2++) {
-    uint32_t l[32], dw[32];
-    tmem_ld32(tL + 32 * h2, l);
-    tmem_ld32(tD + 32 * h2, dw);
-    tmem_wait_ld2(l, dw);
-    uint32_t dh[16], dl[16], wh[16], wl[16];
-    uint64_t t2 = 0, sb2 = 0;  // (+0, +0)
+  uint32_t l[32], dw[32];
+  tmem_ld32(tL, l);
+  tmem_ld32(tD, dw);
+  tmem_wait_ld2(l, dw);
+  loaded();
+  uint32_t dh[16], dl[16], wh[16], wl[16];
+  uint64_t t2 = 0, sb2 = 0;  // (+0, +0)
 #pragma unroll
-    for (int k = 0; k < 16; k++) {
-      const uint64_t L2 = pack2(l[2 * k], l[2 * k + 1]);
-      const uint64_t w2 = pack2(__float_as_uint(ex2(__uint_as_float(l[2 * k]))),
-                                __float_as_uint(ex2(__uint_as_float(l[2 * k + 1]))));
-      const uint64_t a2 = mul2(w2, pack2(dw[2 * k], dw[2 * k + 1]));
-      if (kSums) {
-        t2 = fma2(a2, L2, t2);
-        sb2 = add2(sb2, a2);
-      }
-      const uint32_t p = pack_bf16(lo_f(a2), hi_f(a2));
-      dh[k] = p;
-      if (kSplit) {
-        const uint64_t r2 = fma2(pack2(p << 16, p & 0xFFFF0000u), neg1, a2);  // a - bf16(a)
-        dl[k] = pack_bf16(lo_f(r2), hi_f(r2));
-      }
-      if (kW) {
-        const uint32_t q = pack_bf16(lo_f(w2), hi_f(w2));
-        wh[k] = q;
-        if (kSplit) {
-          const uint64_t r2 = fma2(pack2(q << 16, q & 0xFFFF0000u), neg1, w2);
-          wl[k] = pack_bf16(lo_f(r2), hi_f(r2));
-        }
-      }
-    }
-    tmem_st16(tL + 32 * h2, dh);
-    if (kSplit) tmem_st16(tL + 32 * h2 + 16, dl);
-    if (kW) {
-      tmem_st16(tD + 32 * h2, wh);
-      if (kSplit) tmem_st16(tD + 32 * h2 + 16, wl);
-    }
+  for (int k = 0; k < 16; k++) {
+    const uint64_t L2 = pack2(l[2 * k], l[2 * k + 1]);
+    const uint64_t w2 = pack2(__float_as_uint(ex2(__uint_as_float(l[2 * k]))),
+                              __float_as_uint(ex2(__uint_as_float(l[2 * k + 1]))));
+    const uint64_t a2 = mul2(w2, pack2(dw[2 * k], dw[2 * k + 1]));
     if (kSums) {
-      dt += lo_f(t2) + hi_f(t2);
-      db += lo_f(sb2) + hi_f(sb2);
+      t2 = fma2(a2, L2, t2);
+      sb2 = add2(sb2, a2);
     }
-  }
-}
-// TMEM column (within a unit) of the hi pairs of K-step kk (16 entries).
-__device__ __forceinline__ uint32_t da_col(int kk) { return (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)); }
-
-// One 64-column unit of a TMEM lane: L (log2 weights) -> w = 2^L in place, as bf16
-// pairs in da_unit's layout (hi pairs, then their residuals with kSplit).
-template <bool kSplit>
-__device__ __forceinline__ void w_unit(uint32_t tL) {
-  const uint64_t neg1 = pack2(__float_as_uint(-1.f), __float_as_uint(-1.f));
-#pragma unroll 1
-  for (int h2 = 0; h2 < 2; h2++) {
-    uint32_t l[32];
-    tmem_ld32(tL + 32 * h2, l);
-    tmem_wait_ld(l);
-    uint32_t wh[16], wl[16];
-#pragma unroll
-    for (int k = 0; k < 16; k++) {
-      const uint64_t w2 = pack2(__float_as_uint(ex2(__uint_as_float(l[2 * k]))),
-                                __float_as_uint(ex2(__uint_as_float(l[2 * k + 1]))));
+    const uint32_t p = pack_bf16(lo_f(a2), hi_f(a2));
+    dh[k] = p;
+    if (kSplit) {
+      const uint64_t r2 = fma2(pack2(p << 16, p & 0xFFFF0000u), neg1, a2);  // a - bf16(a)
+      dl[k] = pack_bf16(lo_f(r2), hi_f(r2));
+    }
+    if (kW) {
       const uint32_t q = pack_bf16(lo_f(w2), hi_f(w2));
       wh[k] = q;
       if (kSplit) {
@@ -219,10 +181,54 @@ __device__ __forceinline__ void w_unit(uint32_t tL) {
         wl[k] = pack_bf16(lo_f(r2), hi_f(r2));
       }
     }
-    tmem_st16(tL + 32 * h2, wh);
-    if (kSplit) tmem_st16(tL + 32 * h2 + 16, wl);
+  }
+  tmem_st16(tL, dh);
+  if (kSplit) tmem_st16(tL + 16, dl);
+  if (kW) {
+    tmem_st16(tD, wh);
+    if (kSplit) tmem_st16(tD + 16, wl);
+  }
+  if (kSums) {
+    dt += lo_f(t2) + hi_f(t2);
+    db += lo_f(sb2) + hi_f(sb2);
   }
 }
+// TMEM column (within a unit) of the hi pairs of K-step kk (16 entries).
+__device__ __forceinline__ uint32_t da_col(int kk) { return (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)); }
+
+// One half of a unit: L (log2 weights) -> w = 2^L in place, as bf16 pairs in da_half's
+// layout (hi pairs, then their residuals with kSplit).
+template <bool kSplit>
+__device__ __forceinline__ void w_half(uint32_t tL) {
+  const uint64_t neg1 = pack2(__float_as_uint(-1.f), __float_as_uint(-1.f));
+  uint32_t l[32];
+  tmem_ld32(tL, l);
+  tmem_wait_ld(l);
+  uint32_t wh[16], wl[16];
+#pragma unroll
+  for (int k = 0; k < 16; k++) {
+    const uint64_t w2 = pack2(__float_as_uint(ex2(__uint_as_float(l[2 * k]))),
+                              __float_as_uint(ex2(__uint_as_float(l[2 * k + 1]))));
+    const uint32_t q = pack_bf16(lo_f(w2), hi_f(w2));
+    wh[k] = q;
+    if (kSplit) {
+      const uint64_t r2 = fma2(pack2(q << 16, q & 0xFFFF0000u), neg1, w2);
+      wl[k] = pack_bf16(lo_f(r2), hi_f(r2));
+    }
+  }
+  tmem_st16(tL, wh);
+  if (kSplit) tmem_st16(tL + 16, wl);
+}
+
+// TMEM buffers of a unit's logits L (which become da) and of its dw - delta.  da stays until
+// its products have read it; dw - delta is dead once a softmax warp has loaded it, so two
+// buffers of it feed four of L and four units are under way instead of three.  (The slot
+// pass's MODE 1 writes the weights over dw, for its second product: three of each.)
+template <bool kKeepDw>
+struct UnitBufs {
+  static constexpr int kL = kKeepDw ? 3 : 4, kD = kKeepDw ? 3 : 2;
+  static constexpr uint32_t kDCol = kL * 64;  // column of the first dw buffer
+};
 
 // The slot pass's accumulators are flushed into registers every kSlotFlush of an
 // issuer's units (64 points each), for the reason the slice's are: the tensor cores'
@@ -235,8 +241,8 @@ __device__ __forceinline__ bool slot_flush_at(int u) { return ((u >> 1) % kSlotF
 // u & 1 (64 points) of point tile u >> 1.  Per unit, warp 1 forms, transposed
 // (M = 128 slots, N = 64 points, TMEM lane = slot),
 //   L = a2 - lse2 (W block vs [x | 1, 1, -lse2]) and dw - delta (T block vs [v | 1, 1, -delta]);
-// softmax warpgroup u % 2 turns them into da (and, MODE 1, w) in place and sums
-// da (a2 - lse2) and da per slot in registers; warp 2 + u % 2 issues
+// (warp 2 the latter); softmax warpgroup u % 2 turns them into da (and, MODE 1, w) in place,
+// a half at a time, and sums da (a2 - lse2) and da per slot in registers; warp 3 issues, per half,
 //   dWx += da^T x   (K = points; x's 64B-swizzled tile read as an MN-major B operand)
 //   MODE 1: dZ += w^T dO (the token gradient), from dO's tile the same way.
 // Writes part[p][bh][g] = MODE 1: (dZ(32), dWx(32), sum da, 0); MODE 2: (dWx, sum da, 0)
@@ -248,8 +254,16 @@ __device__ __forceinline__ bool slot_flush_at(int u) { return ((u >> 1) % kSlotF
 //     (its extra block [dS_hi, dS_lo, 1, 1, 1] meets delta's rows), delta = delta_D +
 //     delta_S), written like MODE 2.
 // smem: [W block: hi 8K | extra 4K | lo 8K][T block: same][stages][zero 2K][red 1.5K][bars]
-// TMEM: unit u uses set u % 3: L [128 s, +64), dw [128 s + 64, +64); accumulators
-// dWx_j [384 + 32 j), dZ_j [448 + 32 j).
+// TMEM: [0, 384) the units' L and dw buffers (UnitBufs); accumulators dWx_j [384 + 32 j),
+// dZ_j [448 + 32 j).
+//
+// What bounds it is the cycle of a unit's buffers (logits -> da -> products -> logits): ~1100
+// clocks a unit where the MMAs alone need ~750 and the exponentials 256; the softmax warps wait
+// half of their time.  So the halves of a unit are handed over as they are written, and four
+// units are under way.  Whole backward at B = 2, N = 131,072, H = 8, G = 512, this pass and the
+// point pass changed together: 2261 us with whole units, two warps issuing the products and
+// three units under way; 2198 with halves (and the point pass's third warpgroup), 2184 with one
+// warp per chain, 2165 with four units.
 // =========================================================================================
 template <int MODE, bool split>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -275,9 +289,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* x_full = bars + 1;
   uint64_t* st_empty = x_full + kNSt;
   uint64_t* s_full = st_empty + kNSt;
-  uint64_t* p_ready = s_full + kSBuf;  // [issuer][set]
-  uint64_t* pv_done = p_ready + 2 * kSBuf;
-  uint64_t* acc_full = pv_done + kSBuf;
+  using Bufs = UnitBufs<MODE == 1>;
+  uint64_t* p_ready = s_full + Bufs::kL;  // [L buffer][half of the unit]
+  uint64_t* pv_done = p_ready + 2 * Bufs::kL;
+  uint64_t* dw_free = pv_done + Bufs::kL;
+  uint64_t* acc_full = dw_free + Bufs::kD;
   uint64_t* acc_done = acc_full + 1;  // [issuer]: products of each of its units complete
   uint64_t* wt_ready = acc_done + 2;  // MODES 2, 3: the W' image is in TMEM
   uint64_t* drain = wt_ready + 1;
@@ -300,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // shared memory.
   constexpr bool kWT = MODE == 2 || MODE == 3;
   constexpr bool kTT = MODE == 3;
-  constexpr uint32_t kAccW = kSBuf * kGC, kAccZ = kAccW + 64;
+  constexpr uint32_t kAccW = 384u, kAccZ = kAccW + 64;
   constexpr uint32_t kAccF = MODE == 0 ? kAccZ : kAccW;  // the flushed accumulator
   constexpr uint32_t kVOff = kXBytes, kPOff = 2 * kXBytes, kDOff = 2 * kXBytes + kPxBytes;
 
@@ -308,15 +324,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(w_full, 1);
     for (int s = 0; s < kNSt; s++) {
       mbar_init(&x_full[s], 1);
-      mbar_init(&st_empty[s], 3);  // the logits issuer and both product issuers
+      mbar_init(&st_empty[s], MODE == 0 ? 2 : 3);  // the issuers
     }
-    for (int i = 0; i < kSBuf; i++) {
-      mbar_init(&s_full[i], 1);
-      mbar_init(&p_ready[i], 4);
-      mbar_init(&p_ready[kSBuf + i], 4);
+    for (int i = 0; i < Bufs::kL; i++) {
+      mbar_init(&s_full[i], MODE == 0 ? 1 : 2);  // logits and dw
+      mbar_init(&p_ready[2 * i], 4);
+      mbar_init(&p_ready[2 * i + 1], 4);
       mbar_init(&pv_done[i], 1);
     }
-    mbar_init(acc_full, 2);
+    for (int i = 0; i < Bufs::kD; i++) mbar_init(&dw_free[i], 4);
+    mbar_init(acc_full, 1);
     mbar_init(&acc_done[0], 1);
     mbar_init(&acc_done[1], 1);
     mbar_init(wt_ready, 4);
@@ -371,76 +388,82 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_wait(&x_full[j % kNSt], (uint32_t)((j / kNSt) & 1), ab, nullptr, kWaitNs);
       mbar_wait(w_full, 0, ab, nullptr, kWaitNs);
     }
-  } else if (warp == 1) {
-    // ------------------------------ logits and dw issuer ------------------------------
+  } else if (warp == 1 || (warp == 2 && MODE != 0)) {
+    // ------------------------------ logits (warp 1) and dw (warp 2) issuers ------------------------------
     const uint32_t w = sdesc_lo(smem_u32(s_w), 16), t = sdesc_lo(smem_u32(s_t), 16), t2 = sdesc_lo(smem_u32(s_t2), 16);
     const uint32_t sz = smem_u32(s_zero);
     constexpr uint32_t kExt = kGC * 4, kLo = kGC * 6;  // the extra and residual rows of a slot block, in 16 bytes
-    constexpr uint32_t idesc = idesc_bf16(128, 64, false, false);
     bool ok = mbar_wait_w(w_full, 0, ab, status);
     if (kWT && ok) {
       ok = mbar_wait_w(wt_ready, 0, ab, status);
       tc_fence_after();
     }
     Ring<kNSt> stg;
-    Ring<kSBuf> sb;
+    Ring<Bufs::kL> sb;
+    Ring<Bufs::kD> db;
     for (int i = 0, u = 0; ok && i < wk.ntiles; i++, stg.next()) {
       if (!(ok = mbar_wait_w(&x_full[stg.i], stg.pass, ab, status))) break;
       const uint32_t st = smem_u32(s_st + stg.i * kStgS);
       uint32_t x = sdesc_lo(st, 16);
-      uint32_t px = px_lo(st + kPOff, sz), dpx = px_lo(st + kDOff, sz);
+      uint32_t px = px_lo(st + (warp == 1 ? kPOff : kDOff), sz);  // lse's rows, delta's rows
       // the second half's 64 points: 64-byte-row tiles, then 16-byte extra rows (whose
       // leading offset to the zero block shrinks as the address grows)
       constexpr uint32_t kHalf = 64 * 64 / 16, kHalfP = 64 * 16 / 16 - ((64u * 16 / 16) << 16);
 #pragma unroll 1
-      for (int half = 0; half < 2; half++, u++, sb.next(), x += kHalf, px += kHalfP, dpx += kHalfP) {
-        if (u >= kSBuf && !(ok = mbar_wait_w(&pv_done[sb.i], sb.pass ^ 1u, ab, status))) break;
+      for (int half = 0; half < 2; half++, u++, sb.next(), db.next(), x += kHalf, px += kHalfP) {
+        // L: the products of the unit kL back; dw: loaded by the unit kD back
+        const bool is_l = warp == 1 || MODE == 1;
+        if (u >= (is_l ? Bufs::kL : Bufs::kD) &&
+            !(ok = mbar_wait_w(is_l ? &pv_done[sb.i] : &dw_free[db.i], (is_l ? sb.pass : db.pass) ^ 1u, ab, status)))
+          break;
         tc_fence_after();
-        const uint32_t tL = tmem + (uint32_t)sb.i * kGC;
-        const uint32_t v = x + kVOff / 16, f = x + kBStage / 16;
-        if (kTT) {
-          issue_dot64_ts(tL, tmem + kAccZ, x, split);
-          mma_ss_w<kHi32, kHiPx>(tL, w + kExt, px, idesc, 1u);
-          // the deslice's chain: T (and its residual) from TMEM against dO, no extra block;
-          // the slice's extra block [dS_hi, dS_lo, 1, 1, 1] against delta's rows
-          // [1, 1, -delta parts] adds dS - delta in one K step.
-          issue_dot64_ts(tL + 64, tmem + kAccZ + 32, v, split);
-          issue_dot64<true, kHi32, kHiPx>(tL + 64, t2, f, t2 + kExt, dpx, split ? t2 + kLo : 0u, 1u);
-        } else {
-          if (kWT) {
+        const uint32_t tL = tmem + (uint32_t)sb.i * 64, tD = tmem + Bufs::kDCol + (uint32_t)db.i * 64;
+        if (warp == 1) {
+          if (kTT) {
             issue_dot64_ts(tL, tmem + kAccZ, x, split);
-            mma_ts_w<kHiPx>(tL, tmem + kAccZ + 32, px, idesc, 1u);
+            mma_ss_w<kHi32, kHiPx>(tL, w + kExt, px, idesc_bf16(128, 64, false, false), 1u);
+          } else if (kWT) {
+            issue_dot64_ts(tL, tmem + kAccZ, x, split);
+            mma_ts_w<kHiPx>(tL, tmem + kAccZ + 32, px, idesc_bf16(128, 64, false, false), 1u);
           } else {
             issue_dot64<true, kHi32, kHiPx>(tL, w, x, w + kExt, px, split ? w + kLo : 0u);
           }
-          if (MODE == 1 || MODE == 2)
-            issue_dot64<true, kHi32, kHiPx>(tL + 64, t, v, t + kExt, dpx, split ? t + kLo : 0u);
+        } else if (kTT) {
+          // the deslice's chain: T (and its residual) from TMEM against dO, no extra block;
+          // the slice's extra block [dS_hi, dS_lo, 1, 1, 1] against delta's rows
+          // [1, 1, -delta parts] adds dS - delta in one K step.
+          issue_dot64_ts(tD, tmem + kAccZ + 32, x + kVOff / 16, split);
+          issue_dot64<true, kHi32, kHiPx>(tD, t2, x + kBStage / 16, t2 + kExt, px, split ? t2 + kLo : 0u, 1u);
+        } else {
+          issue_dot64<true, kHi32, kHiPx>(tD, t, x + kVOff / 16, t + kExt, px, split ? t + kLo : 0u);
         }
         mma_commit_w(&s_full[sb.i]);
       }
       mma_commit_w(&st_empty[stg.i]);
     }
-    mma_commit_w(&drain[0]);
-    mbar_wait_w(&drain[0], 0, ab, nullptr, kWaitNs);
-  } else if (warp == 2 || warp == 3) {
-    // ------------------------------ product issuers ------------------------------
-    const int j = warp - 2;  // units u with u % 2 == j (half j of every tile)
+    mma_commit_w(&drain[warp - 1]);
+    mbar_wait_w(&drain[warp - 1], 0, ab, nullptr, kWaitNs);
+  } else if (warp == 3) {
+    // ------------------------------ product issuer ------------------------------
+    // Units u (half u & 1 of every tile) into accumulator u & 1.
     constexpr uint32_t idesc = idesc_bf16(128, kD, false, true);
     bool ok = true;
     Ring<kNSt> stg;
-    Ring<kSBuf> sb;
-    uint32_t pass = 0;  // parity of this issuer's uses of a set (its units there are 2 kSBuf apart)
-    if (j == 1) sb.next();
-    for (int u = j; ok && u < units; u += 2, stg.next(), sb.next(), sb.next()) {
-      if (!(ok = mbar_wait_w(&p_ready[j * kSBuf + sb.i], pass, ab, status))) break;
-      tc_fence_after();
+    Ring<Bufs::kL> sb;
+    Ring<Bufs::kD> db;
+    for (int u = 0; ok && u < units; u++, sb.next(), db.next()) {
+      const int j = u & 1;
       // 16 points: two 8-row groups of the 64B-swizzled tile (MN-major: channels contiguous).
       const uint32_t x = sdesc_lo(smem_u32(s_st + stg.i * kStgS) + (uint32_t)j * 64 * 64, 4096), v = x + kVOff / 16;
-      const uint32_t tL = tmem + (uint32_t)sb.i * kGC, tD = tL + 64;
+      const uint32_t tL = tmem + (uint32_t)sb.i * 64, tD = tmem + Bufs::kDCol + (uint32_t)db.i * 64;
       const uint32_t tW = tmem + kAccW + (uint32_t)j * 32, tZ = tmem + kAccZ + (uint32_t)j * 32;
       const bool fresh = u < 2 || (kFl && slot_flush_at(u));
 #pragma unroll
       for (int kk = 0; kk < 4; kk++) {
+        if ((kk & 1) == 0) {  // a half of the unit
+          if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + (kk >> 1)], sb.pass, ab, status))) break;
+          tc_fence_after();
+        }
         const uint32_t acc = (!fresh || kk > 0) ? 1u : 0u;
         if (MODE == 0) {  // the weights are in the L columns: dZ += w^T dO
           mma_ts_w<kHi64>(tZ, tL + da_col(kk), v + kk * 64, idesc, acc);
@@ -455,14 +478,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       mma_commit_w(&pv_done[sb.i]);
-      mma_commit_w(&st_empty[stg.i]);
       if (kFl) mma_commit_w(&acc_done[j]);
-      if ((u >> 1) % kSBuf == kSBuf - 1) pass ^= 1u;
+      if (j == 1) {
+        mma_commit_w(&st_empty[stg.i]);
+        stg.next();
+      }
     }
     if (ok) mma_commit_w(acc_full);
-    mma_commit_w(&drain[1 + j]);
-    mbar_wait_w(&drain[1 + j], 0, ab, nullptr, kWaitNs);
-  } else {
+    mma_commit_w(&drain[2]);
+    mbar_wait_w(&drain[2], 0, ab, nullptr, kWaitNs);
+  } else if (warp >= kSoftmaxWarp0) {
     // ------------------------------ softmax warpgroups ------------------------------
     const int wg = (warp - kSoftmaxWarp0) >> 2;
     const int wq = warp & 3;
@@ -514,28 +539,35 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int k = 0; k < kD; k++) acc[k] += __uint_as_float(a[k]);
     };
     for (int u = wg; ok && u < units; u += 2) {
-      const int bb = u % kSBuf;
-      if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((u / kSBuf) & 1), ab, status))) break;
+      const int bb = u % Bufs::kL, bd = u % Bufs::kD;
+      if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((u / Bufs::kL) & 1), ab, status))) break;
       tc_fence_after();
-      const uint32_t tL = tmem + lane_addr + (uint32_t)bb * kGC;
-      if (MODE == 0) {
-        w_unit<split>(tL);
-      } else {
-        float t = 0.f, sb = 0.f;
-        da_unit<split, MODE == 1, true>(tL, tL + 64, t, sb);
-        dt += t;
-        db += sb;
+      const uint32_t tL = tmem + lane_addr + (uint32_t)bb * 64;
+      const uint32_t tD = tmem + lane_addr + Bufs::kDCol + (uint32_t)bd * 64;
+#pragma unroll
+      for (int hf = 0; hf < 2; hf++) {
+        if constexpr (MODE == 0) {
+          w_half<split>(tL + 32 * hf);
+        } else {
+          da_half<split, MODE == 1, true>(tL + 32 * hf, tD + 32 * hf, dt, db, [&]() {
+            if (MODE != 1 && hf == 1) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&dw_free[bd]);
+            }
+          });
+        }
+        tmem_wait_st();
+        if (hf == 0 && kFl && u >= 2 && slot_flush_at(u)) {
+          // This warpgroup's units up to u - 2 have completed their products.
+          if (!(ok = mbar_wait(&acc_done[wg], (uint32_t)(((u - 2) >> 1) & 1), ab, status))) break;
+          tc_fence_after();
+          add_acc();
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_ready[2 * bb + hf]);
       }
-      tmem_wait_st();
-      if (kFl && u >= 2 && slot_flush_at(u)) {
-        // This warpgroup's units up to u - 2 have completed their products.
-        if (!(ok = mbar_wait(&acc_done[wg], (uint32_t)(((u - 2) >> 1) & 1), ab, status))) break;
-        tc_fence_after();
-        add_acc();
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_ready[wg * kSBuf + bb]);
     }
     // Epilogue.  Warpgroup 1 hands its sums dt, db to warpgroup 0 through shared
     // memory.  Flushed modes: each warpgroup adds what its accumulator holds since
@@ -630,9 +662,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Point pass: dx_n = ln2 * sum_g da_ng W'_g (W' = W log2(e)/tau) over slots [g0, g0 + G) of
 // images of Gi slots; accumulate: added to what dx holds.  CTA (split, bh)
 // walks its point tiles; block q is (tile q / nb, 64-slot chunk q % nb).  Warp 1
-// forms L (x tile vs W rows) and dw - delta (v tile vs T rows), M = 128 points,
-// N = 64 slots, into set q % 3; softmax warpgroup q % 2 writes da in place (hi, lo
-// pairs); warp 2 + j issues K-steps [2 j, 2 j + 2) of the chunk into O_j:
+// forms L (x tile vs W rows) and warp 2 dw - delta (v tile vs T rows), M = 128 points,
+// N = 64 slots; softmax warpgroup q % 3 writes da in place (hi, lo pairs), a half of the
+// chunk at a time; warp 3 issues K-steps [2 j, 2 j + 2) of half j into O_j:
 //   O_j += da W'^T (B: the W'^T image, channel rows, slots along K).
 // kComb (the whole coupling's backward): da is the sum of the deslice's and the
 // slice's, which share the weights, so one pass serves both: dw - delta is two chains
@@ -642,10 +674,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 // also holds the fx tile.
 // smem: [W img G x (96 | 160)][T img G x 96][kComb: T2 img G x 96][W'^T img G x 64]
 //       [stages][zero 2K][bars]
-// TMEM: sets [0, 384) of (L 64 | dw 64); O_(j, tile parity) at [384 + 32 (2 j + parity)).
+// TMEM: [0, 384) the blocks' L and dw buffers (UnitBufs); O_(j, tile parity) at
+// [384 + 32 (2 j + parity)).  o_full: kDxOFull barriers, as in the forward's deslice (the
+// warpgroup that drains tile t has not waited for tile t - 2; it has seen the logits of a block
+// at most three back, so the products four before that: tile t - 7).
 // =========================================================================================
+constexpr int kDxThreads = 512, kDxWGs = 3, kDxOFull = 8;
 template <bool split, bool kComb = false>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kDxThreads, 1)
     k_bwd_dx_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap vmap,
                 const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap dmap,
                 const __grid_constant__ CUtensorMap fmap, const uint8_t* __restrict__ wimg,
@@ -667,10 +703,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* x_full = bars + 1;
   uint64_t* x_empty = x_full + kDxStages;
   uint64_t* s_full = x_empty + kDxStages;
-  uint64_t* p_ready = s_full + kSBuf;
-  uint64_t* pv_done = p_ready + kSBuf;
-  uint64_t* o_full = pv_done + kSBuf;
-  uint64_t* o_free = o_full + 2;
+  using Bufs = UnitBufs<false>;
+  uint64_t* p_ready = s_full + Bufs::kL;  // [L buffer][half of the unit]
+  uint64_t* pv_done = p_ready + 2 * Bufs::kL;
+  uint64_t* dw_free = pv_done + Bufs::kL;
+  uint64_t* o_full = dw_free + Bufs::kD;
+  uint64_t* o_free = o_full + kDxOFull;
   uint64_t* drain = o_free + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 3);
   Abort* ab = reinterpret_cast<Abort*>(tmem_slot + 1);
@@ -681,24 +719,24 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int h = (int)(wk.bh % H);
   const int nch = G / 64;
   const int total = wk.ntiles * nch;
-  constexpr uint32_t kO = kSBuf * kGC;
+  constexpr uint32_t kO = 384u;
   constexpr uint32_t kVOff = kXBytes, kPOff = 2 * kXBytes, kDOff = 2 * kXBytes + kPxBytes;
 
   if (threadIdx.x == 0) {
     mbar_init(wz_full, 1);
     for (int s = 0; s < kDxStages; s++) {
       mbar_init(&x_full[s], 1);
-      mbar_init(&x_empty[s], 1);
+      mbar_init(&x_empty[s], 2);  // logits and dw issuers
     }
-    for (int i = 0; i < kSBuf; i++) {
-      mbar_init(&s_full[i], 1);
-      mbar_init(&p_ready[i], 4);
-      mbar_init(&pv_done[i], 2);
+    for (int i = 0; i < Bufs::kL; i++) {
+      mbar_init(&s_full[i], 2);  // logits and dw
+      mbar_init(&p_ready[2 * i], 4);
+      mbar_init(&p_ready[2 * i + 1], 4);
+      mbar_init(&pv_done[i], 1);
     }
-    for (int i = 0; i < 2; i++) {
-      mbar_init(&o_full[i], 2);
-      mbar_init(&o_free[i], 4);
-    }
+    for (int i = 0; i < Bufs::kD; i++) mbar_init(&dw_free[i], 4);
+    for (int i = 0; i < kDxOFull; i++) mbar_init(&o_full[i], 1);
+    for (int i = 0; i < 2; i++) mbar_init(&o_free[i], 4);
     for (int i = 0; i < 3; i++) mbar_init(&drain[i], 1);
     ab->flag = 0;
     fence_mbar_init();
@@ -742,69 +780,80 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_wait(&x_full[j % kDxStages], (uint32_t)((j / kDxStages) & 1), ab, nullptr, kWaitNs);
       mbar_wait(wz_full, 0, ab, nullptr, kWaitNs);
     }
-  } else if (warp == 1) {
+  } else if (warp == 1 || warp == 2) {
+    // ------------------------------ logits (warp 1) and dw (warp 2) issuers ------------------------------
     if (wk.ntiles > 0) {
       const uint32_t w0 = sdesc_lo(smem_u32(s_w), 16), t0 = sdesc_lo(smem_u32(s_t), 16), t20 = sdesc_lo(smem_u32(s_t2), 16);
       const uint32_t sz = smem_u32(s_zero), ext = (uint32_t)G * 4;
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
       Ring<kDxStages> stg;
-      Ring<kSBuf> sb;
+      Ring<Bufs::kL> sb;
+      Ring<Bufs::kD> db;
       for (int i = 0, q = 0; ok && i < wk.ntiles; i++, stg.next()) {
         if (!(ok = mbar_wait_w(&x_full[stg.i], stg.pass, ab, status))) break;
         const uint32_t st = smem_u32(s_st + stg.i * kStg);
         const uint32_t x = sdesc_lo(st, 16), v = x + kVOff / 16, f = x + kBStage / 16;
-        const uint32_t px = px_lo(st + kPOff, sz), dpx = px_lo(st + kDOff, sz);
+        const uint32_t px = px_lo(st + (warp == 1 ? kPOff : kDOff), sz);
         uint32_t r = 0, e = ext;  // the chunk's rows in the 64-byte and 32-byte images, in 16 bytes
 #pragma unroll 1
-        for (int c = 0; c < nch; c++, q++, sb.next(), r += 64 * 4, e += 64 * 2) {
-          if (q >= kSBuf && !(ok = mbar_wait_w(&pv_done[sb.i], sb.pass ^ 1u, ab, status))) break;
+        for (int c = 0; c < nch; c++, q++, sb.next(), db.next(), r += 64 * 4, e += 64 * 2) {
+          // L: the products of the unit kL back; dw: loaded by the unit kD back
+          if (q >= (warp == 1 ? Bufs::kL : Bufs::kD) &&
+              !(ok = mbar_wait_w(warp == 1 ? &pv_done[sb.i] : &dw_free[db.i], (warp == 1 ? sb.pass : db.pass) ^ 1u, ab,
+                                 status)))
+            break;
           tc_fence_after();
-          const uint32_t tL = tmem + (uint32_t)sb.i * kGC;
-          issue_dot64<false, kHiPx, kHi32>(tL, x, w0 + r, px, w0 + e, hilo ? w0 + (uint32_t)G * 6 + r : 0u);
-          if (kComb) {
+          const uint32_t tL = tmem + (uint32_t)sb.i * 64, tD = tmem + Bufs::kDCol + (uint32_t)db.i * 64;
+          if (warp == 1) {
+            issue_dot64<false, kHiPx, kHi32>(tL, x, w0 + r, px, w0 + e, hilo ? w0 + (uint32_t)G * 6 + r : 0u);
+          } else if (kComb) {
             // As in the slot pass: the deslice's chain without an extra block, the slice's
             // extra block against delta's rows (dS - delta in one K step).
-            issue_dot64<false, 0, 0>(tL + 64, v, t0 + r, 0u, 0u, 0u);
-            issue_dot64<false, kHiPx, kHi32>(tL + 64, f, t20 + r, dpx, t20 + e, 0u, 1u);
+            issue_dot64<false, 0, 0>(tD, v, t0 + r, 0u, 0u, 0u);
+            issue_dot64<false, kHiPx, kHi32>(tD, f, t20 + r, px, t20 + e, 0u, 1u);
           } else {
-            issue_dot64<false, kHiPx, kHi32>(tL + 64, v, t0 + r, dpx, t0 + e, 0u);
+            issue_dot64<false, kHiPx, kHi32>(tD, v, t0 + r, px, t0 + e, 0u);
           }
           mma_commit_w(&s_full[sb.i]);
         }
         mma_commit_w(&x_empty[stg.i]);
       }
-      mma_commit_w(&drain[0]);
-      mbar_wait_w(&drain[0], 0, ab, nullptr, kWaitNs);
+      mma_commit_w(&drain[warp - 1]);
+      mbar_wait_w(&drain[warp - 1], 0, ab, nullptr, kWaitNs);
     }
-  } else if (warp == 2 || warp == 3) {
-    const int j = warp - 2;
+  } else if (warp == 3) {
+    // ------------------------------ product issuer ------------------------------
+    // K-steps [2 j, 2 j + 2) of a 64-slot chunk into O_j.
     if (wk.ntiles > 0) {
       constexpr uint32_t idesc = idesc_bf16(128, kD, false, false);
-      // K-steps [2 j, 2 j + 2) of a 64-slot chunk
-      const uint32_t wt0 = sdesc_lo(smem_u32(s_wt), 16) + (uint32_t)j * 4;
+      const uint32_t wt0 = sdesc_lo(smem_u32(s_wt), 16);
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
-      Ring<kSBuf> sb;
+      Ring<Bufs::kL> sb;
       for (int i = 0; ok && i < wk.ntiles; i++) {
         const int ob = i & 1;
-        const uint32_t tO = tmem + kO + (uint32_t)(j * 2 + ob) * kD;
         if (i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
         uint32_t wt = wt0;
 #pragma unroll 1
         for (int c = 0; c < nch; c++, wt += 256, sb.next()) {
-          if (!(ok = mbar_wait_w(&p_ready[sb.i], sb.pass, ab, status))) break;
-          tc_fence_after();
-          const uint32_t tL = tmem + (uint32_t)sb.i * kGC + (uint32_t)j * 32;  // da_col(2 j)
 #pragma unroll
-          for (int e = 0; e < 2; e++) {
-            mma_ts_w<kHi128>(tO, tL + da_col(e), wt + e * 2, idesc, (c > 0 || e > 0) ? 1u : 0u);
-            if (split) mma_ts_w<kHi128>(tO, tL + da_col(e) + 16, wt + e * 2, idesc, 1u);
+          for (int j = 0; j < 2; j++) {
+            if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + j], sb.pass, ab, status))) break;
+            tc_fence_after();
+            const uint32_t tO = tmem + kO + (uint32_t)(j * 2 + ob) * kD;
+            const uint32_t tL = tmem + (uint32_t)sb.i * 64 + (uint32_t)j * 32;  // da_col(2 j)
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+              mma_ts_w<kHi128>(tO, tL + da_col(e), wt + j * 4 + e * 2, idesc, (c > 0 || e > 0) ? 1u : 0u);
+              if (split) mma_ts_w<kHi128>(tO, tL + da_col(e) + 16, wt + j * 4 + e * 2, idesc, 1u);
+            }
           }
+          if (!ok) break;
           mma_commit_w(&pv_done[sb.i]);
         }
-        mma_commit_w(&o_full[ob]);
+        mma_commit_w(&o_full[i % kDxOFull]);
       }
-      mma_commit_w(&drain[1 + j]);
-      mbar_wait_w(&drain[1 + j], 0, ab, nullptr, kWaitNs);
+      mma_commit_w(&drain[2]);
+      mbar_wait_w(&drain[2], 0, ab, nullptr, kWaitNs);
     }
   } else {
     const int wg = (warp - kSoftmaxWarp0) >> 2;
@@ -814,7 +863,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     auto epilogue = [&](int t) -> bool {
       const int ob = t & 1;
-      if (!mbar_wait(&o_full[ob], (uint32_t)((t >> 1) & 1), ab, status)) return false;
+      if (!mbar_wait(&o_full[t % kDxOFull], (uint32_t)((t / kDxOFull) & 1), ab, status)) return false;
       tc_fence_after();
       uint32_t o0[32], o1[32];
       tmem_ld32(tmem + lane_addr + kO + (uint32_t)ob * kD, o0);
@@ -856,21 +905,31 @@ __global__ void __launch_bounds__(kThreads, 1)
       return true;
     };
     BlockPos pos(wg, nch);
-    for (int q = wg; ok && q < total; q += 2, pos.step(2, nch)) {
+    for (int q = wg; ok && q < total; q += kDxWGs, pos.step(kDxWGs, nch)) {
       const int i = pos.i, c = pos.c;
-      const int bb = q % kSBuf;
-      if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((q / kSBuf) & 1), ab, status))) break;
+      const int bb = q % Bufs::kL, bd = q % Bufs::kD;
+      if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((q / Bufs::kL) & 1), ab, status))) break;
       tc_fence_after();
-      const uint32_t tL = tmem + lane_addr + (uint32_t)bb * kGC;
+      const uint32_t tL = tmem + lane_addr + (uint32_t)bb * 64;
+      const uint32_t tD = tmem + lane_addr + Bufs::kDCol + (uint32_t)bd * 64;
       float unused0 = 0.f, unused1 = 0.f;
-      da_unit<split, false, false>(tL, tL + 64, unused0, unused1);
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_ready[bb]);
+#pragma unroll
+      for (int hf = 0; hf < 2; hf++) {
+        da_half<split, false, false>(tL + 32 * hf, tD + 32 * hf, unused0, unused1, [&]() {
+          if (hf == 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&dw_free[bd]);
+          }
+        });
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_ready[2 * bb + hf]);
+      }
       if (c == 0 && i > 0 && !(ok = epilogue(i - 1))) break;
     }
-    if (ok && total > 0 && total % 2 == wg) epilogue(wk.ntiles - 1);
+    if (ok && total > 0 && total % kDxWGs == wg) epilogue(wk.ntiles - 1);
   }
   tc_fence_before();
   __syncthreads();
@@ -1036,7 +1095,7 @@ struct BwdCall {
     const int P = point_splits(s, (int)s.BH());
     for (int k = 0; k < r.n; k++) {
       const int g0 = k * r.size;
-      if (cudaError_t e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kThreads), sm, st, xmap, vmap, pmap,
+      if (cudaError_t e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kDxThreads), sm, st, xmap, vmap, pmap,
                                  dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, ws + L.wtimg,
                                  static_cast<__nv_bfloat16*>(dx), s.N, padded_n(s), s.H, s.G, g0,
                                  std::min(r.size, s.G - g0), P, hilo ? 1 : 0, (accumulate || k > 0) ? 1 : 0,

@@ -359,15 +359,6 @@ __device__ __forceinline__ void weights_half(uint32_t tS, uint32_t tP) {
   tmem_st16(tP + 16, pk1);
 }
 
-// The 128 log2-weights of one TMEM lane of an S buffer -> bf16 weights written back
-// in place, packed in pairs, into the first 64 columns, in two halves: columns
-// [64 h, 64 h + 64) -> packed weights in columns [32 h, 32 h + 32), which this
-// thread has already read.
-__device__ __forceinline__ void weights_in_halves(uint32_t tS) {
-#pragma unroll 1
-  for (int half = 0; half < 2; half++) weights_half(tS + half * 64, tS + half * 32);
-}
-
 // One 64-column half with split products: the log2-weights in columns [0, 64) from tS
 // -> the bf16 weights packed in pairs into columns [0, 32) and the bf16 pairs of
 // their residuals into [32, 64).  The whole half is in registers before the first
@@ -386,8 +377,8 @@ __device__ __forceinline__ void weights_hilo_half(uint32_t tS) {
   tmem_st16(tS + 48, lo);
 }
 
-// The weight helpers above, plus acc += sum over the block's 128 slots of w_g ds[g]
-// (ds: the block's slice of a per-slot array in shared memory; every lane reads
+// The weight helpers above, plus acc += sum over the half's 64 slots of w_g ds[g]
+// (ds: the half's slice of a per-slot array in shared memory; every lane reads
 // the same address, a broadcast).  The backward of the slice needs this sum for
 // its delta (the dS term).
 __device__ __forceinline__ void weights32_ds(const uint32_t (&v)[32], uint32_t (&p)[16], const float* ds,
@@ -427,19 +418,16 @@ __device__ __forceinline__ void weights32_hilo_ds(const uint32_t (&v)[32], uint3
     }
   }
 }
-__device__ __forceinline__ void weights_in_halves_ds(uint32_t tS, const float* ds, float& acc) {
-#pragma unroll 1
-  for (int half = 0; half < 2; half++) {
-    uint32_t v0[32], v1[32];
-    tmem_ld32(tS + half * 64, v0);
-    tmem_ld32(tS + half * 64 + 32, v1);
-    tmem_wait_ld2(v0, v1);
-    uint32_t pk0[16], pk1[16];
-    weights32_ds(v0, pk0, ds + half * 64, acc);
-    weights32_ds(v1, pk1, ds + half * 64 + 32, acc);
-    tmem_st16(tS + half * 32, pk0);
-    tmem_st16(tS + half * 32 + 16, pk1);
-  }
+__device__ __forceinline__ void weights_half_ds(uint32_t tS, uint32_t tP, const float* ds, float& acc) {
+  uint32_t v0[32], v1[32];
+  tmem_ld32(tS, v0);
+  tmem_ld32(tS + 32, v1);
+  tmem_wait_ld2(v0, v1);
+  uint32_t pk0[16], pk1[16];
+  weights32_ds(v0, pk0, ds, acc);
+  weights32_ds(v1, pk1, ds + 32, acc);
+  tmem_st16(tP, pk0);
+  tmem_st16(tP + 16, pk1);
 }
 // weights_hilo_half with the sum over the half's 64 slots.
 __device__ __forceinline__ void weights_hilo_half_ds(uint32_t tS, const float* ds, float& acc) {

@@ -76,8 +76,11 @@ using namespace tc;
 // it is written, so that its products run under the other half's exponentials (N = 262,144,
 // H = 8, call: G = 1024 373 -> 355 us, G = 512 232 -> 211, G = 256 133 -> 118, against four
 // warpgroups on half rows).  Weights in a buffer of their own with two S buffers, which frees
-// S before the exponentials, was slower (375 with three warpgroups, 411 with four).  The other
-// modes need more registers: two warpgroups, warpgroup q % 2 taking block q.
+// S before the exponentials, was slower (375 with three warpgroups, 411 with four).  The split
+// products (all halves handed over the same way) and MODE 1 run three warpgroups as well: fp32
+// deslice call at B = 1, N = 262,144, G = 512 410 -> 404 us; whole backward at B = 2,
+// N = 131,072, G = 512 2220 -> 2198 (MODE 1 and the point pass).  MODE 2 needs more registers:
+// two warpgroups, warpgroup q % 2 taking block q.
 //
 // The same pass serves the backward (Sec. 3.3): with R_n = sum_g w_ng t_g,
 //   MODE 1 (deslice backward, t = z', v = dO): delta_n = dO_n . R_n (fp32);
@@ -86,8 +89,8 @@ using namespace tc;
 //     softmax warpgroups from the fp32 weights; each warpgroup adds its own
 //     partial per point to wds[wg][bh][n] (cleared beforehand) and the consumer adds them.
 // The pass covers slots [g0, g0 + G) of images of Gi slots.  accumulate (MODES 1, 2, and
-// MODE 0 with X3): a later range of the slots, whose contributions to delta and dfx (to the fp32 out) are added to those of
-// the earlier ranges.
+// MODE 0 with X3): a later range of the slots, whose contributions to delta and dfx (to the
+// fp32 out) are added to those of the earlier ranges.
 // PS (split products): the weights and t as bf16 hi + lo halves, P t = Phi thi +
 // Plo thi + Phi tlo; the image then holds t's residual half after its bf16 half.
 // The split weights of slot half j (slots [64 j, 64 j + 64) of the block) go to
@@ -98,7 +101,7 @@ constexpr uint32_t kDStage = kXBytes + 2 * kPxBytes;  // x tile, point extra (bo
 // X3 (fp32 inputs, MODE 0 with PS): each stage also holds x's residual tile
 // (xrmap), the logits add x_r W'_hi, and out is fp32.
 template <int MODE, bool PS>
-constexpr bool desl_wg3() { return MODE == 0 && !PS; }
+constexpr bool desl_wg3() { return MODE != 2; }
 constexpr int kDesl3Threads = 512;
 // Barriers of completed tiles.  With three warpgroups the one that drains tile t has not
 // waited for tile t - 2 (the accumulator's previous tile), and a parity wait on a barrier
@@ -130,7 +133,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
   uint64_t* x_empty = x_full + kStages;
   uint64_t* s_full = x_empty + kStages;
   constexpr bool kWG3 = desl_wg3<MODE, PS>();
-  uint64_t* p_ready = s_full + kSBuf;  // [S buffer][half] (two warpgroups: half 0 stands for both)
+  uint64_t* p_ready = s_full + kSBuf;  // [S buffer][half]
   uint64_t* pv_done = p_ready + 2 * kSBuf;
   uint64_t* o_full = pv_done + kSBuf;
   uint64_t* o_free = o_full + kOFull;
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
         if (i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
         uint32_t z = z0;
         for (int c = 0; c < nch; c++, z += 512, sb.next()) {
-          if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + (kWG3 ? j : 0)], sb.pass, ab, status))) break;
+          if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + j], sb.pass, ab, status))) break;
           tc_fence_after();
           // weights of slots 64j.. (packed pairs; PS: hi pairs, then lo pairs 32 on)
           const uint32_t tP = tmem + (uint32_t)sb.i * kGC + (uint32_t)j * (PS ? 64 : 32);
@@ -362,34 +365,27 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       const int bb = kWG3 ? wg : q % kSBuf;
       if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((q / kSBuf) & 1), ab, status))) break;
       tc_fence_after();
-      if constexpr (kWG3) {
-        const uint32_t tS = tmem + lane_addr + (uint32_t)bb * kGC;
-        weights_half(tS, tS);
+      const uint32_t tS = tmem + lane_addr + (uint32_t)bb * kGC;
+      if (MODE == 2 && i != wds_tile) {
+        flush_wds();
+        wds_tile = i;
+      }
+#pragma unroll
+      for (int hf = 0; hf < 2; hf++) {
+        const uint32_t tH = tS + (uint32_t)hf * 64;
+        if constexpr (MODE == 2 && PS)
+          weights_hilo_half_ds(tH, s_ds + c * kGC + hf * 64, wds_acc);
+        else if constexpr (MODE == 2)
+          weights_half_ds(tH, tS + (uint32_t)hf * 32, s_ds + c * kGC + hf * 64, wds_acc);
+        else if constexpr (PS)
+          weights_hilo_half(tH);
+        else
+          weights_half(tH, tS + (uint32_t)hf * 32);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&p_ready[2 * bb]);
-        weights_half(tS + 64, tS + 32);
-      } else if constexpr (MODE == 2) {
-        if (i != wds_tile) {
-          flush_wds();
-          wds_tile = i;
-        }
-        if (PS) {
-          weights_hilo_half_ds(tmem + lane_addr + (uint32_t)bb * kGC, s_ds + c * kGC, wds_acc);
-          weights_hilo_half_ds(tmem + lane_addr + (uint32_t)bb * kGC + 64, s_ds + c * kGC + 64, wds_acc);
-        } else
-          weights_in_halves_ds(tmem + lane_addr + (uint32_t)bb * kGC, s_ds + c * kGC, wds_acc);
-      } else if constexpr (PS) {
-        weights_hilo_half(tmem + lane_addr + (uint32_t)bb * kGC);
-        weights_hilo_half(tmem + lane_addr + (uint32_t)bb * kGC + 64);
-      } else {
-        weights_in_halves(tmem + lane_addr + (uint32_t)bb * kGC);
+        if (lane == 0) mbar_arrive(&p_ready[2 * bb + hf]);
       }
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_ready[2 * bb + (kWG3 ? 1 : 0)]);
       // The output of the previous tile is drained by the warpgroup that took the first
       // block of this tile, when the last products of that tile have long finished.
       if (c == 0 && i > 0 && !(ok = epilogue(i - 1))) break;
@@ -664,7 +660,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* x_full = bars + 1;
   uint64_t* st_empty = x_full + kSBuft;
   uint64_t* s_full = st_empty + kSBuft;
-  uint64_t* p_ready = s_full + kSBuf;   // [issuer][S buffer]
+  uint64_t* p_ready = s_full + kSBuf;   // [S buffer][half]
   uint64_t* pv_done = p_ready + 2 * kSBuf;
   uint64_t* acc_full = pv_done + kSBuf;
   uint64_t* acc_done = acc_full + 1;  // [issuer]: products of each of its tiles complete
@@ -803,11 +799,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       Ring<kSBuft> st;
       Ring<kSBuf> sb;
-      uint32_t half = 0;  // parity of this issuer's uses of a buffer (its tiles there are 2 kSBuf apart)
       if (j == 1) st.next(), sb.next();
       for (int i = j; ok && i < wk.ntiles; i += 2) {
-        if (!(ok = mbar_wait_w(&p_ready[j * kSBuf + sb.i], half, ab, status))) break;
-        tc_fence_after();
         const uint32_t tE = tmem + (uint32_t)sb.i * kGC;  // packed weights of the 128 points
         const uint32_t f = sdesc_lo(smem_u32(s_st + st.i * kStB) + kFOff, kFBlock);
         const uint32_t fr = f - kFOff / 16 + kFROff / 16;
@@ -817,6 +810,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool fresh = i < 2 || slice_flush_at<split || X3>(i);
 #pragma unroll
         for (int kk = 0; kk < 8; kk++) {
+          if ((kk & 3) == 0) {  // a half's weights
+            if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + (kk >> 2)], sb.pass, ab, status))) break;
+            tc_fence_after();
+          }
           // 16 points' packed weights: columns kk * 8, or with split products the hi
           // pairs of half kk / 4 at (kk / 4) * 64 + (kk % 4) * 8, their residuals 32 on
           const uint32_t tw = tE + (split ? (uint32_t)(kk >> 2) * 64 + (uint32_t)(kk & 3) * 8 : (uint32_t)kk * 8);
@@ -830,10 +827,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         mma_commit_w(&st_empty[st.i]);
         if (split || X3) mma_commit_w(&acc_done[j]);
         st.next(), st.next();
-        // kSBuf is odd: after each full pass over the ring the issuer has visited every buffer
-        // once, in an order that repeats every kSBuf of its tiles
         sb.next(), sb.next();
-        if ((i >> 1) % kSBuf == kSBuf - 1) half ^= 1u;
       }
       if (ok) mma_commit_w(acc_full);
       mma_commit_w(&drain[1 + j]);
@@ -883,23 +877,24 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((i / kSBuf) & 1), ab, status))) break;
       tc_fence_after();
       const uint32_t tS = tmem + lane_addr + (uint32_t)bb * kGC;
-      if constexpr (split) {
-        weights_hilo_half(tS);
-        weights_hilo_half(tS + 64);
-      } else {
-        weights_in_halves(tS);
+#pragma unroll
+      for (int hf = 0; hf < 2; hf++) {
+        if constexpr (split)
+          weights_hilo_half(tS + (uint32_t)hf * 64);
+        else
+          weights_half(tS + (uint32_t)hf * 64, tS + (uint32_t)hf * 32);
+        tmem_wait_st();
+        if (hf == 0 && i >= 2 && slice_flush_at<split || X3>(i)) {
+          // The products of this warpgroup's tiles up to i - 2 are complete (acc_done
+          // cannot move past that phase before this warpgroup hands over tile i).
+          if (!(ok = mbar_wait(&acc_done[wg], (uint32_t)(((i - 2) >> 1) & 1), ab, status))) break;
+          tc_fence_after();
+          add_acc();
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_ready[2 * bb + hf]);
       }
-      tmem_wait_st();
-      if (i >= 2 && slice_flush_at<split || X3>(i)) {
-        // The products of this warpgroup's tiles up to i - 2 are complete (acc_done
-        // cannot move past that phase before this warpgroup hands over tile i).
-        if (!(ok = mbar_wait(&acc_done[wg], (uint32_t)(((i - 2) >> 1) & 1), ab, status))) break;
-        tc_fence_after();
-        add_acc();
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_ready[wg * kSBuf + bb]);
     }
     const int64_t BH = gridDim.z;
     float* o = part + (((int64_t)blockIdx.y * BH + wk.bh) * G + g_base + r) * (kD + 1);
@@ -1163,7 +1158,7 @@ cudaError_t tc_deslice_fwd(const Shape& s0, const void* x, const float* W, const
   if ((e = set_smem(kernel, sm)) != cudaSuccess) return e;
   for (int k = 0; k < xr.n; k++) {
     const int g0 = k * xr.size;
-    if ((e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(x3 ? kThreads : kDesl3Threads), sm, st, xmap,
+    if ((e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kDesl3Threads), sm, st, xmap,
                     pmap, xrmap, wimg, zimg, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr,
                     s.N, padded_n(s), s.H, s.G, g0, std::min(xr.size, s.G - g0), P, hilo ? 1 : 0,
                     (uint32_t)s.G * (ps ? 128 : 64), k > 0 ? 1 : 0, status)) != cudaSuccess) return e;
@@ -1191,7 +1186,7 @@ cudaError_t tc_rows_bwd(const Shape& s, int Gi, int g0, int mode, const void* x,
                                 : (ps ? k_deslice<2, true> : k_deslice<2, false>);
   cudaError_t e = set_smem(kernel, sm);
   if (e != cudaSuccess) return e;
-  return launch(kernel, grid, dim3(kThreads), sm, st, xmap, pmap, xmap, wimg, zimg, static_cast<__nv_bfloat16*>(dfx),
+  return launch(kernel, grid, dim3(mode == 2 ? kThreads : kDesl3Threads), sm, st, xmap, pmap, xmap, wimg, zimg, static_cast<__nv_bfloat16*>(dfx),
                 static_cast<const __nv_bfloat16*>(v), delta, wds, dS, s.N, Np, s.H, Gi, g0, s.G, P, hilo ? 1 : 0,
                 (uint32_t)Gi * 128, accumulate, status);
 }
