@@ -38,15 +38,18 @@ cudaError_t run_slice(const Shape& s, int G, const void* x, const void* f, const
                       const uint8_t* wimg, void* px, float* tokens, float* wsum, int finalize, float* part,
                       uint32_t* status, cudaStream_t st);
 
-// Rows pass of the backward (the deslice kernel in backward mode 1 or 2) over slots
+// Rows pass of the backward (the deslice kernel in backward mode 1, 2 or 3) over slots
 // [g0, g0 + s.G) of operands prepared for Gi slots: W image, Z-layout image of t (hi then
-// lo, Gi*128 bytes per (b,h)), lse point-extra rows; writes delta (and, mode 2, dfx), or adds
-// to them when accumulate != 0 (a later slot range of the same points), and adds the two
-// per-warpgroup partials of sum_g w dS to wds (which must start at zero).
+// lo, Gi*128 bytes per (b,h); mode 3: zimg2 the second part's), lse point-extra rows; writes
+// delta (and, modes 2 and 3, dfx), or adds to them when accumulate != 0 (a later slot range of
+// the same points), and the per-warpgroup partials (mode 2 two, mode 3 three) of sum_g w dS to
+// wds (which must start at zero).  v: the points that meet t (mode 3: fx, and v2 = dO).
 cudaError_t tc_rows_bwd(const Shape& s, int Gi, int g0, int mode, const void* x, const uint8_t* wimg,
-                        const uint8_t* zimg, const void* px, const void* v, void* dfx, float* delta, float* wds,
-                        const float* dS, int accumulate, uint32_t* status, cudaStream_t st);
-size_t tc_rows_smem(const Shape& s, int mode, bool ps, bool hilo);
+                        const uint8_t* zimg, const uint8_t* zimg2, const void* px, const void* v, const void* v2,
+                        void* dfx, float* delta, float* wds, const float* dS, int accumulate, uint32_t* status,
+                        cudaStream_t st);
+// Shared memory it needs at least.
+size_t tc_rows_smem(const Shape& s);
 
 // ---- tensor-core backward (fs_tc_bwd.cu) ----
 // True when the tensor-core backward implements this shape: bf16, d = 32, N >= 2,

@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(256) k_prep_us(const float* __restrict__ z, co
 // delta_n = delta[bh][n] (+ delta2[bh][n] when given, + wds[0][bh][n] + wds[1][bh][n]
 // when wds is given).
 __global__ void k_prep_dpx(const float* __restrict__ delta, const float* __restrict__ delta2,
-                           const float* __restrict__ wds, uint4* __restrict__ dpx, int64_t BH, int64_t N, int64_t Np) {
+                           const float* __restrict__ wds, int nwds, uint4* __restrict__ dpx, int64_t BH, int64_t N,
+                           int64_t Np) {
   grid_begin(delta, delta2, wds);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= BH * Np) return;
@@ -99,7 +100,11 @@ __global__ void k_prep_dpx(const float* __restrict__ delta, const float* __restr
   if (n < N) {
     d = delta[bh * N + n];
     if (delta2) d += delta2[bh * N + n];
-    if (wds) d += wds[bh * N + n] + wds[(BH + bh) * N + n];
+    if (wds) {
+      float w = wds[bh * N + n] + wds[(BH + bh) * N + n];
+      if (nwds == 3) w += wds[(2 * BH + bh) * N + n];
+      d += w;
+    }
   }
   dpx[i] = extra_row3(-d);
 }
@@ -193,8 +198,6 @@ __device__ __forceinline__ void da_half(uint32_t tL, uint32_t tD, float& dt, flo
     db += lo_f(sb2) + hi_f(sb2);
   }
 }
-// TMEM column (within a unit) of the hi pairs of K-step kk (16 entries).
-__device__ __forceinline__ uint32_t da_col(int kk) { return (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)); }
 
 // One half of a unit: L (log2 weights) -> w = 2^L in place, as bf16 pairs in da_half's
 // layout (hi pairs, then their residuals with kSplit).
@@ -962,7 +965,7 @@ int bwd_slot_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * bwd_
 // (The separate calls' point pass holds the residual half of W' up to 512 slots: past 640,
 // where it runs over ranges anyway, no range is longer, which keeps dx of a sum over many
 // ranges accurate.)
-constexpr int kBwdSlotsMax = 640, kCombSlotsMax = 256, kPointSlotsMax = 512;
+constexpr int kBwdSlotsMax = 640, kCombSlotsMax = 256, kPointSlotsMax = 512, kRowsBothMax = 512;
 struct SlotRanges {
   int n, size;
 };
@@ -970,6 +973,11 @@ SlotRanges slot_ranges(int Gp, int most) {
   const int n = (Gp + most - 1) / most;
   return {n, (Gp / kGC + n - 1) / n * kGC};
 }
+
+// fs_coupling_bwd: one rows pass for both parts where the images of both t fit (512 slots).
+// Ranges cut to fit would round dfx to bf16 once more a range and run the epilogue again, so
+// longer ranges (513 to 640 slots) keep a pass for each part.
+bool rows_both(const Shape& s) { return slot_ranges(s.G, kBwdSlotsMax).size <= kRowsBothMax; }
 
 SlotRanges point_ranges(int Gp, bool comb) {
   return slot_ranges(Gp, comb ? kCombSlotsMax : (Gp <= kBwdSlotsMax ? kBwdSlotsMax : kPointSlotsMax));
@@ -1014,10 +1022,12 @@ BwdLayout bwd_layout(const Shape& s0, BwdKind kind) {
   L.px = take(px_bytes(s));
   L.dpx = take(px_bytes(s));
   L.delta = take(pts * sizeof(float));
-  L.delta_d = take(comb ? pts * sizeof(float) : 0);
-  L.wds = take(kind != kDesliceBwd ? 2 * pts * sizeof(float) : 0);
+  const bool both = comb && rows_both(s);
+  L.delta_d = take(comb && !both ? pts * sizeof(float) : 0);
+  L.wds = take(kind != kDesliceBwd ? (both ? 3 : 2) * pts * sizeof(float) : 0);
   L.ds = take(BHG * sizeof(float));
   L.dtp = take((size_t)s.BH() * P * R * sizeof(float));
+  // (rows_both: the second zimg, whose last reader is done when the slot pass writes here)
   L.part = take((size_t)P * BHG * (kind == kDesliceBwd ? 2 * kD + 2 : kD + 2) * sizeof(float));
   // d z' of the coupling through the forward's slice
   const bool via_slice = comb && tc_forward_supported(split_shape(s0));
@@ -1039,27 +1049,28 @@ struct BwdCall {
   float* f(size_t off) const { return reinterpret_cast<float*>(ws + off); }
 
   // delta and, mode 2, dfx and the sums of w dS, over the slot ranges; zimg holds t.
-  cudaError_t rows(int mode, const void* x, const void* v, void* dfx, float* delta) const {
+  // Mode 3: both parts (v = fx, v2 = dO; zimg holds z', the part region dU).
+  cudaError_t rows(int mode, const void* x, const void* v, const void* v2, void* dfx, float* delta) const {
     const SlotRanges r = slot_ranges(s.G, kBwdSlotsMax);
     for (int k = 0; k < r.n; k++) {
       const int g0 = k * r.size;
       Shape sr = s;
       sr.G = std::min(r.size, s.G - g0);
-      if (cudaError_t e = tc_rows_bwd(sr, s.G, g0, mode, x, ws + L.wimg, ws + L.zimg, ws + L.px, v, dfx, delta,
-                                      mode == 2 ? f(L.wds) : nullptr, f(L.ds), k > 0 ? 1 : 0, status, st))
+      if (cudaError_t e = tc_rows_bwd(sr, s.G, g0, mode, x, ws + L.wimg, ws + L.zimg, ws + L.part, ws + L.px, v, v2, dfx, delta,
+                                      mode != 1 ? f(L.wds) : nullptr, f(L.ds), k > 0 ? 1 : 0, status, st))
         return e;
     }
     return cudaSuccess;
   }
-  // u = dz / (S + eps) and c as images (T at `timg`, zimg) and ds.
-  cudaError_t images_us(const float* z, const float* wsum, const float* dz, size_t timg) const {
+  // u = dz / (S + eps) and c as images (T at `timg`, Z layout at `zimg`) and ds.
+  cudaError_t images_us(const float* z, const float* wsum, const float* dz, size_t timg, size_t zimg) const {
     return launch(k_prep_us, dim3((unsigned)(s.G / 64), (unsigned)s.BH()), dim3(256), 0, st, z, wsum, dz, ws + timg,
-                  ws + L.zimg, f(L.ds), s0.G, s.G, s.eps);
+                  ws + zimg, f(L.ds), s0.G, s.G, s.eps);
   }
   // delta's point rows from delta (+ delta2) (+ the sums of w dS).
-  cudaError_t delta_rows(const float* delta, const float* delta2, const float* wds) const {
+  cudaError_t delta_rows(const float* delta, const float* delta2, const float* wds, int nwds) const {
     const int64_t n = s.BH() * padded_n(s);
-    return launch(k_prep_dpx, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, delta, delta2, wds,
+    return launch(k_prep_dpx, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, delta, delta2, wds, nwds,
                   reinterpret_cast<uint4*>(ws + L.dpx), s.BH(), s.N, padded_n(s));
   }
   // The slot pass over all slots (v, f: the deslice's and the slice's points of MODE 3).
@@ -1129,7 +1140,7 @@ bool tc_backward_supported(const Shape& s0) {
   Shape s = pass_shape(s0);
   s.G = slot_ranges(s.G, kBwdSlotsMax).size;
   return tc_forward_supported(s) && smem_bwd_dx(s.G, false) <= kMaxSmem &&
-         tc_rows_smem(s, 2, false, false) <= kMaxSmem;
+         tc_rows_smem(s) <= kMaxSmem;
 }
 
 size_t tc_backward_bytes(const Shape& s, int mode) {
@@ -1155,8 +1166,8 @@ cudaError_t tc_deslice_bwd(const Shape& s0, const void* x, const float* W, const
   p.tokens(zp, c.ws + c.L.timg, c.ws + c.L.zimg, true);
   p.rows(lse, c.ws + c.L.px);
   FS_TRY(p.run(st));
-  FS_TRY(c.rows(1, x, dout, nullptr, c.f(c.L.delta)));
-  FS_TRY(c.delta_rows(c.f(c.L.delta), nullptr, nullptr));
+  FS_TRY(c.rows(1, x, dout, nullptr, nullptr, c.f(c.L.delta)));
+  FS_TRY(c.delta_rows(c.f(c.L.delta), nullptr, nullptr, 0));
   FS_TRY(c.slot<1>(x, dout, nullptr));
   FS_TRY(c.reduce(tau, dzp, dW, db, dtau, accumulate));
   return c.point<false>(x, dout, nullptr, dx, accumulate);
@@ -1173,9 +1184,9 @@ cudaError_t tc_slice_bwd(const Shape& s0, const void* x, const void* f, const fl
   p.rows(lse, c.ws + c.L.px);
   p.clear(c.f(c.L.wds), 2 * c.s.BH() * c.s.N);
   FS_TRY(p.run(st));
-  FS_TRY(c.images_us(z, wsum, dz, c.L.timg));
-  FS_TRY(c.rows(2, x, f, dfx, c.f(c.L.delta)));
-  FS_TRY(c.delta_rows(c.f(c.L.delta), nullptr, c.f(c.L.wds)));
+  FS_TRY(c.images_us(z, wsum, dz, c.L.timg, c.L.zimg));
+  FS_TRY(c.rows(2, x, f, nullptr, dfx, c.f(c.L.delta)));
+  FS_TRY(c.delta_rows(c.f(c.L.delta), nullptr, c.f(c.L.wds), 2));
   FS_TRY(c.slot<2>(x, f, nullptr));
   FS_TRY(c.reduce(tau, nullptr, dW, db, dtau, accumulate));
   return c.point<false>(x, f, nullptr, dx, accumulate);
@@ -1188,23 +1199,23 @@ size_t tc_coupling_bwd_bytes(const Shape& s) {
 int tc_coupling_bwd_launch_count(const Shape& s) {
   const int G = pass_shape(s).G, n = slot_ranges(G, kBwdSlotsMax).n;
   // prep; d z' (slice or slot pass, reduction), the mix backward, u's images; delta's rows,
-  // slot, reductions; both rows passes and the point pass per range
-  return 1 + 2 + 1 + 1 + 3 + 2 * n + point_ranges(G, true).n;
+  // slot, reductions; the rows passes and the point pass per range
+  return 1 + 2 + 1 + 1 + 3 + (rows_both(pass_shape(s)) ? 1 : 2) * n + point_ranges(G, true).n;
 }
 
 // The coupling's backward in one call (fs_coupling_bwd).  The deslice's and the
 // slice's da share the weights, so their slot-owned and point-owned products can be
 // formed once from da_D + da_S; what has to come first is d z' (it feeds the mix
 // backward, and so dU, dS and the slice's part):
-//   1. the deslice part's rows pass: delta_D;
-//   2. d z' = sum_n w_ng dO_n: the forward's slice with dO for fx (its unnormalised
+//   1. d z' = sum_n w_ng dO_n: the forward's slice with dO for fx (its unnormalised
 //      numerators) where the forward's kernels take the shape, else the slot pass in
 //      mode 0 (the weights alone);
-//   3. the mix backward and the images of dU | dS;
-//   4. the slice part's rows pass: delta_S, dfx, the sum_g w dS partials;
-//   5. delta = delta_S + delta_D + sum_g w dS into the point rows;
-//   6. the slot pass in mode 3: dW, dbias, dtau of da_D + da_S;
-//   7. the point pass for dx.
+//   2. the mix backward and the images of dU | dS;
+//   3. the rows pass in mode 3: delta_D + delta_S, dfx, the sum_g w dS partials (past 512
+//      slots a range: in mode 1 for the deslice part, first, and here in mode 2);
+//   4. delta + sum_g w dS into the point rows;
+//   5. the slot pass in mode 3: dW, dbias, dtau of da_D + da_S;
+//   6. the point pass for dx.
 cudaError_t tc_coupling_bwd(const Shape& s0, const void* x, const void* f, const void* dout, const float* W,
                             const float* bias, const float* tau, const float* M, const float* z, const float* wsum,
                             const float* zp, const float* lse, float* dzp, float* dz, float* dM, void* dx, void* dfx,
@@ -1217,9 +1228,11 @@ cudaError_t tc_coupling_bwd(const Shape& s0, const void* x, const void* f, const
   p.weights_t(W, c.ws + L.wtimg);
   p.tokens(zp, c.ws + L.timg, c.ws + L.zimg, true);
   p.rows(lse, c.ws + L.px);
-  p.clear(c.f(L.wds), 2 * c.s.BH() * c.s.N);
+  const bool both = rows_both(c.s);
+  const int nwds = both ? 3 : 2;
+  p.clear(c.f(L.wds), nwds * c.s.BH() * c.s.N);
   FS_TRY(p.run(st));
-  FS_TRY(c.rows(1, x, dout, nullptr, c.f(L.delta_d)));
+  if (!both) FS_TRY(c.rows(1, x, dout, nullptr, nullptr, c.f(L.delta_d)));
   if (tc_forward_supported(split_shape(s0))) {
     FS_TRY(run_slice(c.s, s0.G, x, dout, nullptr, nullptr, c.ws + L.wimg, c.ws + L.px, dzp, c.f(L.sl_wsum), 0,
                      c.f(L.sl_part), status, st));
@@ -1228,9 +1241,9 @@ cudaError_t tc_coupling_bwd(const Shape& s0, const void* x, const void* f, const
     FS_TRY(simt_reduce_dzp(s0, bwd_slot_splits(c.s), c.f(L.part), c.s.G, kD, dzp, st));
   }
   FS_TRY(mix_bwd(s0, M, z, dzp, dz, dM, st));
-  FS_TRY(c.images_us(z, wsum, dz, L.timg2));
-  FS_TRY(c.rows(2, x, f, dfx, c.f(L.delta)));
-  FS_TRY(c.delta_rows(c.f(L.delta), c.f(L.delta_d), c.f(L.wds)));
+  FS_TRY(c.images_us(z, wsum, dz, L.timg2, both ? L.part : L.zimg));
+  FS_TRY(c.rows(both ? 3 : 2, x, f, dout, dfx, c.f(L.delta)));
+  FS_TRY(c.delta_rows(c.f(L.delta), both ? nullptr : c.f(L.delta_d), c.f(L.wds), nwds));
   FS_TRY(c.slot<3>(x, dout, f));
   FS_TRY(c.reduce(tau, nullptr, dW, db, dtau, accumulate));
   return c.point<true>(x, dout, f, dx, accumulate);

@@ -332,16 +332,22 @@ __device__ __forceinline__ void weights32(const uint32_t (&v)[32], uint32_t (&p)
   for (int k = 0; k < 16; k++) p[k] = pack_bf16(ex2(__uint_as_float(v[2 * k])), ex2(__uint_as_float(v[2 * k + 1])));
 }
 
+// The bf16 halves hi and lo = bf16(w - hi) of a pair of weights.
+__device__ __forceinline__ void split_pair(uint64_t w2, uint32_t& hi, uint32_t& lo) {
+  const uint64_t neg1 = pack2(__float_as_uint(-1.f), __float_as_uint(-1.f));
+  hi = pack_bf16(lo_f(w2), hi_f(w2));
+  const uint64_t r2 = fma2(pack2(hi << 16, hi & 0xFFFF0000u), neg1, w2);
+  lo = pack_bf16(lo_f(r2), hi_f(r2));
+}
+
 // 2^t for 32 log2-weights -> the bf16 pairs (hi) and the bf16 pairs of the
 // residuals w - hi (lo): w = hi + lo to ~2^-16 relative.
 __device__ __forceinline__ void weights32_hilo(const uint32_t (&v)[32], uint32_t (&hi)[16], uint32_t (&lo)[16]) {
 #pragma unroll
   for (int k = 0; k < 16; k++) {
-    const float w0 = ex2(__uint_as_float(v[2 * k])), w1 = ex2(__uint_as_float(v[2 * k + 1]));
-    const uint32_t p = pack_bf16(w0, w1);
-    const float h0 = __uint_as_float(p << 16), h1 = __uint_as_float(p & 0xFFFF0000u);
-    hi[k] = p;
-    lo[k] = pack_bf16(w0 - h0, w1 - h1);
+    const uint64_t w2 = pack2(__float_as_uint(ex2(__uint_as_float(v[2 * k]))),
+                              __float_as_uint(ex2(__uint_as_float(v[2 * k + 1]))));
+    split_pair(w2, hi[k], lo[k]);
   }
 }
 
@@ -359,44 +365,31 @@ __device__ __forceinline__ void weights_half(uint32_t tS, uint32_t tP) {
   tmem_st16(tP + 16, pk1);
 }
 
-// One 64-column half with split products: the log2-weights in columns [0, 64) from tS
-// -> the bf16 weights packed in pairs into columns [0, 32) and the bf16 pairs of
-// their residuals into [32, 64).  The whole half is in registers before the first
-// store, so the stores may land on columns not yet converted.
-__device__ __forceinline__ void weights_hilo_half(uint32_t tS) {
-  uint32_t v0[32], v1[32];
-  tmem_ld32(tS, v0);
-  tmem_ld32(tS + 32, v1);
-  tmem_wait_ld2(v0, v1);
-  uint32_t hi[16], lo[16];
-  weights32_hilo(v0, hi, lo);
+// Split products: 32 columns of log2-weights -> in place the bf16 weights packed in pairs
+// (16 columns), then the bf16 pairs of their residuals (16).
+__device__ __forceinline__ void weights32_hilo_inplace(uint32_t tS) {
+  uint32_t v[32], hi[16], lo[16];
+  tmem_ld32(tS, v);
+  tmem_wait_ld(v);
+  weights32_hilo(v, hi, lo);
   tmem_st16(tS, hi);
-  tmem_st16(tS + 32, lo);
-  weights32_hilo(v1, hi, lo);
-  tmem_st16(tS + 16, hi);
-  tmem_st16(tS + 48, lo);
+  tmem_st16(tS + 16, lo);
+}
+// TMEM column, within a run of such packed columns, of the hi pairs of K-step kk (16
+// entries); their lo pairs are 16 columns on.
+__device__ __forceinline__ uint32_t da_col(int kk) { return (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)); }
+// One 64-column half.  (With 64 columns in registers at a time the fp32 deslice call at
+// N = 262,144, H = 8, G = 512 took 402 us against 372.)
+__device__ __forceinline__ void weights_hilo_half(uint32_t tS) {
+  weights32_hilo_inplace(tS);
+  weights32_hilo_inplace(tS + 32);
 }
 
-// The weight helpers above, plus acc += sum over the half's 64 slots of w_g ds[g]
-// (ds: the half's slice of a per-slot array in shared memory; every lane reads
-// the same address, a broadcast).  The backward of the slice needs this sum for
-// its delta (the dS term).
-__device__ __forceinline__ void weights32_ds(const uint32_t (&v)[32], uint32_t (&p)[16], const float* ds,
-                                             float& acc) {
-  const float4* d4 = reinterpret_cast<const float4*>(ds);
-#pragma unroll
-  for (int k = 0; k < 8; k++) {
-    const float4 q = d4[k];
-    const float w0 = ex2(__uint_as_float(v[4 * k])), w1 = ex2(__uint_as_float(v[4 * k + 1]));
-    const float w2 = ex2(__uint_as_float(v[4 * k + 2])), w3 = ex2(__uint_as_float(v[4 * k + 3]));
-    acc = fmaf(w0, q.x, acc);
-    acc = fmaf(w1, q.y, acc);
-    acc = fmaf(w2, q.z, acc);
-    acc = fmaf(w3, q.w, acc);
-    p[2 * k] = pack_bf16(w0, w1);
-    p[2 * k + 1] = pack_bf16(w2, w3);
-  }
-}
+// The same, plus acc += sum over the half's 64 slots of w_g ds[g] (ds: the half's slice of a
+// per-slot array in shared memory; every lane reads the same address, a broadcast).  The
+// backward of the slice needs this sum for its delta (the dS term).  The loop stays rolled:
+// unrolled, the sums of one 32 overlap the next and spill at 128 registers a thread (whole
+// backward at B = 2, N = 131,072, H = 8, G = 512 1926 us against 1850).
 __device__ __forceinline__ void weights32_hilo_ds(const uint32_t (&v)[32], uint32_t (&hi)[16], uint32_t (&lo)[16],
                                                   const float* ds, float& acc) {
   const float4* d4 = reinterpret_cast<const float4*>(ds);
@@ -411,37 +404,20 @@ __device__ __forceinline__ void weights32_hilo_ds(const uint32_t (&v)[32], uint3
     acc = fmaf(w[2], q.z, acc);
     acc = fmaf(w[3], q.w, acc);
 #pragma unroll
-    for (int e = 0; e < 2; e++) {
-      const uint32_t pk = pack_bf16(w[2 * e], w[2 * e + 1]);
-      hi[2 * k + e] = pk;
-      lo[2 * k + e] = pack_bf16(w[2 * e] - __uint_as_float(pk << 16), w[2 * e + 1] - __uint_as_float(pk & 0xFFFF0000u));
-    }
+    for (int e = 0; e < 2; e++)
+      split_pair(pack2(__float_as_uint(w[2 * e]), __float_as_uint(w[2 * e + 1])), hi[2 * k + e], lo[2 * k + e]);
   }
 }
-__device__ __forceinline__ void weights_half_ds(uint32_t tS, uint32_t tP, const float* ds, float& acc) {
-  uint32_t v0[32], v1[32];
-  tmem_ld32(tS, v0);
-  tmem_ld32(tS + 32, v1);
-  tmem_wait_ld2(v0, v1);
-  uint32_t pk0[16], pk1[16];
-  weights32_ds(v0, pk0, ds, acc);
-  weights32_ds(v1, pk1, ds + 32, acc);
-  tmem_st16(tP, pk0);
-  tmem_st16(tP + 16, pk1);
-}
-// weights_hilo_half with the sum over the half's 64 slots.
 __device__ __forceinline__ void weights_hilo_half_ds(uint32_t tS, const float* ds, float& acc) {
-  uint32_t v0[32], v1[32];
-  tmem_ld32(tS, v0);
-  tmem_ld32(tS + 32, v1);
-  tmem_wait_ld2(v0, v1);
-  uint32_t hi[16], lo[16];
-  weights32_hilo_ds(v0, hi, lo, ds, acc);
-  tmem_st16(tS, hi);
-  tmem_st16(tS + 32, lo);
-  weights32_hilo_ds(v1, hi, lo, ds + 32, acc);
-  tmem_st16(tS + 16, hi);
-  tmem_st16(tS + 48, lo);
+#pragma unroll 1
+  for (int e = 0; e < 64; e += 32) {
+    uint32_t v[32], hi[16], lo[16];
+    tmem_ld32(tS + e, v);
+    tmem_wait_ld(v);
+    weights32_hilo_ds(v, hi, lo, ds + e, acc);
+    tmem_st16(tS + e, hi);
+    tmem_st16(tS + e + 16, lo);
+  }
 }
 
 // A point-extra row [1, 1, -v_1, -v_2, -v_3, 0, 0, 0] (bf16): v = v_1 + v_2 + v_3 in

@@ -77,24 +77,33 @@ using namespace tc;
 // H = 8, call: G = 1024 373 -> 355 us, G = 512 232 -> 211, G = 256 133 -> 118, against four
 // warpgroups on half rows).  Weights in a buffer of their own with two S buffers, which frees
 // S before the exponentials, was slower (375 with three warpgroups, 411 with four).  The split
-// products (all halves handed over the same way) and MODE 1 run three warpgroups as well: fp32
-// deslice call at B = 1, N = 262,144, G = 512 410 -> 404 us; whole backward at B = 2,
-// N = 131,072, G = 512 2220 -> 2198 (MODE 1 and the point pass).  MODE 2 needs more registers:
-// two warpgroups, warpgroup q % 2 taking block q.
+// products (all halves handed over the same way) run three warpgroups as well: fp32 deslice
+// call at B = 1, N = 262,144, H = 8, G = 512 410 us with two, 404 with three, 372 with 32
+// columns at a time in registers.  MODE 2 keeps two (its scratch holds two partial sums of
+// w dS a point), warpgroup q % 2 taking block q.
 //
 // The same pass serves the backward (Sec. 3.3): with R_n = sum_g w_ng t_g,
 //   MODE 1 (deslice backward, t = z', v = dO): delta_n = dO_n . R_n (fp32);
 //   MODE 2 (slice backward, t = dU, v = fx): dfx_n = R_n (bf16, into out) and
 //     delta_n = fx_n . R_n + sum_g w_ng dS_g.  The second sum is formed by the
 //     softmax warpgroups from the fp32 weights; each warpgroup adds its own
-//     partial per point to wds[wg][bh][n] (cleared beforehand) and the consumer adds them.
-// The pass covers slots [g0, g0 + G) of images of Gi slots.  accumulate (MODES 1, 2, and
+//     partial per point to wds[wg][bh][n] (cleared beforehand) and the consumer adds them;
+//   MODE 3, both at once (the whole coupling's backward; z' in zimg, dU in zimg2): the
+//     weights are formed once.  delta_n = dO_n . R_n + fx_n . R2_n, dfx_n = R2_n.  z' and dU
+//     rows of 64 slots lie one after the other, so one MMA (N = 64) multiplies both; warp 3
+//     issues them all into one accumulator per tile parity.  The images take 416 B a slot, so
+//     at 512 slots one x stage is left; three are no faster (G = 256: 1037 us with three,
+//     1042 with one).  What bounds it is the softmax warps: without the w dS sums the whole
+//     backward took 7% less, without the epilogue's loads and stores 6%, without two of three
+//     products 2%.  Whole backward at B = 2, N = 131,072, H = 8, G = 512: 2165 us with a MODE
+//     1 and a MODE 2 pass, 1849 with this one.
+// The pass covers slots [g0, g0 + G) of images of Gi slots.  accumulate (MODES 1 to 3, and
 // MODE 0 with X3): a later range of the slots, whose contributions to delta and dfx (to the
 // fp32 out) are added to those of the earlier ranges.
 // PS (split products): the weights and t as bf16 hi + lo halves, P t = Phi thi +
 // Plo thi + Phi tlo; the image then holds t's residual half after its bf16 half.
-// The split weights of slot half j (slots [64 j, 64 j + 64) of the block) go to
-// columns [64 j, 64 j + 64) of the S buffer: the hi pairs, then the lo pairs.
+// The split weights of slot half j (slots [64 j, 64 j + 64) of the block) go to columns
+// [64 j, 64 j + 64) of the S buffer: per 32 slots the hi pairs, then the lo pairs.
 // =========================================================================================
 constexpr uint32_t kDStage = kXBytes + 2 * kPxBytes;  // x tile, point extra (both halves)
 
@@ -112,22 +121,25 @@ template <int MODE, bool PS, bool X3 = false>
 __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThreads, 1)
     k_deslice(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap pmap,
               const __grid_constant__ CUtensorMap xrmap,
-              const uint8_t* __restrict__ wimg, const uint8_t* __restrict__ zimg, __nv_bfloat16* __restrict__ out,
-              const __nv_bfloat16* __restrict__ v, float* __restrict__ delta, float* __restrict__ wds,
+              const uint8_t* __restrict__ wimg, const uint8_t* __restrict__ zimg, const uint8_t* __restrict__ zimg2,
+              __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ v,
+              const __nv_bfloat16* __restrict__ v2, float* __restrict__ delta, float* __restrict__ wds,
               const float* __restrict__ dS, int64_t N, int64_t Np, int H, int Gi, int g0, int G, int splits,
-              int hilo, uint32_t zstride, int accumulate, uint32_t* status) {
+              int hilo, uint32_t zstride, int nst, int accumulate, uint32_t* status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // hilo: the residual half of W' fits in shared memory too (K = 80 logits, as in
   // the statistics pass); else bf16 W' only (K = 48).
-  const uint32_t wbytes = (uint32_t)G * (hilo ? kWRow : 96), zbytes = (uint32_t)G * (PS ? 128 : 64);
+  const uint32_t wbytes = (uint32_t)G * (hilo ? kWRow : 96), zbytes = (uint32_t)G * (MODE == 3 ? 256 : PS ? 128 : 64);
+  constexpr bool kDs = MODE == 2 || MODE == 3;
+  const int ns = MODE == 3 ? nst : kStages;  // stages
   uint8_t* s_w = smem;
   uint8_t* s_z = s_w + wbytes;
-  float* s_ds = reinterpret_cast<float*>(s_z + zbytes);  // MODE 2: dS of the G slots
+  float* s_ds = reinterpret_cast<float*>(s_z + zbytes);  // kDs: dS of the G slots
   // (the stages stay 1024-byte aligned for their swizzled tiles)
-  uint8_t* s_x = s_z + zbytes + (MODE == 2 ? (((uint32_t)G * 4 + 1023u) & ~1023u) : 0u);  // stage s at s_x + s * kDSt
+  uint8_t* s_x = s_z + zbytes + (kDs ? (((uint32_t)G * 4 + 1023u) & ~1023u) : 0u);  // stage s at s_x + s * kDSt
   constexpr uint32_t kDSt = kDStage + (X3 ? kXBytes : 0u);  // stage: x | px (2 halves) [| x residual]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_x + kStages * kDSt);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_x + ns * kDSt);
   uint64_t* wz_full = bars;
   uint64_t* x_full = bars + 1;
   uint64_t* x_empty = x_full + kStages;
@@ -160,15 +172,15 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       mbar_init(&s_full[i], 1);
       mbar_init(&p_ready[2 * i], 4);  // the four warps of the warpgroup that owns the block
       mbar_init(&p_ready[2 * i + 1], 4);
-      mbar_init(&pv_done[i], 2);
+      mbar_init(&pv_done[i], MODE == 3 ? 1 : 2);
     }
-    for (int i = 0; i < kOFull; i++) mbar_init(&o_full[i], 2);
+    for (int i = 0; i < kOFull; i++) mbar_init(&o_full[i], MODE == 3 ? 1 : 2);
     for (int i = 0; i < 2; i++) mbar_init(&o_free[i], 4);
     for (int i = 0; i < 3; i++) mbar_init(&drain[i], 1);
     ab->flag = 0;
     fence_mbar_init();
   }
-  for (int s = 0; s < kStages; s++) zero_smem(s_x + s * kDSt + kXBytes + kPxBytes, kPxBytes);
+  for (int s = 0; s < ns; s++) zero_smem(s_x + s * kDSt + kXBytes + kPxBytes, kPxBytes);
   fence_proxy_async_smem();
   if (warp == 1) tmem_alloc(tmem_slot, 512);
   tc_fence_before();
@@ -176,9 +188,11 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   grid_trigger();
-  grid_wait(wimg, zimg, out, v, delta, wds, dS);
-  if (MODE == 2) {
-    for (int g = threadIdx.x; g < G; g += kThreads) s_ds[g] = dS[wk.bh * Gi + g0 + g];
+  // (The softmax warps' pointers take the zero through the row index r: seven opaque 64-bit
+  // pointers cost registers that the 512-thread launch does not have.)
+  const int after_wait = (int)grid_wait(wimg, zimg, zimg2, dS);
+  if (kDs) {
+    for (int g = threadIdx.x; g < G; g += blockDim.x) s_ds[g] = dS[wk.bh * Gi + g0 + g];
     __syncthreads();
   }
 
@@ -193,12 +207,24 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       mbar_expect_tx(wz_full, wbytes + zbytes);
       load_slots(s_w, wimg + (size_t)h * Gi * kWRow, Gi, g0, G, hilo, wz_full);
       const uint8_t* zi = zimg + (size_t)wk.bh * zstride + (size_t)g0 * 64;
-      load_images(s_z, zi, (uint32_t)G * 64, wz_full);
-      if (PS) load_images(s_z + (uint32_t)G * 64, zi + (size_t)Gi * 64, (uint32_t)G * 64, wz_full);
-      Ring<kStages> st;
+      if (MODE == 3) {
+        // per 64 slots z' then t2, 32 channel rows each; all hi halves, then all lo halves
+        const uint8_t* zi2 = zimg2 + (size_t)wk.bh * zstride + (size_t)g0 * 64;
+        for (int hl = 0; hl < 2; hl++)
+          for (int k = 0; k < G / 64; k++) {
+            uint8_t* dst = s_z + (size_t)hl * G * 128 + (size_t)k * 8192;
+            const size_t src = (size_t)hl * Gi * 64 + (size_t)k * 4096;
+            bulk_load(dst, zi + src, 4096, wz_full);
+            bulk_load(dst + 4096, zi2 + src, 4096, wz_full);
+          }
+      } else {
+        load_images(s_z, zi, (uint32_t)G * 64, wz_full);
+      }
+      if (PS && MODE != 3) load_images(s_z + (uint32_t)G * 64, zi + (size_t)Gi * 64, (uint32_t)G * 64, wz_full);
+      RingOf st(ns);
       int i = 0;
       for (; i < wk.ntiles; i++, st.next()) {
-        if (i >= kStages && !mbar_wait(&x_empty[st.i], st.pass ^ 1u, ab, status)) break;
+        if (i >= ns && !mbar_wait(&x_empty[st.i], st.pass ^ 1u, ab, status)) break;
         uint8_t* stage = s_x + st.i * kDSt;
         const int n0 = (int)((wk.tile0 + i) * kTile);
         mbar_expect_tx(&x_full[st.i], kXBytes + kPxBytes + (X3 ? kXBytes : 0u));
@@ -207,8 +233,8 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
         if (X3) tma_load_3d(stage + kDStage, &xrmap, h * kD, n0, (int)b, &x_full[st.i]);
       }
       // Drain: the newest load of each stage has landed before the CTA exits.
-      for (int j = (i > kStages ? i - kStages : 0); j < i; j++)
-        mbar_wait(&x_full[j % kStages], (uint32_t)((j / kStages) & 1), ab, nullptr, kWaitNs);
+      for (int j = (i > ns ? i - ns : 0); j < i; j++)
+        mbar_wait(&x_full[j % ns], (uint32_t)((j / ns) & 1), ab, nullptr, kWaitNs);
       mbar_wait(wz_full, 0, ab, nullptr, kWaitNs);
     }
   } else if (warp == 1) {
@@ -220,7 +246,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       const uint32_t wl0 = hilo ? w0 + (uint32_t)G * 6 : 0u, wl_step = hilo ? kGC * 4u : 0u;
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
       Ring<kSBuf> sb;
-      Ring<kStages> st;
+      RingOf st(ns);
       int q = 0;
       for (int i = 0; ok && i < wk.ntiles; i++, st.next()) {
         if (!(ok = mbar_wait_w(&x_full[st.i], st.pass, ab, status))) break;
@@ -242,7 +268,41 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       mma_commit_w(&drain[0]);
       mbar_wait_w(&drain[0], 0, ab, nullptr, kWaitNs);
     }
-  } else if (warp == 2 || warp == 3) {
+  } else if (MODE == 3 && warp == 3) {
+    // ------------------------------ P x [Z' | T2] issuer ------------------------------
+    if (wk.ntiles > 0) {
+      constexpr uint32_t idesc_pv = idesc_bf16(128, 2 * kD, false, false);
+      const uint32_t z0 = sdesc_lo(smem_u32(s_z), 16);
+      bool ok = mbar_wait_w(wz_full, 0, ab, status);
+      Ring<kSBuf> sb;
+      for (int i = 0; ok && i < wk.ntiles; i++) {
+        const int ob = i & 1;
+        const uint32_t tO = tmem + kO + (uint32_t)ob * 2 * kD;
+        if (i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
+        uint32_t z = z0;
+        for (int c = 0; ok && c < nch; c++, sb.next()) {
+#pragma unroll
+          for (int j = 0; j < 2; j++, z += 512) {
+            if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + j], sb.pass, ab, status))) break;
+            tc_fence_after();
+            const uint32_t tP = tmem + (uint32_t)sb.i * kGC + (uint32_t)j * 64;
+#pragma unroll
+            for (int kk = 0; kk < 4; kk++) {
+              const uint32_t hi = tP + da_col(kk), lo = hi + 16;
+              mma_ts_w<kHi128>(tO, hi, z + kk * 2, idesc_pv, (c > 0 || j > 0 || kk > 0) ? 1u : 0u);
+              mma_ts_w<kHi128>(tO, lo, z + kk * 2, idesc_pv, 1u);
+              mma_ts_w<kHi128>(tO, hi, z + (uint32_t)G * 8 + kk * 2, idesc_pv, 1u);
+            }
+          }
+          if (!ok) break;
+          mma_commit_w(&pv_done[sb.i]);
+        }
+        mma_commit_w(&o_full[i % kOFull]);
+      }
+      mma_commit_w(&drain[1]);
+      mbar_wait_w(&drain[1], 0, ab, nullptr, kWaitNs);
+    }
+  } else if (MODE != 3 && (warp == 2 || warp == 3)) {
     // ------------------------------ P x Z' issuers ------------------------------
     const int j = warp - 2;  // K-steps [4j, 4j + 4) of every block, accumulator O_j
     if (wk.ntiles > 0) {
@@ -259,14 +319,15 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
         for (int c = 0; c < nch; c++, z += 512, sb.next()) {
           if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + j], sb.pass, ab, status))) break;
           tc_fence_after();
-          // weights of slots 64j.. (packed pairs; PS: hi pairs, then lo pairs 32 on)
+          // weights of slots 64j.. (packed pairs; PS: at da_col(kk), lo pairs 16 on)
           const uint32_t tP = tmem + (uint32_t)sb.i * kGC + (uint32_t)j * (PS ? 64 : 32);
 #pragma unroll
           for (int kk = 0; kk < 4; kk++) {
-            mma_ts_w<kHi128>(tO, tP + (uint32_t)kk * 8, z + kk * 2, idesc_pv, (c > 0 || kk > 0) ? 1u : 0u);
+            const uint32_t tw = tP + (PS ? da_col(kk) : (uint32_t)kk * 8);
+            mma_ts_w<kHi128>(tO, tw, z + kk * 2, idesc_pv, (c > 0 || kk > 0) ? 1u : 0u);
             if (PS) {
-              mma_ts_w<kHi128>(tO, tP + 32 + (uint32_t)kk * 8, z + kk * 2, idesc_pv, 1u);
-              mma_ts_w<kHi128>(tO, tP + (uint32_t)kk * 8, z + (uint32_t)G * 4 + kk * 2, idesc_pv, 1u);
+              mma_ts_w<kHi128>(tO, tw + 16, z + kk * 2, idesc_pv, 1u);
+              mma_ts_w<kHi128>(tO, tw, z + (uint32_t)G * 4 + kk * 2, idesc_pv, 1u);
             }
           }
           mma_commit_w(&pv_done[sb.i]);
@@ -280,7 +341,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
     // ------------------------------ softmax warpgroups ------------------------------
     const int wg = (warp - kSoftmaxWarp0) >> 2;
     const int wq = warp & 3;  // TMEM sub-partition of this warp
-    const int r = wq * 32 + lane;
+    const int r = wq * 32 + lane + after_wait;
     const uint32_t lane_addr = (uint32_t)(wq * 32) << 16;
     bool ok = true;
     // Output of tile t: O_0 + O_1 (fixed order) -> bf16 -> global, 64 B per point.
@@ -347,13 +408,78 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       }
       return true;
     };
-    // MODE 2: this warpgroup's sum_g w dS_g for point r of its current tile.
+    // MODE 3: delta_n = v_n . R2_n + v2_n . R_n and dfx_n = R2_n (R of z', R2 of t2).
+    auto epilogue3 = [&](int t) -> bool {
+      const int ob = (int)(t & 1);
+      const int64_t n = (wk.tile0 + t) * kTile + r;
+      const int64_t row = ((b * N + n) * H + h) * kD;
+      uint4 va[4], vb[4];
+      if (n < N) {
+        const uint4* sa = reinterpret_cast<const uint4*>(v2 + row);
+        const uint4* sb = reinterpret_cast<const uint4*>(v + row);
+#pragma unroll
+        for (int k = 0; k < 4; k++) va[k] = sa[k], vb[k] = sb[k];
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; k++) va[k] = vb[k] = make_uint4(0u, 0u, 0u, 0u);
+      }
+      if (!mbar_wait(&o_full[t % kOFull], (uint32_t)((t / kOFull) & 1), ab, status)) return false;
+      tc_fence_after();
+      uint32_t o[32];
+      tmem_ld32(tmem + lane_addr + kO + (uint32_t)ob * 2 * kD, o);
+      tmem_wait_ld(o);
+      float da = 0.f, db = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const uint32_t w[4] = {va[k].x, va[k].y, va[k].z, va[k].w};
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          da = fmaf(__uint_as_float(w[e] << 16), __uint_as_float(o[8 * k + 2 * e]), da);
+          da = fmaf(__uint_as_float(w[e] & 0xFFFF0000u), __uint_as_float(o[8 * k + 2 * e + 1]), da);
+        }
+      }
+      tmem_ld32(tmem + lane_addr + kO + (uint32_t)ob * 2 * kD + kD, o);
+      tmem_wait_ld(o);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&o_free[ob]);
+      if (n < N) {
+        uint4* dst = reinterpret_cast<uint4*>(out + row);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+          const uint32_t wb[4] = {vb[k].x, vb[k].y, vb[k].z, vb[k].w};
+          uint4 p4 = make_uint4(0u, 0u, 0u, 0u);
+          if (accumulate) p4 = dst[k];
+          const uint32_t pw[4] = {p4.x, p4.y, p4.z, p4.w};
+          uint32_t w[4];
+#pragma unroll
+          for (int e = 0; e < 4; e++) {
+            const int c0 = 8 * k + 2 * e;
+            const float r0 = __uint_as_float(o[c0]), r1 = __uint_as_float(o[c0 + 1]);
+            w[e] = pack_bf16(r0 + __uint_as_float(pw[e] << 16), r1 + __uint_as_float(pw[e] & 0xFFFF0000u));
+            db = fmaf(__uint_as_float(wb[e] << 16), r0, db);
+            db = fmaf(__uint_as_float(wb[e] & 0xFFFF0000u), r1, db);
+          }
+          dst[k] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        delta[wk.bh * N + n] = accumulate ? delta[wk.bh * N + n] + (db + da) : db + da;
+      }
+      return true;
+    };
+    auto finish = [&](int t) -> bool {
+      if constexpr (MODE == 3)
+        return epilogue3(t);
+      else
+        return epilogue(t);
+    };
+    // kDs: this warpgroup's sum_g w dS_g for point r of its current tile.
     float wds_acc = 0.f;
     int wds_tile = -1;
     auto flush_wds = [&]() {
-      if (MODE == 2 && wds_tile >= 0) {
+      if (kDs && wds_tile >= 0) {
         const int64_t n = (wk.tile0 + wds_tile) * kTile + r;
-        if (n < N) wds[((int64_t)wg * gridDim.y + wk.bh) * N + n] += wds_acc;
+        float* p = wds + ((int64_t)wg * gridDim.y + wk.bh) * N + n;
+        if (n < N) *p = accumulate ? *p + wds_acc : wds_acc;
       }
       wds_acc = 0.f;
     };
@@ -366,17 +492,15 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       if (!(ok = mbar_wait(&s_full[bb], (uint32_t)((q / kSBuf) & 1), ab, status))) break;
       tc_fence_after();
       const uint32_t tS = tmem + lane_addr + (uint32_t)bb * kGC;
-      if (MODE == 2 && i != wds_tile) {
+      if (kDs && i != wds_tile) {
         flush_wds();
         wds_tile = i;
       }
 #pragma unroll
       for (int hf = 0; hf < 2; hf++) {
         const uint32_t tH = tS + (uint32_t)hf * 64;
-        if constexpr (MODE == 2 && PS)
+        if constexpr (kDs)
           weights_hilo_half_ds(tH, s_ds + c * kGC + hf * 64, wds_acc);
-        else if constexpr (MODE == 2)
-          weights_half_ds(tH, tS + (uint32_t)hf * 32, s_ds + c * kGC + hf * 64, wds_acc);
         else if constexpr (PS)
           weights_hilo_half(tH);
         else
@@ -388,9 +512,9 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       }
       // The output of the previous tile is drained by the warpgroup that took the first
       // block of this tile, when the last products of that tile have long finished.
-      if (c == 0 && i > 0 && !(ok = epilogue(i - 1))) break;
+      if (c == 0 && i > 0 && !(ok = finish(i - 1))) break;
     }
-    if (ok && total > 0 && total % kWGs == wg) epilogue(wk.ntiles - 1);
+    if (ok && total > 0 && total % kWGs == wg) finish(wk.ntiles - 1);
     if (ok) flush_wds();
   }
   tc_fence_before();
@@ -814,12 +938,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + (kk >> 2)], sb.pass, ab, status))) break;
             tc_fence_after();
           }
-          // 16 points' packed weights: columns kk * 8, or with split products the hi
-          // pairs of half kk / 4 at (kk / 4) * 64 + (kk % 4) * 8, their residuals 32 on
-          const uint32_t tw = tE + (split ? (uint32_t)(kk >> 2) * 64 + (uint32_t)(kk & 3) * 8 : (uint32_t)kk * 8);
+          // 16 points' packed weights: columns kk * 8, or with split products at da_col(kk)
+          const uint32_t tw = tE + (split ? da_col(kk) : (uint32_t)kk * 8);
           mma_ts_w<kHi32>(tacc, tw, f + kk * 32, idesc_sl, (!fresh || kk > 0) ? 1u : 0u);
           // The residual halves of the weights: U and S to ~2^-16.
-          if (split) mma_ts_w<kHi32>(tacc, tw + 32, f + kk * 32, idesc_sl, 1u);
+          if (split) mma_ts_w<kHi32>(tacc, tw + 16, f + kk * 32, idesc_sl, 1u);
           if (X3)  // the weights against fx's residual half (U only)
             mma_ts_w<kHi32>(tacc, tw, fr + kk * 32, idesc_bf16(128, 32, false, true), 1u);
         }
@@ -971,8 +1094,9 @@ X3Ranges x3_ranges(const Shape& s0) {
 size_t half_bytes(const Shape& s) { return align_up((size_t)s.B * s.N * s.H * s.d * 2, 256); }
 
 size_t smem_deslice(int G, bool hilo, int mode = 0, bool ps = false, bool x3 = false) {
-  return 1024 + (size_t)G * ((hilo ? kWRow : 96) + (ps ? 128 : 64)) + (mode == 2 ? align_up((size_t)G * 4, 1024) : 0) +
-         kStages * (kDStage + (x3 ? kXBytes : 0)) + 512;
+  return 1024 + (size_t)G * ((hilo ? kWRow : 96) + (mode == 3 ? 256 : ps ? 128 : 64)) +
+         (mode >= 2 ? align_up((size_t)G * 4, 1024) : 0) +
+         (mode == 3 ? 1 : kStages) * (kDStage + (x3 ? kXBytes : 0)) + 512;
 }
 // Shared memory of the statistics pass and, from what W' leaves, its x stages.
 size_t smem_stats(int G, bool split, bool x3, int nst) {
@@ -1159,36 +1283,40 @@ cudaError_t tc_deslice_fwd(const Shape& s0, const void* x, const float* W, const
   for (int k = 0; k < xr.n; k++) {
     const int g0 = k * xr.size;
     if ((e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kDesl3Threads), sm, st, xmap,
-                    pmap, xrmap, wimg, zimg, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr,
+                    pmap, xrmap, wimg, zimg, nullptr, static_cast<__nv_bfloat16*>(out), nullptr, nullptr, nullptr, nullptr, nullptr,
                     s.N, padded_n(s), s.H, s.G, g0, std::min(xr.size, s.G - g0), P, hilo ? 1 : 0,
-                    (uint32_t)s.G * (ps ? 128 : 64), k > 0 ? 1 : 0, status)) != cudaSuccess) return e;
+                    (uint32_t)s.G * (ps ? 128 : 64), kStages, k > 0 ? 1 : 0, status)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-size_t tc_rows_smem(const Shape& s, int mode, bool ps, bool hilo) { return smem_deslice(s.G, hilo, mode, ps); }
+size_t tc_rows_smem(const Shape& s) { return smem_deslice(s.G, false, 2, true); }
 
 cudaError_t tc_rows_bwd(const Shape& s, int Gi, int g0, int mode, const void* x, const uint8_t* wimg,
-                        const uint8_t* zimg, const void* px, const void* v, void* dfx, float* delta, float* wds,
-                        const float* dS, int accumulate, uint32_t* status, cudaStream_t st) {
-  const bool split = s.dot == FS_DOT_BF16X2;
-  const bool ps = split && smem_deslice(s.G, false, mode, true) <= kMaxSmem;
-  const bool hilo = split && smem_deslice(s.G, true, mode, ps) <= kMaxSmem;
-  const size_t sm = smem_deslice(s.G, hilo, mode, ps);
+                        const uint8_t* zimg, const uint8_t* zimg2, const void* px, const void* v, const void* v2,
+                        void* dfx, float* delta, float* wds, const float* dS, int accumulate, uint32_t* status,
+                        cudaStream_t st) {
+  const bool hilo = smem_deslice(s.G, true, mode, true) <= kMaxSmem;
+  size_t sm = smem_deslice(s.G, hilo, mode, true);
   if (sm > kMaxSmem) return cudaErrorInvalidValue;
+  int nst = kStages;
+  if (mode == 3) {
+    nst = std::min(kStages, 1 + (int)((kMaxSmem - sm) / kDStage));
+    sm += (size_t)(nst - 1) * kDStage;
+  }
   const int64_t Np = padded_n(s);
   CUtensorMap xmap, pmap;
   if (!make_point_map(&xmap, x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B)) return cudaErrorInvalidValue;
   if (!make_px_map(&pmap, px, s.BH(), Np)) return cudaErrorInvalidValue;
   const int P = point_splits(s, (int)s.BH());
   dim3 grid((unsigned)P, (unsigned)s.BH());
-  const auto kernel = mode == 1 ? (ps ? k_deslice<1, true> : k_deslice<1, false>)
-                                : (ps ? k_deslice<2, true> : k_deslice<2, false>);
+  const auto kernel = mode == 1 ? k_deslice<1, true> : mode == 2 ? k_deslice<2, true> : k_deslice<3, true>;
   cudaError_t e = set_smem(kernel, sm);
   if (e != cudaSuccess) return e;
-  return launch(kernel, grid, dim3(mode == 2 ? kThreads : kDesl3Threads), sm, st, xmap, pmap, xmap, wimg, zimg, static_cast<__nv_bfloat16*>(dfx),
-                static_cast<const __nv_bfloat16*>(v), delta, wds, dS, s.N, Np, s.H, Gi, g0, s.G, P, hilo ? 1 : 0,
-                (uint32_t)Gi * 128, accumulate, status);
+  return launch(kernel, grid, dim3(mode == 2 ? kThreads : kDesl3Threads), sm, st, xmap, pmap, xmap,
+                wimg, zimg, zimg2, static_cast<__nv_bfloat16*>(dfx), static_cast<const __nv_bfloat16*>(v),
+                static_cast<const __nv_bfloat16*>(v2), delta, wds, dS, s.N, Np, s.H, Gi, g0, s.G, P, hilo ? 1 : 0,
+                (uint32_t)Gi * 128, nst, accumulate, status);
 }
 
 }  // namespace fs

@@ -291,6 +291,20 @@ struct Ring {
   }
 };
 
+// Ring with a runtime number of buffers.
+struct RingOf {
+  const int n;
+  int i = 0;
+  uint32_t pass = 0;
+  __device__ __forceinline__ explicit RingOf(int n_) : n(n_) {}
+  __device__ __forceinline__ void next() {
+    if (++i == n) {
+      i = 0;
+      pass ^= 1u;
+    }
+  }
+};
+
 // Instruction descriptor for kind::f16 with bf16 A/B and fp32 D.
 //   a_mn / b_mn: operand is MN-major (else K-major).
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool b_mn) {
