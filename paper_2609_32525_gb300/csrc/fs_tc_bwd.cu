@@ -572,86 +572,62 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) mbar_arrive(&p_ready[2 * bb + hf]);
       }
     }
-    // Epilogue.  Warpgroup 1 hands its sums dt, db to warpgroup 0 through shared
-    // memory.  Flushed modes: each warpgroup adds what its accumulator holds since
-    // its last flush; warpgroup 1 passes its share through the partial row and
-    // warpgroup 0 adds the two in a fixed order (MODE 0: dZ; MODES 2, 3: dWx and the
-    // sums).  MODE 1: warpgroup 0 writes dWx (both accumulators) and the sums,
+    // Epilogue.  The block's partial rows are gathered in the stages' memory (every load has
+    // landed and been read) and leave as one bulk copy.  Warpgroup 1 hands its sums dt, db to
+    // warpgroup 0 the same way.  Flushed modes: each warpgroup adds what its accumulator holds
+    // since its last flush, and the two shares are added in a fixed order (MODE 0: dZ; MODES 2,
+    // 3: dWx and the sums).  MODE 1: warpgroup 0 writes dWx (both accumulators) and the sums,
     // warpgroup 1 dZ.
     const int64_t BH = gridDim.z;
-    const int PS = MODE == 1 ? 2 * kD + 2 : (MODE == 0 ? kD : kD + 2);
-    float* o = part + (((int64_t)blockIdx.y * BH + wk.bh) * G + g_base + r) * PS;
+    constexpr int PS = MODE == 1 ? 2 * kD + 2 : (MODE == 0 ? kD : kD + 2);
+    float* s_out = reinterpret_cast<float*>(s_st);
+    float* o = s_out + r * PS;
     const bool have = ok && wk.ntiles > 0 && mbar_wait(acc_full, 0, ab, status);
     if (have) tc_fence_after();
     if (kFl) {
       if (have) add_acc();
-      if (wg == 1) {
+    } else if (have) {  // MODE 1: the sum of a product's two accumulators
+      uint32_t a0[32], a1[32];
+      tmem_ld32(tmem + lane_addr + (wg == 0 ? kAccW : kAccZ), a0);
+      tmem_ld32(tmem + lane_addr + (wg == 0 ? kAccW : kAccZ) + 32, a1);
+      tmem_wait_ld2(a0, a1);
 #pragma unroll
-        for (int k = 0; k < kD; k++) o[k] = acc[k];
-        if (MODE != 0) {
-          s_red[r] = dt;
-          s_red[kGC + r] = db;
-        }
-      }
-      named_barrier(1, 256);
-      if (wg == 0) {
+      for (int k = 0; k < kD; k++) acc[k] = __uint_as_float(a0[k]) + __uint_as_float(a1[k]);
+    }
+    if (wg == 1) {
 #pragma unroll
-        for (int k = 0; k < kD; k++) o[k] = acc[k] + o[k];
-        if (MODE != 0) {
-          dt += s_red[r];
-          db += s_red[kGC + r];
-          o[kD] = db;
-          o[kD + 1] = 0.f;
-          s_red[2 * kGC + r] = dt;
-          named_barrier(2, 128);
-          if (r == 0) {
-            float sum = 0.f;
-            for (int k = 0; k < kGC; k++) sum += s_red[2 * kGC + k];
-            dt_part[wk.bh * ((int64_t)gridDim.x * gridDim.y) + (int64_t)blockIdx.y * gridDim.x + blockIdx.x] =
-                sum * kLn2;
-          }
-        }
-      }
-    } else {
-      if (wg == 1) {
+      for (int k = 0; k < kD; k++) o[k] = acc[k];
+      if (MODE != 0) {
         s_red[r] = dt;
         s_red[kGC + r] = db;
       }
-      named_barrier(1, 256);
-      if (wg == 0) {
+      fence_proxy_async_smem();
+    }
+    named_barrier(1, 256);
+    if (wg == 0) {
+#pragma unroll
+      for (int k = 0; k < kD; k++) {
+        if (kFl)
+          o[k] = acc[k] + o[k];
+        else
+          o[kD + k] = acc[k];
+      }
+      if (MODE != 0) {
         dt += s_red[r];
         db += s_red[kGC + r];
-        constexpr int off = kD;
-        if (have) {
-          uint32_t a0[32], a1[32];
-          tmem_ld32(tmem + lane_addr + kAccW, a0);
-          tmem_ld32(tmem + lane_addr + kAccW + 32, a1);
-          tmem_wait_ld2(a0, a1);
+        o[PS - 2] = db;
+        o[PS - 1] = 0.f;
 #pragma unroll
-          for (int k = 0; k < kD; k++) o[off + k] = __uint_as_float(a0[k]) + __uint_as_float(a1[k]);
-        } else {
-          for (int k = 0; k < kD; k++) o[off + k] = 0.f;
-        }
-        o[off + kD] = db;
-        o[off + kD + 1] = 0.f;
-        s_red[2 * kGC + r] = dt;
-        named_barrier(2, 128);
-        if (r == 0) {
-          float sum = 0.f;
-          for (int k = 0; k < kGC; k++) sum += s_red[2 * kGC + k];
-          dt_part[wk.bh * ((int64_t)gridDim.x * gridDim.y) + (int64_t)blockIdx.y * gridDim.x + blockIdx.x] = sum * kLn2;
-        }
-      } else {
-        if (have) {
-          uint32_t z0[32], z1[32];
-          tmem_ld32(tmem + lane_addr + kAccZ, z0);
-          tmem_ld32(tmem + lane_addr + kAccZ + 32, z1);
-          tmem_wait_ld2(z0, z1);
-#pragma unroll
-          for (int k = 0; k < kD; k++) o[k] = __uint_as_float(z0[k]) + __uint_as_float(z1[k]);
-        } else {
-          for (int k = 0; k < kD; k++) o[k] = 0.f;
-        }
+        for (int e = 16; e; e >>= 1) dt += __shfl_xor_sync(0xffffffffu, dt, e);
+        if (lane == 0) s_red[2 * kGC + wq] = dt;
+      }
+      fence_proxy_async_smem();
+      named_barrier(2, 128);
+      if (r == 0) {
+        if (MODE != 0)
+          dt_part[wk.bh * ((int64_t)gridDim.x * gridDim.y) + (int64_t)blockIdx.y * gridDim.x + blockIdx.x] =
+              ((s_red[2 * kGC] + s_red[2 * kGC + 1]) + (s_red[2 * kGC + 2] + s_red[2 * kGC + 3])) * kLn2;
+        bulk_store(part + (((int64_t)blockIdx.y * BH + wk.bh) * G + g_base) * PS, s_out, kGC * PS * 4);
       }
     }
   }
@@ -953,7 +929,7 @@ size_t smem_bwd_dx(int G, bool hilo, bool comb = false) {
 }
 
 int bwd_slot_blocks(const Shape& s) { return s.G / kGC; }
-int bwd_slot_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * bwd_slot_blocks(s))); }
+int bwd_slot_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * bwd_slot_blocks(s)), 2); }
 
 // Slot ranges.  The images of a call cover all of its slots; the rows and point passes, which
 // hold images in shared memory (a rows pass W' and t with their residuals, the point pass
@@ -1103,7 +1079,7 @@ struct BwdCall {
     if (sm > kMaxSmem) return cudaErrorInvalidValue;
     const auto kernel = k_bwd_dx_tc<true, kComb>;
     if (cudaError_t e = set_smem(kernel, sm)) return e;
-    const int P = point_splits(s, (int)s.BH());
+    const int P = point_splits(s, (int)s.BH(), r.size / 64);
     for (int k = 0; k < r.n; k++) {
       const int g0 = k * r.size;
       if (cudaError_t e = launch(kernel, dim3((unsigned)P, (unsigned)s.BH()), dim3(kDxThreads), sm, st, xmap, vmap, pmap,

@@ -490,19 +490,36 @@ size_t z_image_bytes(const Shape& s) { return (size_t)s.BH() * s.G * (s.dtype ==
 int64_t padded_n(const Shape& s) { return (s.N + kTile - 1) / kTile * kTile; }
 size_t px_bytes(const Shape& s) { return (size_t)s.BH() * padded_n(s) * 16; }
 
-// Point splits per work unit for one-CTA-per-SM kernels: the split count P that
-// minimises the makespan in units of one unit's work, ceil(units * P / SMs) / P
-// (whole waves of CTAs), smallest P on ties; at most one split per point tile.
-int point_splits(const Shape& s, int units) {
+// Point splits P per work unit for one-CTA-per-SM kernels: the P that minimises the makespan
+// waves * (tiles a split * blocks + kFixedBlocks), where a tile is `blocks` blocks of 0.35 to
+// 0.6 us and a CTA's start and end (set-up, images, first loads, last products, partial rows)
+// cost as much as kFixedBlocks.  Measured: statistics and deslice 2.6 and 2.9 us, slice 4.7 to
+// 6.  Counting whole waves alone takes P = 19 for most shapes, up to eight waves of short CTAs
+// (against P = 6 at B = 3, N = 20,011, G = 100: statistics 24.4 us against 19.2, slice 33.3
+// against 23.8, deslice 27.1 against 21.3, backward 235 against 184; slice against P = 7 at
+// B = 1, N = 262,144, G = 1024 374 against 355; the other way round statistics at B = 4,
+// N = 262,144, G = 256: 351 at P = 19, 362 at 9).  P is no larger than whole waves alone would
+// take it, and at most one split per point tile, which bounds the partials' workspace.
+constexpr int kFixedBlocks = 8;
+int point_splits(const Shape& s, int units, int blocks) {
   const int64_t tiles = (s.N + kTile - 1) / kTile;
   const int64_t sms = num_sms();
   if (units < 1) units = 1;
-  int64_t best = 1;
-  double best_t = 1e30;
+  auto waves = [&](int64_t p) { return (units * p + sms - 1) / sms; };
+  int64_t best = 1, best_w = 1;
+  double w_t = 1e30;
+  int64_t t_min = INT64_MAX;
   for (int64_t p = 1; p <= 2 * sms && p <= tiles; p++) {
-    const double t = (double)((units * p + sms - 1) / sms) / (double)p;
-    if (t < best_t - 1e-12) {
-      best_t = t;
+    const double t = (double)waves(p) / (double)p;
+    if (t < w_t - 1e-12) {
+      w_t = t;
+      best_w = p;
+    }
+  }
+  for (int64_t p = 1; p <= best_w; p++) {
+    const int64_t t = waves(p) * ((tiles + p - 1) / p * blocks + kFixedBlocks);
+    if (t < t_min) {
+      t_min = t;
       best = p;
     }
   }

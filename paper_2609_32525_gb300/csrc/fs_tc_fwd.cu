@@ -749,13 +749,13 @@ constexpr uint32_t kWBlock = 128 * kWRow;                               // one 1
 // gradient magnifies errors of the token gradients many times over (its sum over
 // (n, g) cancels to ~1e-5 of its terms' magnitude).  So each accumulator's chain is
 // restarted every kSliceFlush of its issuer's tiles, after its warpgroup has added
-// what it holds into fp32 registers (round to nearest).  Only with split products
-// and fp32 inputs: with single bf16 products the weights' own rounding (~3e-3
-// relative in the tokens) dwarfs the drift (~1e-4 at 55,000 points per CTA), and
-// the waits on each flushed chain cost the plain slice 4%.
-constexpr int kSliceFlush = 4;
-template <bool kOn>
-__device__ __forceinline__ bool slice_flush_at(int i) { return kOn && ((i >> 1) % kSliceFlush) == 0; }
+// what it holds into fp32 registers (round to nearest).  With single bf16 products the
+// weights' own rounding (~3e-3 relative in the tokens) dwarfs the drift (~1e-4 at 55,000
+// points per CTA), and the waits on a chain flushed every 4 tiles cost the plain slice 4%:
+// there a chain of 64 tiles (512 K steps) keeps the drift at the level of a short CTA's
+// however long the CTA's range is, at no measurable cost.
+template <bool split>
+__device__ __forceinline__ bool slice_flush_at(int i) { return ((i >> 1) % (split ? 4 : 64)) == 0; }
 
 // X3 (fp32 inputs): each stage also holds the residual tiles of x and fx (xrmap,
 // frmap); the logits add x_r W'_hi and the products add P_hi F_r (N = 32: U only).
@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t tacc = tmem + kA + (uint32_t)j * 48;
         // A chain restarts at this issuer's first tile and at every flush tile (its
         // warpgroup has moved the earlier tiles' sums to registers by then).
-        const bool fresh = i < 2 || slice_flush_at<split || X3>(i);
+        const bool fresh = i < 2 || slice_flush_at<split>(i);
 #pragma unroll
         for (int kk = 0; kk < 8; kk++) {
           if ((kk & 3) == 0) {  // a half's weights
@@ -948,7 +948,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         mma_commit_w(&pv_done[sb.i]);
         mma_commit_w(&st_empty[st.i]);
-        if (split || X3) mma_commit_w(&acc_done[j]);
+        mma_commit_w(&acc_done[j]);
         st.next(), st.next();
         sb.next(), sb.next();
       }
@@ -1007,7 +1007,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         else
           weights_half(tS + (uint32_t)hf * 64, tS + (uint32_t)hf * 32);
         tmem_wait_st();
-        if (hf == 0 && i >= 2 && slice_flush_at<split || X3>(i)) {
+        if (hf == 0 && i >= 2 && slice_flush_at<split>(i)) {
           // The products of this warpgroup's tiles up to i - 2 are complete (acc_done
           // cannot move past that phase before this warpgroup hands over tile i).
           if (!(ok = mbar_wait(&acc_done[wg], (uint32_t)(((i - 2) >> 1) & 1), ab, status))) break;
@@ -1020,46 +1020,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     const int64_t BH = gridDim.z;
-    float* o = part + (((int64_t)blockIdx.y * BH + wk.bh) * G + g_base + r) * (kD + 1);
     const bool have = ok && wk.ntiles > 0 && mbar_wait(acc_full, 0, ab, status);
-    if (split || X3) {
-      // Epilogue with flushes: what A_wg holds since the last flush, then the two
-      // warpgroups' shares added in a fixed order (warpgroup 1 passes its share
-      // through the partial row).
-      if (have && wg < wk.ntiles) {
-        tc_fence_after();
-        add_acc();
-      }
-      if (wg == 1)
-        for (int k = 0; k <= kD; k++) o[k] = acc[k];
-      named_barrier(1, 256);
-      if (wg == 0)
-        for (int k = 0; k <= kD; k++) o[k] = acc[k] + o[k];
-    } else if (have) {
-      // Without flushes: warpgroup 0 writes the numerators U (A_0 + A_1), warpgroup 1
-      // the weight sums S.
+    // What the accumulators hold since the last flush, then the two warpgroups' shares added
+    // in a fixed order.  The 128 rows of the partials are contiguous: gathered in the stages'
+    // memory (every load has landed and been read) they leave as one bulk copy.  (Stored by
+    // their threads, 132 bytes apart, and the shares added through global memory, split slice
+    // call at N = 32,768, H = 8, G = 64: 27.3 us against 21.)
+    if (have && wg < wk.ntiles) {
       tc_fence_after();
-      const bool two = wk.ntiles >= 2;  // A_1 holds tiles only when there are two (else unwritten)
-      if (wg == 0) {
-        uint32_t u0[32], u1[32];
-        tmem_ld32(tmem + lane_addr + kA, u0);
-        tmem_ld32(tmem + lane_addr + kA + 48, u1);
-        tmem_wait_ld2(u0, u1);
-#pragma unroll
-        for (int k = 0; k < kD; k++) o[k] = two ? __uint_as_float(u0[k]) + __uint_as_float(u1[k]) : __uint_as_float(u0[k]);
-      } else {
-        uint32_t s0[16], s1[16];
-        tmem_ld16(tmem + lane_addr + kA + 32, s0);
-        tmem_ld16(tmem + lane_addr + kA + 48 + 32, s1);
-        tmem_wait_ld(s0);
-        tmem_wait_ld(s1);
-        o[kD] = two ? __uint_as_float(s0[0]) + __uint_as_float(s1[0]) : __uint_as_float(s0[0]);
-      }
-    } else if (ok && wk.ntiles == 0) {
-      if (wg == 0)
-        for (int k = 0; k < kD; k++) o[k] = 0.f;
-      else
-        o[kD] = 0.f;
+      add_acc();
+    }
+    float* s_out = reinterpret_cast<float*>(s_st);
+    float* row = s_out + r * (kD + 1);
+    if (wg == 1)
+      for (int k = 0; k <= kD; k++) row[k] = acc[k];
+    named_barrier(1, 256);
+    if (wg == 0) {
+      for (int k = 0; k <= kD; k++) row[k] = acc[k] + row[k];
+      fence_proxy_async_smem();
+      named_barrier(2, 128);
+      if (r == 0)
+        bulk_store(part + (((int64_t)blockIdx.y * BH + wk.bh) * G + g_base) * (kD + 1), s_out, kGC * (kD + 1) * 4);
     }
   }
   tc_fence_before();
@@ -1070,7 +1051,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // One slice CTA per (point split, batch-head, 128-slot block).
 int slice_blocks(const Shape& s) { return s.G / kGC < 1 ? 1 : s.G / kGC; }
-int slice_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * slice_blocks(s))); }
+int slice_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * slice_blocks(s)), 1); }
 
 // fp32 point tensors take the tensor-core path with every operand as two bf16 halves
 // (x, fx and W', the weights, z'): the X3 kernels.  Their inputs are first split
@@ -1115,7 +1096,7 @@ cudaError_t run_stats(const Shape& s, const void* x, const void* xr, const uint8
   CUtensorMap xmap, xrmap;
   if (!make_point_map(&xmap, x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B)) return cudaErrorInvalidValue;
   if (!make_point_map(&xrmap, xr ? xr : x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B)) return cudaErrorInvalidValue;
-  const int P = point_splits(s, (int)s.BH());
+  const int P = point_splits(s, (int)s.BH(), s.G / kGC);
   const bool x3 = xr != nullptr;
   const bool split = s.dot == FS_DOT_BF16X2 || x3;
   int nst = kStatsMaxStages;
@@ -1272,7 +1253,7 @@ cudaError_t tc_deslice_fwd(const Shape& s0, const void* x, const float* W, const
   if (!make_point_map(&xrmap, x3 ? xh + half_bytes(s) : x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B))
     return cudaErrorInvalidValue;
   if (!make_px_map(&pmap, px, s.BH(), padded_n(s))) return cudaErrorInvalidValue;
-  const int P = point_splits(s, (int)s.BH());
+  const int P = point_splits(s, (int)s.BH(), s.G / kGC);
   const bool split = s.dot == FS_DOT_BF16X2 || x3;
   const bool ps = x3;
   const bool hilo = split && smem_deslice(xr.size, true, 0, ps, x3) <= kMaxSmem;  // up to G = 768 (bf16)
@@ -1308,7 +1289,7 @@ cudaError_t tc_rows_bwd(const Shape& s, int Gi, int g0, int mode, const void* x,
   CUtensorMap xmap, pmap;
   if (!make_point_map(&xmap, x, s, kD, CU_TENSOR_MAP_SWIZZLE_64B)) return cudaErrorInvalidValue;
   if (!make_px_map(&pmap, px, s.BH(), Np)) return cudaErrorInvalidValue;
-  const int P = point_splits(s, (int)s.BH());
+  const int P = point_splits(s, (int)s.BH(), s.G / 64);
   dim3 grid((unsigned)P, (unsigned)s.BH());
   const auto kernel = mode == 1 ? k_deslice<1, true> : mode == 2 ? k_deslice<2, true> : k_deslice<3, true>;
   cudaError_t e = set_smem(kernel, sm);

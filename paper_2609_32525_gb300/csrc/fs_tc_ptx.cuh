@@ -117,6 +117,16 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
+// Plain bulk copy shared -> global by one thread, complete on return (16-byte aligned, size a
+// multiple of 16; the writes to shared memory fenced to the async proxy and ordered before).
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+  asm volatile(
+      "cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n"
+      "cp.async.bulk.commit_group;\n"
+      "cp.async.bulk.wait_group 0;" ::"l"(dst),
+      "r"(smem_u32(src)), "r"(bytes)
+      : "memory");
+}
 
 // ---- TMEM -------------------------------------------------------------------------------
 // Allocation is warp-collective; the base address is written to *slot (shared).
