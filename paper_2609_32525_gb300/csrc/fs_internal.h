@@ -64,7 +64,7 @@ cudaError_t simt_deslice_bwd(const Shape& s, int P, const void* x, const float* 
                              const float* lse, const void* dout, float* dzp, void* dx,
                              float* dW, float* db, float* dtau, int accumulate, float* delta,
                              float* part, float* dt_part, bool reset, uint32_t* status, cudaStream_t st);
-// dUS[bh][g] = (dz_g / (S_g + eps), -(dz_g . z_g) / (S_g + eps)) (d + 1 floats per slot).
+// dUS: dU = dz_g / (S_g + eps) [bh][g][d], then dS = -(dz_g . z_g) / (S_g + eps) [bh][g].
 cudaError_t simt_slice_bwd_prep(const Shape& s, const float* z, const float* wsum, const float* dz, float* dUS,
                                 cudaStream_t st);
 // Fixed-order reduction of slot-owned backward partials part[P][B*H][Gs][PS]

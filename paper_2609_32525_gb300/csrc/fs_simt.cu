@@ -339,9 +339,10 @@ __global__ void __launch_bounds__(256) k_mix_bwd(const float* __restrict__ M, co
   dM_tile(sm, z, dzp, dM, B, H, G, D, (int)(i % nt), (int)((i / nt) % nt), (int)(i / ((int64_t)nt * nt)));
 }
 
-// Token-gradient prep for the slice backward: dUS[bh][g] = (dz_g/(S_g+eps),
-// -(dz_g.z_g)/(S_g+eps)).  A warp per slot row (a thread per row read 32-word rows word by
-// word: 20 us at 2,048 rows, 5 us this way).
+// Token-gradient prep for the slice backward: dU = dz_g/(S_g+eps) as rows [bh][g][D], then
+// dS = -(dz_g.z_g)/(S_g+eps) as [bh][g], so that both read in 16-byte pieces.  A warp
+// per slot row (a thread per row read 32-word rows word by word: 20 us at 2,048 rows, 5 us
+// this way).
 __global__ void __launch_bounds__(256) k_slice_bwd_prep(const float* __restrict__ z, const float* __restrict__ wsum,
                                                         const float* __restrict__ dz, float* __restrict__ dUS,
                                                         int64_t BHG, int D, float eps) {
@@ -353,12 +354,12 @@ __global__ void __launch_bounds__(256) k_slice_bwd_prep(const float* __restrict_
   float s = 0.f;
   for (int c = lane; c < D; c += 32) {
     const float g = dz[i * D + c];
-    dUS[i * (D + 1) + c] = g / den;
+    dUS[i * D + c] = g / den;
     s = fmaf(g, z[i * D + c], s);
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) dUS[i * (D + 1) + D] = -s / den;
+  if (lane == 0) dUS[BHG * D + i] = -s / den;
 }
 
 // Fixed-order reduction of slot-owned backward partials over (b, p), one thread

@@ -13,9 +13,9 @@
 // side with more loads goes over lane >> 2 and the other over lane & 3.
 //
 // Measured (B = 2, N = 65,536, H = 8, d = 32, G = 256, fp32, against the thread-per-point and
-// thread-per-slot kernels): statistics 0.82 -> 0.47 ms, d z' 1.50 -> 1.17, delta and dx
-// 5.50 -> 3.29, dW 3.97 -> 1.99; at d = 64 (N = 16,384, H = 4, G = 64, bf16), where a point's
-// rows do not fit a thread's registers, delta and dx 3.85 -> 0.147 ms.
+// thread-per-slot kernels): statistics 0.82 -> 0.41 ms, d z' 1.50 -> 0.98, delta and dx
+// 5.50 -> 2.90, dW 3.97 -> 1.69; at d = 64 (N = 16,384, H = 4, G = 64, bf16), where a point's
+// rows do not fit a thread's registers, delta and dx 3.85 -> 0.15 ms.
 //
 // One layout serves all products of a tile, with rows padded by four floats:
 //   points  [d][128 + 4]  x, dO, fx transposed (channel-major)
@@ -64,11 +64,9 @@ struct Tile {
   static constexpr int kPtRows = kWarps / kPtCols;
   static constexpr int kPtM = TP / (8 * kPtRows);
   static constexpr int kPtN = 4;
-  // slot_products: warps over slots (32 each) x channels
-  static constexpr int kSlRows = TG / 32;
-  static constexpr int kSlCols = kWarps / kSlRows;
-  static constexpr int kSlM = 4;
-  static constexpr int kSlN = D / (4 * kSlCols);
+  // slot_products: warps over two halves of the points x channels
+  static constexpr int kSlM = TG / 8;
+  static constexpr int kSlN = D / (2 * kWarps);
   static_assert((kPairN == 4 || kPairN == 8) && (kPtM == 4 || kPtM == 8) && kSlN >= 1, "register tiles");
 
   static constexpr size_t kPointTile = (size_t)D * LP;
@@ -89,80 +87,121 @@ __device__ __forceinline__ void write_status(bool reset, const float* tau, int H
 }
 
 // ---- staging ---------------------------------------------------------------------------------
+// A tile's operands go from memory through registers to shared memory: load() issues all of a
+// thread's reads at once, store() lays them out.  The passes load the next tile before the
+// second product of the current one (whose register tile is small), so the reads run under it;
+// the backward's slot pass, whose three point tiles would spill there, loads them before the
+// barrier that ends the previous tile.  Staged four reads of a loop at a time, the FMA pipe was
+// 44 to 50% busy (B = 2, N = 65,536, H = 8, d = 32, G = 256, fp32: whole backward with
+// statistics 6944 us, 6047 with this and slot_products over halves of the points; the point
+// pass 3292 -> 2900, its FMA pipe 55% busy).
 
-// Points [n0, n0 + TP) of head h, channel-major; rows past n_end are zero.
-template <int D, int NT>
-__device__ __forceinline__ void stage_points(float* dst, const float* src, int64_t b, int h, int64_t n0,
-                                             int64_t n_end, int64_t N, int H) {
-#pragma unroll 4
-  for (int i = threadIdx.x; i < TP * (D / 4); i += NT) {
-    const int p = i % TP, c = i / TP * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (n0 + p < n_end) v = *reinterpret_cast<const float4*>(src + ((b * N + n0 + p) * H + h) * D + c);
-    dst[c * LP + p] = v.x;
-    dst[(c + 1) * LP + p] = v.y;
-    dst[(c + 2) * LP + p] = v.z;
-    dst[(c + 3) * LP + p] = v.w;
-  }
-}
-template <int D, int NT>
-__device__ __forceinline__ void stage_points(float* dst, const __nv_bfloat16* src, int64_t b, int h, int64_t n0,
-                                             int64_t n_end, int64_t N, int H) {
-#pragma unroll 2
-  for (int i = threadIdx.x; i < TP * (D / 8); i += NT) {
-    const int p = i % TP, c = i / TP * 8;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (n0 + p < n_end) v = *reinterpret_cast<const uint4*>(src + ((b * N + n0 + p) * H + h) * D + c);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+// Points [n0, n0 + TP) of head h, to channel-major; rows past N are zero.
+template <int D, int NT, typename T>
+struct PointRows {
+  static constexpr int kV = 16 / sizeof(T), kN = TP * D / (kV * NT);
+  uint4 v[kN];
+  __device__ __forceinline__ void load(const T* src, int64_t b, int h, int64_t n0, int64_t N, int H) {
+    const int64_t n = n0 + threadIdx.x % TP;
+    const T* row = src + ((b * N + n) * H + h) * D + threadIdx.x / TP * kV;
 #pragma unroll
-    for (int e = 0; e < 4; e++) {
-      dst[(c + 2 * e) * LP + p] = __uint_as_float(w[e] << 16);
-      dst[(c + 2 * e + 1) * LP + p] = __uint_as_float(w[e] & 0xffff0000u);
+    for (int i = 0; i < kN; i++)
+      v[i] = n < N ? *reinterpret_cast<const uint4*>(row + i * (NT / TP) * kV) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  __device__ __forceinline__ void store(float* dst) const {
+    dst += threadIdx.x / TP * kV * LP + threadIdx.x % TP;
+#pragma unroll
+    for (int i = 0; i < kN; i++) {
+      const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+      float* d = dst + i * (NT / TP) * kV * LP;
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        if (sizeof(T) == 4) {
+          d[e * LP] = __uint_as_float(w[e]);
+        } else {
+          d[2 * e * LP] = __uint_as_float(w[e] << 16);
+          d[(2 * e + 1) * LP] = __uint_as_float(w[e] & 0xffff0000u);
+        }
+      }
     }
   }
-}
-// Slots [g0, g0 + TG) of W[h] (scaled) and the scaled bias.
+};
+// Slots [g0, g0 + TG) of W[h] and the bias, scaled on their way to shared memory.  Rows of W
+// are G floats: read by fours where G is a multiple of four, else by ones.
 template <int D, int TG, int NT>
-__device__ __forceinline__ void stage_w(float* dst, float* sB, const float* W, const float* bias, int h, int G,
-                                        int g0, float scale) {
-#pragma unroll 4
-  for (int i = threadIdx.x; i < TG * D; i += NT) {
-    const int g = i % TG, k = i / TG;
-    dst[k * (TG + 4) + g] = (g0 + g < G) ? W[((int64_t)h * D + k) * G + g0 + g] * scale : 0.f;
+struct SlotW {
+  static constexpr int kN = TG * D / NT;
+  static_assert(kN % 4 == 0 && TG <= NT, "whole pieces");
+  float v[kN], bias;
+  __device__ __forceinline__ void load(const float* W, const float* bs, int h, int G, int g0) {
+    W += (int64_t)h * D * G + g0;
+    if (G % 4 == 0) {
+#pragma unroll
+      for (int i = 0; i < kN / 4; i++) {
+        const int t = threadIdx.x + i * NT, g = t % (TG / 4) * 4, k = t / (TG / 4);
+        const float4 f = g0 + g < G ? *reinterpret_cast<const float4*>(W + (int64_t)k * G + g)
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[4 * i] = f.x, v[4 * i + 1] = f.y, v[4 * i + 2] = f.z, v[4 * i + 3] = f.w;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < kN; i++) {
+        const int t = threadIdx.x + i * NT, g = t % TG, k = t / TG;
+        v[i] = g0 + g < G ? W[(int64_t)k * G + g] : 0.f;
+      }
+    }
+    const int g = g0 + (int)threadIdx.x;
+    bias = (int)threadIdx.x < TG && g < G ? bs[(int64_t)h * G + g] : 0.f;
   }
-  for (int i = threadIdx.x; i < TG; i += NT) sB[i] = (g0 + i < G) ? bias[(int64_t)h * G + g0 + i] * scale : -kFar;
-}
-// Token rows [g0, g0 + TG) of t [G][D], channel-major.
+  __device__ __forceinline__ void store(float* dst, float* sB, int G, int g0, float scale) const {
+    if (G % 4 == 0) {
+#pragma unroll
+      for (int i = 0; i < kN / 4; i++) {
+        const int t = threadIdx.x + i * NT, g = t % (TG / 4) * 4, k = t / (TG / 4);
+        *reinterpret_cast<float4*>(dst + k * (TG + 4) + g) =
+            make_float4(v[4 * i] * scale, v[4 * i + 1] * scale, v[4 * i + 2] * scale, v[4 * i + 3] * scale);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < kN; i++) {
+        const int t = threadIdx.x + i * NT;
+        dst[t / TG * (TG + 4) + t % TG] = v[i] * scale;
+      }
+    }
+    if (threadIdx.x < TG) sB[threadIdx.x] = g0 + (int)threadIdx.x < G ? bias * scale : -kFar;
+  }
+};
+// Token rows [g0, g0 + TG) of t [G][D], to channel-major.
 template <int D, int TG, int NT>
-__device__ __forceinline__ void stage_tokens(float* dst, const float* t, int G, int g0) {
-#pragma unroll 4
-  for (int i = threadIdx.x; i < TG * (D / 4); i += NT) {
-    const int g = i % TG, c = i / TG * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (g0 + g < G) v = *reinterpret_cast<const float4*>(t + (int64_t)(g0 + g) * D + c);
-    dst[c * (TG + 4) + g] = v.x;
-    dst[(c + 1) * (TG + 4) + g] = v.y;
-    dst[(c + 2) * (TG + 4) + g] = v.z;
-    dst[(c + 3) * (TG + 4) + g] = v.w;
+struct TokenRows {
+  static constexpr int kN = TG * D / (4 * NT);
+  static_assert(kN >= 1, "whole pieces");
+  float4 v[kN];
+  __device__ __forceinline__ void load(const float* t, int G, int g0) {
+#pragma unroll
+    for (int i = 0; i < kN; i++) {
+      const int e = threadIdx.x + i * NT, g = e % TG, c = e / TG * 4;
+      v[i] = g0 + g < G ? *reinterpret_cast<const float4*>(t + (int64_t)(g0 + g) * D + c)
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
-}
-// Rows [g0, g0 + TG) of dU | dS [G][D + 1]: dU channel-major, dS to its vector.
-template <int D, int TG, int NT>
-__device__ __forceinline__ void stage_dus(float* dst, float* sS, const float* t, int G, int g0) {
-#pragma unroll 4
-  for (int i = threadIdx.x; i < TG * (D + 1); i += NT) {
-    const int g = i / (D + 1), k = i % (D + 1);
-    const float v = (g0 + g < G) ? t[(int64_t)(g0 + g) * (D + 1) + k] : 0.f;
-    if (k < D)
-      dst[k * (TG + 4) + g] = v;
-    else
-      sS[g] = v;
+  __device__ __forceinline__ void store(float* dst) const {
+#pragma unroll
+    for (int i = 0; i < kN; i++) {
+      const int e = threadIdx.x + i * NT, g = e % TG, c = e / TG * 4;
+      dst[c * (TG + 4) + g] = v[i].x;
+      dst[(c + 1) * (TG + 4) + g] = v[i].y;
+      dst[(c + 2) * (TG + 4) + g] = v[i].z;
+      dst[(c + 3) * (TG + 4) + g] = v[i].w;
+    }
   }
+};
+// One value per point (lse, delta) or slot (dS), by the first threads.
+__device__ __forceinline__ float load_one(const float* src, int64_t i, int64_t n, int count) {
+  return (int)threadIdx.x < count && i + threadIdx.x < n ? src[i + threadIdx.x] : 0.f;
 }
-template <int NT>
-__device__ __forceinline__ void stage_lse2(float* dst, const float* lse, int64_t bh, int64_t n0, int64_t n_end,
-                                           int64_t N) {
-  for (int i = threadIdx.x; i < TP; i += NT) dst[i] = (n0 + i < n_end) ? lse[bh * N + n0 + i] * kLog2e : kFar;
+__device__ __forceinline__ void store_lse2(float* dst, float lse, int64_t n0, int64_t N) {
+  if (threadIdx.x < TP) dst[threadIdx.x] = n0 + threadIdx.x < N ? lse * kLog2e : kFar;
 }
 
 // ---- products --------------------------------------------------------------------------------
@@ -210,11 +249,13 @@ __device__ __forceinline__ void point_products(float (&acc)[M][N], const float* 
     }
   }
 }
-// Slots 32 wr + m + 8 i, channels wc 4 N + n + 4 j.
+// Slots m + 8 i, channels wc 4 N + n + 4 j, over the warp's half of the points.  (With the warps
+// over slots instead, 4 x 4 outputs a thread, the reads took 1.6 clocks per clock of FMAs
+// against 1.1.)
 template <int M, int N>
 __device__ __forceinline__ void slot_products(float (&acc)[M][N], const float* wts, const float* pts) {
 #pragma unroll 2
-  for (int p = 0; p < TP; p += 4) {
+  for (int p = 0; p < TP / 2; p += 4) {
     float a[M][4], b[N][4];
 #pragma unroll
     for (int i = 0; i < M; i++) ld4(a[i], wts + 8 * i * LP + p);
@@ -236,7 +277,7 @@ struct Place {
   int m, n;
   int p1, g1, c1;  // pair_products: first point and slot; its warp column
   int p2, c2, w2;  // point_products: first point and channel; its warp column
-  int g3, c3;      // slot_products: first slot and channel
+  int p3, c3;      // slot_products: first point and channel (first slot: m)
   __device__ __forceinline__ Place() {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     m = lane >> 2, n = lane & 3;
@@ -246,8 +287,8 @@ struct Place {
     w2 = warp / C::kPtRows;
     p2 = (warp % C::kPtRows) * 8 * C::kPtM + 4 * m;
     c2 = w2 * 16 + n;
-    g3 = (warp % C::kSlRows) * 32 + m;
-    c3 = (warp / C::kSlRows) * 4 * C::kSlN + n;
+    p3 = (warp & 1) * (TP / 2);
+    c3 = (warp >> 1) * 4 * C::kSlN + n;
   }
   // point i (of 8) and slot j (of kPairN) of the thread, counted in the tile
   __device__ __forceinline__ int point(int i) const { return p1 + (i >> 2) * 32 + (i & 3); }
@@ -263,6 +304,26 @@ __device__ __forceinline__ void store_weights(float* wts, const Place<D, TG>& pl
     *reinterpret_cast<float4*>(row) = make_float4(w[0][j], w[1][j], w[2][j], w[3][j]);
     *reinterpret_cast<float4*>(row + 32) = make_float4(w[4][j], w[5][j], w[6][j], w[7][j]);
   }
+}
+
+// The two halves' slot_products, the second added to the first through `stage` (free for the
+// block, TG D floats); the threads of the first half (p3 = 0) hold the sum.
+template <int D, int TG>
+__device__ __forceinline__ void add_halves(float (&acc)[Tile<D, TG>::kSlM][Tile<D, TG>::kSlN], float* stage,
+                                           const Place<D, TG>& pl) {
+  using C = Tile<D, TG>;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < C::kSlM; i++)
+#pragma unroll
+    for (int j = 0; j < C::kSlN; j++)
+      if (pl.p3 != 0) stage[(pl.m + 8 * i) * D + pl.c3 + 4 * j] = acc[i][j];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < C::kSlM; i++)
+#pragma unroll
+    for (int j = 0; j < C::kSlN; j++)
+      if (pl.p3 == 0) acc[i][j] += stage[(pl.m + 8 * i) * D + pl.c3 + 4 * j];
 }
 
 // Sum over the four lanes of a run (lane & 3), in a fixed order; every lane gets it.
@@ -324,7 +385,7 @@ constexpr int resident(int blocks) { return D == 64 ? 1 : blocks; }
 
 // ---- statistics --------------------------------------------------------------------------------
 template <int D, int TG, typename T>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads)
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(3))
     k_tile_stats(const T* __restrict__ x, const float* __restrict__ W, const float* __restrict__ bias,
                  const float* __restrict__ tau, float* __restrict__ lse, int64_t N, int H, int G, int reset,
                  uint32_t* status) {
@@ -343,7 +404,11 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads)
   const float scale = kLog2e / tau[h];
   const int64_t n0 = (int64_t)blockIdx.x * TP;
   const Place<D, TG> pl;
-  stage_points<D, NT>(sx, x, b, h, n0, N, N, H);
+  PointRows<D, NT, T> xr;
+  SlotW<D, TG, NT> wr;
+  xr.load(x, b, h, n0, N, H);
+  wr.load(W, bias, h, G, 0);
+  xr.store(sx);
   // Running (max, sum) of the thread's slots; the maximum starts finite so that a thread
   // whose slots are all masked (-inf) stays free of NaN.
   float mx[8], l[8];
@@ -351,8 +416,9 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads)
   for (int i = 0; i < 8; i++) mx[i] = -kFar, l[i] = 0.f;
   for (int g0 = 0; g0 < G; g0 += TG) {
     __syncthreads();
-    stage_w<D, TG, NT>(sw, sB, W, bias, h, G, g0, scale);
+    wr.store(sw, sB, G, g0, scale);
     __syncthreads();
+    if (g0 + TG < G) wr.load(W, bias, h, G, g0 + TG);
     float a[8][NJ];
 #pragma unroll
     for (int j = 0; j < NJ; j++) {
@@ -440,7 +506,18 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   const int h = (int)(bh % H);
   if (!tau_ok(tau[h])) return;
   const Place<D, TG> pl;
-  stage_w<D, TG, NT>(sw, sB, W, bias, h, G, g0, kLog2e / tau[h]);
+  PointRows<D, NT, T> xr, fr;
+  float lr;
+  auto load = [&](int64_t t) {
+    xr.load(x, b, h, t * TP, N, H);
+    fr.load(f, b, h, t * TP, N, H);
+    lr = load_one(lse + bh * N, t * TP, N, TP);
+  };
+  {
+    SlotW<D, TG, NT> wr;
+    wr.load(W, bias, h, G, g0);
+    wr.store(sw, sB, G, g0, kLog2e / tau[h]);
+  }
   float U[C::kSlM][C::kSlN], S[NJ];
 #pragma unroll
   for (int i = 0; i < C::kSlM; i++)
@@ -448,12 +525,13 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     for (int j = 0; j < C::kSlN; j++) U[i][j] = 0.f;
 #pragma unroll
   for (int j = 0; j < NJ; j++) S[j] = 0.f;
-  const int64_t tiles = (N + TP - 1) / TP, t1 = tiles * (blockIdx.z + 1) / P;
-  for (int64_t t = tiles * blockIdx.z / P; t < t1; t++) {
+  const int64_t tiles = (N + TP - 1) / TP, t0 = tiles * blockIdx.z / P, t1 = tiles * (blockIdx.z + 1) / P;
+  if (t0 < t1) load(t0);
+  for (int64_t t = t0; t < t1; t++) {
     __syncthreads();
-    stage_points<D, NT>(sx, x, b, h, t * TP, N, N, H);
-    stage_points<D, NT>(sf, f, b, h, t * TP, N, N, H);
-    stage_lse2<NT>(sl, lse, bh, t * TP, N, N);
+    xr.store(sx);
+    fr.store(sf);
+    store_lse2(sl, lr, t * TP, N);
     __syncthreads();
     float w[8][NJ];
     log_weights<D, TG>(w, pl, sx, sw, sB, sl);
@@ -469,7 +547,8 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     }
     store_weights<D, TG>(wt, pl, w);
     __syncthreads();
-    slot_products<C::kSlM, C::kSlN>(U, wt + pl.g3 * LP, sf + pl.c3 * LP);
+    if (t + 1 < t1) load(t + 1);
+    slot_products<C::kSlM, C::kSlN>(U, wt + pl.m * LP + pl.p3, sf + pl.c3 * LP + pl.p3);
   }
   // S: the eight runs of a warp, then its two rows of warps.
 #pragma unroll
@@ -478,12 +557,12 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     for (int d = 4; d <= 16; d <<= 1) S[j] += __shfl_xor_sync(0xffffffffu, S[j], d);
     if (pl.m == 0) red[(threadIdx.x >> 5 & 1) * TG + pl.slot(j)] = S[j];
   }
-  __syncthreads();
+  add_halves<D, TG>(U, wt, pl);
   float* o = part + (((int64_t)blockIdx.z * gridDim.y + bh) * G + g0) * (D + 1);
 #pragma unroll
   for (int i = 0; i < C::kSlM; i++) {
-    const int g = pl.g3 + 8 * i;
-    if (g0 + g >= G) continue;
+    const int g = pl.m + 8 * i;
+    if (pl.p3 != 0 || g0 + g >= G) continue;
 #pragma unroll
     for (int j = 0; j < C::kSlN; j++) o[g * (D + 1) + pl.c3 + 4 * j] = U[i][j];
   }
@@ -514,8 +593,19 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   const float scale = kLog2e / tau[h];
   const int64_t n0 = (int64_t)blockIdx.x * TP;
   const Place<D, TG> pl;
-  stage_points<D, NT>(sx, x, b, h, n0, N, N, H);
-  stage_lse2<NT>(sl, lse, bh, n0, N, N);
+  SlotW<D, TG, NT> wr;
+  TokenRows<D, TG, NT> zr;
+  auto load = [&](int g0) {
+    wr.load(W, bias, h, G, g0);
+    zr.load(zp + bh * G * D, G, g0);
+  };
+  {
+    PointRows<D, NT, T> xr;
+    xr.load(x, b, h, n0, N, H);
+    load(0);
+    xr.store(sx);
+  }
+  store_lse2(sl, load_one(lse + bh * N, n0, N, TP), n0, N);
   float acc[C::kPtM][4];
 #pragma unroll
   for (int i = 0; i < C::kPtM; i++)
@@ -523,8 +613,8 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
   for (int g0 = 0; g0 < G; g0 += TG) {
     __syncthreads();
-    stage_w<D, TG, NT>(sw, sB, W, bias, h, G, g0, scale);
-    stage_tokens<D, TG, NT>(sz, zp + bh * G * D, G, g0);
+    wr.store(sw, sB, G, g0, scale);
+    zr.store(sz);
     __syncthreads();
     float w[8][NJ];
     log_weights<D, TG>(w, pl, sx, sw, sB, sl);
@@ -534,6 +624,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
       for (int j = 0; j < NJ; j++) w[i][j] = exp2f(w[i][j]);
     store_weights<D, TG>(wt, pl, w);
     __syncthreads();
+    if (g0 + TG < G) load(g0 + TG);
     point_products<TG>(acc, wt + pl.p2, sz + pl.c2 * C::LG);
   }
   write_rows<D, TG, T>(acc, 1.f, false, wt, pl, out, b, h, n0, N, H);
@@ -582,19 +673,36 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   const float scale = kLog2e / tau[h];
   const int64_t n0 = (int64_t)blockIdx.x * TP;
   const Place<D, TG> pl;
-  stage_points<D, NT>(sx, x, b, h, n0, N, N, H);
-  if (kD) stage_points<D, NT>(sd, dO, b, h, n0, N, N, H);
-  if (kS) stage_points<D, NT>(sf, fx, b, h, n0, N, N, H);
-  stage_lse2<NT>(sl, lse, bh, n0, N, N);
+  {
+    PointRows<D, NT, T> r;
+    r.load(x, b, h, n0, N, H);
+    r.store(sx);
+    if (kD) r.load(dO, b, h, n0, N, H), r.store(sd);
+    if (kS) r.load(fx, b, h, n0, N, H), r.store(sf);
+  }
+  store_lse2(sl, load_one(lse + bh * N, n0, N, TP), n0, N);
   const float* zb = kD ? zp + bh * G * D : nullptr;
-  const float* ub = kS ? dUS + bh * G * (D + 1) : nullptr;
+  const float* ub = kS ? dUS + bh * G * D : nullptr;
+  const float* sb = kS ? dUS + ((int64_t)gridDim.y * D + bh) * G : nullptr;
+  SlotW<D, TG, NT> wr;
+  TokenRows<D, TG, NT> zr, ur;
+  float sr;
+  auto load = [&](int g0) {
+    wr.load(W, bias, h, G, g0);
+    if (kD) zr.load(zb, G, g0);
+    if (kS) ur.load(ub, G, g0), sr = load_one(sb, g0, G, TG);
+  };
   auto stage = [&](int g0) {
     __syncthreads();
-    stage_w<D, TG, NT>(sw, sB, W, bias, h, G, g0, scale);
-    if (kD) stage_tokens<D, TG, NT>(sz, zb, G, g0);
-    if (kS) stage_dus<D, TG, NT>(su, sS, ub, G, g0);
+    wr.store(sw, sB, G, g0, scale);
+    if (kD) zr.store(sz);
+    if (kS) {
+      ur.store(su);
+      if (threadIdx.x < TG) sS[threadIdx.x] = sr;
+    }
     __syncthreads();
   };
+  load(0);
   // Sweep 1: R, dfx, sum_g w dS.
   {
     float R[M2][4], F[M2][4], ws[8];
@@ -619,6 +727,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
       }
       store_weights<D, TG>(wt, pl, w);
       __syncthreads();
+      load(g0 + TG < G ? g0 + TG : 0);  // (the second sweep's first tile at last)
       if (kD) point_products<TG>(R, wt + pl.p2, sz + pl.c2 * C::LG);
       if (kS) point_products<TG>(F, wt + pl.p2, su + pl.c2 * C::LG);
     }
@@ -693,6 +802,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     }
     store_weights<D, TG>(wt, pl, dw);
     __syncthreads();
+    if (g0 + TG < G) load(g0 + TG);
     point_products<TG>(acc, wt + pl.p2, sw + pl.c2 * C::LG);
   }
   // acc = sum_g da_g W[:,g] log2e/tau; dx = acc ln2.
@@ -740,9 +850,18 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   const int h = (int)(bh % H);
   if (!tau_ok(tau[h])) return;
   const Place<D, TG> pl;
-  stage_w<D, TG, NT>(sw, sB, W, bias, h, G, g0, kLog2e / tau[h]);
-  if (kD) stage_tokens<D, TG, NT>(sz, zp + bh * G * D, G, g0);
-  if (kS) stage_dus<D, TG, NT>(su, sS, dUS + bh * G * (D + 1), G, g0);
+  {
+    SlotW<D, TG, NT> wr;
+    TokenRows<D, TG, NT> tr;
+    wr.load(W, bias, h, G, g0);
+    wr.store(sw, sB, G, g0, kLog2e / tau[h]);
+    if (kD) tr.load(zp + bh * G * D, G, g0), tr.store(sz);
+    if (kS) {
+      tr.load(dUS + bh * G * D, G, g0), tr.store(su);
+      const float v = load_one(dUS + ((int64_t)gridDim.y * D + bh) * G, g0, G, TG);
+      if (threadIdx.x < TG) sS[threadIdx.x] = v;
+    }
+  }
   float dW[C::kSlM][C::kSlN], dZ[C::kSlM][C::kSlN], db[NJ];
 #pragma unroll
   for (int i = 0; i < C::kSlM; i++)
@@ -750,14 +869,19 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     for (int j = 0; j < C::kSlN; j++) dW[i][j] = 0.f, dZ[i][j] = 0.f;
 #pragma unroll
   for (int j = 0; j < NJ; j++) db[j] = 0.f;
-  const int64_t tiles = (N + TP - 1) / TP, t1 = tiles * (blockIdx.z + 1) / P;
-  for (int64_t t = tiles * blockIdx.z / P; t < t1; t++) {
+  const int64_t tiles = (N + TP - 1) / TP, t0 = tiles * blockIdx.z / P, t1 = tiles * (blockIdx.z + 1) / P;
+  for (int64_t t = t0; t < t1; t++) {
+    PointRows<D, NT, T> xr, dr, fr;
+    xr.load(x, b, h, t * TP, N, H);
+    if (kD) dr.load(dO, b, h, t * TP, N, H);
+    if (kS) fr.load(fx, b, h, t * TP, N, H);
+    const float lr = load_one(lse + bh * N, t * TP, N, TP), er = load_one(delta + bh * N, t * TP, N, TP);
     __syncthreads();
-    stage_points<D, NT>(sx, x, b, h, t * TP, N, N, H);
-    if (kD) stage_points<D, NT>(sd, dO, b, h, t * TP, N, N, H);
-    if (kS) stage_points<D, NT>(sf, fx, b, h, t * TP, N, N, H);
-    stage_lse2<NT>(sl, lse, bh, t * TP, N, N);
-    for (int i = threadIdx.x; i < TP; i += NT) sdl[i] = (t * TP + i < N) ? delta[bh * N + t * TP + i] : 0.f;
+    xr.store(sx);
+    if (kD) dr.store(sd);
+    if (kS) fr.store(sf);
+    store_lse2(sl, lr, t * TP, N);
+    if (threadIdx.x < TP) sdl[threadIdx.x] = er;
     __syncthreads();
     float a[8][NJ], dw[8][NJ];
     log_weights<D, TG>(a, pl, sx, sw, sB, sl);
@@ -787,12 +911,12 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     }
     store_weights<D, TG>(wt, pl, dw);
     __syncthreads();
-    slot_products<C::kSlM, C::kSlN>(dW, wt + pl.g3 * LP, sx + pl.c3 * LP);
+    slot_products<C::kSlM, C::kSlN>(dW, wt + pl.m * LP + pl.p3, sx + pl.c3 * LP + pl.p3);
     if (MODE == 0) {
       __syncthreads();
       store_weights<D, TG>(wt, pl, a);
       __syncthreads();
-      slot_products<C::kSlM, C::kSlN>(dZ, wt + pl.g3 * LP, sd + pl.c3 * LP);
+      slot_products<C::kSlM, C::kSlN>(dZ, wt + pl.m * LP + pl.p3, sd + pl.c3 * LP + pl.p3);
     }
   }
 #pragma unroll
@@ -801,12 +925,13 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     for (int d = 4; d <= 16; d <<= 1) db[j] += __shfl_xor_sync(0xffffffffu, db[j], d);
     if (pl.m == 0) red[(threadIdx.x >> 5 & 1) * TG + pl.slot(j)] = db[j];
   }
-  __syncthreads();
+  add_halves<D, TG>(dW, wt, pl);
+  if (MODE == 0) add_halves<D, TG>(dZ, wt, pl);
   float* o = part + (((int64_t)blockIdx.z * gridDim.y + bh) * G + g0) * PS;
 #pragma unroll
   for (int i = 0; i < C::kSlM; i++) {
-    const int g = pl.g3 + 8 * i;
-    if (g0 + g >= G) continue;
+    const int g = pl.m + 8 * i;
+    if (pl.p3 != 0 || g0 + g >= G) continue;
 #pragma unroll
     for (int j = 0; j < C::kSlN; j++) {
       if (MODE == 0) o[g * PS + pl.c3 + 4 * j] = dZ[i][j];
