@@ -21,12 +21,16 @@ int num_sms() {
 // its point tiles plus about half a tile (its slot tile, its partial rows), so P minimises
 // waves * (tiles per split + 1/2); the smallest such P within 1%.  P stays below two
 // splits per SM and 128-slot block, which bounds the partials' workspace.
+int slot_splits_most(const Shape& s) {
+  const int64_t blocks = s.BH() * ((s.G + 127) / 128);
+  return (int)std::max<int64_t>(1, std::min<int64_t>({(s.N + 63) / 64, (2LL * num_sms() + blocks - 1) / blocks, 1024}));
+}
 int slot_splits(const Shape& s) {
   const int64_t tg = simt_tile_slots(s);
-  const int64_t units = s.BH() * ((s.G + tg - 1) / tg), blocks = s.BH() * ((s.G + 127) / 128);
+  const int64_t units = s.BH() * ((s.G + tg - 1) / tg);
   const int64_t cap = (int64_t)num_sms() * (s.d == 64 ? 1 : 2);
   const int64_t tiles = (s.N + kSimtTP - 1) / kSimtTP;
-  const int64_t max_p = std::min<int64_t>({tiles, (2LL * num_sms() + blocks - 1) / blocks, 1024});
+  const int64_t max_p = std::min<int64_t>(tiles, slot_splits_most(s));
   int64_t best = 1;
   double best_t = 1e300;
   for (int64_t p = 1; p <= max_p; p++) {
@@ -103,7 +107,8 @@ Regions regions(const Shape& s, int op) {
   r.status = take(sizeof(uint32_t));
   switch (op) {
     case FS_OP_SLICE_FWD: {
-      size_t part = (size_t)P * BHG * (s.d + 1) * sizeof(float);
+      // (for the most splits, as the tensor-core partials)
+      size_t part = (size_t)slot_splits_most(s) * BHG * (s.d + 1) * sizeof(float);
       const size_t tcb = tc_slice_partials_bytes(s);
       if (tcb > part) part = tcb;
       r.partials = take(part);

@@ -501,25 +501,29 @@ size_t px_bytes(const Shape& s) { return (size_t)s.BH() * padded_n(s) * 16; }
 // N = 262,144, G = 256: 351 at P = 19, 362 at 9).  P is no larger than whole waves alone would
 // take it, and at most one split per point tile, which bounds the partials' workspace.
 constexpr int kFixedBlocks = 8;
-int point_splits(const Shape& s, int units, int blocks) {
-  const int64_t tiles = (s.N + kTile - 1) / kTile;
-  const int64_t sms = num_sms();
-  if (units < 1) units = 1;
-  auto waves = [&](int64_t p) { return (units * p + sms - 1) / sms; };
-  int64_t best = 1, best_w = 1;
-  double w_t = 1e30;
-  int64_t t_min = INT64_MAX;
+// The P of the fewest whole waves per split alone, smallest on ties.
+int wave_splits(const Shape& s, int units) {
+  const int64_t tiles = (s.N + kTile - 1) / kTile, sms = num_sms();
+  int64_t best = 1;
+  double best_t = 1e30;
   for (int64_t p = 1; p <= 2 * sms && p <= tiles; p++) {
-    const double t = (double)waves(p) / (double)p;
-    if (t < w_t - 1e-12) {
-      w_t = t;
-      best_w = p;
+    const double t = (double)((units * p + sms - 1) / sms) / (double)p;
+    if (t < best_t - 1e-12) {
+      best_t = t;
+      best = p;
     }
   }
-  for (int64_t p = 1; p <= best_w; p++) {
-    const int64_t t = waves(p) * ((tiles + p - 1) / p * blocks + kFixedBlocks);
-    if (t < t_min) {
-      t_min = t;
+  return (int)best;
+}
+int point_splits(const Shape& s, int units, int blocks) {
+  const int64_t tiles = (s.N + kTile - 1) / kTile, sms = num_sms();
+  if (units < 1) units = 1;
+  const int64_t most = wave_splits(s, units);
+  int64_t best = 1, best_t = INT64_MAX;
+  for (int64_t p = 1; p <= most; p++) {
+    const int64_t t = (units * p + sms - 1) / sms * ((tiles + p - 1) / p * blocks + kFixedBlocks);
+    if (t < best_t) {
+      best_t = t;
       best = p;
     }
   }

@@ -1136,7 +1136,9 @@ int tc_forward_launch_count(const Shape& s) {
 size_t tc_slice_partials_bytes(const Shape& s0) {
   if (!tc_forward_supported(s0)) return 0;
   const Shape s = tc_padded(s0);
-  return (size_t)slice_splits(s) * s.BH() * s.G * (kD + 1) * sizeof(float);
+  // (sized for the most splits that a size can take, so that a shape's scratch, and with it
+  // what fits a fixed one, does not hang on the choice of splits)
+  return (size_t)wave_splits(s, (int)(s.BH() * slice_blocks(s))) * s.BH() * s.G * (kD + 1) * sizeof(float);
 }
 // Layouts of the prepared operands: slice [W img | px | (X3) x hi, x r, fx hi, fx r];
 // deslice and statistics [W img | Z' img | px | (X3) x hi, x r].
