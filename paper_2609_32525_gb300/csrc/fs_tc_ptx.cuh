@@ -70,14 +70,17 @@ struct Abort {
 // each; after `limit_ns` of wall time it records FS timeout in *status, raises the
 // CTA abort flag and returns false.  Also returns false as soon as the abort flag
 // is up.
+// The wall time also runs while a kernel is preempted (a profiler that replays the kernel
+// launched after it, for seconds), so a wait has to have polled kMinPolls times as well.
+constexpr uint32_t kMinPolls = 2000;
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Abort* ab, uint32_t* status,
                                           uint64_t limit_ns = 2000000000ull) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = globaltimer();
-  for (;;) {
+  for (uint32_t polls = 0;; polls++) {
     if (mbar_try_wait_sleep(bar, parity, 20000u)) return true;
     if (ab->flag) return false;
-    if (globaltimer() - t0 > limit_ns) {
+    if (polls > kMinPolls && globaltimer() - t0 > limit_ns) {
       ab->flag = 1;
       if (status) atomicCAS(status, 0u, 4u /* FS_ERR_TIMEOUT */);
       return false;
