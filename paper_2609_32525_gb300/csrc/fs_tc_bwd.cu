@@ -929,7 +929,21 @@ size_t smem_bwd_dx(int G, bool hilo, bool comb = false) {
 }
 
 int bwd_slot_blocks(const Shape& s) { return s.G / kGC; }
-int bwd_slot_splits(const Shape& s) { return point_splits(s, (int)(s.BH() * bwd_slot_blocks(s)), 2); }
+// Point splits of the slot pass.  MODE 1 (fs_deslice_bwd) keeps dW and d z' in one accumulator
+// chain a half for a CTA's whole range, and a chain of tensor-core sums drifts towards zero with
+// its length, ~2^-26 relative per 16 points (d z' at B = 1, N = 262,144, H = 8, G = 1024 in 19
+// splits 1.3e-5 from 64 bits, in 7 splits 3.4e-5); so a range longer than kChainTiles, whose drift
+// of 5e-7 the other errors (3e-6) hide, takes more splits, up to those of whole waves.  (Whole
+// waves' splits for every range: separate backward calls at B = 2, N = 4,096, H = 8, G = 256 149
+// us against 132.)  The other modes flush their chains.
+constexpr int kChainTiles = 4;
+int bwd_slot_splits(const Shape& s, int mode) {
+  const int units = (int)(s.BH() * bwd_slot_blocks(s));
+  const int P = point_splits(s, units, 2);
+  if (mode != 1) return P;
+  const int64_t tiles = padded_n(s) / kTile;
+  return (int)std::min<int64_t>(wave_splits(s, units), std::max<int64_t>(P, (tiles + kChainTiles - 1) / kChainTiles));
+}
 
 // Slot ranges.  The images of a call cover all of its slots; the rows and point passes, which
 // hold images in shared memory (a rows pass W' and t with their residuals, the point pass
@@ -988,7 +1002,7 @@ BwdLayout bwd_layout(const Shape& s0, BwdKind kind) {
   const Shape s = pass_shape(s0);
   const size_t BHG = (size_t)s.BH() * s.G;
   const size_t pts = (size_t)s.BH() * s.N;
-  const int P = bwd_slot_splits(s), R = bwd_slot_blocks(s);
+  const int P = bwd_slot_splits(s, kind == kDesliceBwd ? 1 : 2), R = bwd_slot_blocks(s);
   const bool comb = kind == kCouplingBwd;
   L.wimg = take(w_image_bytes(s));
   L.wtimg = take((size_t)s.H * s.G * 128);
@@ -1057,14 +1071,14 @@ struct BwdCall {
     const size_t sm = smem_bwd_slot(MODE);
     const auto kernel = k_bwd_slot_tc<MODE, true>;
     if (cudaError_t e = set_smem(kernel, sm)) return e;
-    const int P = bwd_slot_splits(s);
+    const int P = bwd_slot_splits(s, MODE);
     return launch(kernel, dim3((unsigned)bwd_slot_blocks(s), (unsigned)P, (unsigned)s.BH()), dim3(kThreads), sm, st,
                   xmap, vmap, pmap, dmap, fmap, ws + L.wimg, ws + L.timg, ws + L.timg2, f(L.part), f(L.dtp), s.N,
                   padded_n(s), s.H, s.G, P, status);
   }
   // dW, dbias, dtau (and d z' into dzp) from the slot pass's partials.
   cudaError_t reduce(const float* tau, float* dzp, float* dW, float* db, float* dtau, int accumulate) const {
-    const int P = bwd_slot_splits(s);
+    const int P = bwd_slot_splits(s, dzp ? 1 : 2);
     return reduce_bwd(s0, P, f(L.part), s.G, dzp ? 2 * kD + 2 : kD + 2, tau, dzp, dW, db, dtau, f(L.dtp),
                       (int64_t)P * bwd_slot_blocks(s), accumulate, st);
   }
@@ -1214,7 +1228,7 @@ cudaError_t tc_coupling_bwd(const Shape& s0, const void* x, const void* f, const
                      c.f(L.sl_part), status, st));
   } else {
     FS_TRY(c.slot<0>(x, dout, nullptr));
-    FS_TRY(simt_reduce_dzp(s0, bwd_slot_splits(c.s), c.f(L.part), c.s.G, kD, dzp, st));
+    FS_TRY(simt_reduce_dzp(s0, bwd_slot_splits(c.s, 0), c.f(L.part), c.s.G, kD, dzp, st));
   }
   FS_TRY(mix_bwd(s0, M, z, dzp, dz, dM, st));
   FS_TRY(c.images_us(z, wsum, dz, L.timg2, both ? L.part : L.zimg));
