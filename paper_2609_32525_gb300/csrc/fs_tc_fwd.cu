@@ -63,7 +63,7 @@ using namespace tc;
 // Deslice: out_n = sum_g w_ng z'_g.
 // smem: [W img G*96][Z' img G*64][stages: x | point extra (TMA half, zero half)][barriers]
 // TMEM: S buffers [0, 384); P x Z' accumulators O_0 [384, 448), O_1 [448, 512), each
-// double-buffered by tile parity.  Block q (tile q / nb, slot block q % nb) uses S buffer
+// double-buffered by tile parity (MODE 3: 64 columns wide and single).  Block q (tile q / nb, slot block q % nb) uses S buffer
 // q % 3; a softmax warpgroup writes the bf16 weights of its 128 slots, packed in pairs,
 // into columns [0, 64) of the same buffer; warp 2 + j turns slots [64 j, 64 j + 64) of every
 // block into products (K-steps [4 j, 4 j + 4)) accumulated in O_j.
@@ -91,9 +91,14 @@ using namespace tc;
 //   MODE 3, both at once (the whole coupling's backward; z' in zimg, dU in zimg2): the
 //     weights are formed once.  delta_n = dO_n . R_n + fx_n . R2_n, dfx_n = R2_n.  z' and dU
 //     rows of 64 slots lie one after the other, so one MMA (N = 64) multiplies both; warp 3
-//     issues them all into one accumulator per tile parity.  The images take 416 B a slot, so
-//     at 512 slots one x stage is left; three are no faster (G = 256: 1037 us with three,
-//     1042 with one).  What bounds it is the softmax warps: without the w dS sums the whole
+//     issues them all, slot half j of every block into O_j as in the other modes: a chain of
+//     tensor-core sums drifts towards zero with its length, and one chain of all slots, with an
+//     accumulator per tile parity, left sum_g da_ng at 4.0e-6 of delta_n against 1.7e-6
+//     (G = 512) and dbias and dW 5% further off.  Two chains leave no columns for a second tile,
+//     so a tile is drained before the next one's products (whole backward at B = 2, N = 131,072,
+//     H = 8: G = 512 1727 -> 1740 us, 256 933 -> 936, 64 574 -> 575).  The images take 416 B a
+//     slot, so at 512 slots one x stage is left; three are no faster (G = 256: 1037 us with
+//     three, 1042 with one).  What bounds it is the softmax warps: without the w dS sums the whole
 //     backward took 7% less, without the epilogue's loads and stores 6%, without two of three
 //     products 2%.  Whole backward at B = 2, N = 131,072, H = 8, G = 512: 2165 us with a MODE
 //     1 and a MODE 2 pass, 1849 with this one.
@@ -276,9 +281,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       bool ok = mbar_wait_w(wz_full, 0, ab, status);
       Ring<kSBuf> sb;
       for (int i = 0; ok && i < wk.ntiles; i++) {
-        const int ob = i & 1;
-        const uint32_t tO = tmem + kO + (uint32_t)ob * 2 * kD;
-        if (i >= 2 && !(ok = mbar_wait_w(&o_free[ob], (uint32_t)(((i >> 1) - 1) & 1), ab, status))) break;
+        if (i >= 1 && !(ok = mbar_wait_w(&o_free[0], (uint32_t)((i - 1) & 1), ab, status))) break;
         uint32_t z = z0;
         for (int c = 0; ok && c < nch; c++, sb.next()) {
 #pragma unroll
@@ -286,10 +289,11 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
             if (!(ok = mbar_wait_w(&p_ready[2 * sb.i + j], sb.pass, ab, status))) break;
             tc_fence_after();
             const uint32_t tP = tmem + (uint32_t)sb.i * kGC + (uint32_t)j * 64;
+            const uint32_t tO = tmem + kO + (uint32_t)j * 2 * kD;
 #pragma unroll
             for (int kk = 0; kk < 4; kk++) {
               const uint32_t hi = tP + da_col(kk), lo = hi + 16;
-              mma_ts_w<kHi128>(tO, hi, z + kk * 2, idesc_pv, (c > 0 || j > 0 || kk > 0) ? 1u : 0u);
+              mma_ts_w<kHi128>(tO, hi, z + kk * 2, idesc_pv, (c > 0 || kk > 0) ? 1u : 0u);
               mma_ts_w<kHi128>(tO, lo, z + kk * 2, idesc_pv, 1u);
               mma_ts_w<kHi128>(tO, hi, z + (uint32_t)G * 8 + kk * 2, idesc_pv, 1u);
             }
@@ -410,7 +414,6 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
     };
     // MODE 3: delta_n = v_n . R2_n + v2_n . R_n and dfx_n = R2_n (R of z', R2 of t2).
     auto epilogue3 = [&](int t) -> bool {
-      const int ob = (int)(t & 1);
       const int64_t n = (wk.tile0 + t) * kTile + r;
       const int64_t row = ((b * N + n) * H + h) * kD;
       uint4 va[4], vb[4];
@@ -425,24 +428,37 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
       }
       if (!mbar_wait(&o_full[t % kOFull], (uint32_t)((t / kOFull) & 1), ab, status)) return false;
       tc_fence_after();
-      uint32_t o[32];
-      tmem_ld32(tmem + lane_addr + kO + (uint32_t)ob * 2 * kD, o);
-      tmem_wait_ld(o);
+      // Columns [col, col + 16) of the tile's accumulators, O_0 + O_1.
+      auto load_sum = [&](uint32_t col, uint32_t (&o)[16]) {
+        uint32_t o1[16];
+        tmem_ld16(tmem + lane_addr + kO + col, o);
+        tmem_ld16(tmem + lane_addr + kO + col + 2 * kD, o1);
+        tmem_wait_ld(o);
+        tmem_wait_ld(o1);
+#pragma unroll
+        for (int k = 0; k < 16; k++) o[k] = __float_as_uint(__uint_as_float(o[k]) + __uint_as_float(o1[k]));
+      };
+      uint32_t o[2][16];
       float da = 0.f, db = 0.f;
 #pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const uint32_t w[4] = {va[k].x, va[k].y, va[k].z, va[k].w};
+      for (int p = 0; p < 2; p++) {
+        load_sum(16 * p, o[p]);
 #pragma unroll
-        for (int e = 0; e < 4; e++) {
-          da = fmaf(__uint_as_float(w[e] << 16), __uint_as_float(o[8 * k + 2 * e]), da);
-          da = fmaf(__uint_as_float(w[e] & 0xFFFF0000u), __uint_as_float(o[8 * k + 2 * e + 1]), da);
+        for (int k = 0; k < 2; k++) {
+          const uint4 q = va[2 * p + k];
+          const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+          for (int e = 0; e < 4; e++) {
+            da = fmaf(__uint_as_float(w[e] << 16), __uint_as_float(o[p][8 * k + 2 * e]), da);
+            da = fmaf(__uint_as_float(w[e] & 0xFFFF0000u), __uint_as_float(o[p][8 * k + 2 * e + 1]), da);
+          }
         }
       }
-      tmem_ld32(tmem + lane_addr + kO + (uint32_t)ob * 2 * kD + kD, o);
-      tmem_wait_ld(o);
+      load_sum(kD, o[0]);
+      load_sum(kD + 16, o[1]);
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&o_free[ob]);
+      if (lane == 0) mbar_arrive(&o_free[0]);
       if (n < N) {
         uint4* dst = reinterpret_cast<uint4*>(out + row);
 #pragma unroll
@@ -455,7 +471,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
 #pragma unroll
           for (int e = 0; e < 4; e++) {
             const int c0 = 8 * k + 2 * e;
-            const float r0 = __uint_as_float(o[c0]), r1 = __uint_as_float(o[c0 + 1]);
+            const float r0 = __uint_as_float(o[c0 >> 4][c0 & 15]), r1 = __uint_as_float(o[c0 >> 4][(c0 & 15) + 1]);
             w[e] = pack_bf16(r0 + __uint_as_float(pw[e] << 16), r1 + __uint_as_float(pw[e] & 0xFFFF0000u));
             db = fmaf(__uint_as_float(wb[e] << 16), r0, db);
             db = fmaf(__uint_as_float(wb[e] & 0xFFFF0000u), r1, db);
@@ -465,12 +481,6 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
         delta[wk.bh * N + n] = accumulate ? delta[wk.bh * N + n] + (db + da) : db + da;
       }
       return true;
-    };
-    auto finish = [&](int t) -> bool {
-      if constexpr (MODE == 3)
-        return epilogue3(t);
-      else
-        return epilogue(t);
     };
     // kDs: this warpgroup's sum_g w dS_g for point r of its current tile.
     float wds_acc = 0.f;
@@ -510,11 +520,17 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
         __syncwarp();
         if (lane == 0) mbar_arrive(&p_ready[2 * bb + hf]);
       }
-      // The output of the previous tile is drained by the warpgroup that took the first
-      // block of this tile, when the last products of that tile have long finished.
-      if (c == 0 && i > 0 && !(ok = finish(i - 1))) break;
+      if constexpr (MODE == 3) {
+        // A tile's output is drained by the warpgroup that took its last block, at once, as the
+        // next tile's products wait for the accumulators.
+        if (c == nch - 1 && !(ok = epilogue3(i))) break;
+      } else {
+        // The output of the previous tile is drained by the warpgroup that took the first
+        // block of this tile, when the last products of that tile have long finished.
+        if (c == 0 && i > 0 && !(ok = epilogue(i - 1))) break;
+      }
     }
-    if (ok && total > 0 && total % kWGs == wg) finish(wk.ntiles - 1);
+    if (MODE != 3 && ok && total > 0 && total % kWGs == wg) epilogue(wk.ntiles - 1);
     if (ok) flush_wds();
   }
   tc_fence_before();

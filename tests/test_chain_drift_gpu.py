@@ -43,3 +43,24 @@ def test_deslice_bwd_long_ranges(lib, B, N, G):
         ref += torch.softmax(a, 1).T @ dout[0, n:n + 65536, h].double()
     e = float((c.d_tokens_mixed[0, h].double() - ref).norm() / ref.norm())
     assert e <= (1.3e-5 if G == 1024 else 6.5e-6) + 6e-6, e
+
+
+@pytest.mark.parametrize("G", [256, 512, 1024])
+def test_fused_backward_keeps_the_balance_of_da(lib, G):
+    """sum_g da_ng is 0 for every point, so sum_g dbias_hg is 0 but for the error of delta_n, which
+    has one sign; with dout = out, delta_n is |out_n|^2 (the slice's part sums to 0).  The fused
+    call forms delta from chains as long as the separate calls' (half of a range's slots each),
+    so its imbalance is theirs; chains twice as long would double it."""
+    B, N, H = 1, 65536, 4
+    x, fx, W, bias, tau, M, _ = _inputs(B, N, H, G, 3 + G)
+    fx = fx + 2
+    c = lib.Coupling(B, N, H, 32, G, torch.bfloat16, backward=True)
+    out = c.forward(x, fx, W, bias, tau, M).clone()
+    scale = (out.double() ** 2).sum((0, 1, 3)) / tau.double()
+    off = {}
+    for fused in (True, False):
+        g = c.backward(x, fx, W, bias, tau, M, out, fused=fused)
+        off[fused] = float((g["dbias"].double().sum(1) / scale).abs().mean())
+    torch.cuda.synchronize()
+    assert c.device_status() == lib.FS_OK
+    assert off[True] <= 1.4 * off[False], off
