@@ -32,6 +32,8 @@
  *      wsum                              : [B, H, G]      fp32
  *      lse                               : [B, H, N]      fp32, natural log
  *    Channel c of a point's C = H*d features is head c / d, lane c % d.
+ *  - A bias of -inf, or one that overflows to it in the scaling by 1/tau, masks its slot: weight 0
+ *    for every point, gradients 0.  Each head needs at least one slot that is not masked.
  *  - Every pointer must be 16-byte aligned.
  *  - `ws` is caller-owned scratch of at least fs_workspace_bytes(shape, op)
  *    bytes (16-byte aligned).  Its first word is a device status word that

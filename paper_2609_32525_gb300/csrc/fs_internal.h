@@ -10,6 +10,11 @@
 namespace fs {
 
 constexpr float kLog2e = 1.4426950408889634f;
+// The lowest scaled bias (base-2 units): a slot masked with -inf, or with a bias that overflows in
+// the scaling, gets this one, whose weight is exactly 0 and whose products with 0 stay 0 (with
+// -inf itself the low bf16 half of the bias and the temperature's terms da (a - lse) are NaN).
+// A NaN stays NaN.
+constexpr float kMaskedBias = -3e38f;
 constexpr float kLn2 = 0.6931471805599453f;
 
 // Status word codes written by kernels (same values as fs_status).

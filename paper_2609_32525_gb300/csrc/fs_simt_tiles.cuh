@@ -33,8 +33,8 @@
 //
 // Logits are a2 = x . (W log2e/tau) + beta log2e/tau, the temperature-scaled logit in
 // base-2 units, so w = exp2(a2 - lse2) with lse2 = lse log2e.  Slots past G get W = 0 and
-// beta = -1e30 and points past N lse2 = 1e30: their weights are exactly 0 and every sum
-// stays finite.
+// beta = kLowest and points past N lse2 = 1e30, and a masked slot's bias is finite (kMaskedBias):
+// their weights are exactly 0 and every sum stays finite.
 #pragma once
 
 #include "fs_launch.h"
@@ -48,7 +48,8 @@ namespace {
 
 constexpr int TP = kSimtTP;
 constexpr int LP = TP + 4;  // row length of the point and weight tiles
-constexpr float kFar = 1e30f;
+constexpr float kFar = 1e30f;        // lse2 of points past N
+constexpr float kLowest = -3.4e38f;  // base-2 logit of slots past G, below every masked slot's
 
 // Threads and register tiles: with d = 64 one block of 256 threads fills an SM's shared
 // memory, with smaller d two or more blocks of 128.
@@ -77,6 +78,7 @@ struct Tile {
 };
 
 __device__ __forceinline__ bool tau_ok(float t) { return t > 0.f && t < INFINITY; }
+__device__ __forceinline__ float masked_bias(float b) { return b < kMaskedBias ? kMaskedBias : b; }
 // The call's first launch writes the status word: one block looks at every temperature.
 __device__ __forceinline__ void write_status(bool reset, const float* tau, int H, uint32_t* status) {
   if (!reset || blockIdx.x + blockIdx.y + blockIdx.z != 0) return;
@@ -168,7 +170,7 @@ struct SlotW {
         dst[t / TG * (TG + 4) + t % TG] = v[i] * scale;
       }
     }
-    if (threadIdx.x < TG) sB[threadIdx.x] = g0 + (int)threadIdx.x < G ? bias * scale : -kFar;
+    if (threadIdx.x < TG) sB[threadIdx.x] = g0 + (int)threadIdx.x < G ? masked_bias(bias * scale) : kLowest;
   }
 };
 // Token rows [g0, g0 + TG) of t [G][D], to channel-major.
@@ -409,11 +411,10 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(3))
   xr.load(x, b, h, n0, N, H);
   wr.load(W, bias, h, G, 0);
   xr.store(sx);
-  // Running (max, sum) of the thread's slots; the maximum starts finite so that a thread
-  // whose slots are all masked (-inf) stays free of NaN.
+  // Running (max, sum) of the thread's slots.
   float mx[8], l[8];
 #pragma unroll
-  for (int i = 0; i < 8; i++) mx[i] = -kFar, l[i] = 0.f;
+  for (int i = 0; i < 8; i++) mx[i] = kLowest, l[i] = 0.f;
   for (int g0 = 0; g0 < G; g0 += TG) {
     __syncthreads();
     wr.store(sw, sB, G, g0, scale);
@@ -453,7 +454,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(3))
   }
   __syncthreads();
   for (int p = threadIdx.x; p < TP; p += NT) {
-    float M = -kFar, L = 0.f;
+    float M = kLowest, L = 0.f;
 #pragma unroll
     for (int c = 0; c < C::kWarps / 2; c++) M = fmaxf(M, red[c * TP + p].x);
 #pragma unroll

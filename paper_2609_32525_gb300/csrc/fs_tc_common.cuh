@@ -78,6 +78,7 @@ struct Prep {
 };
 
 __device__ __forceinline__ bool good_tau(float t) { return t > 0.f && t < INFINITY; }
+__device__ __forceinline__ float masked_bias(float b) { return b < kMaskedBias ? kMaskedBias : b; }
 // 8 floats -> 8 bf16 (hi) and the bf16 of the residuals (lo).
 __device__ __forceinline__ void split8(const float (&v)[8], uint4& hi, uint4& lo) {
   uint32_t h[4], l[4];
@@ -114,7 +115,7 @@ __device__ __forceinline__ void prep_w_piece(const Prep& a, int64_t i) {
     split8(v, *reinterpret_cast<uint4*>(base + off), *reinterpret_cast<uint4*>(base + (size_t)a.Gp * 96 + off));
     return;
   }
-  const float b2 = real ? a.bias[(int64_t)h * a.G + g] * scale : -1e30f;
+  const float b2 = real ? masked_bias(a.bias[(int64_t)h * a.G + g] * scale) : -1e30f;
   const uint32_t bp = pack_bf16(b2, 0.f) & 0xFFFFu;
   const float bhi = __uint_as_float(bp << 16);
   const uint32_t blo = pack_bf16(b2 - bhi, 0.f) & 0xFFFFu;
