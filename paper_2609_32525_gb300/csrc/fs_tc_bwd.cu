@@ -297,8 +297,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* pv_done = p_ready + 2 * Bufs::kL;
   uint64_t* dw_free = pv_done + Bufs::kL;
   uint64_t* acc_full = dw_free + Bufs::kD;
-  uint64_t* acc_done = acc_full + 1;  // [issuer]: products of each of its units complete
-  uint64_t* wt_ready = acc_done + 2;  // MODES 2, 3: the W' image is in TMEM
+  uint64_t* acc_done = acc_full + 1;  // [half][its units' parity]: a unit's products complete
+  uint64_t* wt_ready = acc_done + 4;  // MODES 2, 3: the W' image is in TMEM
   uint64_t* drain = wt_ready + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 3);
   Abort* ab = reinterpret_cast<Abort*>(tmem_slot + 1);
@@ -337,8 +337,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int i = 0; i < Bufs::kD; i++) mbar_init(&dw_free[i], 4);
     mbar_init(acc_full, 1);
-    mbar_init(&acc_done[0], 1);
-    mbar_init(&acc_done[1], 1);
+    for (int i = 0; i < 4; i++) mbar_init(&acc_done[i], 1);
     mbar_init(wt_ready, 4);
     for (int i = 0; i < 3; i++) mbar_init(&drain[i], 1);
     ab->flag = 0;
@@ -481,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       mma_commit_w(&pv_done[sb.i]);
-      if (kFl) mma_commit_w(&acc_done[j]);
+      if (kFl) mma_commit_w(&acc_done[acc_done_of(u)]);
       if (j == 1) {
         mma_commit_w(&st_empty[stg.i]);
         stg.next();
@@ -563,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_wait_st();
         if (hf == 0 && kFl && u >= 2 && slot_flush_at(u)) {
           // This warpgroup's units up to u - 2 have completed their products.
-          if (!(ok = mbar_wait(&acc_done[wg], (uint32_t)(((u - 2) >> 1) & 1), ab, status))) break;
+          if (!(ok = mbar_wait(&acc_done[acc_done_of(u - 2)], acc_done_phase(u - 2), ab, status))) break;
           tc_fence_after();
           add_acc();
         }

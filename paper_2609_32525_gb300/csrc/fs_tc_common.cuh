@@ -251,6 +251,15 @@ struct BlockPos {
   }
 };
 
+// Barriers on which the warpgroup that flushes an accumulator waits for its products: tile (or
+// unit) i goes into accumulator i & 1, and that one's tiles take two barriers in turn.  A parity
+// wait passes at once on a barrier two phases behind.  A warpgroup at tile i has seen logits that
+// were issued after the products of tile i - 4, so it knows the commits issued before those
+// products, tile i - 6's; with one barrier for all tiles it would have to know tile i - 4's own,
+// which stands behind the commit that let those logits go.
+__host__ __device__ constexpr int acc_done_of(int i) { return 2 * (i & 1) + ((i >> 1) & 1); }
+__host__ __device__ constexpr uint32_t acc_done_phase(int i) { return (uint32_t)(i >> 2) & 1u; }
+
 // CTA (split p of unit bh) processes a contiguous range of point tiles.
 __device__ __forceinline__ Work work_of(int64_t N, int splits, int p, int64_t bh) {
   Work w;

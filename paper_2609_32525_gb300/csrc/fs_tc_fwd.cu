@@ -803,8 +803,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* p_ready = s_full + kSBuf;   // [S buffer][half]
   uint64_t* pv_done = p_ready + 2 * kSBuf;
   uint64_t* acc_full = pv_done + kSBuf;
-  uint64_t* acc_done = acc_full + 1;  // [issuer]: products of each of its tiles complete
-  uint64_t* wt_ready = acc_done + 2;  // single-level products: the W' image is in TMEM
+  uint64_t* acc_done = acc_full + 1;  // [issuer][its tiles' parity]: a tile's products complete
+  uint64_t* wt_ready = acc_done + 4;  // single-level products: the W' image is in TMEM
   uint64_t* drain = wt_ready + 1;  // one per issuing warp
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 3);
   Abort* ab = reinterpret_cast<Abort*>(tmem_slot + 1);
@@ -834,8 +834,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&pv_done[i], 1);
     }
     mbar_init(acc_full, 2);
-    mbar_init(&acc_done[0], 1);
-    mbar_init(&acc_done[1], 1);
+    for (int i = 0; i < 4; i++) mbar_init(&acc_done[i], 1);
     mbar_init(wt_ready, 4);
     for (int i = 0; i < 3; i++) mbar_init(&drain[i], 1);
     ab->flag = 0;
@@ -964,7 +963,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         mma_commit_w(&pv_done[sb.i]);
         mma_commit_w(&st_empty[st.i]);
-        mma_commit_w(&acc_done[j]);
+        mma_commit_w(&acc_done[acc_done_of(i)]);
         st.next(), st.next();
         sb.next(), sb.next();
       }
@@ -1024,9 +1023,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           weights_half(tS + (uint32_t)hf * 64, tS + (uint32_t)hf * 32);
         tmem_wait_st();
         if (hf == 0 && i >= 2 && slice_flush_at<split>(i)) {
-          // The products of this warpgroup's tiles up to i - 2 are complete (acc_done
-          // cannot move past that phase before this warpgroup hands over tile i).
-          if (!(ok = mbar_wait(&acc_done[wg], (uint32_t)(((i - 2) >> 1) & 1), ab, status))) break;
+          // The products of this warpgroup's tiles up to i - 2 are complete.
+          if (!(ok = mbar_wait(&acc_done[acc_done_of(i - 2)], acc_done_phase(i - 2), ab, status))) break;
           tc_fence_after();
           add_acc();
         }
