@@ -51,11 +51,11 @@ constexpr int LP = TP + 4;  // row length of the point and weight tiles
 constexpr float kFar = 1e30f;        // lse2 of points past N
 constexpr float kLowest = -3.4e38f;  // base-2 logit of slots past G, below every masked slot's
 
-// Threads and register tiles: with d = 64 one block of 256 threads fills an SM's shared
-// memory, with smaller d two or more blocks of 128.
+// Threads and register tiles: with d = 64 and 64 slots one block of 256 threads fills an SM's
+// shared memory, else there are two or more blocks of 128.
 template <int D, int TG>
 struct Tile {
-  static constexpr int kThreads = D == 64 ? 256 : 128;
+  static constexpr int kThreads = D == 64 && TG == 64 ? 256 : 128;
   static constexpr int kWarps = kThreads / 32;
   static constexpr int LG = TG + 4;  // row length of the slot tiles
   // pair_products: two rows of warps over the points, 8 points per thread
@@ -68,12 +68,14 @@ struct Tile {
   // slot_products: warps over two halves of the points x channels
   static constexpr int kSlM = TG / 8;
   static constexpr int kSlN = D / (2 * kWarps);
-  static_assert((kPairN == 4 || kPairN == 8) && (kPtM == 4 || kPtM == 8) && kSlN >= 1, "register tiles");
+  static_assert((kPairN == 4 || kPairN == 8) && (kPtM == 4 || kPtM == 8 || kPtM == 16) && kSlN >= 1, "register tiles");
 
   static constexpr size_t kPointTile = (size_t)D * LP;
   static constexpr size_t kSlotTile = (size_t)D * LG;
   static constexpr size_t kWeightTile = (size_t)TG * LP;
-  static_assert(kWeightTile >= (size_t)TP * (D + 1), "write_rows fits in the weight tile");
+  // write_rows goes through the weight tile where it is large enough, else through the x tile.
+  static constexpr bool kRowsInWeights = kWeightTile >= (size_t)TP * (D + 1);
+  static_assert(kRowsInWeights || kPointTile >= (size_t)TP * (D + 1), "write_rows fits");
   static constexpr size_t kVectors = 2 * TP + 2 * TG + kWarps * TP;  // lse2, delta | beta, dS | sums of a pass
 };
 
@@ -232,22 +234,27 @@ __device__ __forceinline__ void pair_products(float (&acc)[8][N], const float* p
 }
 // The thread's points as above with M points (M / 4 runs, 32 apart), channels
 // 16 wc + n + 4 j.
+// Over the tile's first `left` slots, rounded up to eight (the rest have weight 0).
 template <int TG, int M, int N>
-__device__ __forceinline__ void point_products(float (&acc)[M][N], const float* wts, const float* slots) {
-#pragma unroll 2
-  for (int g = 0; g < TG; g += 4) {
-    float b[N][4];
+__device__ __forceinline__ void point_products(float (&acc)[M][N], const float* wts, const float* slots, int left) {
+  const int end = min(TG, left);
+#pragma unroll 1
+  for (int g0 = 0; g0 < end; g0 += 8) {
 #pragma unroll
-    for (int j = 0; j < N; j++) ld4(b[j], slots + 4 * j * (TG + 4) + g);
+    for (int g = g0; g < g0 + 8; g += 4) {
+      float b[N][4];
 #pragma unroll
-    for (int e = 0; e < 4; e++) {
-      float a[M];
+      for (int j = 0; j < N; j++) ld4(b[j], slots + 4 * j * (TG + 4) + g);
 #pragma unroll
-      for (int q = 0; q < M / 4; q++) ld4(a + 4 * q, wts + (g + e) * LP + 32 * q);
+      for (int e = 0; e < 4; e++) {
+        float a[M];
 #pragma unroll
-      for (int i = 0; i < M; i++)
+        for (int q = 0; q < M / 4; q++) ld4(a + 4 * q, wts + (g + e) * LP + 32 * q);
 #pragma unroll
-        for (int j = 0; j < N; j++) acc[i][j] = fmaf(a[i], b[j][e], acc[i][j]);
+        for (int i = 0; i < M; i++)
+#pragma unroll
+          for (int j = 0; j < N; j++) acc[i][j] = fmaf(a[i], b[j][e], acc[i][j]);
+      }
     }
   }
 }
@@ -295,6 +302,10 @@ struct Place {
   // point i (of 8) and slot j (of kPairN) of the thread, counted in the tile
   __device__ __forceinline__ int point(int i) const { return p1 + (i >> 2) * 32 + (i & 3); }
   __device__ __forceinline__ int slot(int j) const { return g1 + (j >> 2) * 16 + (j & 3); }
+  // Whether the warp's slots of a tile with `left` slots hold any: the pair_products of a warp
+  // whose slots are all past G are left out (a tile of 64 and one of 1 slot take G = 65: deslice
+  // at N = 131,072, H = 8, d = 16, fp32 272 us with them and all of point_products, 229 without).
+  __device__ __forceinline__ bool live(int left) const { return c1 * 4 * C::kPairN < left; }
 };
 
 // The thread's 8 x N weights to the tile [slot][point].
@@ -382,12 +393,20 @@ __host__ __device__ constexpr size_t tile_bytes(int points, int slots, int weigh
   using C = Tile<D, TG>;
   return (points * C::kPointTile + slots * C::kSlotTile + weights * C::kWeightTile + C::kVectors) * sizeof(float);
 }
-template <int D>
-constexpr int resident(int blocks) { return D == 64 ? 1 : blocks; }
+template <int D, int TG>
+constexpr int resident(int blocks) { return Tile<D, TG>::kThreads == 256 ? 1 : blocks; }
+// The statistics and the deslice do little per tile at d = 16 and with the narrow tile: more
+// resident blocks hide its barriers and reads (deslice at N = 131,072, H = 8, fp32: d = 16,
+// G = 65 229 us with two blocks, 194 with three; d = 16, G = 16 83 with three, 73 with four;
+// d = 32, G = 8 154 with two, 130 with three).
+template <int D, int TG>
+constexpr int resident_fwd(int blocks) {
+  return D == 16 ? (TG == 32 ? 4 : 3) : D == 32 && TG == 32 ? 3 : resident<D, TG>(blocks);
+}
 
 // ---- statistics --------------------------------------------------------------------------------
 template <int D, int TG, typename T>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(3))
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident_fwd<D, TG>(3))
     k_tile_stats(const T* __restrict__ x, const float* __restrict__ W, const float* __restrict__ bias,
                  const float* __restrict__ tau, float* __restrict__ lse, int64_t N, int H, int G, int reset,
                  uint32_t* status) {
@@ -427,6 +446,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(3))
 #pragma unroll
       for (int i = 0; i < 8; i++) a[i][j] = bj;
     }
+    if (!pl.live(G - g0)) continue;
     pair_products<D, NJ, C::LG>(a, sx + pl.p1, sw + pl.g1);
 #pragma unroll
     for (int i = 0; i < 8; i++) {
@@ -463,10 +483,11 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(3))
   }
 }
 
-// The thread's log2-weights a2 - lse2 of the staged tile.
+// The thread's log2-weights a2 - lse2 of the staged tile of `left` slots.
 template <int D, int TG>
 __device__ __forceinline__ void log_weights(float (&a)[8][Tile<D, TG>::kPairN], const Place<D, TG>& pl,
-                                            const float* sx, const float* sw, const float* sB, const float* sl) {
+                                            const float* sx, const float* sw, const float* sB, const float* sl,
+                                            int left) {
   using C = Tile<D, TG>;
 #pragma unroll
   for (int j = 0; j < C::kPairN; j++) {
@@ -474,7 +495,7 @@ __device__ __forceinline__ void log_weights(float (&a)[8][Tile<D, TG>::kPairN], 
 #pragma unroll
     for (int i = 0; i < 8; i++) a[i][j] = bj;
   }
-  pair_products<D, C::kPairN, C::LG>(a, sx + pl.p1, sw + pl.g1);
+  if (pl.live(left)) pair_products<D, C::kPairN, C::LG>(a, sx + pl.p1, sw + pl.g1);
 #pragma unroll
   for (int i = 0; i < 8; i++) {
     const float l2 = sl[pl.point(i)];
@@ -486,7 +507,7 @@ __device__ __forceinline__ void log_weights(float (&a)[8][Tile<D, TG>::kPairN], 
 // ---- slice: slot-owned partials over a split of the points ---------------------------------------
 // grid (slot tiles, B*H, P).  part[p][bh][g][0..D] = (U, S).
 template <int D, int TG, typename T>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D, TG>(2))
     k_tile_slice(const T* __restrict__ x, const T* __restrict__ f, const float* __restrict__ W,
                  const float* __restrict__ bias, const float* __restrict__ tau, const float* __restrict__ lse,
                  float* __restrict__ part, int64_t N, int H, int G, int P, int reset, uint32_t* status) {
@@ -535,7 +556,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     store_lse2(sl, lr, t * TP, N);
     __syncthreads();
     float w[8][NJ];
-    log_weights<D, TG>(w, pl, sx, sw, sB, sl);
+    log_weights<D, TG>(w, pl, sx, sw, sB, sl, G - g0);
 #pragma unroll
     for (int j = 0; j < NJ; j++) {
       float s = 0.f;
@@ -573,7 +594,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
 
 // ---- deslice: point-owned ------------------------------------------------------------------------
 template <int D, int TG, typename T>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident_fwd<D, TG>(2))
     k_tile_deslice(const T* __restrict__ x, const float* __restrict__ W, const float* __restrict__ bias,
                    const float* __restrict__ tau, const float* __restrict__ zp, const float* __restrict__ lse,
                    T* __restrict__ out, int64_t N, int H, int G, int reset, uint32_t* status) {
@@ -618,7 +639,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     zr.store(sz);
     __syncthreads();
     float w[8][NJ];
-    log_weights<D, TG>(w, pl, sx, sw, sB, sl);
+    log_weights<D, TG>(w, pl, sx, sw, sB, sl, G - g0);
 #pragma unroll
     for (int i = 0; i < 8; i++)
 #pragma unroll
@@ -626,9 +647,9 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     store_weights<D, TG>(wt, pl, w);
     __syncthreads();
     if (g0 + TG < G) load(g0 + TG);
-    point_products<TG>(acc, wt + pl.p2, sz + pl.c2 * C::LG);
+    point_products<TG>(acc, wt + pl.p2, sz + pl.c2 * C::LG, G - g0);
   }
-  write_rows<D, TG, T>(acc, 1.f, false, wt, pl, out, b, h, n0, N, H);
+  write_rows<D, TG, T>(acc, 1.f, false, C::kRowsInWeights ? wt : sx, pl, out, b, h, n0, N, H);
 }
 
 // ---- backward, point-owned -----------------------------------------------------------------------
@@ -644,7 +665,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
 // logits centred on lse (exact, since sum_g da_g = 0) they carry no large cancelling parts
 // (App. G.2).
 template <int D, int TG, typename T, int MODE>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D, TG>(2))
     k_tile_bwd_point(const T* __restrict__ x, const T* __restrict__ dO, const T* __restrict__ fx,
                      const float* __restrict__ W, const float* __restrict__ bias, const float* __restrict__ tau,
                      const float* __restrict__ zp, const float* __restrict__ dUS, const float* __restrict__ lse,
@@ -716,7 +737,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     for (int g0 = 0; g0 < G; g0 += TG) {
       stage(g0);
       float w[8][NJ];
-      log_weights<D, TG>(w, pl, sx, sw, sB, sl);
+      log_weights<D, TG>(w, pl, sx, sw, sB, sl, G - g0);
 #pragma unroll
       for (int j = 0; j < NJ; j++) {
         const float s = kS ? sS[pl.slot(j)] : 0.f;
@@ -729,8 +750,8 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
       store_weights<D, TG>(wt, pl, w);
       __syncthreads();
       load(g0 + TG < G ? g0 + TG : 0);  // (the second sweep's first tile at last)
-      if (kD) point_products<TG>(R, wt + pl.p2, sz + pl.c2 * C::LG);
-      if (kS) point_products<TG>(F, wt + pl.p2, su + pl.c2 * C::LG);
+      if (kD) point_products<TG>(R, wt + pl.p2, sz + pl.c2 * C::LG, G - g0);
+      if (kS) point_products<TG>(F, wt + pl.p2, su + pl.c2 * C::LG, G - g0);
     }
     // delta: the dot products of the thread's channels, over the run, then the warp
     // columns in order; then the columns' sums of w dS.
@@ -782,15 +803,17 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
   for (int g0 = 0; g0 < G; g0 += TG) {
     stage(g0);
     float a[8][NJ], dw[8][NJ];
-    log_weights<D, TG>(a, pl, sx, sw, sB, sl);
+    log_weights<D, TG>(a, pl, sx, sw, sB, sl, G - g0);
 #pragma unroll
     for (int j = 0; j < NJ; j++) {
       const float s = kS ? sS[pl.slot(j)] : 0.f;
 #pragma unroll
       for (int i = 0; i < 8; i++) dw[i][j] = s;
     }
-    if (kD) pair_products<D, NJ, C::LG>(dw, sd + pl.p1, sz + pl.g1);
-    if (kS) pair_products<D, NJ, C::LG>(dw, sf + pl.p1, su + pl.g1);
+    if (pl.live(G - g0)) {
+      if (kD) pair_products<D, NJ, C::LG>(dw, sd + pl.p1, sz + pl.g1);
+      if (kS) pair_products<D, NJ, C::LG>(dw, sf + pl.p1, su + pl.g1);
+    }
 #pragma unroll
     for (int i = 0; i < 8; i++) {
       const float dl = sdl[pl.point(i)];
@@ -804,7 +827,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     store_weights<D, TG>(wt, pl, dw);
     __syncthreads();
     if (g0 + TG < G) load(g0 + TG);
-    point_products<TG>(acc, wt + pl.p2, sw + pl.c2 * C::LG);
+    point_products<TG>(acc, wt + pl.p2, sw + pl.c2 * C::LG, G - g0);
   }
   // acc = sum_g da_g W[:,g] log2e/tau; dx = acc ln2.
   write_rows<D, TG, T>(acc, kLn2, accumulate != 0, wt, pl, dx, b, h, n0, N, H);
@@ -823,7 +846,7 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
 //   dWa_g = sum_n da x_n,  dba_g = sum_n da;  MODE 0 also dz'_g = sum_n w dO_n.
 // part[p][bh][g] = (MODE 0: dz' (D)), dWa (D), dba, 0   (un-scaled by 1/tau).
 template <int D, int TG, typename T, int MODE>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D, TG>(2))
     k_tile_bwd_slot(const T* __restrict__ x, const T* __restrict__ dO, const T* __restrict__ fx,
                     const float* __restrict__ W, const float* __restrict__ bias, const float* __restrict__ tau,
                     const float* __restrict__ zp, const float* __restrict__ dUS, const float* __restrict__ lse,
@@ -885,15 +908,17 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D>(2))
     if (threadIdx.x < TP) sdl[threadIdx.x] = er;
     __syncthreads();
     float a[8][NJ], dw[8][NJ];
-    log_weights<D, TG>(a, pl, sx, sw, sB, sl);
+    log_weights<D, TG>(a, pl, sx, sw, sB, sl, G - g0);
 #pragma unroll
     for (int j = 0; j < NJ; j++) {
       const float s = kS ? sS[pl.slot(j)] : 0.f;
 #pragma unroll
       for (int i = 0; i < 8; i++) dw[i][j] = s;
     }
-    if (kD) pair_products<D, NJ, C::LG>(dw, sd + pl.p1, sz + pl.g1);
-    if (kS) pair_products<D, NJ, C::LG>(dw, sf + pl.p1, su + pl.g1);
+    if (pl.live(G - g0)) {
+      if (kD) pair_products<D, NJ, C::LG>(dw, sd + pl.p1, sz + pl.g1);
+      if (kS) pair_products<D, NJ, C::LG>(dw, sf + pl.p1, su + pl.g1);
+    }
 #pragma unroll
     for (int i = 0; i < 8; i++) {
       const float dl = sdl[pl.point(i)];
@@ -957,8 +982,10 @@ dim3 slot_grid(const Shape& s, int P) {
   return dim3((unsigned)((s.G + TG - 1) / TG), (unsigned)s.BH(), (unsigned)P);
 }
 
-// Calls fn with (d, slots per tile) of the shape as compile-time constants.
-template <typename Fn>
+// Calls fn with (d, slots per tile) of the shape as compile-time constants.  kNarrow64: d = 64 has
+// the narrow tile too (the statistics and the deslice, whose sweeps over the slots are all of
+// their work: N = 131,072, H = 8, G = 16, fp32, 348 and 576 us with the wide tile, 158 and 288 with the narrow one).
+template <bool kNarrow64 = false, typename Fn>
 cudaError_t with_tile(const Shape& s, Fn fn) {
   const bool narrow = simt_tile_slots(s) == 32;
 #define FS_TILE(D_)                                                                                    \
@@ -967,7 +994,10 @@ cudaError_t with_tile(const Shape& s, Fn fn) {
   switch (s.d) {
     case 16: FS_TILE(16);
     case 32: FS_TILE(32);
-    case 64: return fn(std::integral_constant<int, 64>{}, std::integral_constant<int, 64>{});
+    case 64:
+      if constexpr (kNarrow64)
+        if (s.G <= 32) return fn(std::integral_constant<int, 64>{}, std::integral_constant<int, 32>{});
+      return fn(std::integral_constant<int, 64>{}, std::integral_constant<int, 64>{});
     default: return cudaErrorInvalidValue;
   }
 #undef FS_TILE
@@ -978,7 +1008,7 @@ cudaError_t with_tile(const Shape& s, Fn fn) {
 template <typename T>
 cudaError_t SimtTiles<T>::stats(const Shape& s, const T* x, const float* W, const float* bias, const float* tau,
                                 float* lse, bool reset, uint32_t* status, cudaStream_t st) {
-  return with_tile(s, [&](auto d, auto tg) {
+  return with_tile<true>(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value;
     constexpr size_t sm = tile_bytes<D, TG>(1, 1, 0);
     const auto k = k_tile_stats<D, TG, T>;
@@ -1006,7 +1036,7 @@ template <typename T>
 cudaError_t SimtTiles<T>::deslice(const Shape& s, const T* x, const float* W, const float* bias, const float* tau,
                                   const float* zp, const float* lse, T* out, bool reset, uint32_t* status,
                                   cudaStream_t st) {
-  return with_tile(s, [&](auto d, auto tg) {
+  return with_tile<true>(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value;
     constexpr size_t sm = tile_bytes<D, TG>(1, 2, 1);
     const auto k = k_tile_deslice<D, TG, T>;
