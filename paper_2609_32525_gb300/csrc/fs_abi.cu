@@ -296,10 +296,8 @@ int fs_backward_launch_count(const fs_shape* s, int lse_given) {
 int fs_coupling_bwd_launch_count(const fs_shape* s, int lse_given) {
   if (!valid_shape(s) || !supported_shape(s)) return -1;
   const Shape sh = to_shape(s);
-  if (!tc_backward_supported(sh)) return backward_stats_launches(sh, lse_given) + simt_coupling_bwd_launch_count();
-  const bool tc = tc_forward_supported(sh);
-  const int stats = (lse_given && sh.dot == FS_DOT_BF16X2) ? 0 : (tc ? 2 : 1);  // the statistics once
-  return stats + tc_coupling_bwd_launch_count(sh);
+  return backward_stats_launches(sh, lse_given) /* once */ +
+         (tc_backward_supported(sh) ? tc_coupling_bwd_launch_count(sh) : simt_coupling_bwd_launch_count());
 }
 
 fs_status fs_slice_fwd(const fs_shape* s, const void* x_mid, const void* fx, const float* W_slice,
