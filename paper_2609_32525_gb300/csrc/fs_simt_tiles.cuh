@@ -395,18 +395,19 @@ __host__ __device__ constexpr size_t tile_bytes(int points, int slots, int weigh
 }
 template <int D, int TG>
 constexpr int resident(int blocks) { return Tile<D, TG>::kThreads == 256 ? 1 : blocks; }
-// The statistics and the deslice do little per tile at d = 16 and with the narrow tile: more
-// resident blocks hide its barriers and reads (deslice at N = 131,072, H = 8, fp32: d = 16,
-// G = 65 229 us with two blocks, 194 with three; d = 16, G = 16 83 with three, 73 with four;
-// d = 32, G = 8 154 with two, 130 with three).
+// The statistics and the deslice do little per tile at d = 16 and with the narrow tile: on grids of
+// many waves more resident blocks hide its barriers and reads (deslice at N = 131,072, H = 8, fp32:
+// d = 16, G = 65 229 us with two blocks, 194 with three; d = 16, G = 16 83 with three, 73 with
+// four; d = 32, G = 8 154 with two, 130 with three).  Below three blocks an SM the extra ones only
+// pile up on some SMs (N = 4,096, G = 32: d = 32 7.4 us with two, 10.0 with three).
 template <int D, int TG>
-constexpr int resident_fwd(int blocks) {
+constexpr int resident_many(int blocks) {
   return D == 16 ? (TG == 32 ? 4 : 3) : D == 32 && TG == 32 ? 3 : resident<D, TG>(blocks);
 }
 
 // ---- statistics --------------------------------------------------------------------------------
-template <int D, int TG, typename T>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident_fwd<D, TG>(3))
+template <int D, int TG, typename T, int kBlocks>
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, kBlocks)
     k_tile_stats(const T* __restrict__ x, const float* __restrict__ W, const float* __restrict__ bias,
                  const float* __restrict__ tau, float* __restrict__ lse, int64_t N, int H, int G, int reset,
                  uint32_t* status) {
@@ -593,8 +594,8 @@ __global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident<D, TG>(2))
 }
 
 // ---- deslice: point-owned ------------------------------------------------------------------------
-template <int D, int TG, typename T>
-__global__ void __launch_bounds__(Tile<D, TG>::kThreads, resident_fwd<D, TG>(2))
+template <int D, int TG, typename T, int kBlocks>
+__global__ void __launch_bounds__(Tile<D, TG>::kThreads, kBlocks)
     k_tile_deslice(const T* __restrict__ x, const float* __restrict__ W, const float* __restrict__ bias,
                    const float* __restrict__ tau, const float* __restrict__ zp, const float* __restrict__ lse,
                    T* __restrict__ out, int64_t N, int H, int G, int reset, uint32_t* status) {
@@ -976,6 +977,7 @@ template <typename K>
 cudaError_t allow_smem(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
+inline bool many_waves(const Shape& s) { return simt_point_blocks(s) * s.BH() > 3 * num_sms(); }
 inline dim3 point_grid(const Shape& s) { return dim3((unsigned)((s.N + TP - 1) / TP), (unsigned)s.BH()); }
 template <int TG>
 dim3 slot_grid(const Shape& s, int P) {
@@ -1011,7 +1013,7 @@ cudaError_t SimtTiles<T>::stats(const Shape& s, const T* x, const float* W, cons
   return with_tile<true>(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value;
     constexpr size_t sm = tile_bytes<D, TG>(1, 1, 0);
-    const auto k = k_tile_stats<D, TG, T>;
+    const auto k = many_waves(s) ? k_tile_stats<D, TG, T, resident_many<D, TG>(3)> : k_tile_stats<D, TG, T, resident<D, TG>(3)>;
     if (cudaError_t e = allow_smem(k, sm)) return e;
     return launch(k, point_grid(s), dim3(Tile<D, TG>::kThreads), sm, st, x, W, bias, tau, lse, s.N, s.H, s.G, reset,
                   status);
@@ -1039,7 +1041,8 @@ cudaError_t SimtTiles<T>::deslice(const Shape& s, const T* x, const float* W, co
   return with_tile<true>(s, [&](auto d, auto tg) {
     constexpr int D = decltype(d)::value, TG = decltype(tg)::value;
     constexpr size_t sm = tile_bytes<D, TG>(1, 2, 1);
-    const auto k = k_tile_deslice<D, TG, T>;
+    const auto k =
+        many_waves(s) ? k_tile_deslice<D, TG, T, resident_many<D, TG>(2)> : k_tile_deslice<D, TG, T, resident<D, TG>(2)>;
     if (cudaError_t e = allow_smem(k, sm)) return e;
     return launch(k, point_grid(s), dim3(Tile<D, TG>::kThreads), sm, st, x, W, bias, tau, zp, lse, out, s.N, s.H, s.G,
                   reset, status);
