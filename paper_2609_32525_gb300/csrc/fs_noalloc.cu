@@ -90,8 +90,8 @@ extern "C" fs_status fs_slice_fwd_noalloc(const fs_shape* s, const void* x_mid, 
   void* ws = nullptr;
   if (fs_status e = scratch_address(&ws)) return e;
   if (scratch) *scratch = ws;
-  // fs_slice_fwd clears the status word at the start of ws (the only part of
-  // the workspace that must start at zero) before its first kernel.
+  // The first kernel of fs_slice_fwd writes the status word at the start of ws; no part of the
+  // workspace has to start at zero.
   return fs_slice_fwd(s, x_mid, fx, W_slice, bias, tau, tokens, wsum, lse, finalize, ws, FS_NOALLOC_SCRATCH_BYTES,
                       stream);
 }

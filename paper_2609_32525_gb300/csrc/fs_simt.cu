@@ -465,6 +465,8 @@ cudaError_t simt_reduce_bwd(const Shape& s, int P, const float* part, int Gs, in
   return launch(k_reduce_dtau, dim3(s.H), dim3(256), 0, st, dt_part, s.B, s.H, nblk, tau, dtau, accumulate);
 }
 
+// The one-launch forms of the reductions and of the mix backward serve the tensor-core calls, whose
+// chains of launches they shorten; the SIMT calls and fs_mix_bwd still launch the parts one by one.
 cudaError_t reduce_bwd(const Shape& s, int P, const float* part, int Gs, int PS, const float* tau, float* dzp,
                        float* dW, float* db, float* dtau, const float* dt_part, int64_t nblk, int accumulate,
                        cudaStream_t st) {

@@ -87,8 +87,8 @@ __global__ void __launch_bounds__(256) k_prep_us(const float* __restrict__ z, co
 }
 
 // delta's point-extra rows [1, 1, -delta in three bf16 parts, 0, 0, 0] into dpx [BH, Np, 8];
-// delta_n = delta[bh][n] (+ delta2[bh][n] when given, + wds[0][bh][n] + wds[1][bh][n]
-// when wds is given).
+// delta_n = delta[bh][n] (+ delta2[bh][n] when given, + the nwds (two or three) partials
+// wds[.][bh][n] when wds is given).
 __global__ void k_prep_dpx(const float* __restrict__ delta, const float* __restrict__ delta2,
                            const float* __restrict__ wds, int nwds, uint4* __restrict__ dpx, int64_t BH, int64_t N,
                            int64_t Np) {

@@ -18,12 +18,12 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 384;
+constexpr int kThreads = 384;     // kernels with two softmax warpgroups
 constexpr int kTile = 128;        // points per tile
 constexpr int kGC = 128;          // slots per logits block
 constexpr int kD = 32;            // head width of the tensor-core path
-constexpr int kSoftmaxWarp0 = 4;  // warps 4..11: two softmax warpgroups
-constexpr int kStages = 3;        // x-tile pipeline depth (stats / deslice)
+constexpr int kSoftmaxWarp0 = 4;  // warps 4 and up: two to four softmax warpgroups
+constexpr int kStages = 3;        // x-tile pipeline depth of the deslice
 constexpr int kSliceStages = 8;   // slice pipeline depth (it streams x, F and px for every 128 slots)
 constexpr int kSBuf = 3;          // S buffers (logits run up to two blocks ahead)
 constexpr uint32_t kXBytes = kTile * 64;   // 128 points x 32 bf16

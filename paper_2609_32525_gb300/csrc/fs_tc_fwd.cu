@@ -41,7 +41,7 @@
 // CTA: warp 0 TMA producer, warps 1..3 MMA issuers, warps 4 and up softmax warpgroups
 // (two to four) that take blocks in turn (so they run out of phase);
 // a thread owns one TMEM lane (tcgen05.ld/st 32x32b).  Every wait is bounded
-// (2 s): a wait that gives up writes FS_ERR_TIMEOUT to the status word, the CTA
+// (2 s and 2,000 polls): a wait that gives up writes FS_ERR_TIMEOUT to the status word, the CTA
 // drains its copies and MMAs, frees TMEM and exits.
 //
 // Shared-memory operand layouts (all bases 1024-byte aligned):
@@ -114,7 +114,7 @@ constexpr uint32_t kDStage = kXBytes + 2 * kPxBytes;  // x tile, point extra (bo
 
 // X3 (fp32 inputs, MODE 0 with PS): each stage also holds x's residual tile
 // (xrmap), the logits add x_r W'_hi, and out is fp32.
-template <int MODE, bool PS>
+template <int MODE>
 constexpr bool desl_wg3() { return MODE != 2; }
 constexpr int kDesl3Threads = 512;
 // Barriers of completed tiles.  With three warpgroups the one that drains tile t has not
@@ -123,7 +123,7 @@ constexpr int kDesl3Threads = 512;
 // blocks back, so the products three blocks before that: tile t - 5) covers tile t - 8.
 constexpr int kOFull = 8;
 template <int MODE, bool PS, bool X3 = false>
-__global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThreads, 1)
+__global__ void __launch_bounds__(desl_wg3<MODE>() ? kDesl3Threads : kThreads, 1)
     k_deslice(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap pmap,
               const __grid_constant__ CUtensorMap xrmap,
               const uint8_t* __restrict__ wimg, const uint8_t* __restrict__ zimg, const uint8_t* __restrict__ zimg2,
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(desl_wg3<MODE, PS>() ? kDesl3Threads : kThread
   uint64_t* x_full = bars + 1;
   uint64_t* x_empty = x_full + kStages;
   uint64_t* s_full = x_empty + kStages;
-  constexpr bool kWG3 = desl_wg3<MODE, PS>();
+  constexpr bool kWG3 = desl_wg3<MODE>();
   uint64_t* p_ready = s_full + kSBuf;  // [S buffer][half]
   uint64_t* pv_done = p_ready + 2 * kSBuf;
   uint64_t* o_full = pv_done + kSBuf;
